@@ -144,7 +144,6 @@ __global__ void __launch_bounds__(kGemmThreads, 1) dst_gemm_kernel(const GemmDst
   const int KB = a.ktiles;
   const unsigned polls = a.polls ? a.polls : kWaitPolls;
   const int ntile_all = a.m * a.mtiles * a.ntiles;
-  if (a.gate != nullptr && *a.gate == 0) return;  // nothing selected: before any set-up
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < kStages; ++s) {
@@ -291,6 +290,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) dst_gemm_kernel(const GemmDst
         const float *pog = nullptr;
         float *png = nullptr, *xg = nullptr;
         float beta = 0.f, alpha = 0.f;
+        bool xnew = false;  // x = alpha p_old (see RhsState::xbase)
         if (pupd) {
           const bool odd = a.st[m].iters & 1;
           pog = odd ? a.pb : a.pa;
@@ -302,6 +302,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) dst_gemm_kernel(const GemmDst
             xg = a.x;
             xr = a.x + roff;
             alpha = (float)a.st[m].alpha;
+            xnew = a.st[m].iters == a.st[m].xbase;
           }
         }
         const unsigned tP = tmem + ((unsigned)(q * 32) << 16) + (unsigned)b * kTileCols;
@@ -387,7 +388,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) dst_gemm_kernel(const GemmDst
                     const int r = h + j;
                     const bool ok = colok && row0 + r < a.nr;
                     po[j] = ok ? __ldg(pog + cbase + (size_t)r * a.pitch) : 0.f;
-                    xv[j] = (ok && xg) ? xg[cbase + (size_t)r * a.pitch] : 0.f;
+                    xv[j] = (ok && xg && !xnew) ? xg[cbase + (size_t)r * a.pitch] : 0.f;
                   }
 #pragma unroll
                   for (int j = 0; j < 16; ++j) {
@@ -496,7 +497,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) dst_gemm_kernel(const GemmDst
       __syncwarp();
       if (lane == 0) mbar_arrive(&tempty_bar[b]);
       if (a.partial) {
-        const double sw = warp_sum((double)acc);
+        const double sw = warp_sum_of(acc);
         if (lane == 0) red[ew] = sw;
         asm volatile("bar.sync 1, %0;" ::"r"(32 * kEpiWarps) : "memory");
         if (ew == 0 && lane == 0) {

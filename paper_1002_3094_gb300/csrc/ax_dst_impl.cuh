@@ -33,7 +33,7 @@
 // rows (forward) or form the (r, z) partial while storing (inverse).
 #pragma once
 #include <cmath>
-#include "ax_common.cuh"
+#include "ax_finish.cuh"
 
 namespace ax {
 
@@ -491,9 +491,11 @@ __global__ void __launch_bounds__(256, DstOcc<T>::min_blocks) dst_kernel(const D
   const size_t base = (size_t)m * (size_t)a.field + (size_t)row0 * a.pitch;
   T alpha = T(0);
   const T *__restrict__ p = nullptr;
+  bool x_fresh = false;  // x is overwritten (see RhsState::xbase)
   if (MODE == kDstPcgForward) {
     alpha = (T)a.st[m].alpha;
     p = (a.st[m].iters & 1) ? a.pa : a.pb;
+    x_fresh = sizeof(T) == 4 && a.st[m].iters == a.st[m].xbase;
   }
   T acc = T(0);
 
@@ -513,7 +515,12 @@ __global__ void __launch_bounds__(256, DstOcc<T>::min_blocks) dst_kernel(const D
       T v[V];
       if (MODE == kDstPcgForward) {
         T xv[V], pv[V], rv[V], qv[V];
-        load_vec<T>(xg + e, xv);
+        if (x_fresh) {
+#pragma unroll
+          for (int t = 0; t < V; ++t) xv[t] = T(0);
+        } else {
+          load_vec<T>(xg + e, xv);
+        }
         load_vec<T>(p + e, pv);
         load_vec<T>(rg + e, rv);
         load_vec<T>(ing + e, qv);
@@ -660,8 +667,9 @@ __global__ void __launch_bounds__(256, DstOcc<T>::min_blocks) dst_kernel(const D
     }
   }
   if (MODE == kDstPcgForward || MODE == kDstPcgInverse) {
-    const double s = block_sum((double)acc, red);
+    const double s = block_sum_of(acc, red);
     if (threadIdx.x == 0) a.partial[(size_t)m * kPartialStride + blockIdx.y] = s;
+    finish_rhs(a.fin, m, gridDim.y, a.partial + (size_t)m * kPartialStride, (int)gridDim.y, red);
   }
 }
 

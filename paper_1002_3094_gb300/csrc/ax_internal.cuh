@@ -113,17 +113,46 @@ struct RhsState {
   int status;      // AX_* status
   int max_iter;
   int due;         // mixed PCG: residual replacement due at the end of this iteration
+  int use_prev;    // kRedo: the new beta refers to rho_prev (mixed PCG residual replacement)
+  int xbase;       // mixed PCG: the x update at this iteration count overwrites x32 (which was
+                   // folded into the double-float iterate) instead of adding to it
   int pad_;
 };
 
-enum { kActive = 0, kCheck = 1, kDone = 2, kFailed = 3, kIdle = 4 };
-// Selection mask of the replacement step: active right-hand sides marked due.
-constexpr int kDue = 8;
+// kCheck: the FP64 PCG's true residual is to be formed and tested.  kRedo: r was
+// replaced by a true residual; the next iteration skips A p and, with alpha = 0
+// (x and r unchanged), recomputes z = B^-1 r, beta and p from it.
+enum { kActive = 0, kCheck = 1, kDone = 2, kFailed = 3, kIdle = 4, kRedo = 5 };
+// Selection masks that are not a single state.  kDue: active right-hand sides
+// marked due for residual replacement; kLive: kActive or kRedo (the kernels of
+// an iteration behind A p).
+constexpr int kDue = 8, kLive = 16;
+
+// Scalar step that a kernel's last CTA of a right-hand side performs on its
+// state once all CTAs of that right-hand side have written their partial
+// sums (finish_rhs): the iteration then needs no separate scalar launches.
+// The partials are summed in a fixed order, so results do not depend on which
+// CTA is last.
+enum { kFinNone = 0, kFinAlpha, kFinUpdate, kFinBeta, kFinRho, kFinTrueCheck, kFinReplace, kFinCheb, kFinStart,
+       kFinGatePhi, kFinGateRes };
+struct Finish {
+  int kind;
+  RhsState *st;
+  unsigned *count;     // arrivals per right-hand side, zero between launches
+  int on_converge;     // kFinUpdate, kFinCheb: state of a right-hand side that passes its threshold
+  int check;           // kFinCheb: the partials hold the residual norm
+  int xoff;            // kFinReplace, kFinStart: xbase = iters + xoff
+  const double *par;   // kFinReplace, kFinStart: device {tol^2, delta^2}
+  const double *bb;    // kFinStart: partials of ||phi||^2 (null: those of the kernel itself)
+  int nbb;
+  int max_iter;        // kFinStart
+  const double *chp;   // kFinCheb: (tau_0, rho_0^2) per right-hand side
+  int *chk;            // kFinReplace: count of the kRedo right-hand sides (option "replace_checks")
+};
 
 // Launch geometry shared by producers and consumers of per-CTA partial sums.
-constexpr int kStencilRows = 16;     // rows per stencil CTA
 constexpr int kStencilWarps = 8;     // warps per stencil CTA (along z)
-constexpr int kPartialStride = 8192; // max partials per RHS per kind
+constexpr int kPartialStride = 16384; // max partials per RHS per kind
 constexpr int kMaxNr = 8192, kMaxNz = 7000;
 
 struct Workspace;
@@ -199,6 +228,7 @@ struct StencilArgs {
   const RhsState *st;    // per RHS state (Pcg reads beta)
   int mask;
   double *partial;       // [m][kPartialStride] per-CTA sums: Pcg (p,q); Residual, Cheb ||res||^2
+  Finish fin;
 };
 
 template <typename T>
@@ -209,21 +239,27 @@ int stencil_blocks_per_rhs(int nr, int nz, int vec);
 // Double-float true residual r = phi - A x of the mixed method: x, phi and the
 // coefficients as pairs of FP32 numbers (hi + lo), all arithmetic in FP32 with
 // error-free transformations; r is returned rounded to FP32 with per-CTA
-// partials of ||r||^2.
+// partials of ||r||^2.  With d (the FP32 correction gathered since the last
+// replacement) x is first advanced, x <- x + d, in the same pass: the pair is
+// read from one of two buffers and written to the other (neighbouring CTAs
+// read the old pair), chosen by the parity of the replacement count st.tmp.
 struct DfResidualArgs {
   const float *CRh, *CRl, *CZh, *CZl, *Wh, *Wl;
   long long cstride, czstride;  // coefficient elements per RHS (0: one operator for all RHS)
   int nr, nz, pitch, pitchz;
   long long field;
   int m;
-  const float *xh, *xl, *ph, *pl;
+  float *xh[2], *xl[2];  // the two x buffers ([0] at an even replacement count)
+  const float *d;        // x32, or null: no fold (x from buffer [0])
+  int zero_start;        // 1: x is zero before the first replacement (buffer [0] is not read)
+  const float *ph, *pl;
   float *r32;
   const RhsState *st;
   int mask;
-  double *partial;  // [m][kPartialStride], slot blockIdx.y * gridDim.x + blockIdx.x
+  double *partial;  // [m][kPartialStride]
+  Finish fin;
 };
 void launch_residual_df(const DfResidualArgs &a, cudaStream_t s);
-int residual_df_blocks(int nr, int nz);
 
 // Persistent FP64 PCG of one right-hand side on a small grid (ax_small.cu):
 // the whole iteration in one cooperative launch, phases separated by bounded
@@ -285,6 +321,7 @@ struct DstArgs {
   const RhsState *st;
   int mask;
   double *partial;        // [m][kPartialStride]: PcgForward ||r||^2, PcgInverse (r, z)
+  Finish fin;
 };
 
 template <typename T>
@@ -347,10 +384,6 @@ struct GemmDstArgs {
   // the run out[(m n + l) tpitch + i], i < nr (no p update, no partials); the
   // input of the mode-solve kernel 14
   int tout, tpitch;
-  // non-null: the launch returns at once while *gate == 0 (a count, kept by
-  // the scalar kernels, of the right-hand sides its mask can select; for the
-  // masked launches of the residual-replacement step)
-  const int *gate;
 };
 void launch_dst_gemm(const GemmDstArgs &a, cudaStream_t s);
 size_t dst_gemm_smem_bytes(int three);
@@ -401,12 +434,7 @@ struct TriArgs {
   const T *IPST;
   long long tcstride;
   int tpitch;
-  // kernel 14, for a mask that rarely selects a right-hand side: short_grid =
-  // 1 runs a few CTAs per SM that loop over the tiles (instead of one CTA per
-  // tile), returning at once while *gate == 0 if gate is set (see
-  // GemmDstArgs::gate)
-  int short_grid;
-  const int *gate;
+  Finish fin;  // kernel 14 only
 };
 
 template <typename T>

@@ -7,9 +7,9 @@
 // ||A y - phi|| / ||phi|| <= tol.
 //
 // GPU organisation.  Scalars (alpha, beta, rho, norms) live on the device in
-// one RhsState per right-hand side and are produced by tiny "scalar" kernels
-// that reduce per-CTA FP64 partial sums in a fixed order (deterministic, no
-// atomics).  Every iteration kernel reads its RHS's state and returns at once
+// one RhsState per right-hand side and are produced by the last CTA of the
+// kernel that forms the sum, which reduces the per-CTA FP64 partial sums in a
+// fixed order (ax_finish.cuh; deterministic).  Every iteration kernel reads its RHS's state and returns at once
 // unless the state matches the kernel's mask, so converged right-hand sides
 // stop costing bandwidth while the others continue.  A block of iterations is
 // captured once into a CUDA graph and replayed; the host reads the states
@@ -30,7 +30,7 @@
 #include <string>
 #include <vector>
 
-#include "ax_common.cuh"
+#include "ax_finish.cuh"
 
 namespace ax {
 
@@ -41,6 +41,7 @@ struct GraphCache {
   cudaGraphExec_t exec = nullptr;
   int key = -1;
   size_t nodes = 0;
+  int direct_key = -1, direct = 0;  // iteration blocks launched without a graph (see run_graph)
 };
 
 struct ProfEvent {
@@ -55,7 +56,10 @@ struct Workspace {
   double *phi64 = nullptr, *x64 = nullptr;
   double *r64 = nullptr, *pa64 = nullptr, *pb64 = nullptr, *q64 = nullptr, *z64 = nullptr, *y64prev = nullptr;
   // FP32 vectors
-  float *xh = nullptr, *xl = nullptr, *phh = nullptr, *phl = nullptr;  // double-float x and phi (mixed PCG)
+  // double-float x (two buffers, see DfResidualArgs) and phi (mixed PCG)
+  float *xh[2] = {nullptr, nullptr}, *xl[2] = {nullptr, nullptr}, *phh = nullptr, *phl = nullptr;
+  float *arena32 = nullptr;  // one allocation holds the FP32 vectors
+  bool df32 = false;         // it holds the double-float vectors too
   float *x32 = nullptr, *r32 = nullptr, *pa32 = nullptr, *pb32 = nullptr, *q32 = nullptr, *z32 = nullptr,
         *y32prev = nullptr;
   // partial sums [4][m][kPartialStride]
@@ -63,11 +67,12 @@ struct Workspace {
   double *chp = nullptr;      // Chebyshev (tau, rho0^2) per right-hand side [m][2]
   double *rscale = nullptr;   // mixed methods: power-of-two scale of phi and x per right-hand side [m]
   RhsState *st = nullptr, *st_outer = nullptr;
-  // [0] right-hand sides the residual-replacement step has put in kCheck (the
-  // gate of its masked launches; reset at the end of the step), [1] the same
-  // counted over the current solve (option "replace_checks")
+  int mfield64 = 0;           // right-hand sides that phi64 and x64 hold
+  unsigned *arrive = nullptr; // CTA arrivals per right-hand side (Finish::count)
+  double *par = nullptr;      // mixed PCG: tol^2, delta^2 of the current solve (Finish::par)
+  // residual replacements of the current solve that recomputed z (option "replace_checks")
   int *chk = nullptr;
-  int replace_gate = 1;         // 0: the replacement step's launches are not gated
+  int replace_gate = 1;         // option "replace_gate": accepted, without effect
   RhsState *h_st = nullptr;   // pinned host mirror [2 m]
   // dense FP64 staging for host buffers and single-step entry points
   double *stage_a = nullptr, *stage_b = nullptr;
@@ -194,18 +199,20 @@ void free_vectors64(Workspace *w) {
   free_graph(w->gc64);
 }
 void free_vectors32(Workspace *w) {
-  dfree(w->x32); dfree(w->r32); dfree(w->pa32); dfree(w->pb32); dfree(w->q32); dfree(w->z32); dfree(w->y32prev);
-  dfree(w->xh); dfree(w->xl); dfree(w->phh); dfree(w->phl);
+  dfree(w->arena32);
+  w->x32 = w->r32 = w->pa32 = w->pb32 = w->q32 = w->z32 = w->y32prev = nullptr;
+  w->xh[0] = w->xh[1] = w->xl[0] = w->xl[1] = w->phh = w->phl = nullptr;
   w->m32 = 0;
+  w->df32 = false;
   free_graph(w->g32);
   free_graph(w->gc32);
 }
 void free_base(Workspace *w) {
   dfree(w->phi64); dfree(w->x64); dfree(w->part); dfree(w->chp); dfree(w->rscale); dfree(w->st);
-  dfree(w->st_outer); dfree(w->chk);
+  dfree(w->st_outer); dfree(w->chk); dfree(w->arrive); dfree(w->par);
   if (w->h_st) cudaFreeHost(w->h_st);
   w->h_st = nullptr;
-  w->mbase = 0;
+  w->mbase = w->mfield64 = 0;
   free_graph(w->g64); free_graph(w->g32); free_graph(w->gc64); free_graph(w->gc32);
 }
 
@@ -216,18 +223,32 @@ int ensure_base(ax_operator *op, int m) {
   Workspace *w = op->ws;
   if (w->mbase >= m) return AX_OK;
   free_base(w);
-  const size_t f = field_elems(op) * m;
-  AX_TRY(dalloc(&w->phi64, f));
-  AX_TRY(dalloc(&w->x64, f));
   AX_TRY(dalloc(&w->part, (size_t)4 * m * kPartialStride));
   AX_TRY(dalloc(&w->chp, (size_t)2 * m));
   AX_TRY(dalloc(&w->rscale, (size_t)m));
   AX_TRY(dalloc(&w->st, (size_t)m));
   AX_TRY(dalloc(&w->st_outer, (size_t)m));
-  AX_TRY(dalloc(&w->chk, 2));
-  AX_TRY(cudaMemset(w->chk, 0, 2 * sizeof(int)));
+  AX_TRY(dalloc(&w->chk, 1));
+  AX_TRY(dalloc(&w->arrive, (size_t)m));
+  AX_TRY(dalloc(&w->par, 2));
   AX_TRY(cudaMallocHost((void **)&w->h_st, sizeof(RhsState) * 2 * m));
   w->mbase = m;
+  return AX_OK;
+}
+
+// FP64 phi and x (every method but the mixed PCG with residual replacement).
+int ensure_field64(ax_operator *op, int m) {
+  std::lock_guard<std::recursive_mutex> lock(g_alloc_capture_mutex);
+  Workspace *w = op->ws;
+  if (w->mfield64 >= m) return AX_OK;
+  dfree(w->phi64);
+  dfree(w->x64);
+  w->mfield64 = 0;
+  free_graph(w->g64); free_graph(w->gc64);
+  const size_t f = field_elems(op) * m;
+  AX_TRY(dalloc(&w->phi64, f));
+  AX_TRY(dalloc(&w->x64, f));
+  w->mfield64 = m;
   return AX_OK;
 }
 
@@ -247,24 +268,31 @@ int ensure_vec64(ax_operator *op, int m, bool cheb) {
   return AX_OK;
 }
 
-int ensure_vec32(ax_operator *op, int m, bool cheb) {
+// FP32 vectors for m right-hand sides, with the Chebyshev iteration's second
+// iterate (cheb) or the double-float x and phi of the mixed PCG (df), in one
+// allocation.  z also holds the mode-major field of the forward transform
+// (nz tpitch floats per right-hand side, which can exceed nr pitch).
+int ensure_vec32(ax_operator *op, int m, bool cheb, bool df = false) {
   std::lock_guard<std::recursive_mutex> lock(g_alloc_capture_mutex);
   Workspace *w = op->ws;
-  if (w->m32 >= m && (!cheb || w->y32prev)) return AX_OK;
+  if (w->m32 >= m && (!cheb || w->y32prev) && (!df || w->df32)) return AX_OK;
+  if (w->m32 >= m) {  // grows by what is missing
+    m = w->m32;
+    cheb = cheb || w->y32prev != nullptr;
+    df = df || w->df32;
+  }
   free_vectors32(w);
-  const size_t f = field_elems(op) * m;
-  AX_TRY(dalloc(&w->x32, f));
-  AX_TRY(dalloc(&w->r32, f));
-  AX_TRY(dalloc(&w->pa32, f));
-  AX_TRY(dalloc(&w->pb32, f));
-  AX_TRY(dalloc(&w->q32, f));
-  AX_TRY(dalloc(&w->z32, f));
-  AX_TRY(dalloc(&w->xh, f));
-  AX_TRY(dalloc(&w->xl, f));
-  AX_TRY(dalloc(&w->phh, f));
-  AX_TRY(dalloc(&w->phl, f));
-  if (cheb) AX_TRY(dalloc(&w->y32prev, f));
+  const size_t f = field_elems(op) * m, fz = std::max(f, (size_t)m * op->nz * op->tpitch);
+  float **rest[12] = {&w->x32, &w->r32, &w->pa32, &w->pb32, &w->q32};
+  int n = 5;
+  if (cheb) rest[n++] = &w->y32prev;
+  if (df)
+    for (float **p : {&w->xh[0], &w->xl[0], &w->xh[1], &w->xl[1], &w->phh, &w->phl}) rest[n++] = p;
+  AX_TRY(dalloc(&w->arena32, f * n + fz));
+  for (int i = 0; i < n; ++i) *rest[i] = w->arena32 + f * i;
+  w->z32 = w->arena32 + f * n;
   w->m32 = m;
+  w->df32 = df;
   return AX_OK;
 }
 
@@ -286,6 +314,7 @@ int ensure_split(ax_operator *op, size_t bytes) {
   Workspace *w = op->ws;
   if (w->split_bytes >= bytes) return AX_OK;
   dfree(w->split);
+  free_graph(w->g32); free_graph(w->gc32);  // they hold its address
   w->split_bytes = 0;
   AX_TRY(dalloc(&w->split, bytes));  // zero: padding rows and columns stay zero
   w->split_bytes = bytes;
@@ -463,63 +492,185 @@ __global__ void add_correction(double *__restrict__ x, const float *__restrict__
     x[b + e] += (double)d[b + e];
 }
 
-// Task t of a right-hand side: the 8 consecutive columns 8 (t % nch) ..
-// of row t / nch (nch = chunks of 8 columns per row): consecutive threads walk
-// along a row, so every warp reads 1 KB of contiguous row data per field.
+// Task t of a right-hand side: 8 consecutive columns of one row, so that the 32
+// tasks of a warp are an 8-row x 32-column patch: its rows are whole 128-byte
+// lines of the field, and its part of the split operand whole 128-byte core
+// matrices (with the 32 tasks along one row instead, every 8-byte store of the
+// operand fell in a sector of its own: the store pipe was the limit).  nch =
+// chunks of 8 columns per row; patches past the last row or chunk have row >=
+// nr or col >= 8 nch.
+__device__ __forceinline__ int split_tasks(int nr, int nch) { return ((nr + 7) >> 3) * ((nch + 3) >> 2) * 32; }
 __device__ __forceinline__ void split_task(int t, int nch, int &row, int &col) {
-  row = t / nch;
-  col = (t - row * nch) * 8;
+  const int patch = t >> 5, l = t & 31, px = (nch + 3) >> 2;
+  const int pr = patch / px;
+  row = pr * 8 + (l >> 2);
+  col = ((patch - pr * px) * 4 + (l & 3)) * 8;
 }
 
-// FP64 field -> double-float pair (hi = fl(x), lo = fl(x - hi)) and back.
-// n is a multiple of 32 (whole rows of pitch elements): pairs of elements.
-__global__ void to_df(const double *__restrict__ x, float *__restrict__ h, float *__restrict__ l, size_t n) {
-  const double2 *x2 = reinterpret_cast<const double2 *>(x);
-  float2 *h2 = reinterpret_cast<float2 *>(h), *l2 = reinterpret_cast<float2 *>(l);
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n / 2; i += (size_t)gridDim.x * blockDim.x) {
-    const double2 v = x2[i];
-    const float hx = (float)v.x, hy = (float)v.y;
-    h2[i] = make_float2(hx, hy);
-    l2[i] = make_float2((float)(v.x - (double)hx), (float)(v.y - (double)hy));
+// v as a pair of FP32 numbers, v = h + l to 48 bits (h within half an ulp of v).
+// GB300 issues two FP64 operations per clock and SM against 64 integer ones, so
+// the pair is cut from the bits of v: the 53-bit significand rounded to its top
+// 24 bits and the signed 29-bit rest.  (float)v and (float)(v - (double)h) take
+// four FP64-pipe operations per value, 0.45 ms for 1024^2 x 64 values.
+__device__ __forceinline__ void split_df(double v, float &h, float &l) {
+  const long long b = __double_as_longlong(v);
+  const int ex = (int)((b >> 52) & 0x7FF) - 1023;
+  if (ex < -160) {  // 0, or below half the smallest FP32 number
+    h = l = 0.f;
+    return;
   }
-}
-__global__ void from_df(const float *__restrict__ h, const float *__restrict__ l, double *__restrict__ x, size_t n) {
-  const float2 *h2 = reinterpret_cast<const float2 *>(h), *l2 = reinterpret_cast<const float2 *>(l);
-  double2 *x2 = reinterpret_cast<double2 *>(x);
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n / 2; i += (size_t)gridDim.x * blockDim.x) {
-    const float2 a = h2[i], b = l2[i];
-    x2[i] = make_double2((double)a.x + (double)b.x, (double)a.y + (double)b.y);
+  if (ex < -103 || ex > 126) {  // near or outside the FP32 range, or not finite
+    h = (float)v;
+    l = isfinite(h) ? (float)(v - (double)h) : 0.f;
+    return;
   }
+  const unsigned long long sig = ((unsigned long long)b & 0xFFFFFFFFFFFFFull) | 0x10000000000000ull;
+  int top = (int)(sig >> 29), rest = (int)(sig & 0x1FFFFFFFu);
+  if (rest >= 0x10000000) {
+    top += 1;
+    rest -= 0x20000000;
+  }
+  const float sgn = b < 0 ? -1.f : 1.f;
+  const float unit = __int_as_float((ex - 23 + 127) << 23) * sgn;  // 2^(ex - 23): normal
+  h = (float)top * unit;
+  l = (float)rest * unit * 1.862645149230957e-9f;  // 2^-29
 }
-// Replacement of the selected right-hand sides in double-float: (xh, xl) +=
-// x32 (two-sum, then renormalised) and x32 = 0 in one pass.  Launched with
-// many CTAs per right-hand side, since only the few that are due at a step
-// do work (the others return at once).
-__global__ void fold_df(float *__restrict__ xh, float *__restrict__ xl, float *__restrict__ d, size_t field,
-                        const RhsState *st, int mask) {
-  const int m = blockIdx.y;
-  if (!rhs_selected(st, mask, m)) return;
-  // field is a multiple of 32 (rows of pitch elements): whole float4 groups
-  float4 *h4 = reinterpret_cast<float4 *>(xh + (size_t)m * field);
-  float4 *l4 = reinterpret_cast<float4 *>(xl + (size_t)m * field);
-  float4 *d4 = reinterpret_cast<float4 *>(d + (size_t)m * field);
-  const size_t n4 = field / 4;
-  auto fold = [](float a, float c, float lo, float &h, float &l) {
-    const float s = a + c, bb = s - a;
-    const float err = ((a - (s - bb)) + (c - bb)) + lo;
-    h = s + err;
-    l = err - (h - s);
+
+// Mixed PCG: sigma of every right-hand side, the power of two that brings
+// max |r f| into [1/2, 1) (1 for a zero or non-finite right-hand side), so that
+// the FP32 inner iteration works on values of order one whatever the units of f.
+// |f| is compared as integers (its bits, sign cleared), and r >= 0 multiplies the
+// row maxima only (rounding is monotone).  grid (m, .); par: tol^2, delta^2.
+__global__ void __launch_bounds__(256) mixed_peak(const double *__restrict__ f, const double *__restrict__ R, int nr,
+                                                  int nz, double *__restrict__ pmax, double *__restrict__ scale,
+                                                  unsigned *count, double *par, double tol2, double delta2, int *chk) {
+  __shared__ double red[8];
+  __shared__ int s_last;
+  const int m = blockIdx.x;
+  if (m == 0 && blockIdx.y == 0 && threadIdx.x == 0) {
+    par[0] = tol2;
+    par[1] = delta2;
+    *chk = 0;
+  }
+  double mx = 0.0;
+  bool bad = false;
+  for (int i = blockIdx.y; i < nr; i += gridDim.y) {
+    const unsigned long long *fr = reinterpret_cast<const unsigned long long *>(f + ((size_t)m * nr + i) * nz);
+    unsigned long long top = 0;
+#pragma unroll 4
+    for (int k = threadIdx.x; k < nz; k += 256) {
+      const unsigned long long b = fr[k] & 0x7FFFFFFFFFFFFFFFull;
+      top = b > top ? b : top;
+    }
+    const double v = R[i] * __longlong_as_double((long long)top);
+    bad = bad || !isfinite(v);
+    mx = fmax(mx, v);
+  }
+  if (bad) mx = INFINITY;
+  auto cta_max = [&](double v) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
+    __syncthreads();
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
+    __syncthreads();
+    double b = 0.0;
+    for (int w = 0; w < 8; ++w) b = fmax(b, red[w]);
+    return b;
   };
-  for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < n4; e += (size_t)gridDim.x * blockDim.x) {
-    const float4 a = h4[e], c = d4[e], lo = l4[e];
-    float4 h, l;
-    fold(a.x, c.x, lo.x, h.x, l.x);
-    fold(a.y, c.y, lo.y, h.y, l.y);
-    fold(a.z, c.z, lo.z, h.z, l.z);
-    fold(a.w, c.w, lo.w, h.w, l.w);
-    h4[e] = h;
-    l4[e] = l;
-    d4[e] = make_float4(0.f, 0.f, 0.f, 0.f);
+  mx = cta_max(mx);
+  if (threadIdx.x == 0) {
+    pmax[(size_t)m * kPartialStride + blockIdx.y] = mx;
+    __threadfence();
+    s_last = atomicAdd(count + m, 1u) == gridDim.y - 1;
+    if (s_last) {
+      count[m] = 0;
+      __threadfence();
+    }
+  }
+  __syncthreads();
+  if (!s_last) return;
+  mx = 0.0;
+  for (int i = threadIdx.x; i < (int)gridDim.y; i += 256)
+    mx = fmax(mx, __ldcg(pmax + (size_t)m * kPartialStride + i));
+  mx = cta_max(mx);
+  if (threadIdx.x == 0) {
+    double sc = 1.0;
+    if (mx > 0.0 && isfinite(mx)) {
+      int e = 0;
+      frexp(mx, &e);
+      sc = ldexp(1.0, -e);
+    }
+    scale[m] = sc;
+  }
+}
+
+constexpr int kPrepRows = 4;  // rows per CTA of the two kernels below
+
+// phi = sigma r f (Eq. diff_approx1) as a double-float pair with the ||phi||^2
+// partials; with r32 the residual of the zero start too, r = phi.  With u (a
+// guess, dense) instead x = sigma u as a pair.  grid (m, ceil(nr / kPrepRows)).
+__global__ void __launch_bounds__(256) mixed_prep(const double *__restrict__ f, const double *__restrict__ u,
+                                                  const double *__restrict__ R, const double *__restrict__ scale,
+                                                  int nr, int nz, int pitch, float *__restrict__ ph,
+                                                  float *__restrict__ pl, float *__restrict__ r32,
+                                                  float *__restrict__ xh, float *__restrict__ xl,
+                                                  double *__restrict__ part, const Finish fin) {
+  __shared__ double red[8];
+  const int m = blockIdx.x;
+  const int i0 = blockIdx.y * kPrepRows, i1 = min(i0 + kPrepRows, nr);
+  const double sc = scale[m];
+  double acc = 0.0;
+  for (int i = i0; i < i1; ++i) {
+    const double rs = R[i] * sc;  // exact: sc is a power of two
+    const size_t src = ((size_t)m * nr + i) * nz, dst = ((size_t)m * nr + i) * pitch;
+#pragma unroll 4
+    for (int k = threadIdx.x; k < nz; k += 256) {
+      const double v = rs * f[src + k];
+      float h, l;
+      split_df(v, h, l);
+      ph[dst + k] = h;
+      pl[dst + k] = l;
+      if (r32 != nullptr) r32[dst + k] = h;
+      acc = fma(v, v, acc);
+      if (u != nullptr) {
+        split_df(u[src + k] * sc, h, l);
+        xh[dst + k] = h;
+        xl[dst + k] = l;
+      }
+    }
+  }
+  const double s = block_sum(acc, red);
+  if (threadIdx.x == 0) part[(size_t)m * kPartialStride + blockIdx.y] = s;
+  finish_rhs(fin, m, gridDim.y, part + (size_t)m * kPartialStride, (int)gridDim.y, red);
+}
+
+// u = x / sigma (dense rows), x from the buffer of its last replacement; zero
+// where x was never formed (zero_start and no replacement).  The pair's parts
+// are widened and scaled by their exponent bits (see split_df), so that one FP64
+// addition per value remains.  grid (m, .).
+__global__ void __launch_bounds__(256) mixed_result(const float *__restrict__ xh0, const float *__restrict__ xl0,
+                                                    const float *__restrict__ xh1, const float *__restrict__ xl1,
+                                                    const double *__restrict__ scale, const RhsState *st,
+                                                    int zero_start, int nr, int nz, int pitch,
+                                                    double *__restrict__ u) {
+  const int m = blockIdx.x;
+  const int nrep = (int)st[m].tmp;
+  const bool zero = zero_start && nrep == 0;
+  const float *xh = (nrep & 1) ? xh1 : xh0, *xl = (nrep & 1) ? xl1 : xl0;
+  // scale is a power of two, normal: its inverse 2^e2 from the exponent bits
+  const int e2 = 1023 - (int)((__double_as_longlong(scale[m]) >> 52) & 0x7FF);
+  auto widen = [&](float v) -> double {
+    const unsigned b = __float_as_uint(v);
+    const int ex = (int)((b >> 23) & 0xFF), en = ex - 127 + e2;
+    if (ex == 0 || ex == 255 || en < -1022 || en > 1023) return ldexp((double)v, e2);
+    const unsigned long long o = ((unsigned long long)(b >> 31) << 63) | ((unsigned long long)(en + 1023) << 52) |
+                                 ((unsigned long long)(b & 0x7FFFFFu) << 29);
+    return __longlong_as_double((long long)o);
+  };
+  for (int i = blockIdx.y; i < nr; i += gridDim.y) {
+    const size_t src = ((size_t)m * nr + i) * pitch, dst = ((size_t)m * nr + i) * nz;
+#pragma unroll 4
+    for (int k = threadIdx.x; k < nz; k += 256) u[dst + k] = zero ? 0.0 : widen(xh[src + k]) + widen(xl[src + k]);
   }
 }
 
@@ -528,7 +679,9 @@ __global__ void fold_df(float *__restrict__ xh, float *__restrict__ xl, float *_
 // tensor-core transform: the update that the FFT forward transform fuses into
 // its load phase.  p is pb for an even iteration count, pa for an odd one (as
 // in the stencil).  x == nullptr: r only (the iterate update then happens in
-// the inverse transform's epilogue, with the next direction).
+// the inverse transform's epilogue, with the next direction).  For the cosine
+// transform, whose input is folded, a thread updates 8 columns and their 8
+// mirror images, so that it holds both halves of every fold.
 // CTAs per right-hand side of the update and split passes: about four
 // 8-column tasks per thread (at least 64, at most 4096 CTAs), so that large
 // fields keep enough loads in flight.
@@ -537,54 +690,101 @@ int update_blocks(int rows, int nz) {
   const long long b = (tasks + 4 * 256 - 1) / (4 * 256);
   return (int)std::max(64LL, std::min(4096LL, b));
 }
-__global__ void __launch_bounds__(256) pcg_update(float *__restrict__ x, float *__restrict__ r,
-                                                  const float *__restrict__ q, const float *__restrict__ pa,
-                                                  const float *__restrict__ pb, int nr, int n, int pitch,
-                                                  size_t field, int mtiles, int ktiles, int kbe,
-                                                  unsigned char *__restrict__ split,
-                                                  const RhsState *st, int mask, double *__restrict__ partial,
-                                                  int cosine) {
+struct UpdateArgs {
+  float *x, *r;
+  const float *q, *pa, *pb;
+  int nr, n, pitch;
+  size_t field;
+  int mtiles, ktiles, kbe;
+  unsigned char *split;
+  const RhsState *st;
+  int mask;
+  double *partial;
+  Finish fin;
+};
+template <bool COSINE>
+__global__ void __launch_bounds__(256) pcg_update(const UpdateArgs a) {
   __shared__ double red[8];
   const int m = blockIdx.y;
-  if (!rhs_selected(st, mask, m)) return;
-  const float alpha = (float)st[m].alpha;
-  const float *p = (st[m].iters & 1) ? pa : pb;
-  const int nch = (n + 7) >> 3;
-  const int tasks = nr * nch;
+  if (!rhs_selected(a.st, a.mask, m)) return;
+  const float alpha = (float)a.st[m].alpha;
+  const float *p = (a.st[m].iters & 1) ? a.pa : a.pb;
+  const bool x_fresh = a.st[m].iters == a.st[m].xbase;  // x is overwritten (see RhsState::xbase)
+  const int n = a.n;
   float acc = 0.f;
-  for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < tasks; t += gridDim.x * blockDim.x) {
-    int row, col;
-    split_task(t, nch, row, col);  // row < nr, col < n, col + 8 <= n rounded up to 8 <= pitch
-    const size_t e = (size_t)m * field + (size_t)row * pitch + col;
-    float rv[8], qv[8];
-    *reinterpret_cast<float4 *>(rv) = *reinterpret_cast<const float4 *>(r + e);
-    *reinterpret_cast<float4 *>(rv + 4) = *reinterpret_cast<const float4 *>(r + e + 4);
-    *reinterpret_cast<float4 *>(qv) = *reinterpret_cast<const float4 *>(q + e);
-    *reinterpret_cast<float4 *>(qv + 4) = *reinterpret_cast<const float4 *>(q + e + 4);
-    if (x != nullptr) {
+  // 8 consecutive columns at e (aligned)
+  auto update8 = [&](size_t e, float (&rv)[8]) {
+    float qv[8];
+    *reinterpret_cast<float4 *>(rv) = *reinterpret_cast<const float4 *>(a.r + e);
+    *reinterpret_cast<float4 *>(rv + 4) = *reinterpret_cast<const float4 *>(a.r + e + 4);
+    *reinterpret_cast<float4 *>(qv) = *reinterpret_cast<const float4 *>(a.q + e);
+    *reinterpret_cast<float4 *>(qv + 4) = *reinterpret_cast<const float4 *>(a.q + e + 4);
+    if (a.x != nullptr) {
       float xv[8], pv[8];
-      *reinterpret_cast<float4 *>(xv) = *reinterpret_cast<const float4 *>(x + e);
-      *reinterpret_cast<float4 *>(xv + 4) = *reinterpret_cast<const float4 *>(x + e + 4);
+#pragma unroll
+      for (int i = 0; i < 8; ++i) xv[i] = 0.f;
+      if (!x_fresh) {
+        *reinterpret_cast<float4 *>(xv) = *reinterpret_cast<const float4 *>(a.x + e);
+        *reinterpret_cast<float4 *>(xv + 4) = *reinterpret_cast<const float4 *>(a.x + e + 4);
+      }
       *reinterpret_cast<float4 *>(pv) = *reinterpret_cast<const float4 *>(p + e);
       *reinterpret_cast<float4 *>(pv + 4) = *reinterpret_cast<const float4 *>(p + e + 4);
 #pragma unroll
       for (int i = 0; i < 8; ++i) xv[i] = fmaf(alpha, pv[i], xv[i]);
-      *reinterpret_cast<float4 *>(x + e) = *reinterpret_cast<const float4 *>(xv);
-      *reinterpret_cast<float4 *>(x + e + 4) = *reinterpret_cast<const float4 *>(xv + 4);
+      *reinterpret_cast<float4 *>(a.x + e) = *reinterpret_cast<const float4 *>(xv);
+      *reinterpret_cast<float4 *>(a.x + e + 4) = *reinterpret_cast<const float4 *>(xv + 4);
     }
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
       rv[i] = fmaf(-alpha, qv[i], rv[i]);
       acc = fmaf(rv[i], rv[i], acc);
     }
-    *reinterpret_cast<float4 *>(r + e) = *reinterpret_cast<const float4 *>(rv);
-    *reinterpret_cast<float4 *>(r + e + 4) = *reinterpret_cast<const float4 *>(rv + 4);
-    // the cosine transform folds mirrored columns, which other threads update:
-    // its split input is written by a separate pass (split_field)
-    if (!cosine) split_store8(split, m, row, col, mtiles, ktiles, kbe, rv);
+    *reinterpret_cast<float4 *>(a.r + e) = *reinterpret_cast<const float4 *>(rv);
+    *reinterpret_cast<float4 *>(a.r + e + 4) = *reinterpret_cast<const float4 *>(rv + 4);
+  };
+  auto update1 = [&](size_t e) -> float {
+    if (a.x != nullptr) a.x[e] = fmaf(alpha, p[e], x_fresh ? 0.f : a.x[e]);
+    const float v = fmaf(-alpha, a.q[e], a.r[e]);
+    a.r[e] = v;
+    acc = fmaf(v, v, acc);
+    return v;
+  };
+  // sine: chunks of 8 columns; cosine: chunks of 8 columns of the first half
+  // (with the middle one of an odd n) and their mirrors
+  const int half = COSINE ? (n + 1) >> 1 : n;
+  const int nch = (half + 7) >> 3;
+  const int tasks = split_tasks(a.nr, nch);
+  for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < tasks; t += gridDim.x * blockDim.x) {
+    int row, col;
+    split_task(t, nch, row, col);
+    if (row >= a.nr || col >= 8 * nch) continue;  // col < half; col + 8 <= n rounded up to 8 <= pitch
+    const size_t rowe = (size_t)m * a.field + (size_t)row * a.pitch;
+    float rv[8];
+    if (!COSINE) {
+      update8(rowe + col, rv);
+      split_store8(a.split, m, row, col, a.mtiles, a.ktiles, a.kbe, rv);
+    } else {
+      float rm[8];  // the mirrors n - 1 - col - i
+      if ((n & 7) == 0 && col + 8 <= n / 2) {  // whole aligned chunks on both sides
+        float rb[8];
+        update8(rowe + col, rv);
+        update8(rowe + n - 8 - col, rb);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) rm[i] = rb[7 - i];
+      } else {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          const int k = col + i;
+          rv[i] = k < half ? update1(rowe + k) : 0.f;
+          rm[i] = k < n / 2 ? update1(rowe + n - 1 - k) : 0.f;  // the middle column of odd n once
+        }
+      }
+      fold_store8(a.split, m, row, col, n, a.mtiles, a.ktiles, a.kbe, rv, rm);
+    }
   }
-  const double sum = block_sum((double)acc, red);
-  if (threadIdx.x == 0) partial[(size_t)m * kPartialStride + blockIdx.x] = sum;
+  const double sum = block_sum_of(acc, red);
+  if (threadIdx.x == 0) a.partial[(size_t)m * kPartialStride + blockIdx.x] = sum;
+  finish_rhs(a.fin, m, gridDim.x, a.partial + (size_t)m * kPartialStride, (int)gridDim.x, red);
 }
 
 // The rows of a field written split into BF16 halves (tensor-core transform input).
@@ -592,16 +792,15 @@ __global__ void __launch_bounds__(256) pcg_update(float *__restrict__ x, float *
 __global__ void __launch_bounds__(256) split_field(const float *__restrict__ in, int nr, int n, int pitch,
                                                    size_t field, int mtiles, int ktiles, int kbe,
                                                    unsigned char *__restrict__ split,
-                                                   const RhsState *st, int mask, int cosine,
-                                                   const int *gate) {
-  if (gate != nullptr && *gate == 0) return;  // nothing selected (see GemmDstArgs::gate)
+                                                   const RhsState *st, int mask, int cosine) {
   const int m = blockIdx.y;
   if (!rhs_selected(st, mask, m)) return;
   const int nch = (n + 7) >> 3;
-  const int tasks = nr * nch;
+  const int tasks = split_tasks(nr, nch);
   for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < tasks; t += gridDim.x * blockDim.x) {
     int row, col;
-    split_task(t, nch, row, col);  // row < nr, col < n, col + 8 <= n rounded up to 8 <= pitch
+    split_task(t, nch, row, col);
+    if (row >= nr || col >= 8 * nch) continue;  // col < n, col + 8 <= n rounded up to 8 <= pitch
     const size_t e = (size_t)m * field + (size_t)row * pitch + col;
     float v[8];
     *reinterpret_cast<float4 *>(v) = *reinterpret_cast<const float4 *>(in + e);
@@ -645,6 +844,7 @@ __global__ void sc_start(RhsState *st, const double *prr, int nbr, const double 
     s.cheb_a = 2.0;
     s.status = AX_OK;
     s.due = 0;
+    s.xbase = -1;
     if (!isfinite(rr) || !isfinite(bb)) {
       s.state = kFailed;
       s.status = AX_ERR_BREAKDOWN;
@@ -655,209 +855,16 @@ __global__ void sc_start(RhsState *st, const double *prr, int nbr, const double 
   }
 }
 
-__global__ void sc_rho_init(RhsState *st, const double *p, int nb, int mask) {
+// The scalar step of `f` on its own (one CTA per right-hand side), where the
+// kernel that forms the partials cannot do it.
+__global__ void __launch_bounds__(256) sc_finish(const Finish f, int mask, const double *part, int nb) {
+  __shared__ double red[8];
   const int m = blockIdx.x;
-  if (!rhs_selected(st, mask, m)) return;
-  const double rz = reduce_part(p + (size_t)m * kPartialStride, nb);
-  if (threadIdx.x == 0) {
-    st[m].rho = rz;
-    st[m].beta = 0.0;
-    if (!isfinite(rz)) {
-      st[m].state = kFailed;
-      st[m].status = AX_ERR_BREAKDOWN;
-    }
-  }
-}
-
-__global__ void sc_alpha(RhsState *st, const double *p, int nb) {
-  const int m = blockIdx.x;
-  if (st[m].state != kActive) return;
-  const double pq = reduce_part(p + (size_t)m * kPartialStride, nb);
-  if (threadIdx.x == 0) {
-    if (!(pq > 0.0) || !isfinite(pq) || !isfinite(st[m].rho)) {
-      st[m].state = kFailed;
-      st[m].status = AX_ERR_BREAKDOWN;
-    } else {
-      st[m].alpha = st[m].rho / pq;
-    }
-  }
-}
-
-// After x, r update: count the iteration and test the recursive residual.
-// on_converge == kDue: a right-hand side that passes its threshold stays
-// active for the rest of the iteration and is marked due for the replacement
-// step at its end (mixed PCG).
-__global__ void sc_after_update(RhsState *st, const double *p, int nb, int on_converge) {
-  const int m = blockIdx.x;
-  if (st[m].state != kActive) return;
-  const double rr = reduce_part(p + (size_t)m * kPartialStride, nb);
-  if (threadIdx.x == 0) {
-    RhsState s = st[m];
-    s.rr = rr;
-    s.iters += 1;
-    if (!isfinite(rr)) {
-      s.state = kFailed;
-      s.status = AX_ERR_BREAKDOWN;
-    } else if (rr <= s.thresh2) {
-      if (on_converge == kDue) s.due = 1;
-      else s.state = on_converge;
-    } else if (s.iters >= s.max_iter) {
-      s.state = (on_converge == kDone) ? kDone : kFailed;
-      if (on_converge != kDone) s.status = AX_ERR_NO_CONVERGENCE;
-    }
-    st[m] = s;
-  }
-}
-
-// use_prev: the right-hand side already took this iteration's direction
-// update from its recursive residual; the new beta refers to the rho before
-// that update (mixed PCG residual replacement).
-__global__ void sc_beta(RhsState *st, const double *p, int nb, int mask, int next_state, int use_prev = 0) {
-  const int m = blockIdx.x;
-  if (st[m].state != mask) return;
-  const double rz = reduce_part(p + (size_t)m * kPartialStride, nb);
-  if (threadIdx.x == 0) {
-    const double rho = use_prev ? st[m].rho_prev : st[m].rho;
-    if (!isfinite(rz) || rho == 0.0) {
-      st[m].state = kFailed;
-      st[m].status = AX_ERR_BREAKDOWN;
-    } else {
-      if (!use_prev) st[m].rho_prev = rho;
-      st[m].beta = rz / rho;
-      st[m].rho = rz;
-      st[m].state = next_state;
-    }
-  }
-}
-
-// Right-hand sides (of n) in state `from` move to `to`.
-__global__ void sc_promote(RhsState *st, int n, int from, int to, int *reset) {
-  const int m = blockIdx.x * blockDim.x + threadIdx.x;
-  if (m < n && st[m].state == from) st[m].state = to;
-  if (reset != nullptr && m == 0) *reset = 0;
-}
-
-// True-residual test of right-hand sides in kCheck.
-__global__ void sc_true_check(RhsState *st, const double *p, int nb) {
-  const int m = blockIdx.x;
-  if (st[m].state != kCheck) return;
-  const double rr = reduce_part(p + (size_t)m * kPartialStride, nb);
-  if (threadIdx.x == 0) {
-    st[m].rr = rr;
-    if (rr <= st[m].thresh2) st[m].state = kDone;
-    else if (st[m].iters >= st[m].max_iter) {
-      st[m].state = kFailed;
-      st[m].status = AX_ERR_NO_CONVERGENCE;
-    }
-  }
-}
-
-// Chebyshev: rr = ||A y - phi||^2 of the current iterate; stop or continue and
-// advance alpha_{k+1} = 4 / (4 - rho0^2 alpha_k) (alpha for the first step is 1).
-// check = 0: a step without the residual norm (no reduction): only the
-// recurrence advances.
-__global__ void sc_cheb(RhsState *st, const double *p, int nb, const double *chp, int on_converge, int check = 1) {
-  const int m = blockIdx.x;
-  if (st[m].state != kActive) return;
-  const double rho0sq = chp[2 * m + 1];
-  const double rr = check ? reduce_part(p + (size_t)m * kPartialStride, nb) : st[m].rr;
-  if (threadIdx.x == 0) {
-    RhsState s = st[m];
-    s.rr = rr;
-    if (!isfinite(rr)) {
-      s.state = kFailed;
-      s.status = AX_ERR_BREAKDOWN;
-    } else if (check && rr <= s.thresh2) {
-      s.state = on_converge;
-    } else if (s.iters >= s.max_iter) {
-      s.state = (on_converge == kDone) ? kDone : kFailed;
-      if (on_converge != kDone) s.status = AX_ERR_NO_CONVERGENCE;
-    } else {
-      if (s.iters == 0) {
-        s.cheb_a = 1.0;  // y_1 = y_0 - tau B^-1 (A y_0 - phi) (the y_{-1} term drops out)
-      } else {
-        const double prev = (s.iters == 1) ? 2.0 : s.cheb_a;
-        s.cheb_a = 4.0 / (4.0 - rho0sq * prev);
-      }
-      s.iters += 1;
-    }
-    st[m] = s;
-  }
-}
-
-// Mixed PCG with residual replacement: start.  rr = ||phi - A x||^2 (FP64),
-// bb = ||phi||^2; the FP32 iteration runs until its recursive residual falls
-// below thresh2 = max(delta^2 rr_true, (tol/2)^2 bb), then the true residual
-// replaces it.
-__global__ void sc_mixed_start(RhsState *st, const double *prr, int nbr, const double *pbb, int nbb, double tol2,
-                               double delta2, int max_iter) {
-  const int m = blockIdx.x;
-  const double rr = reduce_part(prr + (size_t)m * kPartialStride, nbr);
-  const double bb = reduce_part(pbb + (size_t)m * kPartialStride, nbb);
-  if (threadIdx.x == 0) {
-    RhsState s;
-    memset(&s, 0, sizeof(s));
-    s.rr = rr;
-    s.bb = bb;
-    s.max_iter = max_iter;
-    s.status = AX_OK;
-    if (!isfinite(rr) || !isfinite(bb)) {
-      s.state = kFailed;
-      s.status = AX_ERR_BREAKDOWN;
-    } else if (rr <= tol2 * bb || bb == 0.0) {
-      s.state = kDone;
-    } else {
-      s.state = kActive;
-      s.thresh2 = fmax(delta2 * rr, 0.25 * tol2 * bb);
-    }
-    st[m] = s;
-  }
-}
-
-// Residual replacement: rr = ||phi - A x64||^2 just computed in FP64 for the
-// right-hand sides in kCheck.  Done, failed, or a new threshold (the caller
-// then recomputes z = B^-1 r and resumes with sc_beta).
-__global__ void sc_mixed_replace(RhsState *st, const double *prr, int nbr, double tol2, double delta2, int *chk) {
-  const int m = blockIdx.x;
-  if (!rhs_selected(st, kDue, m)) return;
-  const double rr = reduce_part(prr + (size_t)m * kPartialStride, nbr);
-  if (threadIdx.x == 0) {
-    RhsState s = st[m];
-    // the iteration's z and rho came from the recursive residual: when the
-    // true one differs noticeably (||r||^2 by more than 1%: typically once the
-    // recursion has run below the FP32 accuracy of x), the right-hand side goes
-    // to kCheck for z = B^-1 r and beta from the new (r, z)
-    const bool consistent = fabs(rr - s.rr) <= 1e-2 * rr;
-    s.rr = rr;
-    s.due = 0;
-    s.tmp += 1.0;  // replacements
-    if (!isfinite(rr)) {
-      s.state = kFailed;
-      s.status = AX_ERR_BREAKDOWN;
-    } else if (rr <= tol2 * s.bb) {
-      s.state = kDone;
-    } else if (s.iters >= s.max_iter) {
-      s.state = kFailed;
-      s.status = AX_ERR_NO_CONVERGENCE;
-    } else {
-      s.thresh2 = fmax(delta2 * rr, 0.25 * tol2 * s.bb);
-      if (!consistent) {
-        s.state = kCheck;
-        atomicAdd(chk, 1);  // opens the gate of the step's masked launches
-        atomicAdd(chk + 1, 1);
-      }
-    }
-    st[m] = s;
-  }
-}
-
-template <typename T>
-__global__ void zero_masked(T *x, size_t field, const RhsState *st, int mask) {
-  const int m = blockIdx.y;
-  if (!rhs_selected(st, mask, m)) return;
-  const size_t b = (size_t)m * field;
-  for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < field; e += (size_t)gridDim.x * blockDim.x)
-    x[b + e] = T(0);
+  if (!rhs_selected(f.st, mask, m)) return;
+  double v = 0.0;
+  for (int i = threadIdx.x; i < nb; i += blockDim.x) v += part[(size_t)m * kPartialStride + i];
+  v = block_sum(v, red);
+  if (threadIdx.x == 0) finish_rule(f, m, v, 0.0);
 }
 
 // Outer refinement step: rr = ||phi - A x||^2 (FP64).  Converged RHS -> done;
@@ -910,6 +917,7 @@ __global__ void sc_outer(RhsState *so, RhsState *si, const double *prr, int nbr,
         in.beta = 0.0;
         in.cheb_a = 2.0;
         in.status = AX_OK;
+        in.xbase = -1;
       }
     }
     so[m] = s;
@@ -1350,11 +1358,10 @@ int tc_mode_variant(const ax_operator *op, int m) {
 }
 bool tc_scaled(const ax_operator *op, int m) { return tc_mode_variant(op, m) >= 2; }
 // The forward transform of a preconditioner application writes mode-major
-// for the mode-solve kernel 14, when that layout fits the buffer it writes
-// (m nr pitch floats: nz tpitch <= nr pitch) and its factor table exists.
+// for the mode-solve kernel 14 (the buffer holds either layout: see
+// ensure_vec32), when its factor table exists.
 bool tc_tr_mode(const ax_operator *op, int m) {
-  return tc_mode_variant(op, m) == 14 && op->c32.IPST != nullptr && op->tpitch > 0 &&
-         (long long)op->nz * op->tpitch <= (long long)op->nr * op->pitch;
+  return tc_mode_variant(op, m) == 14 && op->c32.IPST != nullptr && op->tpitch > 0;
 }
 
 // scaled: multiply every output row by D (the row scale of the pipelined mode
@@ -1363,9 +1370,8 @@ bool tc_tr_mode(const ax_operator *op, int m) {
 void tc_transform(const ax_operator *op, int m, int rows, const unsigned char *A, bool inverse, float *out,
                   const RhsState *st, int mask, const float *r, double *partial, cudaStream_t s, int three = -1,
                   float *pa = nullptr, float *pb = nullptr, float *x = nullptr, bool scaled = false,
-                  bool tout = false, const int *gate = nullptr) {
+                  bool tout = false) {
   GemmDstArgs g{};
-  g.gate = gate;
   if (tout) {  // mode-major output for the mode-solve kernel 14 (forward only)
     g.tout = 1;
     g.tpitch = op->tpitch;
@@ -1409,26 +1415,22 @@ void tc_transform(const ax_operator *op, int m, int rows, const unsigned char *A
 
 // FP32 field -> split operand (rows per RHS `rows`).
 void tc_split(const ax_operator *op, int m, int rows, const float *in, unsigned char *split, const RhsState *st,
-              int mask, cudaStream_t s, const int *gate = nullptr) {
+              int mask, cudaStream_t s) {
   const SplitGeom g = split_geom(op, rows);
-  // kCheck (the replacement step's recomputation of z) selects a right-hand
-  // side rarely: fewer CTAs per right-hand side, so that the usual launch in
-  // which none is selected ends soon (the CTAs loop over the rows)
-  const int bx = mask == kCheck ? std::min(update_blocks(rows, op->nz), 8) : update_blocks(rows, op->nz);
   note_launch();
-  split_field<<<dim3(bx, m), 256, 0, s>>>(in, rows, op->nz, op->pitch,
-                                                                   (size_t)rows * op->pitch,
-                                                      g.mtiles, g.ktiles, g.kbe, split, st, mask, op->bc_z == 1,
-                                                      gate);
+  split_field<<<dim3(update_blocks(rows, op->nz), m), 256, 0, s>>>(in, rows, op->nz, op->pitch,
+                                                                   (size_t)rows * op->pitch, g.mtiles, g.ktiles,
+                                                                   g.kbe, split, st, mask, op->bc_z == 1);
 }
 
 // Mode solves z -> split operand (the tile kernel writes it directly; otherwise
 // through the FP32 buffer tmp).
 // With `prz` (tile kernel only), the mode solves also form the partials of
 // (rhat, yhat), equal to (r, z) up to the rounding of the split input: S is
-// symmetric, so (r, S yhat) = (S r, yhat).
+// symmetric, so (r, S yhat) = (S r, yhat).  fin: the scalar step on them.
 void tc_mode_solve(const ax_operator *op, int m, const float *z, float *tmp, unsigned char *split,
-                   const RhsState *st, int mask, cudaStream_t s, double *prz = nullptr, const int *gate = nullptr) {
+                   const RhsState *st, int mask, cudaStream_t s, double *prz = nullptr,
+                   const Finish &fin = Finish{}) {
   const SplitGeom g = split_geom(op, op->nr);
   TriArgs<float> t = tri_args<float>(op, m, z, tmp, st, mask);
   t.variant = tc_mode_variant(op, m);
@@ -1437,10 +1439,6 @@ void tc_mode_solve(const ax_operator *op, int m, const float *z, float *tmp, uns
     t.IPST = op->c32.IPST;
     t.tcstride = op->cstride != 0 ? (long long)op->nz * op->tpitch : 0;
     t.tpitch = op->tpitch;
-    if (mask == kCheck) {  // rarely selected: a short grid, gated where the caller keeps the count
-      t.short_grid = 1;
-      t.gate = gate;
-    }
   } else if (t.variant == 14) {
     t.variant = 9;
   }
@@ -1450,10 +1448,17 @@ void tc_mode_solve(const ax_operator *op, int m, const float *z, float *tmp, uns
     t.split_ktiles = g.ktiles;
     t.split_kbe = g.kbe;
     t.partial = prz;
+    const bool own = t.variant == 14;  // kernel 14 performs the scalar step itself
+    if (own) t.fin = fin;
     launch_tridiag<float>(t, s);
+    if (!own && fin.kind != kFinNone) {
+      const int cols = tridiag_reg_cols(op->nr, tc_mode_variant(op, m));
+      note_launch();
+      sc_finish<<<m, 256, 0, s>>>(fin, mask, prz, (op->nz + cols - 1) / cols);
+    }
   } else {
     launch_tridiag<float>(t, s);
-    tc_split(op, m, op->nr, tmp, split, st, mask, s, gate);
+    tc_split(op, m, op->nr, tmp, split, st, mask, s);
   }
 }
 
@@ -1474,12 +1479,17 @@ int precond_partials(const ax_operator *op, int m) {
   return dst_blocks(op, op->nr, (int)sizeof(T));
 }
 
-// z = B^-1 r for selected RHS, with (r, z) partials into `prz`.  The
-// tensor-core path goes through the workspace's split operand (and tmp when
-// the mode solves cannot write it directly); the FFT path works in place in z.
+// z = B^-1 r for selected RHS, with (r, z) partials into `prz` and the scalar
+// step `fin` on them.  The tensor-core path goes through the workspace's split
+// operand (and tmp when the mode solves cannot write it directly); the FFT path
+// works in place in z.  out: where the result goes (null: z).  dot_only: the
+// (r, z) sum alone is wanted; where the mode solves form it the inverse
+// transform is left out.
 template <typename T>
 void precond_apply(const ax_operator *op, int m, const T *r, T *z, const RhsState *st, int mask, double *prz,
-                   cudaStream_t s, T *tmp = nullptr) {
+                   cudaStream_t s, T *tmp = nullptr, const Finish &fin = Finish{}, T *out = nullptr,
+                   bool dot_only = false) {
+  if (out == nullptr) out = z;
   if constexpr (sizeof(T) == 4) {
     if (use_tc<T>(op) && tmp != nullptr) {
       unsigned char *sp = op->ws->split;
@@ -1488,9 +1498,14 @@ void precond_apply(const ax_operator *op, int m, const T *r, T *z, const RhsStat
       const bool sc = tc_scaled(op, m);
       tc_transform(op, m, op->nr, sp, false, z, st, mask, nullptr, nullptr, s, -1, nullptr, nullptr, nullptr, sc,
                    tc_tr_mode(op, m));
-      tc_mode_solve(op, m, z, tmp, sp, st, mask, s, dm ? prz : nullptr);
-      tc_transform(op, m, op->nr, sp, true, z, st, mask, dm ? nullptr : r, dm ? nullptr : prz, s, -1, nullptr, nullptr,
-                   nullptr, sc);
+      tc_mode_solve(op, m, z, tmp, sp, st, mask, s, dm ? prz : nullptr, dm ? fin : Finish{});
+      if (dm && dot_only) return;
+      tc_transform(op, m, op->nr, sp, true, out, st, mask, dm ? nullptr : r, dm ? nullptr : prz, s, -1, nullptr,
+                   nullptr, nullptr, sc);
+      if (!dm && fin.kind != kFinNone) {
+        note_launch();
+        sc_finish<<<m, 256, 0, s>>>(fin, mask, prz, precond_partials<T>(op, m));
+      }
       return;
     }
   }
@@ -1501,9 +1516,10 @@ void precond_apply(const ax_operator *op, int m, const T *r, T *z, const RhsStat
   launch_tridiag<T>(tri_args<T>(op, m, z, z, st, mask), s);
   DstArgs<T> b = dst_args<T>(op, m, op->nr, st, mask);
   b.in = z;
-  b.out = z;
+  b.out = out;
   b.r = const_cast<T *>(r);
   b.partial = prz;
+  b.fin = fin;
   launch_dst<T>(kDstPcgInverse, b, s);
 }
 
@@ -1521,15 +1537,26 @@ struct PcgVecs {
 // so z is never stored, the stencil reads p alone and the update pass only r.
 bool tc_fused(const ax_operator *op) { return use_tc<float>(op) && tc_dot_in_modes(op) && !op->ws->tc_unfused; }
 
-// One PCG iteration for the right-hand sides in kActive.  fused (FP32
+Finish make_fin(const Workspace *w, RhsState *st, int kind, int on_converge = kDone) {
+  Finish f{};
+  f.kind = kind;
+  f.st = st;
+  f.count = w->arrive;
+  f.on_converge = on_converge;
+  f.par = w->par;
+  f.chp = w->chp;
+  f.chk = w->chk;
+  return f;
+}
+
+// One PCG iteration for the right-hand sides in kActive; those in kRedo only
+// take the part behind A p, with alpha = 0 (see kRedo).  fused (FP32
 // tensor-core path with tc_fused only): p was formed by the previous
-// iteration's inverse transform (or the start), see tc_fused.
+// iteration's inverse transform (or the start), see tc_fused.  Every scalar
+// step is taken by the kernel that forms its sum (ax_finish.cuh).
 template <typename T>
 void pcg_iteration(const ax_operator *op, int m, const PcgVecs<T> &v, RhsState *st, Workspace *w,
                    int on_converge, cudaStream_t s, double units = 0.0, bool fused = false) {
-  const int V = VecT<T>::n;
-  const int nbs = stencil_blocks_per_rhs(op->nr, op->nz, V);
-  const int nbd = dst_blocks(op, op->nr, (int)sizeof(T));
   double *pq = part_ptr(w, kPartA), *prr = part_ptr(w, kPartB), *prz = part_ptr(w, kPartC);
   StencilArgs<T> sa = stencil_args<T>(op, m, st, kActive);
   sa.in = v.z;
@@ -1537,70 +1564,56 @@ void pcg_iteration(const ax_operator *op, int m, const PcgVecs<T> &v, RhsState *
   sa.pb = v.pb;
   sa.out = v.q;
   sa.partial = pq;
+  sa.fin = make_fin(w, st, kFinAlpha);
   {
     ProfScope ps(w, kProfStencil, units, s);
     launch_stencil<T>(fused ? kStencilPcgP : kStencilPcg, sa, s);
   }
-  {
-    ProfScope ps(w, kProfScalar, 0.0, s);
-    note_launch();
-    sc_alpha<<<m, 32, 0, s>>>(st, pq, nbs);
-  }
+  const Finish upd = make_fin(w, st, kFinUpdate, on_converge), beta = make_fin(w, st, kFinBeta);
   if constexpr (sizeof(T) == 4) {
     if (use_tc<T>(op)) {
       // update pass (r written split too), transform r -> z, mode solves
-      // z -> split, inverse transform split -> z with the (r, z) partials
+      // z -> split, inverse transform split -> z (or the next direction) with
+      // the (r, z) partials
       const SplitGeom g = split_geom(op, op->nr);
       unsigned char *sp = w->split;
       {
         ProfScope ps(w, kProfUpdate, units, s);
+        UpdateArgs u{fused ? nullptr : v.x, v.r, v.q, v.pa, v.pb, op->nr, op->nz, op->pitch, field_elems(op),
+                     g.mtiles, g.ktiles, g.kbe, sp, st, kLive, prr, upd};
+        const dim3 grid(update_blocks(op->nr, op->nz), m);
         note_launch();
-        pcg_update<<<dim3(update_blocks(op->nr, op->nz), m), 256, 0, s>>>(fused ? nullptr : v.x, v.r, v.q, v.pa,
-                                                                           v.pb, op->nr,
-                                                          op->nz, op->pitch, field_elems(op), g.mtiles, g.ktiles,
-                                                          g.kbe, sp, st, kActive, prr, op->bc_z == 1);
-        if (op->bc_z == 1) tc_split(op, m, op->nr, v.r, sp, st, kActive, s);
+        if (op->bc_z == 1) pcg_update<true><<<grid, 256, 0, s>>>(u);
+        else pcg_update<false><<<grid, 256, 0, s>>>(u);
       }
       const bool sc = tc_scaled(op, m);
       {
         ProfScope ps(w, kProfDstFwd, units, s);
-        tc_transform(op, m, op->nr, sp, false, v.z, st, kActive, nullptr, nullptr, s, -1, nullptr, nullptr, nullptr, sc,
+        tc_transform(op, m, op->nr, sp, false, v.z, st, kLive, nullptr, nullptr, s, -1, nullptr, nullptr, nullptr, sc,
                      tc_tr_mode(op, m));
-      }
-      {
-        ProfScope ps(w, kProfScalar, 0.0, s);
-        note_launch();
-        sc_after_update<<<m, 32, 0, s>>>(st, prr, update_blocks(op->nr, op->nz), on_converge);
       }
       const bool dm = tc_dot_in_modes(op);
       {
         ProfScope ps(w, kProfTridiag, units, s);
-        tc_mode_solve(op, m, v.z, v.q, sp, st, kActive, s, dm ? prz : nullptr);
-      }
-      if (fused) {
-        {
-          ProfScope ps(w, kProfScalar, 0.0, s);
-          note_launch();
-          sc_beta<<<m, 32, 0, s>>>(st, prz, precond_partials<T>(op, m), kActive, kActive);
-        }
-        ProfScope ps(w, kProfDstInv, units, s);
-        tc_transform(op, m, op->nr, sp, true, v.z, st, kActive, nullptr, nullptr, s, -1, v.pa, v.pb, v.x, sc);
-        return;
+        tc_mode_solve(op, m, v.z, v.q, sp, st, kLive, s, dm ? prz : nullptr, dm ? beta : Finish{});
       }
       {
         ProfScope ps(w, kProfDstInv, units, s);
-        tc_transform(op, m, op->nr, sp, true, v.z, st, kActive, dm ? nullptr : v.r, dm ? nullptr : prz, s, -1, nullptr,
-                     nullptr, nullptr, sc);
+        if (fused)
+          tc_transform(op, m, op->nr, sp, true, v.z, st, kLive, nullptr, nullptr, s, -1, v.pa, v.pb, v.x, sc);
+        else
+          tc_transform(op, m, op->nr, sp, true, v.z, st, kLive, dm ? nullptr : v.r, dm ? nullptr : prz, s, -1, nullptr,
+                       nullptr, nullptr, sc);
       }
-      {
+      if (!dm) {
         ProfScope ps(w, kProfScalar, 0.0, s);
         note_launch();
-        sc_beta<<<m, 32, 0, s>>>(st, prz, precond_partials<T>(op, m), kActive, kActive);
+        sc_finish<<<m, 256, 0, s>>>(beta, kLive, prz, precond_partials<T>(op, m));
       }
       return;
     }
   }
-  DstArgs<T> f = dst_args<T>(op, m, op->nr, st, kActive);
+  DstArgs<T> f = dst_args<T>(op, m, op->nr, st, kLive);
   f.in = v.q;
   f.out = v.z;
   f.x = v.x;
@@ -1608,24 +1621,16 @@ void pcg_iteration(const ax_operator *op, int m, const PcgVecs<T> &v, RhsState *
   f.pa = v.pa;
   f.pb = v.pb;
   f.partial = prr;
+  f.fin = upd;
   { ProfScope ps(w, kProfDstFwd, units, s); launch_dst<T>(kDstPcgForward, f, s); }
-  {
-    ProfScope ps(w, kProfScalar, 0.0, s);
-    note_launch();
-    sc_after_update<<<m, 32, 0, s>>>(st, prr, nbd, on_converge);
-  }
-  { ProfScope ps(w, kProfTridiag, units, s); launch_tridiag<T>(tri_args<T>(op, m, v.z, v.z, st, kActive), s); }
-  DstArgs<T> b = dst_args<T>(op, m, op->nr, st, kActive);
+  { ProfScope ps(w, kProfTridiag, units, s); launch_tridiag<T>(tri_args<T>(op, m, v.z, v.z, st, kLive), s); }
+  DstArgs<T> b = dst_args<T>(op, m, op->nr, st, kLive);
   b.in = v.z;
   b.out = v.z;
   b.r = v.r;
   b.partial = prz;
+  b.fin = beta;
   { ProfScope ps(w, kProfDstInv, units, s); launch_dst<T>(kDstPcgInverse, b, s); }
-  {
-    ProfScope ps(w, kProfScalar, 0.0, s);
-    note_launch();
-    sc_beta<<<m, 32, 0, s>>>(st, prz, nbd, kActive, kActive);
-  }
 }
 
 // Chebyshev step for RHS in kActive: res = A y - phi, test, ybar = y - tau
@@ -1639,8 +1644,6 @@ struct ChebVecs {
 template <typename T>
 void cheb_iteration(const ax_operator *op, int m, const ChebVecs<T> &v, RhsState *st, Workspace *w,
                     int on_converge, int parity, cudaStream_t s, bool check = true) {
-  const int V = VecT<T>::n;
-  const int nbs = stencil_blocks_per_rhs(op->nr, op->nz, V);
   double *prr = part_ptr(w, kPartB);
   T *y = parity ? v.yb : v.ya;
   T *yprev = parity ? v.ya : v.yb;
@@ -1649,9 +1652,9 @@ void cheb_iteration(const ax_operator *op, int m, const ChebVecs<T> &v, RhsState
   sa.out = v.res;
   sa.phi = v.phi;
   sa.partial = check ? prr : nullptr;  // no reduction on the steps between checks
+  sa.fin = make_fin(w, st, kFinCheb, on_converge);
+  sa.fin.check = check ? 1 : 0;
   launch_stencil<T>(kStencilCheb, sa, s);
-  note_launch();
-  sc_cheb<<<m, 32, 0, s>>>(st, prr, nbs, w->chp, on_converge, check ? 1 : 0);
   DstArgs<T> f = dst_args<T>(op, m, op->nr, st, kActive);
   f.in = v.res;
   f.out = v.res;
@@ -1681,9 +1684,26 @@ void lat_mark(Workspace *w, const RhsState *h, int m) {
     if (w->lat_ms[i] < 0.0 && (h[i].state == kDone || h[i].state == kFailed)) w->lat_ms[i] = now;
 }
 
-// Runs `iters` captured iterations of `body` on stream s (graph cached by key).
+// Runs a block of iterations, `body`, on stream s: as a captured graph (cached
+// by key), or launch by launch the first kDirectBlocks times a key is met.
+// Capturing and instantiating a block of 16 iterations costs the host about as
+// much as launching its kernels twice, and unlike the launches does not
+// overlap the GPU's work: an operator that is used once never pays for it.
+constexpr int kDirectBlocks = 2;
 template <typename F>
 int run_graph(Workspace *w, GraphCache &g, int key, cudaStream_t s, F body) {
+  if (g.exec == nullptr || g.key != key) {
+    if (g.direct_key != key) {
+      g.direct_key = key;
+      g.direct = 0;
+    }
+    if (g.direct < kDirectBlocks) {
+      ++g.direct;
+      body(s);
+      AX_CHECK_LAUNCH();
+      return AX_OK;
+    }
+  }
   if (g.exec == nullptr || g.key != key) {
     std::lock_guard<std::recursive_mutex> lock(g_alloc_capture_mutex);
     free_graph(g);
@@ -1721,6 +1741,10 @@ bool any_state(const RhsState *h, int m, int state) {
   return false;
 }
 
+bool unfinished(const RhsState *h, int m) {
+  return any_state(h, m, kActive) || any_state(h, m, kCheck) || any_state(h, m, kRedo);
+}
+
 // PCG for the vectors v with right-hand side phi (in v.r on entry as the
 // residual).  Assumes st has been started (sc_start) and x holds the start.
 // If `true_check`, right-hand sides whose recursive residual passes get an
@@ -1730,20 +1754,15 @@ template <typename T>
 int pcg_loop(ax_operator *op, int m, const PcgVecs<T> &v, const T *phi, RhsState *st, GraphCache &g, bool true_check,
              cudaStream_t s) {
   Workspace *w = op->ws;
-  const int V = VecT<T>::n;
-  const int nbs = stencil_blocks_per_rhs(op->nr, op->nz, V);
-  const int nbd = precond_partials<T>(op, m);
-  // z = B^-1 r, rho = (r, z), p = 0 so that p_1 = z
-  precond_apply<T>(op, m, v.r, v.z, st, kActive, part_ptr(w, kPartC), s, v.q);
-  note_launch();
-  sc_rho_init<<<m, 32, 0, s>>>(st, part_ptr(w, kPartC), nbd, kActive);
-  AX_TRY(cudaMemsetAsync(v.pa, 0, sizeof(T) * field_elems(op) * m, s));
+  // z = B^-1 r, rho = (r, z), beta = 0 so that p_1 = z
+  precond_apply<T>(op, m, v.r, v.z, st, kActive, part_ptr(w, kPartC), s, v.q, make_fin(w, st, kFinRho));
   AX_CHECK_LAUNCH();
   const int on_conv = true_check ? kCheck : kDone;
   const int K = w->graph_iters;
   const int key = m * 4 + (true_check ? 1 : 0);
   // True-residual test of the right-hand sides in kCheck, inside the graph
-  // after every iteration (the kernels return at once for the others).
+  // after every iteration (the kernel returns at once for the others); one that
+  // fails it takes z, beta and p from the new r in the next iteration (kRedo).
   auto check_step = [&](cudaStream_t ss) {
     if (!true_check) return;
     StencilArgs<T> ra = stencil_args<T>(op, m, st, kCheck);
@@ -1751,12 +1770,8 @@ int pcg_loop(ax_operator *op, int m, const PcgVecs<T> &v, const T *phi, RhsState
     ra.phi = phi;
     ra.out_res = v.r;
     ra.partial = part_ptr(w, kPartB);
+    ra.fin = make_fin(w, st, kFinTrueCheck);
     launch_stencil<T>(kStencilResidual, ra, ss);
-    note_launch();
-    sc_true_check<<<m, 32, 0, ss>>>(st, part_ptr(w, kPartB), nbs);
-    precond_apply<T>(op, m, v.r, v.z, st, kCheck, part_ptr(w, kPartC), ss, v.q);
-    note_launch();
-    sc_beta<<<m, 32, 0, ss>>>(st, part_ptr(w, kPartC), nbd, kCheck, kActive);
   };
   const double per_rhs = (double)op->nr * op->nz;
   for (int guard = 0; guard < 1000000; ++guard) {
@@ -1780,7 +1795,7 @@ int pcg_loop(ax_operator *op, int m, const PcgVecs<T> &v, const T *phi, RhsState
     if (rc != AX_OK) return rc;
     if ((rc = read_states(w, st, m, s, h)) != AX_OK) return rc;
     if (true_check) lat_mark(w, h, m);
-    if (!any_state(h, m, kActive) && !any_state(h, m, kCheck)) break;
+    if (!unfinished(h, m)) break;
   }
   return AX_OK;
 }
@@ -1902,6 +1917,7 @@ int cheb_estimate(ax_operator *op, int m, cudaStream_t s, std::vector<int> *step
       init[i].max_iter = k;
       init[i].thresh2 = 0.0;
       init[i].bb = 1.0;
+      init[i].xbase = -1;
     }
     AX_TRY(cudaMemcpyAsync(w->st, init.data(), sizeof(RhsState) * m, cudaMemcpyHostToDevice, s));
   }
@@ -1909,11 +1925,7 @@ int cheb_estimate(ax_operator *op, int m, cudaStream_t s, std::vector<int> *step
   note_launch();
   sc_lanczos_stop<<<m, 32, 0, s>>>(w->st, part_ptr(w, kPartD), (op->nr + 15) / 16, 1e-12);
   PcgVecs<float> v{w->x32, w->r32, w->pa32, w->pb32, w->q32, w->z32};
-  const int nbd = precond_partials<float>(op, m);
-  precond_apply<float>(op, m, v.r, v.z, w->st, kActive, part_ptr(w, kPartC), s, v.q);
-  note_launch();
-  sc_rho_init<<<m, 32, 0, s>>>(w->st, part_ptr(w, kPartC), nbd, kActive);
-  AX_TRY(cudaMemsetAsync(v.pa, 0, sizeof(float) * n, s));
+  precond_apply<float>(op, m, v.r, v.z, w->st, kActive, part_ptr(w, kPartC), s, v.q, make_fin(w, w->st, kFinRho));
   for (int j = 0; j < k; ++j) {
     pcg_iteration<float>(op, m, v, w->st, w, kDone, s);
     note_launch();
@@ -2049,17 +2061,6 @@ int cheb_loop(ax_operator *op, int m, const ChebVecs<T> &v, RhsState *st, GraphC
   return AX_OK;
 }
 
-// Stores sum(partials) of each right-hand side into gate_phi (which = 0) or
-// gate_res (which = 1).
-__global__ void sc_store_gate(RhsState *st, const double *p, int nb, int which) {
-  const int m = blockIdx.x;
-  const double v = reduce_part(p + (size_t)m * kPartialStride, nb);
-  if (threadIdx.x == 0) {
-    if (which == 0) st[m].gate_phi = v;
-    else st[m].gate_res = v;
-  }
-}
-
 // Initial-guess gate.  CG reduces the error in the energy norm, and a learned
 // guess is typically close to the solution in that norm while its small
 // high-frequency errors make the plain residual norm large; so the guess of a
@@ -2069,32 +2070,30 @@ __global__ void sc_store_gate(RhsState *st, const double *p, int nb, int which) 
 // restart from zero; `restart` re-runs the residual and start kernels for all
 // right-hand sides.  phiT and r0T hold phi and the guess residual in the
 // working precision; zbuf and tmp are scratch.  accepted[i] = 1 if kept.
+// zout: where B^-1 r0 goes (null: zbuf; with dot_only it need not be formed).
+// rho of the state becomes (r0, B^-1 r0), so that a solve whose guesses were
+// all kept (*restarted false) starts from zout.
 template <typename T, typename F>
-int gate_guess(ax_operator *op, int m, RhsState *st, const T *phiT, const T *r0T, T *zbuf, T *tmp,
-               std::vector<int> &accepted, cudaStream_t s, F restart) {
+int gate_guess(ax_operator *op, int m, RhsState *st, const T *phiT, const T *r0T, T *zbuf, T *tmp, T *zout,
+               std::vector<int> &accepted, bool *restarted, cudaStream_t s, F reject) {
   Workspace *w = op->ws;
-  const int nbd = precond_partials<T>(op, m);
-  precond_apply<T>(op, m, phiT, zbuf, st, -1, part_ptr(w, kPartC), s, tmp);
-  note_launch();
-  sc_store_gate<<<m, 32, 0, s>>>(st, part_ptr(w, kPartC), nbd, 0);
-  precond_apply<T>(op, m, r0T, zbuf, st, -1, part_ptr(w, kPartC), s, tmp);
-  note_launch();
-  sc_store_gate<<<m, 32, 0, s>>>(st, part_ptr(w, kPartC), nbd, 1);
+  precond_apply<T>(op, m, phiT, zbuf, st, -1, part_ptr(w, kPartC), s, tmp, make_fin(w, st, kFinGatePhi), nullptr,
+                   true);
+  precond_apply<T>(op, m, r0T, zbuf, st, -1, part_ptr(w, kPartC), s, tmp, make_fin(w, st, kFinGateRes), zout);
   AX_CHECK_LAUNCH();
   int rc = read_states(w, st, m, s, w->h_st);
   if (rc != AX_OK) return rc;
-  const size_t field = field_elems(op);
-  bool any = false;
+  *restarted = false;
   for (int i = 0; i < m; ++i) {
     const RhsState &h = w->h_st[i];
     const bool ok = std::isfinite(h.gate_res) && std::isfinite(h.rr) && h.gate_res < h.gate_phi;
     accepted[i] = ok ? 1 : 0;
-    if (!ok) {
-      any = true;
-      AX_TRY(cudaMemsetAsync(w->x64 + (size_t)i * field, 0, field * sizeof(double), s));
-    }
+    if (!ok) *restarted = true;
   }
-  if (any) restart();
+  if (*restarted) {
+    rc = reject(accepted);
+    if (rc != AX_OK) return rc;
+  }
   AX_CHECK_LAUNCH();
   return AX_OK;
 }
@@ -2106,138 +2105,125 @@ int gate_guess(ax_operator *op, int m, RhsState *st, const T *phiT, const T *r0T
 // recursive residual), then x += x32 and the true residual phi - A x
 // (double-float) replaces r; the next iteration continues from it with the
 // same search direction.  It stops when the true residual meets tol.
-int pcg_mixed_loop(ax_operator *op, int m, double tol, double delta, int max_iter, bool check_guess,
-                   std::vector<int> &accepted, cudaStream_t s) {
+//
+// The whole solve, from the dense right-hand sides fd to the dense solutions ud
+// (in: the guesses with `guess`): phi and x are formed and read back as
+// double-float pairs directly, without FP64 fields in between.
+int pcg_mixed_solve(ax_operator *op, const double *fd, double *ud, int m, double tol, double delta, int max_iter,
+                    bool guess, bool check_guess, std::vector<int> &accepted, cudaStream_t s) {
   Workspace *w = op->ws;
   RhsState *st = w->st;
+  const int nr = op->nr, nz = op->nz, P = op->pitch;
   const size_t field = field_elems(op);
-  const int nbdf = residual_df_blocks(op->nr, op->nz);
-  const int nbf = (op->nr + 15) / 16;
-  const int nbd = precond_partials<float>(op, m);
+  const bool fused = tc_fused(op);
+  const int xoff = fused ? 1 : 0;  // the iterate update follows the iteration count (see RhsState::xbase)
   PcgVecs<float> v{w->x32, w->r32, w->pa32, w->pb32, w->q32, w->z32};
-  const size_t nall = field * m;
-  const unsigned cblocks = (unsigned)std::min<size_t>((nall + 255) / 256, 65535);
-  // up to ~8k CTAs in all for the replacement fold (see fold_df): many per
-  // right-hand side, since only the few that are due at a step do work
-  const unsigned fold_x = (unsigned)std::max<size_t>(
-      1, std::min<size_t>((field / 4 + 255) / 256, (size_t)std::max(16, 8192 / std::max(1, m))));
-  const dim3 zg(fold_x, m);
   // The true residual phi - A x in double-float (x and phi as FP32 pairs, the
-  // FP64 coefficients as FP32 + low part): FP32 arithmetic throughout.
-  auto residual64 = [&](int mask, cudaStream_t ss) {
+  // FP64 coefficients as FP32 + low part): FP32 arithmetic throughout.  With
+  // fold, x + x32 becomes the new x first.
+  auto residual = [&](bool fold, int mask, int fin_kind, cudaStream_t ss) {
     DfResidualArgs ra{};
     ra.CRh = op->c32.CR; ra.CRl = op->c32.CRl;
     ra.CZh = op->c32.CZ; ra.CZl = op->c32.CZl;
     ra.Wh = op->c32.W; ra.Wl = op->c32.Wl;
     ra.cstride = op->cstride;
     ra.czstride = op->czstride;
-    ra.nr = op->nr; ra.nz = op->nz; ra.pitch = op->pitch; ra.pitchz = op->pitchz;
+    ra.nr = nr; ra.nz = nz; ra.pitch = P; ra.pitchz = op->pitchz;
     ra.field = (long long)field;
     ra.m = m;
-    ra.xh = w->xh; ra.xl = w->xl; ra.ph = w->phh; ra.pl = w->phl;
+    for (int b = 0; b < 2; ++b) {
+      ra.xh[b] = w->xh[b];
+      ra.xl[b] = w->xl[b];
+    }
+    ra.d = fold ? w->x32 : nullptr;
+    ra.zero_start = guess ? 0 : 1;
+    ra.ph = w->phh; ra.pl = w->phl;
     ra.r32 = w->r32;
     ra.st = st;
     ra.mask = mask;
     ra.partial = part_ptr(w, kPartB);
-    ProfScope ps(w, kProfOuter, (double)op->nr * op->nz * m, ss);
+    ra.fin = make_fin(w, st, fin_kind);
+    ra.fin.xoff = xoff;
+    ra.fin.max_iter = max_iter;
+    ra.fin.bb = part_ptr(w, kPartD);
+    ra.fin.nbb = (nr + kPrepRows - 1) / kPrepRows;
+    ProfScope ps(w, kProfOuter, (double)nr * nz * m, ss);
     launch_residual_df(ra, ss);
   };
-  auto start = [&]() {
+  // sigma, then phi (and the guess) as pairs; without a guess r = phi starts the
+  // iteration at once
+  {
+    const int nb = std::max(1, std::min((nr + 3) / 4, std::max(16, 2432 / m)));
     note_launch();
-    to_df<<<cblocks, 256, 0, s>>>(w->x64, w->xh, w->xl, nall);
-    residual64(-1, s);
+    mixed_peak<<<dim3(m, nb), 256, 0, s>>>(fd, op->c64.R, nr, nz, part_ptr(w, kPartC), w->rscale, w->arrive, w->par,
+                                           tol * tol, delta * delta, w->chk);
+    Finish fin = make_fin(w, st, guess ? kFinNone : kFinStart);
+    fin.xoff = xoff;
+    fin.max_iter = max_iter;
     note_launch();
-    sc_mixed_start<<<m, 32, 0, s>>>(st, part_ptr(w, kPartB), nbdf, part_ptr(w, kPartD), nbf, tol * tol,
-                                    delta * delta, max_iter);
-  };
-  note_launch();
-  to_df<<<cblocks, 256, 0, s>>>(w->phi64, w->phh, w->phl, nall);
-  AX_TRY(cudaMemsetAsync(w->chk, 0, 2 * sizeof(int), s));
-  // Residual replacement, inside the captured graph after every iteration: the
-  // right-hand sides marked due went through the whole iteration (z and beta
-  // from their recursive residual); x32 is folded into the double-float x and
-  // r is replaced by the true residual, which the next iteration's update
-  // continues from.  Where the true residual differs from the recursive one
-  // (kCheck), z and beta are recomputed from it.  Every kernel returns at once
-  // for the others; no right-hand side waits for the host.
-  const bool fused = tc_fused(op);
-  auto replace_step = [&](cudaStream_t ss) {
-    note_launch();
-    fold_df<<<zg, 256, 0, ss>>>(w->xh, w->xl, w->x32, field, st, kDue);
-    residual64(kDue, ss);
-    note_launch();
-    sc_mixed_replace<<<m, 32, 0, ss>>>(st, part_ptr(w, kPartB), nbdf, tol * tol, delta * delta, w->chk);
-    if (fused) {
-      // z = B^-1 r and beta from the true residual, then the direction of this
-      // step again, p_new = z + beta p_old (x already holds alpha p_old).  The
-      // launches are gated by the count of right-hand sides in kCheck, which
-      // is usually 0: they then return at once, where they would otherwise
-      // walk their tile lists or grids (sc_promote resets the count); the mode
-      // solves run on a short grid of CTAs looping over the tiles
-      unsigned char *sp = w->split;
-      const int *gate = w->replace_gate ? w->chk : nullptr;
-      tc_split(op, m, op->nr, v.r, sp, st, kCheck, ss, gate);
-      const bool sc = tc_scaled(op, m);
-      tc_transform(op, m, op->nr, sp, false, v.z, st, kCheck, nullptr, nullptr, ss, -1, nullptr, nullptr, nullptr, sc,
-                   tc_tr_mode(op, m), gate);
-      tc_mode_solve(op, m, v.z, v.q, sp, st, kCheck, ss, part_ptr(w, kPartC), gate);
-      note_launch();
-      sc_beta<<<m, 32, 0, ss>>>(st, part_ptr(w, kPartC), nbd, kCheck, kCheck, 1);
-      tc_transform(op, m, op->nr, sp, true, v.z, st, kCheck, nullptr, nullptr, ss, -1, v.pa, v.pb, nullptr, sc, false,
-                   gate);
-      note_launch();
-      sc_promote<<<(m + 31) / 32, 32, 0, ss>>>(st, m, kCheck, kActive, w->chk);
-      return;
-    }
-    precond_apply<float>(op, m, v.r, v.z, st, kCheck, part_ptr(w, kPartC), ss, v.q);
-    note_launch();
-    sc_beta<<<m, 32, 0, ss>>>(st, part_ptr(w, kPartC), nbd, kCheck, kActive, 1);
-  };
-  start();
-  if (check_guess) {
-    const size_t n = field * m;
-    note_launch();
-    to_precision<float><<<(unsigned)std::min<size_t>((n + 255) / 256, 65535), 256, 0, s>>>(w->phi64, w->pa32, n);
-    int grc = gate_guess<float>(op, m, st, w->pa32, w->r32, w->z32, w->q32, accepted, s, start);
-    if (grc != AX_OK) return grc;
+    mixed_prep<<<dim3(m, (nr + kPrepRows - 1) / kPrepRows), 256, 0, s>>>(
+        fd, guess ? ud : nullptr, op->c64.R, w->rscale, nr, nz, P, w->phh, w->phl, guess ? nullptr : w->r32, w->xh[0],
+        w->xl[0], part_ptr(w, kPartD), fin);
   }
-  AX_TRY(cudaMemsetAsync(w->x32, 0, sizeof(float) * field * m, s));
+  if (guess) residual(false, -1, kFinStart, s);
   AX_CHECK_LAUNCH();
-  precond_apply<float>(op, m, v.r, v.z, st, kActive, part_ptr(w, kPartC), s, v.q);
-  note_launch();
-  sc_rho_init<<<m, 32, 0, s>>>(st, part_ptr(w, kPartC), nbd, kActive);
-  AX_TRY(cudaMemsetAsync(v.pa, 0, sizeof(float) * field * m, s));
-  // fused iteration: the first direction p_0 = z_0, where an even iteration
-  // count finds it (pb)
-  if (fused) AX_TRY(cudaMemcpyAsync(v.pb, v.z, sizeof(float) * field * m, cudaMemcpyDeviceToDevice, s));
+  // z = B^-1 r and rho; the fused iteration finds its first direction p_0 = z_0
+  // where an even iteration count looks (pb)
+  float *z0 = fused ? v.pb : v.z;
+  bool started = false;
+  if (check_guess) {
+    bool restarted = false;
+    auto reject = [&](const std::vector<int> &ok) -> int {
+      for (int i = 0; i < m; ++i)
+        if (!ok[i]) {
+          AX_TRY(cudaMemsetAsync(w->xh[0] + (size_t)i * field, 0, field * sizeof(float), s));
+          AX_TRY(cudaMemsetAsync(w->xl[0] + (size_t)i * field, 0, field * sizeof(float), s));
+        }
+      residual(false, -1, kFinStart, s);
+      return AX_OK;
+    };
+    const int grc = gate_guess<float>(op, m, st, w->phh, w->r32, v.z, v.q, z0, accepted, &restarted, s, reject);
+    if (grc != AX_OK) return grc;
+    started = !restarted;
+  }
+  if (!started)
+    precond_apply<float>(op, m, v.r, v.z, st, kActive, part_ptr(w, kPartC), s, v.q, make_fin(w, st, kFinRho), z0);
   AX_CHECK_LAUNCH();
+  // A block of iterations.  Residual replacement happens inside it after every
+  // iteration: the right-hand sides marked due went through the whole iteration
+  // (z and beta from their recursive residual); x32 is folded into the
+  // double-float x and r is replaced by the true residual, which the next
+  // iteration's update continues from.  Where the true residual differs from
+  // the recursive one the next iteration recomputes z and beta from it (kRedo).
+  // The kernel returns at once for the others; no right-hand side waits for the
+  // host.
   const int K = w->graph_iters;
-  const int key = m * 4 + 3;
-  const double per_rhs = (double)op->nr * op->nz;
+  const int key = m * 8 + 3 + (guess ? 4 : 0);
+  const double per_rhs = (double)nr * nz;
   for (int guard = 0; guard < 1000000; ++guard) {
     int rc = AX_OK;
     RhsState *h = w->h_st;
     if (w->profile) {
       if ((rc = read_states(w, st, m, s, h)) != AX_OK) return rc;
       pcg_iteration<float>(op, m, v, st, w, kDue, s, per_rhs * count_state(h, m, kActive), fused);
-      replace_step(s);
+      residual(true, kDue, kFinReplace, s);
       AX_CHECK_LAUNCH();
     } else {
       rc = run_graph(w, w->g32, key, s, [&](cudaStream_t cs) {
         for (int k = 0; k < K; ++k) {
           pcg_iteration<float>(op, m, v, st, w, kDue, cs, 0.0, fused);
-          replace_step(cs);
+          residual(true, kDue, kFinReplace, cs);
         }
       });
     }
     if (rc != AX_OK) return rc;
     if ((rc = read_states(w, st, m, s, h)) != AX_OK) return rc;
     lat_mark(w, h, m);
-    if (!any_state(h, m, kActive) && !any_state(h, m, kCheck)) break;
+    if (!unfinished(h, m)) break;
   }
-  // the iterate back in FP64
   note_launch();
-  from_df<<<cblocks, 256, 0, s>>>(w->xh, w->xl, w->x64, nall);
+  mixed_result<<<dim3(m, std::max(1, std::min(nr, std::max(64, 9728 / m)))), 256, 0, s>>>(
+      w->xh[0], w->xl[0], w->xh[1], w->xl[1], w->rscale, st, guess ? 0 : 1, nr, nz, P, ud);
   AX_CHECK_LAUNCH();
   return AX_OK;
 }
@@ -2497,6 +2483,7 @@ int ax_autotune(ax_operator *op, int32_t m, int32_t reps, void *stream) {
     init[i].max_iter = 1 << 30;
     init[i].thresh2 = -1.0;
     init[i].bb = 1.0;
+    init[i].xbase = -1;
   }
   TuneChoice best;
   best.ms = -1.0;
@@ -2505,12 +2492,9 @@ int ax_autotune(ax_operator *op, int32_t m, int32_t reps, void *stream) {
     const bool fused = tc_fused(op);
     AX_TRY(cudaMemsetAsync(w->r32, 0x3f, sizeof(float) * n, s));  // 0x3f3f3f3f: 0.747
     AX_TRY(cudaMemsetAsync(w->x32, 0, sizeof(float) * n, s));
-    AX_TRY(cudaMemsetAsync(v.pa, 0, sizeof(float) * n, s));
     AX_TRY(cudaMemcpyAsync(w->st, init.data(), sizeof(RhsState) * m, cudaMemcpyHostToDevice, s));
-    precond_apply<float>(op, m, v.r, v.z, w->st, kActive, part_ptr(w, kPartC), s, v.q);
-    note_launch();
-    sc_rho_init<<<m, 32, 0, s>>>(w->st, part_ptr(w, kPartC), precond_partials<float>(op, m), kActive);
-    if (fused) AX_TRY(cudaMemcpyAsync(v.pb, v.z, sizeof(float) * n, cudaMemcpyDeviceToDevice, s));
+    precond_apply<float>(op, m, v.r, v.z, w->st, kActive, part_ptr(w, kPartC), s, v.q, make_fin(w, w->st, kFinRho),
+                         fused ? v.pb : v.z);
     for (int i = 0; i < 2; ++i) pcg_iteration<float>(op, m, v, w->st, w, kDone, s, 0.0, fused);
     cudaEventRecord(e0, s);
     for (int i = 0; i < reps; ++i) pcg_iteration<float>(op, m, v, w->st, w, kDone, s, 0.0, fused);
@@ -2562,7 +2546,7 @@ int ax_get_option(const ax_operator *op, const char *name, double *value) {
   else if (!strcmp(name, "replace_gate")) *value = w->replace_gate;
   else if (!strcmp(name, "replace_checks")) {  // read-only: synchronises the device
     int h = 0;
-    if (w->chk != nullptr && cudaMemcpy(&h, w->chk + 1, sizeof(int), cudaMemcpyDeviceToHost) != cudaSuccess)
+    if (w->chk != nullptr && cudaMemcpy(&h, w->chk, sizeof(int), cudaMemcpyDeviceToHost) != cudaSuccess)
       return AX_ERR_CUDA;
     *value = h;
   }
@@ -2620,12 +2604,10 @@ int ax_set_option(ax_operator *op, const char *name, double value) {
     w->tc_unfused = value == 0.0;
     free_graph(w->g32);
   } else if (!strcmp(name, "replace_gate")) {
-    // 1 (default): the z recomputation of the residual-replacement step
-    // (tensor-core path) returns at once when no right-hand side needs it; 0:
-    // its launches walk their grids regardless.  Results are the same
+    // accepted for callers that set it: the z recomputation of the
+    // residual-replacement step is part of the iteration's own launches
     if (value != 0.0 && value != 1.0) return AX_ERR_INVALID_ARG;
     w->replace_gate = (int)value;
-    free_graph(w->g32);
   } else if (!strcmp(name, "small_path")) {
     // AX_PCG_FP64 of one right-hand side on a small grid as one persistent
     // launch (1, default) or through the graph-replayed kernels (0)
@@ -2938,12 +2920,14 @@ static int apply_step(ax_operator *op, const double *in, double *out, int m, int
                       cudaStream_t s, bool tc = false, int tc_three = 0) {
   Workspace *w = op->ws;
   const size_t field = (size_t)rows_per * op->pitch;
-  int rc = ensure_scratch(op, 2 * field * m * sizeof(T));
+  // b also holds the mode-major field between the tensor-core transforms
+  const size_t fb = tc ? std::max(field, (size_t)op->nz * op->tpitch) : field;
+  int rc = ensure_scratch(op, (field + fb) * m * sizeof(T));
   if (rc != AX_OK) return rc;
   if (tc && (rc = ensure_split(op, (size_t)m * split_geom(op, rows_per).bytes_per_rhs)) != AX_OK) return rc;
   T *a = reinterpret_cast<T *>(w->scratch);
   T *b = a + field * m;
-  AX_TRY(cudaMemsetAsync(w->scratch, 0, 2 * field * m * sizeof(T), s));
+  AX_TRY(cudaMemsetAsync(w->scratch, 0, (field + fb) * m * sizeof(T), s));
   const long long rows = (long long)rows_per * m;
   const int blocks = (int)std::min<long long>(rows, 65535);
   note_launch();
@@ -3132,6 +3116,8 @@ int ax_solve(ax_operator *op, const double *f, double *u, int32_t m, double tol,
   const size_t field = field_elems(op), dense = (size_t)nr * nz * m;
   int rc;
   if ((rc = ensure_base(op, m)) != AX_OK) return rc;
+  const bool direct_mixed = method == AX_PCG_MIXED && !w->mixed_restart;  // forms phi and x by itself
+  if (!direct_mixed && (rc = ensure_field64(op, m)) != AX_OK) return rc;
   if (method == AX_PCG_FP64 && !(flags & (AX_FLAG_HOST_BUFFERS | AX_FLAG_USE_GUESS)) && small_applies(op, m)) {
     // the whole solve as one persistent launch
     if ((rc = ensure_vec64(op, m, false)) != AX_OK) return rc;
@@ -3152,22 +3138,24 @@ int ax_solve(ax_operator *op, const double *f, double *u, int32_t m, double tol,
   }
   const long long rows = (long long)nr * m;
   const int cblocks = (int)std::min<long long>(rows, 65535);
-  // phi = r f (FP64) and ||phi||^2 partials
-  note_launch();
-  prep_rhs<<<dim3(m, (nr + 15) / 16), 256, 0, s>>>(fd, w->phi64, op->c64.R, nr, nz, P, part_ptr(w, kPartD),
-                                                   part_ptr(w, kPartC));
   const int nbf = (nr + 15) / 16;
-  // x64: guess or zero
-  if (guess) {
-    note_launch();
-    dense_to_padded<double><<<cblocks, 256, 0, s>>>(ud, w->x64, rows, nz, P);
-  } else {
-    AX_TRY(cudaMemsetAsync(w->x64, 0, field * m * sizeof(double), s));
-  }
-  // the mixed methods solve A (sigma u) = sigma phi (see rhs_scale)
-  const bool scaled = (method == AX_PCG_MIXED || method == AX_CHEB_MIXED);
+  // the Chebyshev and restarted mixed methods solve A (sigma u) = sigma phi (see rhs_scale)
+  const bool scaled = !direct_mixed && (method == AX_PCG_MIXED || method == AX_CHEB_MIXED);
   const unsigned sblocks =
       (unsigned)std::max<size_t>(1, std::min<size_t>((field + 1023) / 1024, (8192 + (size_t)m - 1) / (size_t)m));
+  if (!direct_mixed) {
+    // phi = r f (FP64) and ||phi||^2 partials
+    note_launch();
+    prep_rhs<<<dim3(m, nbf), 256, 0, s>>>(fd, w->phi64, op->c64.R, nr, nz, P, part_ptr(w, kPartD),
+                                          part_ptr(w, kPartC));
+    // x64: guess or zero
+    if (guess) {
+      note_launch();
+      dense_to_padded<double><<<cblocks, 256, 0, s>>>(ud, w->x64, rows, nz, P);
+    } else {
+      AX_TRY(cudaMemsetAsync(w->x64, 0, field * m * sizeof(double), s));
+    }
+  }
   if (scaled) {
     note_launch();
     rhs_scale<<<(m + 31) / 32, 32, 0, s>>>(w->rscale, part_ptr(w, kPartC), nbf, m);
@@ -3208,9 +3196,18 @@ int ax_solve(ax_operator *op, const double *f, double *u, int32_t m, double tol,
     };
     start();
     AX_CHECK_LAUNCH();
-    if (check_guess &&
-        (rc = gate_guess<double>(op, m, w->st, w->phi64, w->r64, w->z64, w->q64, accepted, s, start)) != AX_OK)
-      return rc;
+    if (check_guess) {
+      bool restarted = false;
+      auto reject = [&](const std::vector<int> &ok) -> int {
+        for (int i = 0; i < m; ++i)
+          if (!ok[i]) AX_TRY(cudaMemsetAsync(w->x64 + (size_t)i * field, 0, field * sizeof(double), s));
+        start();
+        return AX_OK;
+      };
+      if ((rc = gate_guess<double>(op, m, w->st, w->phi64, w->r64, w->z64, w->q64, w->z64, accepted, &restarted, s,
+                                   reject)) != AX_OK)
+        return rc;
+    }
     if (!cheb && small_applies(op, m)) {
       if ((rc = small_pcg_run(op, s)) != AX_OK) return rc;
     } else if (!cheb) {
@@ -3236,7 +3233,7 @@ int ax_solve(ax_operator *op, const double *f, double *u, int32_t m, double tol,
     rc = finish_info(op, m, w->st, info, 0, accepted, s);
   } else {
     // ---- mixed precision
-    if ((rc = ensure_vec32(op, m, cheb)) != AX_OK) return rc;
+    if ((rc = ensure_vec32(op, m, cheb, direct_mixed)) != AX_OK) return rc;
     if (op->dst_tc) {
       // buffers and tables before any graph capture
       if ((rc = ensure_split(op, (size_t)m * split_geom(op, nr).bytes_per_rhs)) != AX_OK) return rc;
@@ -3245,9 +3242,10 @@ int ax_solve(ax_operator *op, const double *f, double *u, int32_t m, double tol,
           !tc_table(op->device, nz, cz ? kTableCosInverse : kTableSine) || !tc_flag(op->device))
         return AX_ERR_OOM;
     }
-    if (!cheb && !w->mixed_restart) {
+    if (direct_mixed) {
       // FP32 PCG with FP64 residual replacement
-      if ((rc = pcg_mixed_loop(op, m, tol, w->replace_delta, max_iter, check_guess, accepted, s)) != AX_OK)
+      if ((rc = pcg_mixed_solve(op, fd, ud, m, tol, w->replace_delta, max_iter, guess, check_guess, accepted, s)) !=
+          AX_OK)
         return rc;
       rc = finish_info(op, m, w->st, info, 1, accepted, s);
     } else {
@@ -3315,8 +3313,10 @@ int ax_solve(ax_operator *op, const double *f, double *u, int32_t m, double tol,
     note_launch();
     apply_rhs_scale<<<dim3(sblocks, m), 256, 0, s>>>(nullptr, w->x64, w->rscale, nullptr, 0, field, true);
   }
-  note_launch();
-  padded_to_dense<double><<<cblocks, 256, 0, s>>>(w->x64, ud, rows, nz, P);
+  if (!direct_mixed) {
+    note_launch();
+    padded_to_dense<double><<<cblocks, 256, 0, s>>>(w->x64, ud, rows, nz, P);
+  }
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return status_from_cuda(e);
   if (host) {

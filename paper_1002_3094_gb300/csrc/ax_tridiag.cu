@@ -25,7 +25,7 @@
 // out for one CTA instead of a multicomputer.  The data are read and written
 // once; IP is re-read from L1/L2.
 #include <algorithm>
-#include "ax_common.cuh"
+#include "ax_finish.cuh"
 
 namespace ax {
 
@@ -352,7 +352,7 @@ __global__ void __launch_bounds__(32 * WPC * CW, (32 * WPC * CW <= 512) ? 2 : 1)
   }
   if (a.partial != nullptr) {
     __shared__ double red[NT / 32];
-    const double sw = warp_sum((double)dot);
+    const double sw = warp_sum_of(dot);
     if (lane == 0) red[warp] = sw;
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -656,7 +656,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) tridiag_pipe_kernel(const TriAr
       dot = fmaf(sd[t * CW], v[t], dot);
     }
     if (a.partial != nullptr) {
-      const double sw = warp_sum((double)dot);
+      const double sw = warp_sum_of(dot);
       if (lane == 0) red[warp] = sw;
     }
     if (a.split == nullptr) {
@@ -882,7 +882,7 @@ __global__ void __launch_bounds__(32 * WPC * CW, (32 * WPC * CW <= 512) ? 2 : 1)
     pd[CW * t + wc(t)] = v[t];
   }
   if (a.partial != nullptr) {
-    const double sw = warp_sum((double)dot);
+    const double sw = warp_sum_of(dot);
     if (lane == 0) red[warp] = sw;
   }
   __syncthreads();
@@ -944,7 +944,7 @@ __global__ void __launch_bounds__(32 * WPC * CW, (32 * WPC * CW <= 512) ? 2 : 1)
 // the split operand are those of tridiag_reg2_kernel, whose layout the tile
 // keeps.
 // ---------------------------------------------------------------------------
-template <int C2, int WPC, int CW, bool LOOP>
+template <int C2, int WPC, int CW>
 __global__ void __launch_bounds__(32 * WPC * CW, (32 * WPC * CW <= 512) ? 2 : 1)
     tridiag_tr_kernel(const TriArgs<float> a) {
   constexpr int NT = 32 * WPC * CW;
@@ -954,7 +954,7 @@ __global__ void __launch_bounds__(32 * WPC * CW, (32 * WPC * CW <= 512) ? 2 : 1)
   __shared__ float xfa[CW][WPC], xfm[CW][WPC], xba[CW][WPC], xbm[CW][WPC];
   __shared__ double red[NT / 32];
   // one tile: column group cg (columns cg CW ..) of right-hand side m
-  auto tile = [&](const int cg, const int m) {
+  const int cg = blockIdx.x, m = blockIdx.y;
   const int nr = a.nr;
   float *ds = tsm3;
   const int col0 = cg * CW;
@@ -1072,7 +1072,7 @@ __global__ void __launch_bounds__(32 * WPC * CW, (32 * WPC * CW <= 512) ? 2 : 1)
     pd[CW * t + wc(t)] = v[t];
   }
   if (a.partial != nullptr) {
-    const double sw = warp_sum((double)dot);
+    const double sw = warp_sum_of(dot);
     if (lane == 0) red[warp] = sw;
   }
   __syncthreads();
@@ -1081,6 +1081,9 @@ __global__ void __launch_bounds__(32 * WPC * CW, (32 * WPC * CW <= 512) ? 2 : 1)
     for (int i = 0; i < NT / 32; ++i) tot += red[i];
     a.partial[(size_t)m * kPartialStride + cg] = tot;
   }
+  // this CTA's arrival for the scalar step, overlapped with the write-back
+  __shared__ int s_last;
+  if (threadIdx.x == 0) s_last = a.fin.kind != kFinNone && finish_arrive(a.fin, m, gridDim.x);
   // ---- write back: one thread per row, its CW columns (as tridiag_reg2_kernel)
   const int ncol = min(CW, a.nz - col0);
   for (int row = threadIdx.x; row < nr; row += NT) {
@@ -1109,43 +1112,18 @@ __global__ void __launch_bounds__(32 * WPC * CW, (32 * WPC * CW <= 512) ? 2 : 1)
       }
     }
   }
-  };
-  if constexpr (LOOP) {
-    // a launch that rarely selects a right-hand side (TriArgs::short_grid):
-    // a few CTAs per SM loop over the tiles t = (right-hand side t / ncg,
-    // column group t % ncg), after the gate (TriArgs::gate) if there is one
-    if (a.gate != nullptr && *a.gate == 0) return;  // nothing selected
-    const int ncg = (a.nz + CW - 1) / CW, ntiles = ncg * a.m;
-    for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
-      tile(t % ncg, t / ncg);
-      __syncthreads();  // the tile's shared arrays are read before the next tile writes them
-    }
-  } else {
-    tile(blockIdx.x, blockIdx.y);  // one CTA per tile
-  }
+  if (a.fin.kind == kFinNone) return;
+  __syncthreads();
+  if (s_last) finish_last(a.fin, m, a.partial + (size_t)m * kPartialStride, (int)gridDim.x, red);
 }
 
 template <int C2, int WPC, int CW>
 void launch_tridiag_tr(const TriArgs<float> &a, cudaStream_t s) {
   constexpr int NT = 32 * WPC * CW;
   const size_t smem = (size_t)(32 * WPC) * (C2 * CW + 2) * sizeof(float);
-  if (a.short_grid) {
-    ensure_smem_attr((const void *)tridiag_tr_kernel<C2, WPC, CW, true>, smem);
-    static int sms = 0;
-    if (sms == 0) {
-      int dev = 0;
-      cudaGetDevice(&dev);
-      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-      if (sms <= 0) sms = 148;
-    }
-    const long long tiles = (long long)((a.nz + CW - 1) / CW) * a.m;
-    const int grid = (int)std::min<long long>(tiles, (long long)sms * (NT <= 512 ? 2 : 1));
-    tridiag_tr_kernel<C2, WPC, CW, true><<<grid, NT, smem, s>>>(a);
-    return;
-  }
-  ensure_smem_attr((const void *)tridiag_tr_kernel<C2, WPC, CW, false>, smem);
+  ensure_smem_attr((const void *)tridiag_tr_kernel<C2, WPC, CW>, smem);
   dim3 grid((a.nz + CW - 1) / CW, a.m);
-  tridiag_tr_kernel<C2, WPC, CW, false><<<grid, NT, smem, s>>>(a);
+  tridiag_tr_kernel<C2, WPC, CW><<<grid, NT, smem, s>>>(a);
 }
 
 // ---------------------------------------------------------------------------
@@ -1304,7 +1282,7 @@ __global__ void __launch_bounds__(32 * WPC * CW, (32 * WPC * CW <= 512) ? 2 : 1)
       pd[CW * t + wc(t)] = v[t];
     }
     if (a.partial != nullptr) {
-      const double sw = warp_sum((double)dot);
+      const double sw = warp_sum_of(dot);
       if (lane == 0) red[warp] = sw;
     }
     __syncthreads();
