@@ -5,10 +5,11 @@
 // from it only if it lowers the initial residual, and always iterates to the
 // same tolerance.
 //
-// Layout: activations [B][C][H][W] (NCHW), BF16 between layers, FP32 for
-// gradients and the final output.  Conv weights [3][3][Cin][Cout]
-// ([dy+1][dx+1][ci][co], "same" cross-correlation with zero padding), FP32
-// master copy + BF16 compute copy; FP32 accumulation everywhere.
+// Inputs [B][3][H][W] (NCHW, FP32) and outputs [B][H][W]; activations between
+// layers in BF16, gradients in FP32 (see Layouts below).  Conv weights
+// [3][3][Cin][Cout] ([dy+1][dx+1][ci][co], "same" cross-correlation with zero
+// padding), FP32 master copy + packed BF16 compute copies; FP32 accumulation
+// everywhere.
 //
 // Architecture (levels H, H/2, H/4, H/8; channels c1..c4):
 //   e1a e1b | pool | e2a e2b | pool | e3a e3b | pool | b1 b2 | up |
@@ -31,370 +32,661 @@ namespace {
 
 using bf16 = __nv_bfloat16;
 
-__device__ __forceinline__ float ld_as_float(const float *p) { return *p; }
-__device__ __forceinline__ float ld_as_float(const bf16 *p) { return __bfloat162float(*p); }
-__device__ __forceinline__ void st_from_float(float *p, float v) { *p = v; }
-
-constexpr int kTile = 32;   // output tile edge (pixels)
-constexpr int kCib = 8;     // input channels per smem stage
-constexpr int kCob = 16;    // output channels per CTA
-
 // ---------------------------------------------------------------------------
-// 3x3 convolution, forward (also used for the backward-data pass with
-// flipped, transposed weights).  256 threads; each owns a 2x2 pixel block and
-// 16 output channels.  out = act(conv(in) + bias) (+ skip, into out2).
+// Layouts.  Activations are NHWC BF16, channels padded to a multiple of 8 (16
+// bytes; the padding holds zeros); gradients are NHWC FP32 with the same padding
+// (written as zeros).  Convolutions are implicit GEMMs on the tensor cores,
+// mma.sync m16n8k16 (BF16 x BF16 -> FP32): the 3 x 3 taps and chunks of 16 input
+// channels form K.  Weights are kept packed per layer as [chunk of 16 k][tap]
+// [n][16 k] BF16, once for the forward pass (n = output, k = input channel) and
+// once, taps flipped, for the backward-data pass (n = input, k = output).
+// FP32 gradients enter the tensor cores as three BF16 numbers, g = h + m + l
+// (24 bits: all of an FP32 significand), so that products and sums keep FP32
+// accuracy.
 // ---------------------------------------------------------------------------
-template <typename TIn, typename TOut>
-__global__ void __launch_bounds__(256) conv3x3_kernel(const TIn *__restrict__ in, const bf16 *__restrict__ w,
-                                                      const float *__restrict__ bias, TOut *__restrict__ out,
-                                                      const bf16 *__restrict__ skip, bf16 *__restrict__ out2,
-                                                      int Cin, int Cout, int H, int W, int relu) {
-  __shared__ float s_in[kCib][kTile + 2][kTile + 2];
-  __shared__ float s_w[kCib][9][kCob];
-  const int tiles_x = (W + kTile - 1) / kTile;
-  const int tx0 = (blockIdx.x % tiles_x) * kTile, ty0 = (blockIdx.x / tiles_x) * kTile;
-  const int co0 = blockIdx.y * kCob;
-  const int b = blockIdx.z;
-  const int t = threadIdx.x;
-  const int px = (t % 16) * 2, py = (t / 16) * 2;  // 2x2 block inside the tile
-  const size_t plane = (size_t)H * W;
-  const TIn *inb = in + (size_t)b * Cin * plane;
-  float acc[4][kCob];
-#pragma unroll
-  for (int p = 0; p < 4; ++p)
-#pragma unroll
-    for (int c = 0; c < kCob; ++c) acc[p][c] = 0.f;
+__host__ __device__ inline int pad8(int c) { return (c + 7) & ~7; }
+__host__ __device__ inline int chunks16(int c) { return (c + 15) >> 4; }
 
-  for (int ci0 = 0; ci0 < Cin; ci0 += kCib) {
-    __syncthreads();
-    for (int e = t; e < kCib * (kTile + 2) * (kTile + 2); e += 256) {
-      const int ci = e / ((kTile + 2) * (kTile + 2));
-      const int rem = e - ci * (kTile + 2) * (kTile + 2);
-      const int yy = rem / (kTile + 2), xx = rem - yy * (kTile + 2);
-      const int gy = ty0 + yy - 1, gx = tx0 + xx - 1;
-      float v = 0.f;
-      if (ci0 + ci < Cin && gy >= 0 && gy < H && gx >= 0 && gx < W)
-        v = ld_as_float(inb + (size_t)(ci0 + ci) * plane + (size_t)gy * W + gx);
-      s_in[ci][yy][xx] = v;
-    }
-    for (int e = t; e < kCib * 9 * kCob; e += 256) {
-      const int ci = e / (9 * kCob);
-      const int rem = e - ci * 9 * kCob;
-      const int tap = rem / kCob, c = rem - tap * kCob;
-      float v = 0.f;
-      if (ci0 + ci < Cin && co0 + c < Cout) v = __bfloat162float(w[((size_t)tap * Cin + ci0 + ci) * Cout + co0 + c]);
-      s_w[ci][tap][c] = v;
-    }
-    __syncthreads();
-    const int cmax = min(kCib, Cin - ci0);
-    for (int ci = 0; ci < cmax; ++ci) {
-      float nb[4][4];
-#pragma unroll
-      for (int r = 0; r < 4; ++r)
-#pragma unroll
-        for (int c = 0; c < 4; ++c) nb[r][c] = s_in[ci][py + r][px + c];
-#pragma unroll
-      for (int tap = 0; tap < 9; ++tap) {
-        const int dy = tap / 3, dx = tap % 3;
-#pragma unroll
-        for (int c = 0; c < kCob; ++c) {
-          const float wv = s_w[ci][tap][c];
-          acc[0][c] = fmaf(nb[dy][dx], wv, acc[0][c]);
-          acc[1][c] = fmaf(nb[dy][dx + 1], wv, acc[1][c]);
-          acc[2][c] = fmaf(nb[dy + 1][dx], wv, acc[2][c]);
-          acc[3][c] = fmaf(nb[dy + 1][dx + 1], wv, acc[3][c]);
-        }
-      }
-    }
-  }
-  // epilogue
-#pragma unroll
-  for (int p = 0; p < 4; ++p) {
-    const int y = ty0 + py + (p >> 1), x = tx0 + px + (p & 1);
-    if (y >= H || x >= W) continue;
-#pragma unroll
-    for (int c = 0; c < kCob; ++c) {
-      const int co = co0 + c;
-      if (co >= Cout) continue;
-      float v = acc[p][c] + (bias ? bias[co] : 0.f);
-      if (relu) v = fmaxf(v, 0.f);
-      const size_t o = ((size_t)b * Cout + co) * plane + (size_t)y * W + x;
-      st_from_float(out + o, v);
-      if (skip) out2[o] = __float2bfloat16(v + __bfloat162float(skip[o]));
-    }
-  }
-}
-
-// ---------------------------------------------------------------------------
-// 3x3 convolution, forward, on the tensor cores: implicit GEMM with
-// mma.sync m16n8k16 (BF16 inputs, FP32 accumulation).  A CTA computes a
-// 16 x 8 pixel patch (8 warps, one patch row of 16 pixels each) for 32 output
-// channels; K runs over the 9 taps x input channels in chunks of 16.
-// Shared memory holds the haloed input patch as [pixel][16 channels] and the
-// weights as [tap][32 out][16 in], so each (k, k+1) pair of a fragment is one
-// 32-bit word.
-// ---------------------------------------------------------------------------
-constexpr int kPx = 16, kPy = 8, kCo = 32;
-
-__device__ __forceinline__ void mma_bf16_16816(float (&d)[4], const unsigned (&a)[4], const unsigned (&b)[2]) {
+__device__ __forceinline__ void mma_bf16_16816(float (&d)[4], const unsigned (&a)[4], unsigned b0, unsigned b1) {
   asm volatile(
       "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
       "{%0,%1,%2,%3};\n"
       : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
+      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+__device__ __forceinline__ void ldsm4(unsigned addr, unsigned (&r)[4]) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"(addr));
+}
+__device__ __forceinline__ void ldsm4t(unsigned addr, unsigned (&r)[4]) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"(addr));
+}
+__device__ __forceinline__ void ldsm2(unsigned addr, unsigned &r0, unsigned &r1) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x2.shared.b16 {%0,%1}, [%2];" : "=r"(r0), "=r"(r1) : "r"(addr));
+}
+__device__ __forceinline__ void ldsm2t(unsigned addr, unsigned &r0, unsigned &r1) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x2.trans.shared.b16 {%0,%1}, [%2];" : "=r"(r0), "=r"(r1) : "r"(addr));
+}
+__device__ __forceinline__ void cp_async16(unsigned dst, const void *src, bool ok) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(ok ? 16 : 0) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+
+// Byte offset of the 16-byte half `half` of 32-byte row `row` in a shared array
+// of such rows: the halves are swapped in every other group of 4 rows, so that
+// the 8 rows an ldmatrix phase reads fall in distinct banks.
+__device__ __forceinline__ unsigned row32(int row, int half) {
+  return (unsigned)(row * 32 + ((half ^ ((row >> 2) & 1)) << 4));
 }
 
-template <typename TIn>
-__global__ void __launch_bounds__(256) conv3x3_mma_kernel(const TIn *__restrict__ in, const bf16 *__restrict__ w,
-                                                          const float *__restrict__ bias, bf16 *__restrict__ out,
-                                                          const bf16 *__restrict__ skip, bf16 *__restrict__ out2,
-                                                          int Cin, int Cout, int H, int W, int relu) {
-  __shared__ __align__(16) bf16 s_in[(kPy + 2) * (kPx + 2)][16];
-  __shared__ __align__(16) bf16 s_w[9][kCo][16];
-  const int tiles_x = (W + kPx - 1) / kPx;
-  const int x0 = (blockIdx.x % tiles_x) * kPx, y0 = (blockIdx.x / tiles_x) * kPy;
-  const int co0 = blockIdx.y * kCo;
+// a + b as three BF16 pairs: the high, middle and low parts (each the rounding
+// of what the ones before left).
+__device__ __forceinline__ void split3(float a, float b, unsigned &h, unsigned &m, unsigned &l) {
+  h = bf16_pack2(a, b);
+  const float ra = a - bf16_lo(h), rb = b - bf16_hi(h);
+  m = bf16_pack2(ra, rb);
+  l = bf16_pack2(ra - bf16_lo(m), rb - bf16_hi(m));
+}
+
+// ---------------------------------------------------------------------------
+// 3 x 3 convolution.  A CTA computes a patch of 8 MW rows x 16 pixels (warp w: MW
+// rows of 16 pixels) for 8 NT output channels; K runs over chunks of 16 channels
+// and, inside, the 9 taps.  Shared memory holds the haloed patch as [pixel][16
+// channels] and the chunk's weights as [tap][n][16], rows of 32 bytes read with
+// ldmatrix.  What bounds it is the tensor pipe once each fragment feeds several
+// MMAs: per tap MW + NT / 2 ldmatrix for MW NT MMAs (the kernel before read 12
+// words per lane for 4 MMAs of a 16 x 32 warp tile and converted its input
+// element by element: 45 TFLOP/s at 256 x 256, batch 16).
+//   PLANES = 1: BF16 input, forward: out = relu(conv + bias), out2 = out + skip.
+//     The order of accumulation (chunk, then tap) is that of the plain sum over K.
+//   PLANES = 3: FP32 input split in three, backward data: out = conv (* the
+//     ReLU mask of act), out2 = conv unmasked.  The tensor core's accumulation
+//     truncates (emptied once per chunk of 27 products, the gradients of all
+//     layers were 7e-7 off 64 bits against 3e-7 for FP32 FMAs), so every tap's
+//     products, the small parts first, go to a fresh accumulator that is added to
+//     the sum in FP32.
+// ---------------------------------------------------------------------------
+struct ConvArgs {
+  const void *in;       // [B][H >> up][W >> up][pad8(Cin)]
+  const bf16 *w;        // packed [chunk][9][n8][16]
+  const float *bias;    // forward
+  void *out;            // BF16 (forward) or FP32 [B][H][W][pad8(Cout)]
+  void *out2;           // second output or null
+  const bf16 *skip;     // forward with out2: added after the ReLU
+  const bf16 *mask;     // backward: activation whose sign masks out (null: none)
+  int cin, cout, H, W, up;
+};
+template <int NT, int MW, int PLANES>
+struct ConvShape {
+  static constexpr int rows = 8 * MW + 2, pix = rows * 18;
+  static constexpr int in_bytes = pix * 32 * PLANES;
+  static constexpr int w_bytes = 9 * 8 * NT * 32;
+  static constexpr int stages = PLANES == 1 ? 2 : 1;
+  static constexpr int smem = stages * (in_bytes + w_bytes);
+};
+
+template <int NT, int MW, int PLANES>
+__global__ void __launch_bounds__(256, 2) conv3x3_kernel(const ConvArgs a) {
+  using S = ConvShape<NT, MW, PLANES>;
+  extern __shared__ __align__(128) unsigned char csm[];
+  const int H = a.H, W = a.W, up = a.up;
+  const int tiles_x = (W + 15) >> 4;
+  const int x0 = (blockIdx.x % tiles_x) * 16, y0 = (blockIdx.x / tiles_x) * 8 * MW;
+  const int n0 = blockIdx.y * 8 * NT;
   const int b = blockIdx.z;
   const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
-  const int g = lane >> 2, tq = lane & 3;
-  const size_t plane = (size_t)H * W;
-  const TIn *inb = in + (size_t)b * Cin * plane;
-  float acc[4][4];
-#pragma unroll
-  for (int n = 0; n < 4; ++n)
-#pragma unroll
-    for (int c = 0; c < 4; ++c) acc[n][c] = 0.f;
-  const unsigned *sin32 = reinterpret_cast<const unsigned *>(&s_in[0][0]);
-  const unsigned *sw32 = reinterpret_cast<const unsigned *>(&s_w[0][0][0]);
-  for (int ci0 = 0; ci0 < Cin; ci0 += 16) {
-    __syncthreads();
-    for (int e = t; e < (kPy + 2) * (kPx + 2) * 16; e += 256) {
-      const int ci = e / ((kPy + 2) * (kPx + 2));
-      const int pix = e - ci * (kPy + 2) * (kPx + 2);
-      const int yy = pix / (kPx + 2), xx = pix - yy * (kPx + 2);
-      const int gy = y0 + yy - 1, gx = x0 + xx - 1;
-      float v = 0.f;
-      if (ci0 + ci < Cin && gy >= 0 && gy < H && gx >= 0 && gx < W)
-        v = ld_as_float(inb + (size_t)(ci0 + ci) * plane + (size_t)gy * W + gx);
-      s_in[pix][ci] = __float2bfloat16(v);
+  const int cpin = pad8(a.cin), n8 = pad8(a.cout);
+  const int Hs = H >> up, Ws = W >> up;
+  const int nchunk = chunks16(a.cin);
+  auto in_at = [&](int s) { return smem_u32(csm) + s * (S::in_bytes + S::w_bytes); };
+  auto w_at = [&](int s) { return in_at(s) + S::in_bytes; };
+  auto load_w = [&](int s, int k) {
+    for (int e = t; e < 9 * 8 * NT * 2; e += 256) {
+      const int half = e & 1, r = e >> 1, tap = r / (8 * NT), n = r - tap * 8 * NT;
+      const bool ok = n0 + n < n8;
+      cp_async16(w_at(s) + row32(r, half),
+                 a.w + (ok ? ((((size_t)k * 9 + tap) * n8 + n0 + n) * 16 + half * 8) : 0), ok);
     }
-    for (int e = t; e < 9 * kCo * 16; e += 256) {
-      const int tap = e / (kCo * 16);
-      const int rem = e - tap * kCo * 16;
-      const int c = rem / 16, ci = rem - c * 16;
-      bf16 v = __float2bfloat16(0.f);
-      if (ci0 + ci < Cin && co0 + c < Cout) v = w[((size_t)tap * Cin + ci0 + ci) * Cout + co0 + c];
-      s_w[tap][c][ci] = v;
+  };
+  auto load_in = [&](int s, int k) {  // PLANES == 1
+    const bf16 *in = static_cast<const bf16 *>(a.in) + (size_t)b * Hs * Ws * cpin;
+    for (int e = t; e < S::pix * 2; e += 256) {
+      const int half = e & 1, p = e >> 1, yy = p / 18, xx = p - yy * 18;
+      const int gy = y0 + yy - 1, gx = x0 + xx - 1, c = k * 16 + half * 8;
+      const bool ok = gy >= 0 && gy < H && gx >= 0 && gx < W && c < cpin;
+      cp_async16(in_at(s) + row32(p, half), in + (ok ? ((size_t)(gy >> up) * Ws + (gx >> up)) * cpin + c : 0), ok);
     }
-    __syncthreads();
+  };
+  auto load_split = [&](int k) {  // PLANES == 3
+    const float *in = static_cast<const float *>(a.in) + (size_t)b * H * W * cpin;
+    for (int e = t; e < S::pix * 2; e += 256) {
+      const int half = e & 1, p = e >> 1, yy = p / 18, xx = p - yy * 18;
+      const int gy = y0 + yy - 1, gx = x0 + xx - 1, c = k * 16 + half * 8;
+      float4 u = make_float4(0.f, 0.f, 0.f, 0.f), v = u;
+      if (gy >= 0 && gy < H && gx >= 0 && gx < W && c < cpin) {
+        const float4 *src = reinterpret_cast<const float4 *>(in + ((size_t)gy * W + gx) * cpin + c);
+        u = src[0];
+        v = src[1];
+      }
+      uint4 h, m, l;
+      split3(u.x, u.y, h.x, m.x, l.x);
+      split3(u.z, u.w, h.y, m.y, l.y);
+      split3(v.x, v.y, h.z, m.z, l.z);
+      split3(v.z, v.w, h.w, m.w, l.w);
+      unsigned char *dst = csm + row32(p, half);
+      *reinterpret_cast<uint4 *>(dst) = h;
+      *reinterpret_cast<uint4 *>(dst + S::pix * 32) = m;
+      *reinterpret_cast<uint4 *>(dst + 2 * S::pix * 32) = l;
+    }
+  };
+  float sum[MW][NT][4];
+#pragma unroll
+  for (int i = 0; i < MW; ++i)
+#pragma unroll
+    for (int n = 0; n < NT; ++n)
+#pragma unroll
+      for (int c = 0; c < 4; ++c) sum[i][n][c] = 0.f;
+  // one chunk's products into the sums
+  auto products = [&](int s) {
+    const unsigned ib = in_at(s), wb = w_at(s);
+    // ldmatrix row of this lane: A rows (pixels) lane & 15, half lane >> 4; B rows
+    // (channels) (lane & 7) + 8 (lane >> 4), half (lane >> 3) & 1
+    const int ap = lane & 15, ah = lane >> 4, bn = (lane & 7) + ((lane >> 4) << 3), bh = (lane >> 3) & 1;
 #pragma unroll
     for (int tap = 0; tap < 9; ++tap) {
       const int dy = tap / 3, dx = tap % 3;
-      // A rows: pixels x = g and x = g + 8 of patch row `warp`, shifted by the tap
-      const int p0 = (warp + dy) * (kPx + 2) + g + dx;
-      const int p1 = p0 + 8;
-      unsigned a[4];
-      a[0] = sin32[p0 * 8 + tq];
-      a[1] = sin32[p1 * 8 + tq];
-      a[2] = sin32[p0 * 8 + tq + 4];
-      a[3] = sin32[p1 * 8 + tq + 4];
+      unsigned bf[NT][2];
 #pragma unroll
-      for (int n = 0; n < 4; ++n) {
-        const int c = n * 8 + g;
-        unsigned bb[2];
-        bb[0] = sw32[(tap * kCo + c) * 8 + tq];
-        bb[1] = sw32[(tap * kCo + c) * 8 + tq + 4];
-        mma_bf16_16816(acc[n], a, bb);
+      for (int n = 0; n + 1 < NT; n += 2) {
+        unsigned r[4];
+        ldsm4(wb + row32(tap * 8 * NT + n * 8 + bn, bh), r);
+        bf[n][0] = r[0]; bf[n][1] = r[1]; bf[n + 1][0] = r[2]; bf[n + 1][1] = r[3];
+      }
+      if (NT & 1) ldsm2(wb + row32(tap * 8 * NT + (NT - 1) * 8 + (lane & 7), (lane >> 3) & 1), bf[NT - 1][0], bf[NT - 1][1]);
+#pragma unroll
+      for (int i = 0; i < MW; ++i) {
+        const int p = (warp * MW + i + dy) * 18 + dx + ap;
+        if constexpr (PLANES == 1) {
+          unsigned af[4];
+          ldsm4(ib + row32(p, ah), af);
+#pragma unroll
+          for (int n = 0; n < NT; ++n) mma_bf16_16816(sum[i][n], af, bf[n][0], bf[n][1]);
+        } else {
+          unsigned af[PLANES][4];
+#pragma unroll
+          for (int q = 0; q < PLANES; ++q) ldsm4(ib + q * S::pix * 32 + row32(p, ah), af[q]);
+#pragma unroll
+          for (int n = 0; n < NT; ++n) {
+            float acc[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+            for (int q = PLANES - 1; q >= 0; --q) mma_bf16_16816(acc, af[q], bf[n][0], bf[n][1]);
+#pragma unroll
+            for (int c = 0; c < 4; ++c) sum[i][n][c] += acc[c];
+          }
+        }
+      }
+    }
+  };
+  if constexpr (PLANES == 1) {
+    load_in(0, 0);
+    load_w(0, 0);
+    cp_async_commit();
+    for (int k = 0; k < nchunk; ++k) {
+      if (k + 1 < nchunk) {
+        load_in((k + 1) & 1, k + 1);
+        load_w((k + 1) & 1, k + 1);
+        cp_async_commit();
+        cp_async_wait<1>();
+      } else {
+        cp_async_wait<0>();
+      }
+      __syncthreads();
+      products(k & 1);
+      __syncthreads();
+    }
+  } else {
+    for (int k = 0; k < nchunk; ++k) {
+      load_w(0, k);
+      cp_async_commit();
+      load_split(k);
+      cp_async_wait<0>();
+      __syncthreads();
+      products(0);
+      __syncthreads();
+    }
+  }
+  // epilogue: sum[i][n][0..1] pixel g, channels n*8 + 2 tq + {0, 1}; [2..3] pixel g + 8
+  const int g = lane >> 2, tq = lane & 3;
+#pragma unroll
+  for (int i = 0; i < MW; ++i) {
+    const int y = y0 + warp * MW + i;
+    if (y >= H) continue;
+#pragma unroll
+    for (int hf = 0; hf < 2; ++hf) {
+      const int x = x0 + g + 8 * hf;
+      if (x >= W) continue;
+      const size_t pix = ((size_t)b * H + y) * W + x;
+#pragma unroll
+      for (int n = 0; n < NT; ++n) {
+        const int co = n0 + n * 8 + 2 * tq;
+        if (co >= n8) continue;
+        const size_t o = pix * n8 + co;
+        float v0 = sum[i][n][2 * hf], v1 = sum[i][n][2 * hf + 1];
+        if constexpr (PLANES == 1) {
+          // padding channels (their weights are zero) stay zero
+          v0 = co < a.cout ? fmaxf(v0 + a.bias[co], 0.f) : 0.f;
+          v1 = co + 1 < a.cout ? fmaxf(v1 + a.bias[co + 1], 0.f) : 0.f;
+          *reinterpret_cast<unsigned *>(static_cast<bf16 *>(a.out) + o) = bf16_pack2(v0, v1);
+          if (a.out2 != nullptr) {
+            const unsigned s = *reinterpret_cast<const unsigned *>(a.skip + o);
+            *reinterpret_cast<unsigned *>(static_cast<bf16 *>(a.out2) + o) =
+                bf16_pack2(v0 + bf16_lo(s), v1 + bf16_hi(s));
+          }
+        } else {
+          if (a.out2 != nullptr) *reinterpret_cast<float2 *>(static_cast<float *>(a.out2) + o) = make_float2(v0, v1);
+          if (a.mask != nullptr) {
+            const unsigned s = *reinterpret_cast<const unsigned *>(a.mask + o);
+            v0 = bf16_lo(s) > 0.f ? v0 : 0.f;
+            v1 = bf16_hi(s) > 0.f ? v1 : 0.f;
+          }
+          *reinterpret_cast<float2 *>(static_cast<float *>(a.out) + o) = make_float2(v0, v1);
+        }
       }
     }
   }
-  // epilogue: acc[n][0..1] pixel x = g, channels n*8 + 2tq + {0,1}; acc[n][2..3] pixel x = g + 8
-  const int y = y0 + warp;
-#pragma unroll
-  for (int n = 0; n < 4; ++n)
-#pragma unroll
-    for (int c = 0; c < 4; ++c) {
-      const int x = x0 + g + ((c >> 1) ? 8 : 0);
-      const int co = co0 + n * 8 + 2 * tq + (c & 1);
-      if (y >= H || x >= W || co >= Cout) continue;
-      float v = acc[n][c] + bias[co];
-      if (relu) v = fmaxf(v, 0.f);
-      const size_t o = ((size_t)b * Cout + co) * plane + (size_t)y * W + x;
-      out[o] = __float2bfloat16(v);
-      if (skip) out2[o] = __float2bfloat16(v + __bfloat162float(skip[o]));
-    }
 }
 
 // ---------------------------------------------------------------------------
-// Weight gradient of a 3x3 conv over one 32x32 tile of one sample:
-//   partial[tile][tap][ci][co] = sum_{pixels} in[ci][y+dy-1][x+dx-1] gz[co][y][x]
-// 144 threads: (tap, ci) x 2 halves of the 16 output channels.
+// Weight gradient of a 3 x 3 convolution,
+//   dW[tap][ci][co] = sum over pixels of in[pixel + tap][ci] gz[pixel][co],
+// as a GEMM on the tensor cores with M = 16 input channels, N = 24 output
+// channels and K = pixels; both operands are read transposed (ldmatrix.trans)
+// from their NHWC tiles.  A warp keeps all 9 taps' accumulators (108 registers):
+// each k block of 16 pixels takes 9 ldmatrix of the input (the taps' shifts) and
+// feeds 81 MMAs (9 taps x 3 n-tiles x the 3 BF16 parts of gz).  A CTA owns one
+// (ci, co) block and every gridDim.z-th 16 x 16 pixel tile, warp w the rows 2 w,
+// 2 w + 1; the next tile is loaded while one is multiplied.  The truncating
+// accumulators are emptied into FP32 sums after every tile (18 products per
+// element).  The warps' sums are added in order and written as one partial per
+// CTA: deterministic.  (Before: FP32 FMAs on CUDA cores, one partial per 32 x 32
+// tile, 18 ms of a 256 x 256 batch-16 step.)
 // ---------------------------------------------------------------------------
-template <typename TIn>
-__global__ void __launch_bounds__(144) conv3x3_wgrad_kernel(const TIn *__restrict__ in, const float *__restrict__ gz,
-                                                            float *__restrict__ partial, int Cin, int Cout, int H,
-                                                            int W) {
-  extern __shared__ __align__(16) float smem[];
-  float *s_in = smem;                                           // [kCib][34][34]
-  float *s_g = smem + kCib * (kTile + 2) * (kTile + 2);         // [1024][kCob]
-  const int tiles_x = (W + kTile - 1) / kTile, tiles_y = (H + kTile - 1) / kTile;
-  const int tile = blockIdx.x;
-  const int tx0 = (tile % tiles_x) * kTile, ty0 = (tile / tiles_x) * kTile;
-  const int ci0 = blockIdx.y * kCib;
-  const int nco = (Cout + kCob - 1) / kCob;
-  const int co0 = (blockIdx.z % nco) * kCob;
-  const int b = blockIdx.z / nco;
-  const int t = threadIdx.x;
-  const size_t plane = (size_t)H * W;
-  for (int e = t; e < kCib * (kTile + 2) * (kTile + 2); e += blockDim.x) {
-    const int ci = e / ((kTile + 2) * (kTile + 2));
-    const int rem = e - ci * (kTile + 2) * (kTile + 2);
-    const int yy = rem / (kTile + 2), xx = rem - yy * (kTile + 2);
-    const int gy = ty0 + yy - 1, gx = tx0 + xx - 1;
-    float v = 0.f;
-    if (ci0 + ci < Cin && gy >= 0 && gy < H && gx >= 0 && gx < W)
-      v = ld_as_float(in + ((size_t)b * Cin + ci0 + ci) * plane + (size_t)gy * W + gx);
-    s_in[e] = v;
+constexpr int kWgN = 24;                       // output channels per CTA
+constexpr int kWgIn = 18 * 18 * 32;            // input tile bytes (16 channels)
+constexpr int kWgG = 256 * kWgN * 2;           // bytes of one part of the gz tile
+constexpr int kWgSmem = 2 * kWgIn + 3 * kWgG;
+
+struct WgradArgs {
+  const bf16 *in;      // [B][H >> up][W >> up][cpin]
+  const float *gz;     // [B][H][W][pad8(cout)]
+  float *partial;      // [gridDim.z][9][cin][cout]
+  int cin, cpin, cout, B, H, W, up;
+};
+__global__ void __launch_bounds__(256, 1) conv3x3_wgrad_kernel(const WgradArgs a) {
+  extern __shared__ __align__(128) unsigned char wsm[];
+  const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
+  const int ci0 = blockIdx.x * 16, co0 = blockIdx.y * kWgN;
+  const int H = a.H, W = a.W, up = a.up, Hs = H >> up, Ws = W >> up, cpo = pad8(a.cout);
+  const int tx = (W + 15) >> 4, ty = (H + 15) >> 4, ntile = a.B * tx * ty;
+  const unsigned sin0 = smem_u32(wsm), sg = sin0 + 2 * kWgIn;
+  auto load_in = [&](int s, int tile) {
+    const int b = tile / (tx * ty), r = tile - b * tx * ty;
+    const int y0 = (r / tx) * 16, x0 = (r % tx) * 16;
+    const bf16 *in = a.in + (size_t)b * Hs * Ws * a.cpin;
+    for (int e = t; e < 18 * 18 * 2; e += 256) {
+      const int half = e & 1, p = e >> 1, yy = p / 18, xx = p - yy * 18;
+      const int gy = y0 + yy - 1, gx = x0 + xx - 1, c = ci0 + half * 8;
+      const bool ok = gy >= 0 && gy < H && gx >= 0 && gx < W && c < a.cpin;
+      cp_async16(sin0 + s * kWgIn + row32(p, half),
+                 in + (ok ? ((size_t)(gy >> up) * Ws + (gx >> up)) * a.cpin + c : 0), ok);
+    }
+    cp_async_commit();
+  };
+  float4 gv[6];  // the tile's gz: 256 pixels x 6 groups of 4 channels over 256 threads
+  auto load_g = [&](int tile) {
+    const int b = tile / (tx * ty), r = tile - b * tx * ty;
+    const int y0 = (r / tx) * 16, x0 = (r % tx) * 16;
+    const float *g = a.gz + (size_t)b * H * W * cpo;
+#pragma unroll
+    for (int j = 0; j < 6; ++j) {
+      const int e = t + j * 256, p = e / 6, c = co0 + (e - p * 6) * 4;
+      const int gy = y0 + (p >> 4), gx = x0 + (p & 15);
+      gv[j] = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (gy < H && gx < W && c < cpo) gv[j] = *reinterpret_cast<const float4 *>(g + ((size_t)gy * W + gx) * cpo + c);
+    }
+  };
+  auto store_g = [&]() {
+#pragma unroll
+    for (int j = 0; j < 6; ++j) {
+      const int e = t + j * 256, p = e / 6, q = e - p * 6;
+      uint2 h, m, l;
+      split3(gv[j].x, gv[j].y, h.x, m.x, l.x);
+      split3(gv[j].z, gv[j].w, h.y, m.y, l.y);
+      unsigned char *dst = wsm + 2 * kWgIn + p * (kWgN * 2) + q * 8;
+      *reinterpret_cast<uint2 *>(dst) = h;
+      *reinterpret_cast<uint2 *>(dst + kWgG) = m;
+      *reinterpret_cast<uint2 *>(dst + 2 * kWgG) = l;
+    }
+  };
+  float sum[9][3][4];
+#pragma unroll
+  for (int i = 0; i < 9; ++i)
+#pragma unroll
+    for (int n = 0; n < 3; ++n)
+#pragma unroll
+      for (int c = 0; c < 4; ++c) sum[i][n][c] = 0.f;
+  int tile = blockIdx.z, s = 0;
+  if (tile < ntile) {
+    load_in(0, tile);
+    load_g(tile);
   }
-  for (int e = t; e < kTile * kTile * kCob; e += blockDim.x) {
-    const int pix = e / kCob, c = e - pix * kCob;
-    const int y = ty0 + pix / kTile, x = tx0 + pix % kTile;
-    float v = 0.f;
-    if (co0 + c < Cout && y < H && x < W) v = gz[((size_t)b * Cout + co0 + c) * plane + (size_t)y * W + x];
-    s_g[e] = v;
+  for (; tile < ntile; tile += gridDim.z, s ^= 1) {
+    store_g();
+    const int next = tile + gridDim.z;
+    if (next < ntile) {
+      load_in(s ^ 1, next);
+      load_g(next);
+      cp_async_wait<1>();
+    } else {
+      cp_async_wait<0>();
+    }
+    __syncthreads();
+    // B parts of this warp's two k blocks; lanes 0-15 address the rows (pixels)
+    unsigned bfr[2][3][3][2];
+#pragma unroll
+    for (int kb = 0; kb < 2; ++kb)
+#pragma unroll
+      for (int q = 0; q < 3; ++q) {
+        const unsigned base = sg + q * kWgG + ((warp * 2 + kb) * 16 + (lane & 15)) * (kWgN * 2);
+        unsigned r[4];
+        ldsm4t(base + (lane >> 4) * 16, r);  // n-tiles 0 and 1
+        bfr[kb][q][0][0] = r[0]; bfr[kb][q][0][1] = r[1]; bfr[kb][q][1][0] = r[2]; bfr[kb][q][1][1] = r[3];
+        ldsm2t(base + 32, bfr[kb][q][2][0], bfr[kb][q][2][1]);
+      }
+    const unsigned ib = sin0 + s * kWgIn;
+#pragma unroll
+    for (int tap = 0; tap < 9; ++tap) {
+      const int dy = tap / 3, dx = tap % 3;
+      float acc[3][4];
+#pragma unroll
+      for (int n = 0; n < 3; ++n)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) acc[n][c] = 0.f;
+#pragma unroll
+      for (int kb = 0; kb < 2; ++kb) {
+        // A (16 ci x 16 pixels) from [pixel][ci]: matrices (k 0-7, m 0-7),
+        // (k 0-7, m 8-15), (k 8-15, m 0-7), (k 8-15, m 8-15), transposed
+        const int p = (warp * 2 + kb + dy) * 18 + dx + (lane & 7) + ((lane >> 4) << 3);
+        unsigned af[4];
+        ldsm4t(ib + row32(p, (lane >> 3) & 1), af);
+#pragma unroll
+        for (int q = 2; q >= 0; --q)
+#pragma unroll
+          for (int n = 0; n < 3; ++n) mma_bf16_16816(acc[n], af, bfr[kb][q][n][0], bfr[kb][q][n][1]);
+      }
+#pragma unroll
+      for (int n = 0; n < 3; ++n)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) sum[tap][n][c] += acc[n][c];
+    }
+    __syncthreads();
   }
+  // the 8 warps' sums in order (the tiles' shared memory is free now)
+  float *red = reinterpret_cast<float *>(wsm);
+  for (int w = 0; w < 8; ++w) {
+    if (warp == w) {
+#pragma unroll
+      for (int i = 0; i < 9; ++i)
+#pragma unroll
+        for (int n = 0; n < 3; ++n)
+#pragma unroll
+          for (int c = 0; c < 4; ++c) {
+            float *r = red + ((i * 3 + n) * 4 + c) * 32 + lane;
+            *r = (w == 0 ? 0.f : *r) + sum[i][n][c];
+          }
+    }
+    __syncthreads();
+  }
+  float *pp = a.partial + (size_t)blockIdx.z * 9 * a.cin * a.cout;
+  for (int e = t; e < 9 * 16 * kWgN; e += 256) {
+    const int tap = e / (16 * kWgN), r = e - tap * 16 * kWgN, ci = r / kWgN, co = r - ci * kWgN;
+    if (ci0 + ci >= a.cin || co0 + co >= a.cout) continue;
+    // element (row ci, column co) of the accumulator tile: rows g and g + 8 in
+    // registers {0, 1} and {2, 3}, columns 2 tq + {0, 1}
+    const int n = co >> 3, cc = ((ci >> 3) << 1) | (co & 1), ln = ((ci & 7) << 2) | ((co & 7) >> 1);
+    pp[((size_t)tap * a.cin + ci0 + ci) * a.cout + co0 + co] = red[((tap * 3 + n) * 4 + cc) * 32 + ln];
+  }
+}
+
+// out[i] = sum over the slots of partial[slot][i] (a fixed order: 8 groups of
+// slots in FP32, then the groups).  With planes = 3 (the network's FP32 input as
+// three BF16 planes of 3 channels) the three planes' rows of a partial,
+// [9][9][cout], add up to [9][3][cout].  256 threads: 32 elements x 8 groups (one
+// thread per element left most of the chip idle over a chain of up to 304
+// loads: 17 us on average, 30 launches per step).
+__global__ void __launch_bounds__(256) sum_partials(const float *__restrict__ partial, int slots, size_t n,
+                                                    float *__restrict__ out, int planes, int cout) {
+  __shared__ float red[8][32];
+  const size_t i = blockIdx.x * (size_t)32 + (threadIdx.x & 31);
+  const int grp = threadIdx.x >> 5;
+  float s = 0.f;
+  if (i < n) {
+    if (planes == 1) {
+#pragma unroll 8
+      for (int k = grp; k < slots; k += 8) s += partial[(size_t)k * n + i];
+    } else {
+      const size_t co = i % cout, r = i / cout, ci = r % 3, tap = r / 3;
+#pragma unroll 4
+      for (int k = grp; k < slots; k += 8) {
+        const float *p = partial + (size_t)k * 3 * n + (tap * 9 + ci) * cout + co;
+        s += (p[0] + p[3 * (size_t)cout]) + p[6 * (size_t)cout];
+      }
+    }
+  }
+  red[grp][threadIdx.x & 31] = s;
   __syncthreads();
-  const int half = t % 2, pair = t / 2;   // pair = tap * kCib + ci
-  const int tap = pair / kCib, ci = pair % kCib;
-  const int dy = tap / 3, dx = tap % 3;
-  float acc[8];
+  if (grp == 0 && i < n) {
+    float tot = red[0][threadIdx.x];
 #pragma unroll
-  for (int c = 0; c < 8; ++c) acc[c] = 0.f;
-  for (int pix = 0; pix < kTile * kTile; ++pix) {
-    const int y = pix / kTile, x = pix % kTile;
-    const float xv = s_in[(ci * (kTile + 2) + y + dy) * (kTile + 2) + x + dx];
-    const float4 g0 = *reinterpret_cast<const float4 *>(s_g + pix * kCob + half * 8);
-    const float4 g1 = *reinterpret_cast<const float4 *>(s_g + pix * kCob + half * 8 + 4);
-    acc[0] = fmaf(xv, g0.x, acc[0]); acc[1] = fmaf(xv, g0.y, acc[1]);
-    acc[2] = fmaf(xv, g0.z, acc[2]); acc[3] = fmaf(xv, g0.w, acc[3]);
-    acc[4] = fmaf(xv, g1.x, acc[4]); acc[5] = fmaf(xv, g1.y, acc[5]);
-    acc[6] = fmaf(xv, g1.z, acc[6]); acc[7] = fmaf(xv, g1.w, acc[7]);
+    for (int g = 1; g < 8; ++g) tot += red[g][threadIdx.x];
+    out[i] = tot;
   }
-  const size_t slot = (size_t)b * tiles_x * tiles_y + tile;
-  float *pp = partial + slot * 9 * Cin * Cout;
-  if (ci0 + ci < Cin) {
+}
+
+// Per-block sums of gz over pixels, per channel: partial[block][c] (pairs of FP32
+// numbers inside a thread and over the block's threads, fixed order).  blockDim
+// = 256: groups of cp / 4 threads walk the pixels, 4 channels each.
+__global__ void __launch_bounds__(256) channel_sums(const float *__restrict__ g, int C, int cp, size_t pixels,
+                                                    float *__restrict__ partial) {
+  __shared__ float sh[256][4], sl[256][4];
+  const int q = cp / 4, groups = max(1, 256 / q);
+  // channels beyond what one pass of the threads covers are taken in turn
+  for (int c0 = 0; c0 < q; c0 += 256) {
+    const int c = c0 + (q <= 256 ? (int)threadIdx.x % q : (int)threadIdx.x), grp = q <= 256 ? threadIdx.x / q : 0;
+    SumOf<float> s[4];
+    if (c < q && grp < groups) {
+      for (size_t p = (size_t)blockIdx.x * groups + grp; p < pixels; p += (size_t)gridDim.x * groups) {
+        const float4 v = *reinterpret_cast<const float4 *>(g + p * cp + c * 4);
+        s[0].add(v.x); s[1].add(v.y); s[2].add(v.z); s[3].add(v.w);
+      }
+    }
+    __syncthreads();
 #pragma unroll
-    for (int c = 0; c < 8; ++c) {
-      const int co = co0 + half * 8 + c;
-      if (co < Cout) pp[((size_t)tap * Cin + ci0 + ci) * Cout + co] = acc[c];
+    for (int i = 0; i < 4; ++i) {
+      sh[threadIdx.x][i] = s[i].h;
+      sl[threadIdx.x][i] = s[i].l;
+    }
+    __syncthreads();
+    if ((int)threadIdx.x < min(q, 256) && c < q) {
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        SumOf<float> tot;
+        for (int k = 0; k < groups; ++k) tot.add(sh[threadIdx.x + k * q][i], sl[threadIdx.x + k * q][i]);
+        if (c * 4 + i < C) partial[(size_t)blockIdx.x * C + c * 4 + i] = tot.h + tot.l;
+      }
     }
   }
 }
 
-// out[i] = sum_s partial[s][i], fixed order (deterministic).
-__global__ void sum_partials(const float *__restrict__ partial, int slots, size_t n, float *__restrict__ out) {
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-    float s = 0.f;
-    for (int k = 0; k < slots; ++k) s += partial[(size_t)k * n + i];
-    out[i] = s;
-  }
-}
-
-// Per-(sample, channel) sums of gz over the plane -> partial[b][c]; the bias
-// gradient is then the sum over b.
-__global__ void channel_sums(const float *__restrict__ g, int C, size_t plane, float *__restrict__ partial) {
-  __shared__ double red[8];
-  const int c = blockIdx.x, b = blockIdx.y;
-  const float *p = g + ((size_t)b * C + c) * plane;
-  double s = 0.0;
-  for (size_t i = threadIdx.x; i < plane; i += blockDim.x) s += p[i];
-  s = block_sum(s, red);
-  if (threadIdx.x == 0) partial[(size_t)b * C + c] = (float)s;
-}
-
-// gz = g * (a > 0) (ReLU derivative from the stored activation)
-__global__ void relu_mask(const float *__restrict__ g, const bf16 *__restrict__ a, float *__restrict__ gz, size_t n) {
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
-    gz[i] = (__bfloat162float(a[i]) > 0.f) ? g[i] : 0.f;
-}
-
-// 2x2 average pooling (bf16 -> bf16); backward (float -> float) adds into dst
-// when `accumulate` (the pooled tensor is also a skip source).
-__global__ void pool2_fwd(const bf16 *__restrict__ x, bf16 *__restrict__ y, int BC, int H, int W) {
-  const int h = H / 2, w = W / 2;
-  const size_t n = (size_t)BC * h * w;
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-    const int xx = i % w, yy = (i / w) % h;
-    const size_t bc = i / ((size_t)h * w);
-    const bf16 *s = x + bc * H * W + (size_t)(2 * yy) * W + 2 * xx;
-    const float v = __bfloat162float(s[0]) + __bfloat162float(s[1]) + __bfloat162float(s[W]) +
-                    __bfloat162float(s[W + 1]);
-    y[i] = __float2bfloat16(0.25f * v);
-  }
-}
-__global__ void pool2_bwd(const float *__restrict__ gy, const float *__restrict__ gskip, float *__restrict__ gx,
-                          int BC, int H, int W) {
-  const size_t n = (size_t)BC * H * W;
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-    const int xx = i % W, yy = (i / W) % H;
-    const size_t bc = i / ((size_t)H * W);
-    float v = 0.25f * gy[bc * (H / 2) * (W / 2) + (size_t)(yy / 2) * (W / 2) + xx / 2];
-    if (gskip) v += gskip[i];
-    gx[i] = v;
-  }
-}
-// nearest 2x upsampling (bf16) and its adjoint (2x2 sums, float)
-__global__ void up2_fwd(const bf16 *__restrict__ x, bf16 *__restrict__ y, int BC, int h, int w) {
-  const int H = 2 * h, W = 2 * w;
-  const size_t n = (size_t)BC * H * W;
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-    const int xx = i % W, yy = (i / W) % H;
-    const size_t bc = i / ((size_t)H * W);
-    y[i] = x[bc * h * w + (size_t)(yy / 2) * w + xx / 2];
-  }
-}
-__global__ void up2_bwd(const float *__restrict__ gy, float *__restrict__ gx, int BC, int h, int w) {
-  const int W = 2 * w;
-  const size_t n = (size_t)BC * h * w;
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-    const int xx = i % w, yy = (i / w) % h;
-    const size_t bc = i / ((size_t)h * w);
-    const float *s = gy + bc * 4 * h * w + (size_t)(2 * yy) * W + 2 * xx;
-    gx[i] = s[0] + s[1] + s[W] + s[W + 1];
-  }
-}
-
-// 1x1 head (Cin -> 1): y = sum_c w[c] a[c] + b
-__global__ void head_fwd(const bf16 *__restrict__ a, const float *__restrict__ w, const float *__restrict__ bias,
-                         float *__restrict__ y, int B, int C, size_t plane) {
+// x [B][3][plane] FP32 -> NHWC BF16 [pixel][16]: the high, middle and low parts
+// of the 3 channels (the forward weights of all but the high ones are zero).
+__global__ void pack_input(const float *__restrict__ x, bf16 *__restrict__ y, int B, size_t plane) {
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < (size_t)B * plane;
        i += (size_t)gridDim.x * blockDim.x) {
     const size_t b = i / plane, p = i - b * plane;
-    float s = bias[0];
-    for (int c = 0; c < C; ++c) s = fmaf(w[c], __bfloat162float(a[(b * C + c) * plane + p]), s);
-    y[i] = s;
+    const float *s = x + b * 3 * plane + p;
+    const float v[3] = {s[0], s[plane], s[2 * plane]};
+    bf16 o[16];
+#pragma unroll
+    for (int c = 0; c < 16; ++c) o[c] = __float2bfloat16(0.f);
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      const bf16 h = __float2bfloat16(v[c]);
+      const float r = v[c] - __bfloat162float(h);
+      const bf16 m = __float2bfloat16(r);
+      o[c] = h;
+      o[3 + c] = m;
+      o[6 + c] = __float2bfloat16(r - __bfloat162float(m));
+    }
+    uint4 *d = reinterpret_cast<uint4 *>(y + i * 16);
+    d[0] = *reinterpret_cast<const uint4 *>(o);
+    d[1] = *reinterpret_cast<const uint4 *>(o + 8);
   }
 }
-// head backward: ga[c] = w[c] gy; partial[b][c] = sum_p a[c] gy (per CTA-row)
-__global__ void head_bwd_data(const float *__restrict__ gy, const float *__restrict__ w, float *__restrict__ ga, int B,
-                              int C, size_t plane) {
-  const size_t n = (size_t)B * C * plane;
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-    const size_t p = i % plane, bc = i / plane;
-    const int c = bc % C;
-    const size_t b = bc / C;
-    ga[i] = w[c] * gy[b * plane + p];
+
+// 2 x 2 average pooling, 8 channels per thread (BF16 -> BF16); blockIdx.y =
+// sample here and in the next two (32-bit indices within a sample).
+__global__ void pool2_fwd(const bf16 *__restrict__ x, bf16 *__restrict__ y, int h, int w, int cp) {
+  const unsigned q = cp / 8, n = (unsigned)h * w * q;
+  const size_t b = blockIdx.y;
+  for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+    const unsigned c = i % q, p = i / q, xx = p % w, yy = p / w;
+    const uint4 *s = reinterpret_cast<const uint4 *>(x) + (b * 4 * h * w + (size_t)(2 * yy) * (2 * w) + 2 * xx) * q + c;
+    const uint4 v[4] = {s[0], s[q], s[(size_t)2 * w * q], s[(size_t)2 * w * q + q]};
+    unsigned o[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      unsigned u[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) u[j] = reinterpret_cast<const unsigned *>(&v[j])[k];
+      const float a = bf16_lo(u[0]) + bf16_lo(u[1]) + bf16_lo(u[2]) + bf16_lo(u[3]);
+      const float b = bf16_hi(u[0]) + bf16_hi(u[1]) + bf16_hi(u[2]) + bf16_hi(u[3]);
+      o[k] = bf16_pack2(0.25f * a, 0.25f * b);
+    }
+    reinterpret_cast<uint4 *>(y)[b * n + i] = make_uint4(o[0], o[1], o[2], o[3]);
   }
 }
-__global__ void head_bwd_weight(const bf16 *__restrict__ a, const float *__restrict__ gy, float *__restrict__ partial,
-                                int C, size_t plane) {
-  __shared__ double red[8];
-  const int c = blockIdx.x, b = blockIdx.y;
-  double s = 0.0;
-  for (size_t p = threadIdx.x; p < plane; p += blockDim.x)
-    s += (double)__bfloat162float(a[((size_t)b * C + c) * plane + p]) * gy[(size_t)b * plane + p];
-  s = block_sum(s, red);
-  if (threadIdx.x == 0) partial[(size_t)b * C + c] = (float)s;
+// Its adjoint plus the skip gradient, under the ReLU mask of the pooled
+// activation: gx = (gy / 4 + gskip) (act > 0); [B][2h][2w][cp], 4 channels per
+// thread.
+__global__ void pool2_bwd(const float *__restrict__ gy, const float *__restrict__ gskip, const bf16 *__restrict__ act,
+                          float *__restrict__ gx, int h, int w, int cp) {
+  const unsigned q = cp / 4, W = 2 * w, n = 2u * h * W * q;
+  const size_t b = blockIdx.y;
+  for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+    const unsigned c = i % q, p = i / q, x = p % W, y = p / W;
+    const float4 g = reinterpret_cast<const float4 *>(gy)[((b * h + (y >> 1)) * w + (x >> 1)) * q + c];
+    const float4 k = reinterpret_cast<const float4 *>(gskip)[b * n + i];
+    const uint2 a = reinterpret_cast<const uint2 *>(act)[b * n + i];
+    float4 o;
+    o.x = bf16_lo(a.x) > 0.f ? fmaf(0.25f, g.x, k.x) : 0.f;
+    o.y = bf16_hi(a.x) > 0.f ? fmaf(0.25f, g.y, k.y) : 0.f;
+    o.z = bf16_lo(a.y) > 0.f ? fmaf(0.25f, g.z, k.z) : 0.f;
+    o.w = bf16_hi(a.y) > 0.f ? fmaf(0.25f, g.w, k.w) : 0.f;
+    reinterpret_cast<float4 *>(gx)[b * n + i] = o;
+  }
+}
+// Adjoint of the nearest 2x upsampling (2 x 2 sums) under the ReLU mask of the
+// upsampled activation; output [B][h][w][cp].
+__global__ void up2_bwd(const float *__restrict__ gy, const bf16 *__restrict__ act, float *__restrict__ gx, int h,
+                        int w, int cp) {
+  const unsigned q = cp / 4, n = (unsigned)h * w * q;
+  const size_t b = blockIdx.y;
+  for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+    const unsigned c = i % q, p = i / q, x = p % w, y = p / w;
+    const float4 *s = reinterpret_cast<const float4 *>(gy) + (b * 4 * h * w + (size_t)(2 * y) * (2 * w) + 2 * x) * q + c;
+    const float4 v0 = s[0], v1 = s[q], v2 = s[(size_t)2 * w * q], v3 = s[(size_t)2 * w * q + q];
+    const uint2 a = reinterpret_cast<const uint2 *>(act)[b * n + i];
+    float4 o;
+    o.x = bf16_lo(a.x) > 0.f ? v0.x + v1.x + v2.x + v3.x : 0.f;
+    o.y = bf16_hi(a.x) > 0.f ? v0.y + v1.y + v2.y + v3.y : 0.f;
+    o.z = bf16_lo(a.y) > 0.f ? v0.z + v1.z + v2.z + v3.z : 0.f;
+    o.w = bf16_hi(a.y) > 0.f ? v0.w + v1.w + v2.w + v3.w : 0.f;
+    reinterpret_cast<float4 *>(gx)[b * n + i] = o;
+  }
+}
+
+// 1 x 1 head (C -> 1): y = sum_c w[c] a[c] + b, in channel order.
+__global__ void head_fwd(const bf16 *__restrict__ a, const float *__restrict__ w, const float *__restrict__ bias,
+                         float *__restrict__ y, size_t pixels, int C, int cp) {
+  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < pixels; i += (size_t)gridDim.x * blockDim.x) {
+    const uint4 *s = reinterpret_cast<const uint4 *>(a + i * cp);
+    float v = bias[0];
+    for (int c = 0; c < C; c += 8) {
+      const uint4 u = s[c >> 3];
+      const unsigned k[4] = {u.x, u.y, u.z, u.w};
+#pragma unroll
+      for (int j = 0; j < 8; ++j)
+        if (c + j < C) v = fmaf(w[c + j], (j & 1) ? bf16_hi(k[j >> 1]) : bf16_lo(k[j >> 1]), v);
+    }
+    y[i] = v;
+  }
+}
+// Head backward, one pass over the activation: gz[c] = w[c] gy under the ReLU mask
+// of a, and per-block partials of the weight gradient sum_p a[c] gy and (slot C)
+// of the bias gradient sum_p gy.  Threads as in channel_sums (4 channels each).
+__global__ void __launch_bounds__(256) head_bwd(const float *__restrict__ gy, const bf16 *__restrict__ a,
+                                                const float *__restrict__ w, float *__restrict__ gz, size_t pixels,
+                                                int C, int cp, float *__restrict__ partial) {
+  __shared__ float sh[256][5], sl[256][5];
+  const int q = cp / 4, groups = max(1, 256 / q);
+  for (int c0 = 0; c0 < q; c0 += 256) {
+    const int c = c0 + (q <= 256 ? (int)threadIdx.x % q : (int)threadIdx.x), grp = q <= 256 ? threadIdx.x / q : 0;
+    SumOf<float> s[5];
+    if (c < q && grp < groups) {
+      float wv[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) wv[i] = c * 4 + i < C ? w[c * 4 + i] : 0.f;
+      for (size_t p = (size_t)blockIdx.x * groups + grp; p < pixels; p += (size_t)gridDim.x * groups) {
+        const float gv = gy[p];
+        const uint2 u = *reinterpret_cast<const uint2 *>(a + p * cp + c * 4);
+        const float av[4] = {bf16_lo(u.x), bf16_hi(u.x), bf16_lo(u.y), bf16_hi(u.y)};
+        float4 o;
+        o.x = av[0] > 0.f ? wv[0] * gv : 0.f;
+        o.y = av[1] > 0.f ? wv[1] * gv : 0.f;
+        o.z = av[2] > 0.f ? wv[2] * gv : 0.f;
+        o.w = av[3] > 0.f ? wv[3] * gv : 0.f;
+        *reinterpret_cast<float4 *>(gz + p * cp + c * 4) = o;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const float pr = av[i] * gv;
+          s[i].add(pr, fmaf(av[i], gv, -pr));
+        }
+        s[4].add(gv);
+      }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < 5; ++i) {
+      sh[threadIdx.x][i] = s[i].h;
+      sl[threadIdx.x][i] = s[i].l;
+    }
+    __syncthreads();
+    if ((int)threadIdx.x < min(q, 256) && c < q) {
+#pragma unroll
+      for (int i = 0; i < 5; ++i) {
+        SumOf<float> tot;
+        for (int k = 0; k < groups; ++k) tot.add(sh[threadIdx.x + k * q][i], sl[threadIdx.x + k * q][i]);
+        const int slot = i < 4 ? c * 4 + i : C;
+        if (i < 4 ? slot < C : c == 0) partial[(size_t)blockIdx.x * (C + 1) + slot] = tot.h + tot.l;
+      }
+    }
+  }
 }
 
 // Loss over n = B H W lattice values, d = y - t:
@@ -437,21 +729,31 @@ __global__ void loss_kernel(const float *__restrict__ y, const float *__restrict
   if (threadIdx.x == 0) partial[blockIdx.x] = s;
 }
 
-// Weight transform for the backward-data pass: wt[8 - tap][co][ci] = w[tap][ci][co]
-__global__ void flip_transpose(const bf16 *__restrict__ w, bf16 *__restrict__ wt, int Cin, int Cout) {
-  const size_t n = (size_t)9 * Cin * Cout;
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-    const int co = i % Cout;
-    const int ci = (i / Cout) % Cin;
-    const int tap = i / ((size_t)Cin * Cout);
-    wt[((size_t)(8 - tap) * Cout + co) * Cin + ci] = w[i];
+// FP32 weights of every 3 x 3 layer into its two packed BF16 copies (see
+// Layouts); blockIdx.y = layer.
+struct PackLayer {
+  size_t woff, fwd, bwd;  // offsets into the parameters and the packed copies
+  int cin, cout;
+};
+__global__ void pack_weights(const float *__restrict__ p, const PackLayer *__restrict__ ls, bf16 *__restrict__ out) {
+  const PackLayer L = ls[blockIdx.y];
+  const float *w = p + L.woff;
+  const int nf = pad8(L.cout), nb = pad8(L.cin);
+  const unsigned ef = (unsigned)chunks16(L.cin) * 9 * nf * 16, eb = (unsigned)chunks16(L.cout) * 9 * nb * 16;
+  for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < ef + eb; i += gridDim.x * blockDim.x) {
+    const bool back = i >= ef;
+    const unsigned e = back ? i - ef : i, n8 = back ? nb : nf;
+    const int j = e & 15, n = (e >> 4) % n8, r = (e >> 4) / n8, tap = r % 9, k = (r / 9) * 16 + j;
+    const int ci = back ? n : k, co = back ? k : n, tp = back ? 8 - tap : tap;
+    const float v = ci < L.cin && co < L.cout ? w[((size_t)tp * L.cin + ci) * L.cout + co] : 0.f;
+    out[(back ? L.bwd : L.fwd) + e] = __float2bfloat16(v);
   }
 }
 
-// Adam (FP32 master weights) and refresh of the BF16 compute copy.
+// Adam (FP32 master weights).
 __global__ void adam_kernel(float *__restrict__ p, const float *__restrict__ g, float *__restrict__ m,
-                            float *__restrict__ v, bf16 *__restrict__ pb, size_t n, float lr, float b1, float b2,
-                            float eps, float c1, float c2) {
+                            float *__restrict__ v, size_t n, float lr, float b1, float b2, float eps, float c1,
+                            float c2) {
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
     const float gi = g[i];
     const float mi = b1 * m[i] + (1.f - b1) * gi;
@@ -459,15 +761,8 @@ __global__ void adam_kernel(float *__restrict__ p, const float *__restrict__ g, 
     m[i] = mi;
     v[i] = vi;
     const float upd = lr * (mi / c1) / (sqrtf(vi / c2) + eps);
-    const float pi = p[i] - upd;
-    p[i] = pi;
-    if (pb) pb[i] = __float2bfloat16(pi);
+    p[i] = p[i] - upd;
   }
-}
-
-__global__ void to_bf16(const float *__restrict__ x, bf16 *__restrict__ y, size_t n) {
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
-    y[i] = __float2bfloat16(x[i]);
 }
 
 // ---------------------------------------------------------------------------
@@ -550,6 +845,8 @@ struct NetLayer {
   char kind;     // 'c' conv+relu, 's' conv+relu+skip, 'p' pool, 'u' up, 'h' head
   int cin = 0, cout = 0, res = 0;  // res: spatial size of this layer's output
   size_t woff = 0, boff = 0;       // offsets into the flat parameter vector
+  size_t fwd = 0, bwd = 0;         // offsets of the packed weights
+  int in = -1, up = 0;             // input activation buffer (-1: the network's input), read 2x upsampled if up
   int out = -1, out2 = -1;         // activation buffers (out2: relu output + skip)
   int skip = -1;                   // buffer added after ReLU ('s')
 };
@@ -558,24 +855,25 @@ struct GuessNet {
   int hw = 0, cap = 0;   // lattice size, batch capacity
   int ch[4] = {24, 48, 96, 192};
   std::vector<NetLayer> layers;
-  size_t nparams = 0;
+  size_t nparams = 0, npacked = 0;
   float *p = nullptr, *g = nullptr, *m = nullptr, *v = nullptr;  // FP32 master, grads, Adam moments
-  bf16 *pb = nullptr;                                            // BF16 compute copy
-  bf16 *wt = nullptr;                                            // flipped/transposed weights scratch
+  bf16 *pk = nullptr;                                            // packed BF16 weights
+  PackLayer *pl = nullptr;                                       // device: the conv layers' packing
+  int npack = 0;
+  bf16 *xin = nullptr;                                           // packed input [cap][hw][hw][16]
   std::vector<std::pair<int, int>> bufshape;                     // (channels, res) per activation buffer
-  std::vector<bf16 *> act;                                       // activations [cap][C][res][res]
-  float *y = nullptr;                                            // head output [cap][hw][hw]
-  float *gA = nullptr, *gB = nullptr, *gZ = nullptr;             // gradient scratch (largest activation)
+  std::vector<bf16 *> act;                                       // activations [cap][res][res][pad8(C)]
+  float *y = nullptr, *gy = nullptr;                             // head output and its gradient [cap][hw][hw]
+  float *gbuf[3] = {nullptr, nullptr, nullptr};                  // gradients (largest activation)
   std::vector<float *> gskip;                                    // skip gradients per level
-  float *partial = nullptr;                                      // weight-gradient partials
-  size_t partial_n = 0;
+  float *partial = nullptr;                                      // weight- and bias-gradient partials
   double *lpart = nullptr;                                       // loss partials
   float h1 = 0.f;                                                // weight of the loss's edge term
   int step = 0;
 };
 
 size_t act_elems(const GuessNet *n, int buf) {
-  return (size_t)n->cap * n->bufshape[buf].first * n->bufshape[buf].second * n->bufshape[buf].second;
+  return (size_t)n->cap * pad8(n->bufshape[buf].first) * n->bufshape[buf].second * n->bufshape[buf].second;
 }
 
 void build_layers(GuessNet *n) {
@@ -585,10 +883,18 @@ void build_layers(GuessNet *n) {
     n->bufshape.push_back({c, r});
     return (int)n->bufshape.size() - 1;
   };
-  size_t off = 0;
+  size_t off = 0, pack = 0;
+  int cur = -1, up2 = 0;
   auto conv = [&](char kind, int cin, int cout, int res, int skip) {
     NetLayer L;
     L.kind = kind;
+    L.in = cur;
+    L.up = up2;
+    up2 = 0;
+    L.fwd = pack;
+    pack += (size_t)chunks16(cin) * 9 * pad8(cout) * 16;
+    L.bwd = pack;
+    pack += (size_t)chunks16(cout) * 9 * pad8(cin) * 16;
     L.cin = cin;
     L.cout = cout;
     L.res = res;
@@ -602,25 +908,26 @@ void build_layers(GuessNet *n) {
       L.skip = skip;
     }
     n->layers.push_back(L);
-    return (kind == 's') ? L.out2 : L.out;
+    return cur = (kind == 's') ? L.out2 : L.out;
   };
   auto pool = [&](int c, int res) {
     NetLayer L;
     L.kind = 'p';
     L.cin = L.cout = c;
     L.res = res;
-    L.out = buf(c, res);
+    L.in = cur;
+    L.out = cur = buf(c, res);
     n->layers.push_back(L);
     return L.out;
   };
   auto up = [&](int c, int res) {
     NetLayer L;
-    L.kind = 'u';
+    L.kind = 'u';  // read upsampled by the next convolution: no buffer of its own
     L.cin = L.cout = c;
     L.res = res;
-    L.out = buf(c, res);
+    L.in = L.out = cur;
+    up2 = 1;
     n->layers.push_back(L);
-    return L.out;
   };
   conv('c', 3, c1, H, -1);
   const int s1 = conv('c', c1, c1, H, -1);
@@ -647,12 +954,14 @@ void build_layers(GuessNet *n) {
   hd.cin = c1;
   hd.cout = 1;
   hd.res = H;
+  hd.in = cur;
   hd.woff = off;
   off += c1;
   hd.boff = off;
   off += 1;
   n->layers.push_back(hd);
   n->nparams = off;
+  n->npacked = pack;
 }
 
 // deterministic host initialisation: He-normal weights (Box-Muller on a
@@ -693,155 +1002,155 @@ cudaError_t zalloc(P **p, size_t count) {
 }
 
 void net_free(GuessNet *n) {
-  cudaFree(n->p); cudaFree(n->g); cudaFree(n->m); cudaFree(n->v); cudaFree(n->pb); cudaFree(n->wt);
+  cudaFree(n->p); cudaFree(n->g); cudaFree(n->m); cudaFree(n->v); cudaFree(n->pk); cudaFree(n->pl);
+  cudaFree(n->xin); cudaFree(n->gy);
   for (auto *a : n->act) cudaFree(a);
   for (auto *a : n->gskip) cudaFree(a);
-  cudaFree(n->y); cudaFree(n->gA); cudaFree(n->gB); cudaFree(n->gZ); cudaFree(n->partial); cudaFree(n->lpart);
+  cudaFree(n->y);
+  for (float *g : n->gbuf) cudaFree(g);
+  cudaFree(n->partial); cudaFree(n->lpart);
   delete n;
 }
 
 // ---------------------------------------------------------------------------
 // passes
 // ---------------------------------------------------------------------------
-template <typename TIn, typename TOut>
-void launch_conv(const TIn *in, const bf16 *w, const float *bias, TOut *out, const bf16 *skip, bf16 *out2, int B,
-                 int Cin, int Cout, int res, bool relu, cudaStream_t s) {
-  const int tiles = ((res + kTile - 1) / kTile) * ((res + kTile - 1) / kTile);
-  dim3 grid(tiles, (Cout + kCob - 1) / kCob, B);
+// Columns of 8 output channels per CTA: 6 where that divides their number, else
+// 3; rows of pixels per warp: 2, or 1 where the grid would not cover the SMs
+// twice.
+template <int NT, int MW, int PLANES>
+void launch_conv_shape(const ConvArgs &a, int B, cudaStream_t s) {
+  using S = ConvShape<NT, MW, PLANES>;
+  ensure_smem_attr((const void *)conv3x3_kernel<NT, MW, PLANES>, S::smem);
+  const dim3 grid(((a.W + 15) / 16) * ((a.H + 8 * MW - 1) / (8 * MW)), (pad8(a.cout) / 8 + NT - 1) / NT, B);
   note_launch();
-  conv3x3_kernel<TIn, TOut><<<grid, 256, 0, s>>>(in, w, bias, out, skip, out2, Cin, Cout, res, res, relu ? 1 : 0);
+  conv3x3_kernel<NT, MW, PLANES><<<grid, 256, S::smem, s>>>(a);
+}
+template <int PLANES>
+void launch_conv(const ConvArgs &a, int B, cudaStream_t s) {
+  const int nt = pad8(a.cout) / 8;
+  const bool wide = PLANES == 1 && nt % 6 == 0;
+  const long long ctas = (long long)((a.W + 15) / 16) * ((a.H + 15) / 16) * B * ((nt + 2) / 3) / (wide ? 2 : 1);
+  const bool tall = ctas >= 304;
+  if (PLANES == 1 && wide) {
+    if (tall) launch_conv_shape<6, 2, 1>(a, B, s);
+    else launch_conv_shape<6, 1, 1>(a, B, s);
+  } else {
+    // three planes: twice the columns of one row per warp where they divide (an
+    // input patch is split anew for every column block)
+    if (PLANES == 3 && nt % 6 == 0) launch_conv_shape<6, 1, PLANES>(a, B, s);
+    else if (tall) launch_conv_shape<3, 2, PLANES>(a, B, s);
+    else launch_conv_shape<3, 1, PLANES>(a, B, s);
+  }
 }
 
-template <typename TIn>
-void launch_conv_mma(const TIn *in, const bf16 *w, const float *bias, bf16 *out, const bf16 *skip, bf16 *out2, int B,
-                     int Cin, int Cout, int res, cudaStream_t s) {
-  const int tiles = ((res + kPx - 1) / kPx) * ((res + kPy - 1) / kPy);
-  dim3 grid(tiles, (Cout + kCo - 1) / kCo, B);
-  note_launch();
-  conv3x3_mma_kernel<TIn><<<grid, 256, 0, s>>>(in, w, bias, out, skip, out2, Cin, Cout, res, res, 1);
+constexpr int kWgCtas = 304;    // weight-gradient CTAs in all: two rounds of 152 SMs
+constexpr int kSumBlocks = 912; // blocks of the channel sums
+int wgrad_splits(int cin, int cout, long long tiles) {
+  const int blocks = chunks16(cin) * ((cout + kWgN - 1) / kWgN);
+  return (int)std::max<long long>(1, std::min<long long>(tiles, kWgCtas / blocks));
 }
 
-template <typename TIn>
-void launch_wgrad(GuessNet *n, const TIn *in, const float *gz, float *gw, int B, int Cin, int Cout, int res,
-                  cudaStream_t s) {
-  const int tiles = ((res + kTile - 1) / kTile) * ((res + kTile - 1) / kTile);
-  const int nco = (Cout + kCob - 1) / kCob;
-  const size_t smem = sizeof(float) * (kCib * (kTile + 2) * (kTile + 2) + kTile * kTile * kCob);
-  ensure_smem_attr((const void *)conv3x3_wgrad_kernel<TIn>, smem);
-  dim3 grid(tiles, (Cin + kCib - 1) / kCib, nco * B);
+// Writes dW [9][cin][cout].  planes = 3: the network's input (see
+// pack_input), cin = 3.
+void launch_wgrad(GuessNet *n, const bf16 *in, const float *gz, float *gw, int B, int cin, int cout, int res, int up,
+                  int planes, cudaStream_t s) {
+  const int vcin = planes == 3 ? 9 : cin;
+  WgradArgs a{in, gz, n->partial, vcin, planes == 3 ? 16 : pad8(cin), cout, B, res, res, up};
+  const int tiles1 = (res + 15) / 16;
+  const int splits = wgrad_splits(vcin, cout, (long long)B * tiles1 * tiles1);
+  ensure_smem_attr((const void *)conv3x3_wgrad_kernel, kWgSmem);
   note_launch();
-  conv3x3_wgrad_kernel<TIn><<<grid, 144, smem, s>>>(in, gz, n->partial, Cin, Cout, res, res);
-  const size_t nw = (size_t)9 * Cin * Cout;
+  conv3x3_wgrad_kernel<<<dim3(chunks16(vcin), (cout + kWgN - 1) / kWgN, splits), 256, kWgSmem, s>>>(a);
+  const size_t nw = (size_t)9 * cin * cout;
   note_launch();
-  sum_partials<<<grid1d(nw), 256, 0, s>>>(n->partial, B * tiles, nw, gw);
+  sum_partials<<<(unsigned)((nw + 31) / 32), 256, 0, s>>>(n->partial, splits, nw, gw, planes, cout);
 }
 
 void bias_grad(GuessNet *n, const float *gz, float *gb, int B, int C, int res, cudaStream_t s) {
   note_launch();
-  channel_sums<<<dim3(C, B), 256, 0, s>>>(gz, C, (size_t)res * res, n->partial);
+  channel_sums<<<kSumBlocks, 256, 0, s>>>(gz, C, pad8(C), (size_t)B * res * res, n->partial);
   note_launch();
-  sum_partials<<<grid1d(C), 256, 0, s>>>(n->partial, B, (size_t)C, gb);
+  sum_partials<<<(C + 31) / 32, 256, 0, s>>>(n->partial, kSumBlocks, (size_t)C, gb, 1, C);
+}
+
+void pack_all(GuessNet *n, cudaStream_t s) {
+  note_launch();
+  pack_weights<<<dim3(152, n->npack), 256, 0, s>>>(n->p, n->pl, n->pk);
 }
 
 void forward_pass(GuessNet *n, const float *x, int B, cudaStream_t s) {
   const int H = n->hw;
-  int cur = -1;  // current activation buffer (-1: the FP32 input x)
+  note_launch();
+  pack_input<<<grid1d((size_t)B * H * H), 256, 0, s>>>(x, n->xin, B, (size_t)H * H);
   for (const NetLayer &L : n->layers) {
     if (L.kind == 'c' || L.kind == 's') {
-      const bf16 *w = n->pb + L.woff;
-      const float *bias = n->p + L.boff;
-      bf16 *out = n->act[L.out];
-      const bf16 *skip = (L.kind == 's') ? n->act[L.skip] : nullptr;
-      bf16 *out2 = (L.kind == 's') ? n->act[L.out2] : nullptr;
-      if (cur < 0)
-        launch_conv_mma<float>(x, w, bias, out, skip, out2, B, L.cin, L.cout, L.res, s);
-      else
-        launch_conv_mma<bf16>(n->act[cur], w, bias, out, skip, out2, B, L.cin, L.cout, L.res, s);
-      cur = (L.kind == 's') ? L.out2 : L.out;
+      // the packed input has 16 channels, of which the weights use the first 3
+      const bool first = L.in < 0;
+      ConvArgs a{first ? n->xin : n->act[L.in], n->pk + L.fwd, n->p + L.boff, n->act[L.out],
+                 L.kind == 's' ? n->act[L.out2] : nullptr, L.kind == 's' ? n->act[L.skip] : nullptr, nullptr,
+                 first ? 16 : L.cin, L.cout, L.res, L.res, L.up};
+      launch_conv<1>(a, B, s);
     } else if (L.kind == 'p') {
       note_launch();
-      pool2_fwd<<<grid1d((size_t)B * L.cout * L.res * L.res), 256, 0, s>>>(n->act[cur], n->act[L.out], B * L.cout,
-                                                                           2 * L.res, 2 * L.res);
-      cur = L.out;
-    } else if (L.kind == 'u') {
+      pool2_fwd<<<dim3(grid1d((size_t)L.res * L.res * pad8(L.cout) / 8), B), 256, 0, s>>>(
+          n->act[L.in], n->act[L.out], L.res, L.res, pad8(L.cout));
+    } else if (L.kind == 'h') {
       note_launch();
-      up2_fwd<<<grid1d((size_t)B * L.cout * L.res * L.res), 256, 0, s>>>(n->act[cur], n->act[L.out], B * L.cout,
-                                                                         L.res / 2, L.res / 2);
-      cur = L.out;
-    } else {
-      note_launch();
-      head_fwd<<<grid1d((size_t)B * H * H), 256, 0, s>>>(n->act[cur], n->p + L.woff, n->p + L.boff, n->y, B, L.cin,
-                                                         (size_t)H * H);
+      head_fwd<<<grid1d((size_t)B * H * H), 256, 0, s>>>(n->act[L.in], n->p + L.woff, n->p + L.boff, n->y,
+                                                         (size_t)B * H * H, L.cin, pad8(L.cin));
     }
   }
 }
 
-// input buffer of layer li during the forward pass (-1 = x)
-int layer_input(const GuessNet *n, int li) {
-  int cur = -1;
-  for (int k = 0; k < li; ++k) {
-    const NetLayer &L = n->layers[k];
-    if (L.kind == 'h') continue;
-    cur = (L.kind == 's') ? L.out2 : L.out;
+// Backward pass from n->gy (d loss / d y, FP32 [B][H][W]); fills n->g.  Every
+// gradient buffer that a weight gradient reads already carries the ReLU mask of
+// its activation (written so by the kernel that forms it).
+void backward_pass(GuessNet *n, int B, cudaStream_t s) {
+  const int H = n->hw, last = (int)n->layers.size() - 1;
+  float *g = n->gbuf[0], *other = n->gbuf[1], *high = n->gbuf[2];
+  std::vector<float *> skips;
+  {
+    const NetLayer &L = n->layers[last];
+    note_launch();
+    head_bwd<<<kSumBlocks, 256, 0, s>>>(n->gy, n->act[L.in], n->p + L.woff, g, (size_t)B * H * H, L.cin, pad8(L.cin),
+                                        n->partial);
+    note_launch();
+    sum_partials<<<(L.cin + 32) / 32, 256, 0, s>>>(n->partial, kSumBlocks, (size_t)L.cin + 1, n->g + L.woff, 1, L.cin + 1);
   }
-  return cur;
-}
-
-// Backward pass from gy (d loss / d y, FP32 [B][H][W]); fills n->g.
-void backward_pass(GuessNet *n, const float *x, const float *gy, int B, cudaStream_t s) {
-  const int H = n->hw;
-  float *g = n->gA, *gnext = n->gB;
-  int level_skip = 0;  // skip gradients pushed (level 1 first)
-  std::vector<float *> skip_stack;
-  for (int li = (int)n->layers.size() - 1; li >= 0; --li) {
+  for (int li = last - 1; li >= 0; --li) {
     const NetLayer &L = n->layers[li];
-    const int inbuf = layer_input(n, li);
-    if (L.kind == 'h') {
-      note_launch();
-      head_bwd_weight<<<dim3(L.cin, B), 256, 0, s>>>(n->act[inbuf], gy, n->partial, L.cin, (size_t)H * H);
-      note_launch();
-      sum_partials<<<grid1d(L.cin), 256, 0, s>>>(n->partial, B, (size_t)L.cin, n->g + L.woff);
-      // bias gradient: sum of gy over all samples and pixels
-      note_launch();
-      channel_sums<<<dim3(1, B), 256, 0, s>>>(gy, 1, (size_t)H * H, n->partial);
-      note_launch();
-      sum_partials<<<1, 256, 0, s>>>(n->partial, B, 1, n->g + L.boff);
-      note_launch();
-      head_bwd_data<<<grid1d((size_t)B * L.cin * H * H), 256, 0, s>>>(gy, n->p + L.woff, g, B, L.cin, (size_t)H * H);
-    } else if (L.kind == 'c' || L.kind == 's') {
-      const size_t ne = (size_t)B * L.cout * L.res * L.res;
-      if (L.kind == 's') {
-        // the skip source receives the incoming gradient unchanged
-        float *sg = n->gskip[level_skip++];
-        cudaMemcpyAsync(sg, g, ne * sizeof(float), cudaMemcpyDeviceToDevice, s);
-        skip_stack.push_back(sg);
-      }
-      note_launch();
-      relu_mask<<<grid1d(ne), 256, 0, s>>>(g, n->act[L.out], n->gZ, ne);
-      if (inbuf < 0)
-        launch_wgrad<float>(n, x, n->gZ, n->g + L.woff, B, L.cin, L.cout, L.res, s);
-      else
-        launch_wgrad<bf16>(n, n->act[inbuf], n->gZ, n->g + L.woff, B, L.cin, L.cout, L.res, s);
-      bias_grad(n, n->gZ, n->g + L.boff, B, L.cout, L.res, s);
-      if (li > 0) {
-        note_launch();
-        flip_transpose<<<grid1d((size_t)9 * L.cin * L.cout), 256, 0, s>>>(n->pb + L.woff, n->wt, L.cin, L.cout);
-        launch_conv<float, float>(n->gZ, n->wt, nullptr, gnext, nullptr, nullptr, B, L.cout, L.cin, L.res, false, s);
-        std::swap(g, gnext);
-      }
-    } else if (L.kind == 'u') {
-      note_launch();
-      up2_bwd<<<grid1d((size_t)B * L.cin * (L.res / 2) * (L.res / 2)), 256, 0, s>>>(g, gnext, B * L.cin, L.res / 2,
-                                                                                      L.res / 2);
-      std::swap(g, gnext);
-    } else {  // pool: gradient of the pooled input plus its skip gradient
-      float *sg = skip_stack.back();
-      skip_stack.pop_back();
-      note_launch();
-      pool2_bwd<<<grid1d((size_t)B * L.cin * 4 * L.res * L.res), 256, 0, s>>>(g, sg, gnext, B * L.cin, 2 * L.res,
-                                                                                2 * L.res);
-      std::swap(g, gnext);
+    if (L.kind != 'c' && L.kind != 's') continue;  // 'p', 'u': with the convolution behind them
+    const bool first = L.in < 0;
+    launch_wgrad(n, first ? n->xin : n->act[L.in], g, n->g + L.woff, B, L.cin, L.cout, L.res, L.up, first ? 3 : 1, s);
+    bias_grad(n, g, n->g + L.boff, B, L.cout, L.res, s);
+    if (li == 0) break;
+    const NetLayer &prev = n->layers[li - 1];
+    ConvArgs a{g, n->pk + L.bwd, nullptr, other, nullptr, nullptr, nullptr, L.cout, L.cin, L.res, L.res, 0};
+    if (prev.kind == 'c') {
+      a.mask = n->act[prev.out];
+    } else if (prev.kind == 's') {  // the skip source receives the gradient unmasked
+      float *sg = n->gskip[skips.size()];
+      skips.push_back(sg);
+      a.out2 = sg;
+      a.mask = n->act[prev.out];
+    } else {
+      a.out = high;
     }
+    launch_conv<3>(a, B, s);
+    if (prev.kind == 'p') {
+      float *sg = skips.back();
+      skips.pop_back();
+      note_launch();
+      pool2_bwd<<<dim3(grid1d((size_t)4 * L.res * L.res * pad8(L.cin) / 4), B), 256, 0, s>>>(
+          high, sg, n->act[prev.in], other, L.res, L.res, pad8(L.cin));
+    } else if (prev.kind == 'u') {
+      // masked by the ReLU of the convolution whose output is upsampled
+      note_launch();
+      up2_bwd<<<dim3(grid1d((size_t)(L.res / 2) * (L.res / 2) * pad8(L.cin) / 4), B), 256, 0, s>>>(
+          high, n->act[n->layers[li - 2].out], other, L.res / 2, L.res / 2, pad8(L.cin));
+    }
+    std::swap(g, other);
   }
 }
 
@@ -849,7 +1158,7 @@ int loss_and_grad(GuessNet *n, const float *target, int B, cudaStream_t s, doubl
   const size_t N = (size_t)B * n->hw * n->hw;
   const int blocks = std::min<int>(grid1d(N), 1024);
   note_launch();
-  loss_kernel<<<blocks, 256, 0, s>>>(n->y, target, n->gZ, B, n->hw, n->hw, n->h1, n->lpart);
+  loss_kernel<<<blocks, 256, 0, s>>>(n->y, target, n->gy, B, n->hw, n->hw, n->h1, n->lpart);
   std::vector<double> h(blocks);
   if (cudaMemcpyAsync(h.data(), n->lpart, blocks * sizeof(double), cudaMemcpyDeviceToHost, s) != cudaSuccess)
     return AX_ERR_CUDA;
@@ -889,39 +1198,46 @@ int ax_guessnet_create(int32_t hw, const int32_t *channels, int32_t batch_capaci
   if (e == cudaSuccess) e = zalloc(&n->g, n->nparams);
   if (e == cudaSuccess) e = zalloc(&n->m, n->nparams);
   if (e == cudaSuccess) e = zalloc(&n->v, n->nparams);
-  if (e == cudaSuccess) e = zalloc(&n->pb, n->nparams);
-  size_t maxw = 0, maxact = 0;
-  for (const NetLayer &L : n->layers) maxw = std::max(maxw, (size_t)9 * L.cin * L.cout);
-  if (e == cudaSuccess) e = zalloc(&n->wt, maxw);
+  if (e == cudaSuccess) e = zalloc(&n->pk, n->npacked);
+  if (e == cudaSuccess) e = zalloc(&n->xin, (size_t)batch_capacity * hw * hw * 16);
+  std::vector<PackLayer> pls;
+  for (const NetLayer &L : n->layers)
+    if (L.kind == 'c' || L.kind == 's') pls.push_back({L.woff, L.fwd, L.bwd, L.cin, L.cout});
+  n->npack = (int)pls.size();
+  if (e == cudaSuccess) e = zalloc(&n->pl, pls.size());
+  if (e == cudaSuccess) e = cudaMemcpy(n->pl, pls.data(), pls.size() * sizeof(PackLayer), cudaMemcpyHostToDevice);
+  size_t maxact = 0;
   for (size_t b = 0; b < n->bufshape.size() && e == cudaSuccess; ++b) {
     bf16 *a = nullptr;
     e = zalloc(&a, act_elems(n, (int)b));
     n->act.push_back(a);
     maxact = std::max(maxact, act_elems(n, (int)b));
   }
-  maxact = std::max(maxact, (size_t)n->cap * 3 * hw * hw);
+  // a gradient of an upsampled activation has 4 times its pixels
+  for (const NetLayer &L : n->layers)
+    if (L.up) maxact = std::max(maxact, (size_t)n->cap * pad8(L.cin) * L.res * L.res);
   if (e == cudaSuccess) e = zalloc(&n->y, (size_t)n->cap * hw * hw);
-  if (e == cudaSuccess) e = zalloc(&n->gA, maxact);
-  if (e == cudaSuccess) e = zalloc(&n->gB, maxact);
-  if (e == cudaSuccess) e = zalloc(&n->gZ, maxact);
+  if (e == cudaSuccess) e = zalloc(&n->gy, (size_t)n->cap * hw * hw);
+  for (float *&g : n->gbuf)
+    if (e == cudaSuccess) e = zalloc(&g, maxact);
   for (int k = 0; k < 3 && e == cudaSuccess; ++k) {
     float *sg = nullptr;
     e = zalloc(&sg, maxact);
     n->gskip.push_back(sg);
   }
-  // weight-gradient partials: slots (B * tiles) x (9 Cin Cout), largest layer
+  // partials of the weight gradients (splits x 9 cin cout) and of the channel sums
   size_t pn = 0;
   for (const NetLayer &L : n->layers) {
-    const size_t tiles = (size_t)((L.res + kTile - 1) / kTile) * ((L.res + kTile - 1) / kTile);
-    pn = std::max(pn, (size_t)n->cap * tiles * 9 * std::max(L.cin, 1) * std::max(L.cout, 1));
-    pn = std::max(pn, (size_t)n->cap * std::max(L.cout, L.cin));
+    const int cin = L.in < 0 ? 9 : L.cin;
+    if (L.kind == 'c' || L.kind == 's')
+      pn = std::max(pn, (size_t)wgrad_splits(cin, L.cout, 1LL << 40) * 9 * cin * L.cout);
+    pn = std::max(pn, (size_t)kSumBlocks * (std::max(L.cin, L.cout) + 1));
   }
-  n->partial_n = pn;
   if (e == cudaSuccess) e = zalloc(&n->partial, pn);
   if (e == cudaSuccess) e = zalloc(&n->lpart, 1024);
   if (e == cudaSuccess) e = cudaMemcpy(n->p, h.data(), n->nparams * sizeof(float), cudaMemcpyHostToDevice);
   if (e == cudaSuccess) {
-    to_bf16<<<grid1d(n->nparams), 256>>>(n->p, n->pb, n->nparams);
+    pack_all(n, nullptr);
     e = cudaDeviceSynchronize();
   }
   if (e != cudaSuccess) {
@@ -949,8 +1265,7 @@ int ax_guessnet_set_params(void *net, const float *host, int64_t n) {
   GuessNet *g = (GuessNet *)net;
   if (!g || !host || n != (int64_t)g->nparams) return AX_ERR_INVALID_ARG;
   if (cudaMemcpy(g->p, host, n * sizeof(float), cudaMemcpyHostToDevice) != cudaSuccess) return AX_ERR_CUDA;
-  note_launch();
-  to_bf16<<<grid1d(g->nparams), 256>>>(g->p, g->pb, g->nparams);
+  pack_all(g, nullptr);
   cudaMemset(g->m, 0, n * sizeof(float));
   cudaMemset(g->v, 0, n * sizeof(float));
   g->step = 0;
@@ -981,11 +1296,7 @@ int ax_guessnet_gradients(void *net, const float *x, const float *target, int32_
   forward_pass(n, x, batch, s);
   int rc = loss_and_grad(n, target, batch, s, loss);
   if (rc != AX_OK) return rc;
-  // loss_and_grad left d loss / d y in gZ, which the backward pass reuses as
-  // scratch; move it into the output buffer (no longer needed)
-  float *gyc = n->y;
-  cudaMemcpyAsync(gyc, n->gZ, (size_t)batch * n->hw * n->hw * sizeof(float), cudaMemcpyDeviceToDevice, s);
-  backward_pass(n, x, gyc, batch, s);
+  backward_pass(n, batch, s);
   if (grad_host) {
     if (cudaMemcpyAsync(grad_host, n->g, n->nparams * sizeof(float), cudaMemcpyDeviceToHost, s) != cudaSuccess)
       return AX_ERR_CUDA;
@@ -1004,7 +1315,8 @@ int ax_guessnet_train_step(void *net, const float *x, const float *target, int32
   const float b1 = 0.9f, b2 = 0.999f;
   const float c1 = 1.f - std::pow(b1, (float)n->step), c2 = 1.f - std::pow(b2, (float)n->step);
   note_launch();
-  adam_kernel<<<grid1d(n->nparams), 256, 0, s>>>(n->p, n->g, n->m, n->v, n->pb, n->nparams, lr, b1, b2, 1e-8f, c1, c2);
+  adam_kernel<<<grid1d(n->nparams), 256, 0, s>>>(n->p, n->g, n->m, n->v, n->nparams, lr, b1, b2, 1e-8f, c1, c2);
+  pack_all(n, s);
   return cudaGetLastError() == cudaSuccess ? AX_OK : AX_ERR_CUDA;
 }
 
