@@ -76,15 +76,17 @@ __device__ __forceinline__ uint64_t smem_desc(const void *p) {
 }
 // Instruction descriptor, kind::f16: D FP32 (bits 4-5 = 1), A and B BF16
 // (bits 7-9 = 1, 10-12 = 1), both K-major, N >> 3 at bits 17-22, M >> 4 at 24-28.
-constexpr unsigned kIdesc = (1u << 4) | (1u << 7) | (1u << 10) | ((unsigned)(kBN >> 3) << 17) |
+template <int N>
+constexpr unsigned kIdesc = (1u << 4) | (1u << 7) | (1u << 10) | ((unsigned)(N >> 3) << 17) |
                             ((unsigned)(kBM >> 4) << 24);
 
+template <int N = kBN>
 __device__ __forceinline__ void umma(unsigned d_tmem, uint64_t a, uint64_t b, unsigned accumulate) {
   asm volatile(
       "{\n\t.reg .pred p;\n\t"
       "setp.ne.b32 p, %4, 0;\n\t"
       "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
-      "l"(a), "l"(b), "r"(kIdesc), "r"(accumulate)
+      "l"(a), "l"(b), "r"(kIdesc<N>), "r"(accumulate)
       : "memory");
 }
 __device__ __forceinline__ void umma_commit(uint64_t *bar) {
@@ -524,6 +526,219 @@ __global__ void __launch_bounds__(kGemmThreads, 1) dst_gemm_kernel(const GemmDst
   }
 }
 
+// The same transform for few tiles: 128 rows x 32 columns of both P and Q, one
+// tile per CTA.  With one right-hand side at 1024 x 1024 the kernel above has 32
+// tiles for 152 SMs, each a chain of 16 K blocks whose 64 KB copies one SM
+// receives at about 0.1 TB/s, and then an epilogue of 64 columns per warp (28 us
+// per launch).  Here 128 CTAs copy 40 KB per block, each epilogue warp writes 32
+// columns of one of the two output runs, and the p_old and x it needs are
+// loaded while the MMAs run.  MMAs and their order per output are the same, so
+// are the results.  Runs while the kernel above would have at most kSmallTiles
+// tiles (above that the input tiles, read once per 32 instead of 128 columns,
+// cost more L2 traffic than the spread gains).
+constexpr int kSN = 32;               // columns per tile
+constexpr int kSBTileBytes = kSN * kBK * 2;
+constexpr int kSStages = 4;
+constexpr int kSmallTiles = 64;
+template <int THREE> struct SmallStage {
+  static constexpr int bytes = kATileBytes + (1 + THREE) * kSBTileBytes;
+  static constexpr size_t smem = (size_t)kSStages * bytes + (size_t)kEpiWarps * 32 * 32 * sizeof(float) + 1024;
+};
+
+template <int THREE>
+__global__ void __launch_bounds__(kGemmThreads, 1) dst_gemm_small_kernel(const GemmDstArgs a) {
+  constexpr int kStageBytes = SmallStage<THREE>::bytes;
+  extern __shared__ __align__(1024) unsigned char gsm_raw[];
+  unsigned char *gsm =
+      reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(gsm_raw) + 1023) & ~uintptr_t(1023));
+  __shared__ __align__(8) uint64_t full_bar[kSStages], empty_bar[kSStages], tfull_bar;
+  __shared__ unsigned tmem_base;
+  __shared__ int abort_flag;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int KB = a.ktiles, n = a.n, ne = (n + 1) >> 1;
+  const unsigned polls = a.polls ? a.polls : kWaitPolls;
+  const int nts = (ne + kSN - 1) / kSN;
+  const int nt = blockIdx.x % nts, mm = blockIdx.x / nts, m = mm / a.mtiles, mt = mm - m * a.mtiles;
+  if (!rhs_selected(a.st, a.mask, m)) return;  // uniform over the CTA, before any set-up
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < kSStages; ++s) {
+      mbar_init(&full_bar[s], 1);
+      mbar_init(&empty_bar[s], 1);
+    }
+    mbar_init(&tfull_bar, 1);
+    abort_flag = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == 0) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base)),
+                 "r"(2u * kSN)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const unsigned tmem = tmem_base;
+  if (warp == 0) {
+    // ---- MMA issuer ----
+    if (lane == 0) {
+      bool ok = true;
+      for (int kb = 0; kb < KB; ++kb) {
+        const int s = kb % kSStages;
+        if (!mbar_wait(&full_bar[s], (unsigned)(kb / kSStages) & 1u, polls)) {
+          ok = false;
+          break;
+        }
+        tc_fence_after();
+        unsigned char *st = gsm + s * kStageBytes;
+        const bool odd = kb >= a.kbe;  // Q block
+        const unsigned acc_t = odd ? tmem + kSN : tmem;
+        const int first = odd ? a.kbe : 0;
+#pragma unroll
+        for (int j = 0; j < kBK / 16; ++j) {
+          const uint64_t ahi = smem_desc(st + j * 256), alo = smem_desc(st + kATileBytes / 2 + j * 256);
+          const uint64_t bhi = smem_desc(st + kATileBytes + j * 256);
+          umma<kSN>(acc_t, ahi, bhi, (kb != first || j != 0) ? 1u : 0u);
+          umma<kSN>(acc_t, alo, bhi, 1u);
+          if (THREE) umma<kSN>(acc_t, ahi, smem_desc(st + kATileBytes + kSBTileBytes + j * 256), 1u);
+        }
+        umma_commit(&empty_bar[s]);
+      }
+      if (ok) {
+        umma_commit(&tfull_bar);
+      } else {
+        atomicExch(&abort_flag, 1);
+        if (a.err) atomicExch(a.err, 1);
+      }
+    }
+  } else if (warp == 1) {
+    // ---- bulk copies ----
+    if (lane == 0) {
+      bool ok = true;
+      int kb = 0;
+      const unsigned char *ga = a.A + ((size_t)m * a.mtiles + mt) * KB * (size_t)kATileBytes;
+      const unsigned char *gb = reinterpret_cast<const unsigned char *>(a.SB) +
+                                (size_t)(nt / (kBN / kSN)) * KB * 2 * kBTileBytes + (nt % (kBN / kSN)) * kSBTileBytes;
+      for (; kb < KB; ++kb) {
+        const int s = kb % kSStages;
+        if (kb >= kSStages && !mbar_wait(&empty_bar[s], (unsigned)(kb / kSStages - 1) & 1u, polls)) {
+          ok = false;
+          break;
+        }
+        if (abort_flag || kb == a.stall_at) {  // stall_at: test of the expiry path, see GemmDstArgs
+          ok = false;
+          break;
+        }
+        unsigned char *st = gsm + s * kStageBytes;
+        mbar_arrive_tx(&full_bar[s], (unsigned)kStageBytes);
+        bulk_g2s(st, ga + (size_t)kb * kATileBytes, kATileBytes, &full_bar[s]);
+        bulk_g2s(st + kATileBytes, gb + (size_t)kb * 2 * kBTileBytes, kSBTileBytes, &full_bar[s]);
+        if (THREE)
+          bulk_g2s(st + kATileBytes + kSBTileBytes, gb + ((size_t)kb * 2 + 1) * kBTileBytes, kSBTileBytes,
+                   &full_bar[s]);
+      }
+      if (!ok) {
+        atomicExch(&abort_flag, 1);
+        if (a.err) atomicExch(a.err, 1);
+        // wait (bounded) for the copies in flight
+        for (int j = kb > kSStages ? kb - kSStages : 0; j < kb; ++j)
+          mbar_wait(&full_bar[j % kSStages], (unsigned)(j / kSStages) & 1u, polls);
+      }
+    }
+  } else if (warp >= 4) {
+    // ---- epilogue: warp w drains TMEM lane quarter w % 4 for one output run:
+    // run 0 the columns l (cosine forward: 2 l), run 1 their mirrors n - 1 - l
+    // (2 l + 1) ----
+    const int ew = warp - 4, q = warp & 3, run = ew >> 2;
+    const int l0 = nt * kSN, row0 = mt * kBM + q * 32, grow = row0 + lane;
+    const float rsc = (a.rowscale != nullptr && grow < a.nr) ? __ldg(a.rowscale + m * a.rsstride + grow) : 1.f;
+    const int lc = l0 + lane;  // this lane's column of the half range, when a lane is a column
+    const int col = a.cosfwd ? 2 * lc + run : (run ? n - 1 - lc : lc);
+    const bool colok = a.cosfwd ? (lc < ne && col < n) : (lc < ne && (run == 0 || col != lc));
+    const size_t cbase = (size_t)m * (size_t)a.field + (size_t)row0 * a.pitch + col;
+    const bool pupd = a.pa != nullptr;
+    float *png = nullptr, *xg = nullptr;
+    float beta = 0.f, alpha = 0.f;
+    float po[32], xv[32];
+    if (pupd) {  // direction update: p_new = out + beta p_old (and x += alpha p_old)
+      const bool odd = a.st[m].iters & 1;
+      const float *pog = odd ? a.pb : a.pa;
+      png = odd ? a.pa : a.pb;
+      beta = (float)a.st[m].beta;
+      const bool xnew = a.st[m].iters == a.st[m].xbase;  // x = alpha p_old
+      if (a.x != nullptr) {
+        xg = a.x;
+        alpha = (float)a.st[m].alpha;
+      }
+#pragma unroll
+      for (int r = 0; r < 32; ++r) {
+        const bool ok = colok && row0 + r < a.nr;
+        po[r] = ok ? __ldg(pog + cbase + (size_t)r * a.pitch) : 0.f;
+        xv[r] = (ok && xg && !xnew) ? xg[cbase + (size_t)r * a.pitch] : 0.f;
+      }
+    }
+    const bool ok = !abort_flag && mbar_wait(&tfull_bar, 0u, polls);
+    if (!ok) {
+      atomicExch(&abort_flag, 1);
+      if (a.err) atomicExch(a.err, 1);
+    }
+    tc_fence_after();
+    if (__all_sync(0xffffffffu, ok)) {
+      const unsigned tP = tmem + ((unsigned)(q * 32) << 16);
+      float P[32], Q[32];
+      tmem_ld32(tP, P);
+      if (a.ktiles > a.kbe) {
+        tmem_ld32(tP + kSN, Q);
+      } else {
+#pragma unroll
+        for (int i = 0; i < 32; ++i) Q[i] = 0.f;  // n = 1: no odd column
+      }
+#pragma unroll
+      for (int i = 0; i < 32; ++i) {
+        const float v = a.cosfwd ? (run ? Q[i] : P[i]) : (run ? P[i] - Q[i] : P[i] + Q[i]);
+        P[i] = rsc * v;
+      }
+      if (a.tout) {
+        // mode-major output: lane = row, a run of 32 rows per store
+        if (grow < a.nr) {
+          float *ob = a.out + (size_t)m * n * a.tpitch + grow;
+#pragma unroll
+          for (int i = 0; i < 32; ++i) {
+            const int l = l0 + i, c = a.cosfwd ? 2 * l + run : (run ? n - 1 - l : l);
+            if (l < ne && c < n && (a.cosfwd || run == 0 || c != l)) ob[(size_t)c * a.tpitch] = P[i];
+          }
+        }
+      } else {
+        // lane = column, through this warp's 32 x 32 shared tile (XOR-swizzled)
+        float *T = reinterpret_cast<float *>(gsm + kSStages * kStageBytes) + ew * 1024;
+#pragma unroll
+        for (int i = 0; i < 32; ++i) T[lane * 32 + (i ^ lane)] = P[i];
+        __syncwarp();
+        if (pupd) {
+#pragma unroll
+          for (int r = 0; r < 32; ++r)
+            if (colok && row0 + r < a.nr) {
+              const size_t e = cbase + (size_t)r * a.pitch;
+              png[e] = fmaf(beta, po[r], T[r * 32 + (lane ^ r)]);
+              if (xg) xg[e] = fmaf(alpha, po[r], xv[r]);
+            }
+        } else {
+#pragma unroll 8
+          for (int r = 0; r < 32; ++r)
+            if (colok && row0 + r < a.nr) a.out[cbase + (size_t)r * a.pitch] = T[r * 32 + (lane ^ r)];
+        }
+      }
+    }
+  }
+  tc_fence_before();
+  __syncthreads();
+  if (warp == 0) {
+    if (abort_flag) mbar_wait(&tfull_bar, 0u, polls);  // a bounded moment for MMAs in flight
+    tc_fence_after();
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(2u * kSN) : "memory");
+  }
+}
+
 }  // namespace
 
 size_t dst_gemm_smem_bytes(int three) {
@@ -617,8 +832,20 @@ void launch_dst_gemm(const GemmDstArgs &a, cudaStream_t s) {
     if (sms <= 0) sms = 148;
   }
   const int tiles = a.m * a.mtiles * a.ntiles;
-  dim3 grid(std::min(tiles, sms));
   note_launch();
+  if (tiles <= kSmallTiles && a.r == nullptr) {
+    const int nts = ((a.n + 1) / 2 + kSN - 1) / kSN;
+    const unsigned g = (unsigned)(a.m * a.mtiles * nts);
+    if (a.three) {
+      ensure_smem_attr((const void *)dst_gemm_small_kernel<1>, SmallStage<1>::smem);
+      dst_gemm_small_kernel<1><<<g, kGemmThreads, SmallStage<1>::smem, s>>>(a);
+    } else {
+      ensure_smem_attr((const void *)dst_gemm_small_kernel<0>, SmallStage<0>::smem);
+      dst_gemm_small_kernel<0><<<g, kGemmThreads, SmallStage<0>::smem, s>>>(a);
+    }
+    return;
+  }
+  dim3 grid(std::min(tiles, sms));
   if (a.three) {
     ensure_smem_attr((const void *)dst_gemm_kernel<1>, smem);
     dst_gemm_kernel<1><<<grid, kGemmThreads, smem, s>>>(a);

@@ -55,8 +55,11 @@ def test_each_solve_meets_its_own_tolerance(method, tols):
         P.ax_destroy_operator(op)
 
 
+# the last two have one right-hand side below and nine above the tile count at
+# which the tensor-core transform takes its 32-column tiles
 @pytest.mark.parametrize("bc_z", [0, 1])
-@pytest.mark.parametrize("nr,nz", [(1, 5), (2, 128), (3, 129), (17, 131), (40, 256), (64, 33), (65, 260), (259, 127)])
+@pytest.mark.parametrize("nr,nz", [(1, 5), (2, 128), (3, 129), (17, 131), (40, 256), (64, 33), (65, 260), (259, 127),
+                                   (513, 517), (900, 386)])
 def test_strip_edges(nr, nz, bc_z):
     m = 9
     op, ora, f, dev = _problem(nr, nz, m, bc_z)
