@@ -191,6 +191,7 @@ struct ax_operator {
   int device = 0;
   ax::FftPlan plan;
   int *rader_perm = nullptr;  // [2 P] device
+  unsigned char *arena = nullptr;  // set-up: one allocation holds every table (null: each its own)
   int dst_tc = 0;             // 1: the FP32 PCG path transforms with the tensor-core GEMM
   int tri_variant = 0;        // FP32 mode-solve kernel (0: default for nr; option "mode_kernel")
   int *tc_err = nullptr;      // device flag: a bounded wait of the GEMM expired

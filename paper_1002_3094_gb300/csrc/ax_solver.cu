@@ -54,6 +54,7 @@ struct Workspace {
   int m64 = 0, m32 = 0, mbase = 0;
   // FP64 vectors [m][nr][pitch]
   double *phi64 = nullptr, *x64 = nullptr;
+  double *arena64 = nullptr;  // one allocation holds the FP64 vectors
   double *r64 = nullptr, *pa64 = nullptr, *pb64 = nullptr, *q64 = nullptr, *z64 = nullptr, *y64prev = nullptr;
   // FP32 vectors
   // double-float x (two buffers, see DfResidualArgs) and phi (mixed PCG)
@@ -62,6 +63,7 @@ struct Workspace {
   bool df32 = false;         // it holds the double-float vectors too
   float *x32 = nullptr, *r32 = nullptr, *pa32 = nullptr, *pb32 = nullptr, *q32 = nullptr, *z32 = nullptr,
         *y32prev = nullptr;
+  unsigned char *base = nullptr;  // one allocation: part .. chk below
   // partial sums [4][m][kPartialStride]
   double *part = nullptr;
   double *chp = nullptr;      // Chebyshev (tau, rho0^2) per right-hand side [m][2]
@@ -193,7 +195,8 @@ void free_graph(GraphCache &g) {
 }
 
 void free_vectors64(Workspace *w) {
-  dfree(w->r64); dfree(w->pa64); dfree(w->pb64); dfree(w->q64); dfree(w->z64); dfree(w->y64prev);
+  dfree(w->arena64);
+  w->r64 = w->pa64 = w->pb64 = w->q64 = w->z64 = w->y64prev = nullptr;
   w->m64 = 0;
   free_graph(w->g64);
   free_graph(w->gc64);
@@ -208,8 +211,12 @@ void free_vectors32(Workspace *w) {
   free_graph(w->gc32);
 }
 void free_base(Workspace *w) {
-  dfree(w->phi64); dfree(w->x64); dfree(w->part); dfree(w->chp); dfree(w->rscale); dfree(w->st);
-  dfree(w->st_outer); dfree(w->chk); dfree(w->arrive); dfree(w->par);
+  dfree(w->phi64); dfree(w->base);
+  w->x64 = nullptr;
+  w->part = w->chp = w->rscale = w->par = nullptr;
+  w->st = w->st_outer = nullptr;
+  w->arrive = nullptr;
+  w->chk = nullptr;
   if (w->h_st) cudaFreeHost(w->h_st);
   w->h_st = nullptr;
   w->mbase = w->mfield64 = 0;
@@ -223,14 +230,17 @@ int ensure_base(ax_operator *op, int m) {
   Workspace *w = op->ws;
   if (w->mbase >= m) return AX_OK;
   free_base(w);
-  AX_TRY(dalloc(&w->part, (size_t)4 * m * kPartialStride));
-  AX_TRY(dalloc(&w->chp, (size_t)2 * m));
-  AX_TRY(dalloc(&w->rscale, (size_t)m));
-  AX_TRY(dalloc(&w->st, (size_t)m));
-  AX_TRY(dalloc(&w->st_outer, (size_t)m));
-  AX_TRY(dalloc(&w->chk, 1));
-  AX_TRY(dalloc(&w->arrive, (size_t)m));
-  AX_TRY(dalloc(&w->par, 2));
+  // one zeroed allocation (each costs tens of microseconds, as does its release)
+  const size_t mm = (size_t)m, nd = 4 * mm * kPartialStride + 3 * mm + 2;
+  AX_TRY(dalloc(&w->base, nd * sizeof(double) + 2 * mm * sizeof(RhsState) + (mm + 1) * sizeof(unsigned)));
+  w->part = reinterpret_cast<double *>(w->base);
+  w->chp = w->part + 4 * mm * kPartialStride;
+  w->rscale = w->chp + 2 * mm;
+  w->par = w->rscale + mm;
+  w->st = reinterpret_cast<RhsState *>(w->part + nd);
+  w->st_outer = w->st + mm;
+  w->arrive = reinterpret_cast<unsigned *>(w->st_outer + mm);
+  w->chk = reinterpret_cast<int *>(w->arrive + mm);
   AX_TRY(cudaMallocHost((void **)&w->h_st, sizeof(RhsState) * 2 * m));
   w->mbase = m;
   return AX_OK;
@@ -242,12 +252,12 @@ int ensure_field64(ax_operator *op, int m) {
   Workspace *w = op->ws;
   if (w->mfield64 >= m) return AX_OK;
   dfree(w->phi64);
-  dfree(w->x64);
+  w->x64 = nullptr;
   w->mfield64 = 0;
   free_graph(w->g64); free_graph(w->gc64);
   const size_t f = field_elems(op) * m;
-  AX_TRY(dalloc(&w->phi64, f));
-  AX_TRY(dalloc(&w->x64, f));
+  AX_TRY(dalloc(&w->phi64, 2 * f));
+  w->x64 = w->phi64 + f;
   w->mfield64 = m;
   return AX_OK;
 }
@@ -258,12 +268,13 @@ int ensure_vec64(ax_operator *op, int m, bool cheb) {
   if (w->m64 >= m && (!cheb || w->y64prev)) return AX_OK;
   free_vectors64(w);
   const size_t f = field_elems(op) * m;
-  AX_TRY(dalloc(&w->r64, f));
-  AX_TRY(dalloc(&w->pa64, f));
-  AX_TRY(dalloc(&w->pb64, f));
-  AX_TRY(dalloc(&w->q64, f));
-  AX_TRY(dalloc(&w->z64, f));
-  if (cheb) AX_TRY(dalloc(&w->y64prev, f));
+  AX_TRY(dalloc(&w->arena64, f * (cheb ? 6 : 5)));
+  w->r64 = w->arena64;
+  w->pa64 = w->arena64 + f;
+  w->pb64 = w->arena64 + 2 * f;
+  w->q64 = w->arena64 + 3 * f;
+  w->z64 = w->arena64 + 4 * f;
+  if (cheb) w->y64prev = w->arena64 + 5 * f;
   w->m64 = m;
   return AX_OK;
 }
@@ -1031,32 +1042,202 @@ void rader_tables(int R, std::vector<int> &perm, std::vector<double> &rk, std::v
     cr[mm] = std::cos(ang);
     ci[mm] = std::sin(ang);
   }
+  rt.assign(2 * P, 0.0);
+  for (int j = 0; j < P; ++j) {
+    rt[2 * j] = std::cos(2.0 * M_PI * j / P);
+    rt[2 * j + 1] = std::sin(2.0 * M_PI * j / P);
+  }
   rk.assign(2 * P, 0.0);
   for (int k = 0; k < P; ++k) {
     double sr = 0.0, si = 0.0;
-    for (int mm = 0; mm < P; ++mm) {
-      const long long e = ((long long)mm * k) % P;
-      const double c = std::cos(2.0 * M_PI * e / P), sn = -std::sin(2.0 * M_PI * e / P);
+    for (int mm = 0, e = 0; mm < P; ++mm, e = e + k < P ? e + k : e + k - P) {  // e = mm k mod P
+      const double c = rt[2 * e], sn = -rt[2 * e + 1];
       sr += cr[mm] * c - ci[mm] * sn;
       si += cr[mm] * sn + ci[mm] * c;
     }
     rk[2 * k] = sr;
     rk[2 * k + 1] = si;
   }
-  rt.assign(2 * P, 0.0);
-  for (int j = 0; j < P; ++j) {
-    rt[2 * j] = std::cos(2.0 * M_PI * j / P);
-    rt[2 * j + 1] = std::sin(2.0 * M_PI * j / P);
+}
+
+// ---------------------------------------------------------------------------
+// Operator tables on the GPU (the host built them before: 3 ms at 256 x 256, 31
+// ms at 1024 x 1024, most of it passes over FP64 arrays and their copies)
+// ---------------------------------------------------------------------------
+struct SetupRange {
+  unsigned long long kmin, kmax, qmin, qmax;  // FP64 bits (ordered as the values: none is negative)
+  int bad;                                    // a sample is not finite, kappa <= 0 or q < 0
+};
+__global__ void __launch_bounds__(256) setup_range(const double *__restrict__ kr, const double *__restrict__ kz,
+                                                   const double *__restrict__ q, int nr, int nz, SetupRange *out) {
+  unsigned long long kmin = ~0ull, kmax = 0, qmin = ~0ull, qmax = 0;
+  bool bad = false;
+  auto bits = [](double v) { return (unsigned long long)__double_as_longlong(v); };
+  constexpr unsigned long long kInf = 0x7FF0000000000000ull, kSign = 0x8000000000000000ull;
+  auto kappa = [&](double v) {
+    const unsigned long long b = bits(v);
+    bad = bad || b == 0 || b >= kInf;  // zero, negative, infinite or NaN
+    kmin = min(kmin, b);
+    kmax = max(kmax, b);
+  };
+  for (int i = blockIdx.x; i < nr; i += gridDim.x)
+    for (int k = threadIdx.x; k <= nz; k += 256) {
+      kappa(kz[(size_t)i * (nz + 1) + k]);
+      if (k == nz) continue;
+      kappa(kr[(size_t)i * nz + k]);
+      const unsigned long long b = bits(q[(size_t)i * nz + k]), a = b == kSign ? 0 : b;  // -0 is 0
+      bad = bad || a >= kInf;
+      qmin = min(qmin, a);
+      qmax = max(qmax, a);
+    }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    kmin = min(kmin, __shfl_xor_sync(0xffffffffu, kmin, o));
+    kmax = max(kmax, __shfl_xor_sync(0xffffffffu, kmax, o));
+    qmin = min(qmin, __shfl_xor_sync(0xffffffffu, qmin, o));
+    qmax = max(qmax, __shfl_xor_sync(0xffffffffu, qmax, o));
+  }
+  const bool any = __any_sync(0xffffffffu, bad);
+  if ((threadIdx.x & 31) == 0) {
+    atomicMin(&out->kmin, kmin);
+    atomicMax(&out->kmax, kmax);
+    atomicMin(&out->qmin, qmin);
+    atomicMax(&out->qmax, qmax);
+    if (any) atomicExch(&out->bad, 1);
   }
 }
 
-template <typename T>
-cudaError_t upload(T **dst, const std::vector<double> &src) {
-  std::vector<T> tmp(src.size());
-  for (size_t i = 0; i < src.size(); ++i) tmp[i] = (T)src[i];
-  cudaError_t e = dalloc(dst, src.size());
-  if (e != cudaSuccess) return e;
-  return cudaMemcpy(*dst, tmp.data(), tmp.size() * sizeof(T), cudaMemcpyHostToDevice);
+struct SetupArgs {
+  const double *kr, *kz, *q;
+  const double *stage;  // E, R, RS, diagonal of the r-operator, 1 / RS^2 [nr] each; Rader tables RK, RT [p2]
+  Coef<double> c64;
+  Coef<float> c32;
+  int nr, nz, pitch, pitchz, tpitch, L, cosine, p2;
+  double hr, hz, kt, qt;
+};
+
+// Short tables: couplings, radii, row scales and the transforms' factors.
+__global__ void __launch_bounds__(256) setup_small(const SetupArgs a) {
+  const int t0 = blockIdx.x * blockDim.x + threadIdx.x, dt = gridDim.x * blockDim.x;
+  const int nr = a.nr;
+  for (int i = t0; i < nr; i += dt) {
+    const double e = a.stage[i], r = a.stage[nr + i];
+    a.c64.E[i] = e;
+    a.c32.E[i] = (float)e;
+    a.c64.R[i] = r;
+    a.c32.R[i] = (float)r;
+    a.c32.RS[i] = (float)a.stage[2 * nr + i];
+  }
+  for (int j = t0; j < a.L; j += dt) {
+    double sn, cs;
+    sincospi(2.0 * j / a.L, &sn, &cs);
+    a.c64.TW[2 * j] = cs;
+    a.c64.TW[2 * j + 1] = sn;
+    a.c32.TW[2 * j] = (float)cs;
+    a.c32.TW[2 * j + 1] = (float)sn;
+    sincospi((double)j / a.L, &sn, &cs);
+    a.c64.HW[2 * j] = cs;
+    a.c64.HW[2 * j + 1] = sn;
+    a.c32.HW[2 * j] = (float)cs;
+    a.c32.HW[2 * j + 1] = (float)sn;
+  }
+  // Cosine pair, per mode l = 0..nz-1 with phi = pi l / (2 nz): forward
+  // factors s_l / 4 * (cos phi, sin phi, cos 3 phi, sin 3 phi), s_l the
+  // orthonormal scale (sqrt(1/nz) for l = 0, sqrt(2/nz) otherwise); inverse
+  // factors (cos phi, sin phi) (times sqrt 2 for l = 0: X_0 = sqrt(nz) Xhat_0
+  // against sqrt(nz / 2) for the others, which the store scale holds) and
+  // (cos 2 phi, sin 2 phi).
+  if (a.cosine)
+    for (int l = t0; l < a.nz; l += dt) {
+      const double x = l / (2.0 * a.nz);
+      const double f = 0.25 * sqrt(2.0 / a.nz) * (l == 0 ? sqrt(0.5) : 1.0), g0 = l == 0 ? sqrt(2.0) : 1.0;
+      double c1, s1, c2, s2, c3, s3;
+      sincospi(x, &s1, &c1);
+      sincospi(2.0 * x, &s2, &c2);
+      sincospi(3.0 * x, &s3, &c3);
+      const double v[8] = {f * c1, f * s1, f * c3, f * s3, g0 * c1, g0 * s1, c2, s2};
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        a.c64.CW[8 * l + j] = v[j];
+        a.c32.CW[8 * l + j] = (float)v[j];
+      }
+    }
+  for (int j = t0; j < a.p2; j += dt) {
+    const double k = a.stage[5 * nr + j], t = a.stage[5 * nr + a.p2 + j];
+    a.c64.RK[j] = k;
+    a.c32.RK[j] = (float)k;
+    a.c64.RT[j] = t;
+    a.c32.RT[j] = (float)t;
+  }
+}
+
+// Stencil coefficients (Eq. diff_approx1): CR = KR / h_r^2, CZ = KZ / h_z^2, W = r q
+// in FP64, FP32 and the FP32 low parts of the double-float residual (v64 =
+// (float)v64 + lo); the padding columns are written as zeros.
+__global__ void __launch_bounds__(256) setup_fields(const SetupArgs a) {
+  const double hr2 = a.hr * a.hr, hz2 = a.hz * a.hz;
+  for (int i = blockIdx.x; i < a.nr; i += gridDim.x) {
+    const double rbar = (i + 1) * a.hr, ri = (i + 0.5) * a.hr;  // face between r-nodes i + 1 and i + 2 (1-based)
+    for (int k = threadIdx.x; k < a.pitch; k += 256) {
+      const size_t e = (size_t)i * a.pitch + k, src = (size_t)i * a.nz + k;
+      const double cr = k < a.nz ? rbar * a.kr[src] / hr2 : 0.0, w = k < a.nz ? ri * a.q[src] : 0.0;
+      const float crh = (float)cr, wh = (float)w;
+      a.c64.CR[e] = cr;
+      a.c32.CR[e] = crh;
+      a.c32.CRl[e] = (float)(cr - (double)crh);
+      a.c64.W[e] = w;
+      a.c32.W[e] = wh;
+      a.c32.Wl[e] = (float)(w - (double)wh);
+    }
+    for (int k = threadIdx.x; k < a.pitchz; k += 256) {
+      const size_t e = (size_t)i * a.pitchz + k;
+      // zero-flux z: no flux through z = 0 and z = lz (one-sided rows of Eq. scheme_op_r_z)
+      const bool in = k <= a.nz && !(a.cosine && (k == 0 || k == a.nz));
+      const double cz = in ? ri * a.kz[(size_t)i * (a.nz + 1) + k] / hz2 : 0.0;
+      const float h = (float)cz;
+      a.c64.CZ[e] = cz;
+      a.c32.CZ[e] = h;
+      a.c32.CZl[e] = (float)(cz - (double)h);
+    }
+  }
+}
+
+// Per-mode Thomas factors of T_l (Eq. eq_trid) in FP64, delta_a = d_a - E_{a-1}^2
+// / delta_{a-1}: a lane per mode column, a chain of one division per row.  IP = 1 /
+// delta; IPS = IP / RS^2 the inverse pivots of the row-scaled systems D T D, and
+// IPST the same mode-major, through a 32 x 32 shared tile.  One warp per CTA.
+__global__ void __launch_bounds__(32) setup_factors(const SetupArgs a) {
+  __shared__ float tile[32][33];
+  const int lane = threadIdx.x, l = blockIdx.x * 32 + lane, nr = a.nr;
+  const bool ok = l < a.nz;
+  const double *E = a.stage, *R = E + nr, *DG = E + 3 * nr, *I2 = E + 4 * nr;
+  // mode eigenvalue of the z second difference: sine modes l + 1 = 1..nz, or the
+  // cosine modes of Eq. eq_trid, 4/h^2 sin^2(pi l / (2 nz)) (0 for l = 0)
+  const double sn = a.cosine ? sinpi(l / (2.0 * a.nz)) : sinpi((l + 1) / (2.0 * (a.nz + 1)));
+  const double shift = a.kt * (4.0 / (a.hz * a.hz) * sn * sn) + a.qt;
+  double ip = 0.0;
+  for (int a0 = 0; a0 < nr; a0 += 32) {
+    const int cnt = min(32, nr - a0);
+    for (int j = 0; j < cnt; ++j) {
+      const int i = a0 + j;
+      const double e = i > 0 ? E[i - 1] : 0.0;
+      const double delta = fma(-(e * e), ip, fma(R[i], shift, DG[i]));
+      ip = 1.0 / delta;
+      const size_t o = (size_t)i * a.pitch + l;
+      const float ips = ok ? (float)(ip * I2[i]) : 0.f;
+      a.c64.IP[o] = ok ? ip : 0.0;
+      a.c32.IP[o] = ok ? (float)ip : 0.f;
+      a.c32.IPS[o] = ips;
+      tile[j][lane] = ips;
+    }
+    for (int j = cnt; j < 32; ++j) tile[j][lane] = 0.f;
+    __syncwarp();
+    for (int j = 0; j < 32; ++j) {
+      const int col = blockIdx.x * 32 + j;
+      if (col < a.nz) a.c32.IPST[(size_t)col * a.tpitch + a0 + lane] = tile[lane][j];
+    }
+    __syncwarp();
+  }
 }
 
 template <typename T>
@@ -1708,6 +1889,7 @@ int run_graph(Workspace *w, GraphCache &g, int key, cudaStream_t s, F body) {
     std::lock_guard<std::recursive_mutex> lock(g_alloc_capture_mutex);
     free_graph(g);
     cudaGraph_t graph = nullptr;
+    if (!w->cap) AX_TRY(cudaStreamCreateWithFlags(&w->cap, cudaStreamNonBlocking));
     AX_TRY(cudaStreamBeginCapture(w->cap, cudaStreamCaptureModeRelaxed));
     g_capturing = true;
     body(w->cap);
@@ -2334,9 +2516,13 @@ int ax_profile_read(ax_operator *op, int32_t kind, double *ms, double *launches,
 
 int ax_destroy_operator(ax_operator *op) {
   if (!op) return AX_OK;
-  free_coef(op->c64);
-  free_coef(op->c32);
-  dfree(op->rader_perm);
+  if (op->arena) {  // one allocation holds every table
+    dfree(op->arena);
+  } else {
+    free_coef(op->c64);
+    free_coef(op->c32);
+    dfree(op->rader_perm);
+  }
   if (op->ws) {
     Workspace *w = op->ws;
     free_vectors64(w);
@@ -2687,26 +2873,6 @@ int ax_setup_operator(const double *kappa_r, const double *kappa_z, const double
     const int prc = dst_prepare_device();
     if (prc != AX_OK) return prc;
   }
-  const size_t nrz = (size_t)nr * nz, nrz1 = (size_t)nr * (nz + 1);
-  std::vector<double> kr(nrz), kz(nrz1), qq(nrz);
-  AX_TRY(cudaMemcpyAsync(kr.data(), kappa_r, nrz * sizeof(double), cudaMemcpyDeviceToHost, s));
-  AX_TRY(cudaMemcpyAsync(kz.data(), kappa_z, nrz1 * sizeof(double), cudaMemcpyDeviceToHost, s));
-  AX_TRY(cudaMemcpyAsync(qq.data(), q, nrz * sizeof(double), cudaMemcpyDeviceToHost, s));
-  AX_TRY(cudaStreamSynchronize(s));
-  double kmin = INFINITY, kmax = -INFINITY, qmin = INFINITY, qmax = -INFINITY;
-  for (double v : kr) {
-    if (!std::isfinite(v) || !(v > 0.0)) return AX_ERR_INVALID_ARG;
-    kmin = std::min(kmin, v); kmax = std::max(kmax, v);
-  }
-  for (double v : kz) {
-    if (!std::isfinite(v) || !(v > 0.0)) return AX_ERR_INVALID_ARG;
-    kmin = std::min(kmin, v); kmax = std::max(kmax, v);
-  }
-  for (double v : qq) {
-    if (!std::isfinite(v) || v < 0.0) return AX_ERR_INVALID_ARG;
-    qmin = std::min(qmin, v); qmax = std::max(qmax, v);
-  }
-
   ax_operator *op = new ax_operator();
   op->ws = new Workspace();
   op->nr = nr;
@@ -2720,16 +2886,6 @@ int ax_setup_operator(const double *kappa_r, const double *kappa_z, const double
   // zero-flux z: cell-centred nodes, the boundary faces on z = 0 and z = lz
   op->hz = cosine ? g->lz / nz : g->lz / (nz + 1.0);
   cudaGetDevice(&op->device);
-  // Eq. coeff2 with the footnote of Eq. diff_approx2: mean of the extremes.
-  op->kappa_t = 0.5 * (kmin + kmax);
-  op->q_t = 0.5 * (qmin + qmax);
-  // gamma_1, gamma_2 (Eq. energy_rel): face-wise ratios bound the Rayleigh quotient.
-  op->gamma1 = kmin / op->kappa_t;
-  op->gamma2 = kmax / op->kappa_t;
-  if (op->q_t > 0.0) {
-    op->gamma1 = std::min(op->gamma1, qmin / op->q_t);
-    op->gamma2 = std::max(op->gamma2, qmax / op->q_t);
-  }
   // FFT length: the sine transform packs its odd extension of length 2(nz+1),
   // the cosine pair its even extension of length 2 nz
   const int L = cosine ? nz : nz + 1;
@@ -2751,132 +2907,114 @@ int ax_setup_operator(const double *kappa_r, const double *kappa_z, const double
       if (op->plan.radix[i] > 8) op->dst_tc = 1;
   }
 
-  const double hr = op->hr, hz = op->hz, hr2 = hr * hr, hz2 = hz * hz;
-  const int P = op->pitch, PZ = op->pitchz;
-  std::vector<double> ri(nr), CR((size_t)nr * P, 0.0), CZ((size_t)nr * PZ, 0.0), W((size_t)nr * P, 0.0);
-  for (int a = 0; a < nr; ++a) ri[a] = (a + 0.5) * hr;
+  std::vector<int> perm;
+  std::vector<double> rk, rt;
+  const size_t P2 = op->plan.rader ? 2 * (size_t)(op->plan.radix[0] - 1) : 0;
+  op->tpitch = (nr + 31) / 32 * 32;
+  // every table in one allocation, each on a 256-byte boundary; FP64 tables,
+  // then FP32
+  const size_t f = (size_t)nr * op->pitch, fz = (size_t)nr * op->pitchz, ft = (size_t)nz * op->tpitch;
+  size_t bytes = 0;
+  std::vector<std::pair<void **, size_t>> parts;
+  auto want = [&](auto **p, size_t count) {
+    if (count == 0) return;
+    parts.push_back({(void **)p, bytes});
+    bytes += (count * sizeof(**p) + 255) / 256 * 256;
+  };
+  auto common = [&](auto &c) {
+    want(&c.CR, f); want(&c.CZ, fz); want(&c.W, f); want(&c.IP, f); want(&c.E, nr); want(&c.R, nr);
+    want(&c.TW, 2 * (size_t)L); want(&c.HW, 2 * (size_t)L); want(&c.CW, cosine ? 8 * (size_t)nz : 0);
+    want(&c.RK, P2); want(&c.RT, P2);
+  };
+  double *stage = nullptr;
+  SetupRange *range = nullptr;
+  want(&range, 1);
+  common(op->c64);
+  want(&stage, 5 * (size_t)nr + 2 * P2);
+  common(op->c32);
+  want(&op->c32.IPS, f); want(&op->c32.RS, nr); want(&op->c32.IPST, ft);
+  want(&op->c32.CRl, f); want(&op->c32.CZl, fz); want(&op->c32.Wl, f);
+  want(&op->rader_perm, P2);
+  cudaError_t e;
+  {
+    std::lock_guard<std::recursive_mutex> lock(g_alloc_capture_mutex);
+    e = cudaMalloc((void **)&op->arena, bytes);
+  }
+  if (e != cudaSuccess) op->arena = nullptr;
+  if (e == cudaSuccess)
+    for (auto &pr : parts) *pr.first = op->arena + pr.second;
+  // extremes and validity of the samples, on the GPU
+  SetupRange hr_{~0ull, 0ull, ~0ull, 0ull, 0};
+  if (e == cudaSuccess) e = cudaMemcpyAsync(range, &hr_, sizeof(hr_), cudaMemcpyHostToDevice, s);
+  if (e == cudaSuccess) {
+    note_launch();
+    setup_range<<<(unsigned)std::min(nr, 608), 256, 0, s>>>(kappa_r, kappa_z, q, nr, nz, range);
+    e = cudaGetLastError();
+  }
+  if (e == cudaSuccess) e = cudaMemcpyAsync(&hr_, range, sizeof(hr_), cudaMemcpyDeviceToHost, s);
+  if (op->plan.rader) rader_tables(op->plan.radix[0], perm, rk, rt);  // while it runs
+  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+  if (e != cudaSuccess || hr_.bad) {
+    ax_destroy_operator(op);
+    return e != cudaSuccess ? status_from_cuda(e) : AX_ERR_INVALID_ARG;
+  }
+  auto as_double = [](unsigned long long b) {
+    double v;
+    std::memcpy(&v, &b, sizeof(v));
+    return v;
+  };
+  const double kmin = as_double(hr_.kmin), kmax = as_double(hr_.kmax);
+  const double qmin = as_double(hr_.qmin), qmax = as_double(hr_.qmax);
+  // Eq. coeff2 with the footnote of Eq. diff_approx2: mean of the extremes.
+  op->kappa_t = 0.5 * (kmin + kmax);
+  op->q_t = 0.5 * (qmin + qmax);
+  // gamma_1, gamma_2 (Eq. energy_rel): face-wise ratios bound the Rayleigh quotient.
+  op->gamma1 = kmin / op->kappa_t;
+  op->gamma2 = kmax / op->kappa_t;
+  if (op->q_t > 0.0) {
+    op->gamma1 = std::min(op->gamma1, qmin / op->q_t);
+    op->gamma2 = std::max(op->gamma2, qmax / op->q_t);
+  }
+  // Couplings and row scales on the host (short recurrences along r): E_a the
+  // off-diagonal of T_l (Eq. eq_trid); D = diag(rs) the scaling to unit couplings
+  // for the FP32 mode solves, T' = D T D, rs_a rs_{a+1} |E_a| = 1 (rs_0 =
+  // |E_0|^-1/2, so the scale stays near |E_a|^-1/2).
+  const double hr = op->hr;
+  std::vector<double> small(5 * (size_t)nr, 0.0);  // SetupArgs::stage
+  double *E = small.data(), *ri = E + nr, *RS = ri + nr, *DG = RS + nr, *I2 = DG + nr;
   for (int a = 0; a < nr; ++a) {
-    const double rbar = (a + 1) * hr;  // face between r-nodes a+1 and a+2 (1-based)
-    for (int b = 0; b < nz; ++b) {
-      CR[(size_t)a * P + b] = rbar * kr[(size_t)a * nz + b] / hr2;
-      W[(size_t)a * P + b] = ri[a] * qq[(size_t)a * nz + b];
-    }
-    for (int c = 0; c <= nz; ++c) CZ[(size_t)a * PZ + c] = ri[a] * kz[(size_t)a * (nz + 1) + c] / hz2;
-    if (cosine) {  // no flux through z = 0 and z = lz (one-sided rows of Eq. scheme_op_r_z)
-      CZ[(size_t)a * PZ] = 0.0;
-      CZ[(size_t)a * PZ + nz] = 0.0;
-    }
+    ri[a] = (a + 0.5) * hr;
+    RS[a] = 1.0;
+    DG[a] = op->kappa_t * ((a + 1) * hr + a * hr) / (hr * hr);
+    if (a + 1 < nr) E[a] = -op->kappa_t * (a + 1) * hr / (hr * hr);
   }
-  // Per-mode Thomas factors of T_l (Eq. eq_trid), computed in FP64.
-  std::vector<double> E(nr, 0.0), IP((size_t)nr * P, 0.0);
-  const double kt = op->kappa_t, qt = op->q_t;
-  for (int a = 0; a + 1 < nr; ++a) E[a] = -kt * (a + 1) * hr / hr2;
-  for (int l = 1; l <= nz; ++l) {
-    // mode eigenvalue of the z second difference: sine modes l = 1..nz, or the
-    // cosine modes of Eq. eq_trid, 4/h^2 sin^2(pi (l - 1) / (2 nz)) (0 for l = 1)
-    const double sn = cosine ? std::sin(M_PI * (l - 1) / (2.0 * nz)) : std::sin(M_PI * l / (2.0 * (nz + 1)));
-    const double lam = 4.0 / hz2 * sn * sn;
-    double delta = 0.0;
-    for (int a = 0; a < nr; ++a) {
-      const double rbar_hi = (a + 1) * hr, rbar_lo = a * hr;
-      const double d = kt * (rbar_hi + rbar_lo) / hr2 + ri[a] * (kt * lam + qt);
-      delta = (a == 0) ? d : d - E[a - 1] * E[a - 1] / delta;
-      IP[(size_t)a * P + (l - 1)] = 1.0 / delta;
-    }
-  }
-  // The same systems scaled to unit couplings for the FP32 pipelined mode
-  // solves: T' = D T D, D = diag(rs), rs_a rs_{a+1} |E_a| = 1 (rs_0 =
-  // |E_0|^-1/2, so the scale stays near |E_a|^-1/2); pivots of the scaled
-  // diagonal rs_a^2 d_a(l) with off-diagonal -1.
-  std::vector<double> RS(nr, 1.0), IPS((size_t)nr * P, 0.0);
   if (nr > 1) {
     RS[0] = 1.0 / std::sqrt(std::fabs(E[0]));
     for (int a = 0; a + 1 < nr; ++a) RS[a + 1] = 1.0 / (std::fabs(E[a]) * RS[a]);
   }
-  for (int l = 1; l <= nz; ++l) {
-    const double sn = cosine ? std::sin(M_PI * (l - 1) / (2.0 * nz)) : std::sin(M_PI * l / (2.0 * (nz + 1)));
-    const double lam = 4.0 / hz2 * sn * sn;
-    double delta = 0.0;
-    for (int a = 0; a < nr; ++a) {
-      const double rbar_hi = (a + 1) * hr, rbar_lo = a * hr;
-      const double d = (kt * (rbar_hi + rbar_lo) / hr2 + ri[a] * (kt * lam + qt)) * RS[a] * RS[a];
-      delta = (a == 0) ? d : d - 1.0 / delta;
-      IPS[(size_t)a * P + (l - 1)] = 1.0 / delta;
-    }
+  for (int a = 0; a < nr; ++a) I2[a] = 1.0 / (RS[a] * RS[a]);
+  small.insert(small.end(), rk.begin(), rk.end());
+  small.insert(small.end(), rt.begin(), rt.end());
+  if (e == cudaSuccess)
+    e = cudaMemcpyAsync(stage, small.data(), small.size() * sizeof(double), cudaMemcpyHostToDevice, s);
+  if (e == cudaSuccess && !perm.empty())
+    e = cudaMemcpyAsync(op->rader_perm, perm.data(), perm.size() * sizeof(int), cudaMemcpyHostToDevice, s);
+  if (e == cudaSuccess) {
+    SetupArgs a{};
+    a.kr = kappa_r; a.kz = kappa_z; a.q = q; a.stage = stage;
+    a.c64 = op->c64; a.c32 = op->c32;
+    a.nr = nr; a.nz = nz; a.pitch = op->pitch; a.pitchz = op->pitchz; a.tpitch = op->tpitch;
+    a.L = L; a.cosine = cosine; a.p2 = (int)P2;
+    a.hr = hr; a.hz = op->hz; a.kt = op->kappa_t; a.qt = op->q_t;
+    note_launch();
+    setup_small<<<64, 256, 0, s>>>(a);
+    note_launch();
+    setup_fields<<<(unsigned)std::min(nr, 8192), 256, 0, s>>>(a);
+    note_launch();
+    setup_factors<<<(nz + 31) / 32, 32, 0, s>>>(a);
+    e = cudaGetLastError();
   }
-  std::vector<double> TW(2 * (size_t)L), HW(2 * (size_t)L);
-  for (int j = 0; j < L; ++j) {
-    TW[2 * j] = std::cos(2.0 * M_PI * j / L);
-    TW[2 * j + 1] = std::sin(2.0 * M_PI * j / L);
-    HW[2 * j] = std::cos(M_PI * j / L);
-    HW[2 * j + 1] = std::sin(M_PI * j / L);
-  }
-  // Cosine pair, per mode l = 0..nz-1 with phi = pi l / (2 nz): forward
-  // factors s_l / 4 * (cos phi, sin phi, cos 3 phi, sin 3 phi), s_l the
-  // orthonormal scale (sqrt(1/nz) for l = 0, sqrt(2/nz) otherwise); inverse
-  // factors (cos phi, sin phi) (times sqrt 2 for l = 0: X_0 = sqrt(nz) Xhat_0
-  // against sqrt(nz / 2) for the others, which the store scale holds) and
-  // (cos 2 phi, sin 2 phi).
-  std::vector<double> CWt;
-  if (cosine) {
-    CWt.assign(8 * (size_t)nz, 0.0);
-    for (int l = 0; l < nz; ++l) {
-      const double phi = M_PI * l / (2.0 * nz);
-      const double f = 0.25 * std::sqrt(2.0 / nz) * (l == 0 ? std::sqrt(0.5) : 1.0);
-      const double g0 = l == 0 ? std::sqrt(2.0) : 1.0;
-      double *t = &CWt[8 * (size_t)l];
-      t[0] = f * std::cos(phi); t[1] = f * std::sin(phi);
-      t[2] = f * std::cos(3 * phi); t[3] = f * std::sin(3 * phi);
-      t[4] = g0 * std::cos(phi); t[5] = g0 * std::sin(phi);
-      t[6] = std::cos(2 * phi); t[7] = std::sin(2 * phi);
-    }
-  }
-  cudaError_t e = cudaSuccess;
-  if (cosine) {
-    e = upload<double>(&op->c64.CW, CWt);
-    if (e == cudaSuccess) e = upload<float>(&op->c32.CW, CWt);
-  }
-#define AX_UP(T, field, vec) \
-  if (e == cudaSuccess) e = upload<T>(&op->field, vec);
-  AX_UP(double, c64.CR, CR) AX_UP(double, c64.CZ, CZ) AX_UP(double, c64.W, W) AX_UP(double, c64.IP, IP)
-  AX_UP(double, c64.E, E) AX_UP(double, c64.R, ri) AX_UP(double, c64.TW, TW) AX_UP(double, c64.HW, HW)
-  AX_UP(float, c32.CR, CR) AX_UP(float, c32.CZ, CZ) AX_UP(float, c32.W, W) AX_UP(float, c32.IP, IP)
-  AX_UP(float, c32.E, E) AX_UP(float, c32.R, ri) AX_UP(float, c32.TW, TW) AX_UP(float, c32.HW, HW)
-  AX_UP(float, c32.IPS, IPS) AX_UP(float, c32.RS, RS)
-#undef AX_UP
-  {
-    // IPS mode-major for the mode-solve kernel 14: column l is the run of its
-    // nr factors, padded to tpitch with zeros
-    op->tpitch = (nr + 31) / 32 * 32;
-    std::vector<double> ipst((size_t)nz * op->tpitch, 0.0);
-    for (int a2 = 0; a2 < nr; ++a2)
-      for (int l = 0; l < nz; ++l) ipst[(size_t)l * op->tpitch + a2] = IPS[(size_t)a2 * P + l];
-    if (e == cudaSuccess) e = upload<float>(&op->c32.IPST, ipst);
-  }
-  {
-    // low parts for the double-float residual: v64 = (float)v64 + lo
-    auto lo_of = [](const std::vector<double> &v) {
-      std::vector<double> lo(v.size());
-      for (size_t i = 0; i < v.size(); ++i) lo[i] = v[i] - (double)(float)v[i];
-      return lo;
-    };
-    if (e == cudaSuccess) e = upload<float>(&op->c32.CRl, lo_of(CR));
-    if (e == cudaSuccess) e = upload<float>(&op->c32.CZl, lo_of(CZ));
-    if (e == cudaSuccess) e = upload<float>(&op->c32.Wl, lo_of(W));
-  }
-  if (e == cudaSuccess && op->plan.rader) {
-    std::vector<int> perm;
-    std::vector<double> rk, rt;
-    rader_tables(op->plan.radix[0], perm, rk, rt);
-    e = upload<double>(&op->c64.RK, rk);
-    if (e == cudaSuccess) e = upload<double>(&op->c64.RT, rt);
-    if (e == cudaSuccess) e = upload<float>(&op->c32.RK, rk);
-    if (e == cudaSuccess) e = upload<float>(&op->c32.RT, rt);
-    if (e == cudaSuccess) e = dalloc(&op->rader_perm, perm.size());
-    if (e == cudaSuccess)
-      e = cudaMemcpy(op->rader_perm, perm.data(), perm.size() * sizeof(int), cudaMemcpyHostToDevice);
-  }
-  if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&op->ws->cap, cudaStreamNonBlocking);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) {
     ax_destroy_operator(op);
     return status_from_cuda(e);
@@ -3533,7 +3671,6 @@ int ax_batch_create(ax_operator *const *ops, int32_t n, void *stream, ax_batch *
     if (e == cudaSuccess) e = build_group_coef<float>(gop->c32, mops, pick32, s);
     if (e == cudaSuccess && o->plan.rader)
       e = copy_table(&gop->rader_perm, o->rader_perm, 2 * (size_t)(o->plan.radix[0] - 1), s);
-    if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&gop->ws->cap, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&g.stream, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&g.done, cudaEventDisableTiming);
     const size_t dense = (size_t)o->nr * o->nz * g.members.size();
