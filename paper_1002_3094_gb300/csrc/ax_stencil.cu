@@ -31,7 +31,7 @@ struct StencilValue {
 // be a valid global address).
 __device__ __forceinline__ void prefetch_l2(const void *p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
 
-constexpr int kRowsLong = 16;  // rows per CTA of stencil_kernel
+constexpr int kRowsLong = 16;  // rows per CTA of stencil_kernel, at most
 constexpr int kStripRows = 2;  // rows per warp of strip_kernel
 constexpr int kStripChunk = 8; // right-hand sides per CTA of strip_kernel, at most
 
@@ -311,7 +311,7 @@ __global__ void __launch_bounds__(32 * NW, (MODE == kStencilPcg ? 16 : 24) / NW)
 // is read once plus one halo row per CTA edge.  For grids on which the strips'
 // partials would not fit their array (see strip_warps).
 template <typename T, int MODE>
-__global__ void __launch_bounds__(256) stencil_kernel(const StencilArgs<T> a) {
+__global__ void __launch_bounds__(256) stencil_kernel(const StencilArgs<T> a, int rows) {
   constexpr int V = VecT<T>::n;
   __shared__ double red[8];
   const int m = blockIdx.x;
@@ -321,8 +321,8 @@ __global__ void __launch_bounds__(256) stencil_kernel(const StencilArgs<T> a) {
   const int nwarps = blockDim.x >> 5;
   const int k0 = ((blockIdx.z * nwarps + warp) * 32 + lane) * V;
   const int nr = a.nr, nz = a.nz;
-  const int i0 = blockIdx.y * kRowsLong;
-  const int i1 = min(i0 + kRowsLong, nr);
+  const int i0 = blockIdx.y * rows;
+  const int i1 = min(i0 + rows, nr);
   const size_t base = (size_t)m * (size_t)a.field;
   const bool col_ok = k0 < nz;
   const T *__restrict__ CR = a.CR + (size_t)m * a.cstride;
@@ -704,12 +704,24 @@ static int strip_warps(int nr, int nz, int vec, int *gx, int *gy) {
   return (long long)*gx * *gy <= kPartialStride ? nw : 0;
 }
 
+// Rows per CTA of stencil_kernel, by the grid alone (its partials' order): 16, or
+// down to 4 while one right-hand side fills less than two CTAs per SM: a CTA walks
+// its rows one memory round trip after the other, and more of them hide it.  FP64
+// PCG pass, cold caches, 16 rows and 4: 500 x 511, one right-hand side 43 and 18 us,
+// eight 72 and 68 (there the FP64 pipe bounds it).
+static int long_rows(int nr, int nz, int vec) {
+  const int wx = column_warps(nz, vec), gz = (nz + 32 * vec * wx - 1) / (32 * vec * wx);
+  int rows = kRowsLong;
+  while (rows > 4 && (long long)((nr + rows - 1) / rows) * gz < 304) rows /= 2;
+  return rows;
+}
+
 int stencil_blocks_per_rhs(int nr, int nz, int vec) {
   int sx, sy;
   if (strip_warps(nr, nz, vec, &sx, &sy)) return sx * sy;
-  const int wx = column_warps(nz, vec);
+  const int wx = column_warps(nz, vec), rows = long_rows(nr, nz, vec);
   const int gz = (nz + 32 * vec * wx - 1) / (32 * vec * wx);
-  return (nr + kRowsLong - 1) / kRowsLong * gz;
+  return (nr + rows - 1) / rows * gz;
 }
 
 template <typename T, int MODE>
@@ -736,9 +748,9 @@ static void launch_stencil_mode(const StencilArgs<T> &a, cudaStream_t s) {
     }
     return;
   }
-  const int wx = column_warps(a.nz, V);
-  const dim3 grid(a.m, (a.nr + kRowsLong - 1) / kRowsLong, (a.nz + 32 * V * wx - 1) / (32 * V * wx));
-  stencil_kernel<T, MODE><<<grid, 32 * wx, 0, s>>>(a);
+  const int wx = column_warps(a.nz, V), rows = long_rows(a.nr, a.nz, V);
+  const dim3 grid(a.m, (a.nr + rows - 1) / rows, (a.nz + 32 * V * wx - 1) / (32 * V * wx));
+  stencil_kernel<T, MODE><<<grid, 32 * wx, 0, s>>>(a, rows);
 }
 
 template <typename T>

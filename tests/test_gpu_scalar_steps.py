@@ -78,3 +78,20 @@ def test_strip_edges(nr, nz, bc_z):
             assert np.array_equal(one[0].cpu().numpy(), un[m - 1]), tc
     finally:
         P.ax_destroy_operator(op)
+
+
+# FP64 stencil with 4, 8 and 16 rows per CTA, cut at the last row and column.  The
+# tolerance: some 12 roundings per node of terms that together are a few times the
+# result for random data.
+@pytest.mark.parametrize("nr,nz", [(1, 130), (3, 600), (4, 63), (333, 513), (1215, 40), (1217, 64), (2433, 129), (4900, 33)])
+def test_fp64_stencil_rows_per_cta(nr, nz):
+    op, ora, _, dev = _problem(nr, nz, 1)
+    try:
+        x = np.random.default_rng(nr).normal(size=(2, nr, nz))
+        y = torch.zeros((2, nr, nz), dtype=torch.float64, device=dev)
+        P.ax_apply_operator(op, torch.from_numpy(x).to(dev), y, 2)
+        for j in range(2):
+            ref = ora.apply_A(x[j])
+            assert np.linalg.norm(y[j].cpu().numpy() - ref) <= 48 * 2.0 ** -53 * np.linalg.norm(ref)
+    finally:
+        P.ax_destroy_operator(op)
