@@ -400,6 +400,51 @@ int dst_gemm_mtiles(int rows);
 enum { kTableSine = 0, kTableCosForward = 1, kTableCosInverse = 2 };
 std::vector<uint16_t> dst_gemm_table(int n, int kind);
 
+// FP64 transform by exact integer products on the tensor cores (ax_dst_digits.cu)
+struct DigitArgs {
+  int n, rows, pitch;      // n = nz; rows per RHS; pitch and elements per RHS of out and dot
+  long long field;
+  int in_pitch;            // of in (and of x, r, pa, pb)
+  long long in_field;
+  int m, mtiles;
+  // split: the input rows, or with r (PCG forward) q: r -= alpha in, x += alpha p
+  // (p by the parity of the iteration count), ||r||^2 partials, and r is split
+  const double *in;
+  double *x, *r, *pa, *pb;
+  int fold;                // cosine forward: folded input
+  unsigned char *digits;   // [m] of digit_bytes(rows, n)
+  double *scale;           // [m][mtiles 128]: exponent of each row (NaN: not finite)
+  // products
+  const unsigned char *table;
+  int table_exp;
+  int cosfwd;              // table kTableCosForward
+  double *out;
+  const double *dot;       // non-null: (dot, out) partials
+  const RhsState *st;
+  int mask;
+  double *partial;         // split: ||r||^2; products: (dot, out)
+  Finish fin;
+  int *err;
+  unsigned polls;          // see GemmDstArgs
+  int stall_at;
+};
+// The sums stay exact up to 512 positions per half, and one right-hand side's
+// partials fit their array up to 65536 rows.  From 128 columns on: below that the FFT
+// is short.  A transform of few rows takes its MMAs' time whatever their number, the
+// FFT its own (it is short for 255, 511, 1023): 48 rows of 128, 255, 511, 1023, 1024
+// take 21, 25, 35, 57, 59 us (FFT 69, 41, 42, 46, 76), 1024 rows 23, 29, 38, 66, 66
+// (70, 42, 64, 123, 236).  Above 512 columns the lines cross between 128 and 512 rows.
+constexpr int kDigitMinN = 128, kDigitMaxN = 1024, kDigitMinRows = 48, kDigitMinRowsLong = 384, kDigitMaxRows = 65536;
+bool digits_apply(int rows, int n);
+int digit_mtiles(int rows);
+size_t digit_bytes(int rows, int n);       // per RHS
+int digit_table_exp(int n, int kind);
+int digit_split_blocks(int rows);          // partials per RHS of the split
+int digit_gemm_partials(int rows, int n);    // partials per RHS of the products
+const unsigned char *digit_table(int device, int n, int kind, cudaStream_t s);
+void launch_digit_split(const DigitArgs &a, cudaStream_t s);
+void launch_digit_gemm(const DigitArgs &a, cudaStream_t s);
+
 template <typename T>
 struct TriArgs {
   const T *IP, *E;

@@ -83,6 +83,9 @@ struct Workspace {
   size_t scratch_bytes = 0;
   unsigned char *split = nullptr;  // BF16 split operand of the tensor-core transform
   size_t split_bytes = 0;
+  unsigned char *digits = nullptr;  // digits and row exponents of the FP64 tensor-core transform
+  size_t digits_bytes = 0;
+  bool digits_off = false;  // no memory for them: FP64 transforms by FFT
   cudaStream_t cap = nullptr;
   GraphCache g64, g32, gc64, gc32;
   // options
@@ -1648,6 +1651,84 @@ void tc_mode_solve(const ax_operator *op, int m, const float *z, float *tmp, uns
 // inverse transform.
 bool tc_dot_in_modes(const ax_operator *op) { return tridiag_split_ok(op->nr); }
 
+// ---- FP64 transform by integer products (ax_dst_digits.cu) -------------------
+template <typename T>
+bool use_digits(const ax_operator *op) {
+  return sizeof(T) == 8 && !op->ws->digits_off && digits_apply(op->nr, op->nz);
+}
+
+// Buffers and tables for `rows` rows of m right-hand sides (before any capture):
+// 16 bytes per point.  Where they do not fit, the operator's FP64 transforms go
+// back to the FFT, which needs none.
+void digit_prepare(ax_operator *op, int m, int rows, cudaStream_t s) {
+  std::lock_guard<std::recursive_mutex> lock(g_alloc_capture_mutex);
+  Workspace *w = op->ws;
+  const size_t need = m * (digit_bytes(rows, op->nz) + (size_t)digit_mtiles(rows) * 128 * sizeof(double));
+  if (w->digits_bytes < need) {
+    dfree(w->digits);
+    w->digits_bytes = 0;
+    free_graph(w->g64);  // it holds the address
+    if (cudaMalloc((void **)&w->digits, need) != cudaSuccess) {  // padding rows may hold anything
+      cudaGetLastError();
+      w->digits = nullptr;
+      w->digits_off = true;
+      return;
+    }
+    w->digits_bytes = need;
+  }
+  const bool cz = op->bc_z == 1;
+  if (!digit_table(op->device, op->nz, cz ? kTableCosForward : kTableSine, s) ||
+      !digit_table(op->device, op->nz, cz ? kTableCosInverse : kTableSine, s) || !tc_flag(op->device)) {
+    cudaGetLastError();
+    w->digits_off = true;
+    free_graph(w->g64);
+  }
+}
+
+// out = transform of the rows `in`; with upd.r the PCG update of r and x comes
+// first (upd.in = q; upd.partial and upd.fin its ||r||^2).  dot: (dot, out)
+// partials with the scalar step fin.  report: an expired wait sets the device's
+// error flag (callers that read it); it always makes the rows NaN.
+void digit_transform(const ax_operator *op, int m, int rows, const double *in, double *out, bool inverse,
+                     const RhsState *st, int mask, cudaStream_t s, const DigitArgs *upd = nullptr,
+                     const double *dot = nullptr, double *partial = nullptr, const Finish &fin = Finish{},
+                     bool report = true, bool dense_in = false, bool dense_out = false) {
+  Workspace *w = op->ws;
+  DigitArgs a{};
+  if (upd != nullptr) a = *upd;
+  const int kind = op->bc_z == 1 ? (inverse ? kTableCosInverse : kTableCosForward) : kTableSine;
+  a.n = op->nz;
+  a.rows = rows;
+  a.pitch = dense_out ? op->nz : op->pitch;
+  a.field = (long long)rows * a.pitch;
+  a.in_pitch = dense_in ? op->nz : op->pitch;
+  a.in_field = (long long)rows * a.in_pitch;
+  a.m = m;
+  a.mtiles = digit_mtiles(rows);
+  a.in = in;
+  a.fold = kind == kTableCosForward;
+  a.digits = w->digits;
+  a.scale = reinterpret_cast<double *>(w->digits + (size_t)m * digit_bytes(rows, op->nz));
+  a.st = st;
+  a.mask = mask;
+  launch_digit_split(a, s);
+  a.table = digit_table(op->device, op->nz, kind, s);
+  a.table_exp = digit_table_exp(op->nz, kind);
+  a.cosfwd = a.fold;
+  a.out = out;
+  a.dot = dot;
+  a.partial = partial;
+  a.fin = fin;
+  a.err = report ? tc_flag(op->device) : nullptr;
+  a.stall_at = -1;
+  if (w->tc_stall_test) {  // test of the expiry path (option "tc_stall_test"), once
+    a.polls = 1u << 14;
+    a.stall_at = 0;
+    w->tc_stall_test = 0;
+  }
+  launch_digit_gemm(a, s);
+}
+
 // Number of (r, z) partial slots per RHS that precond_apply writes for m
 // right-hand sides.
 template <typename T>
@@ -1687,6 +1768,14 @@ void precond_apply(const ax_operator *op, int m, const T *r, T *z, const RhsStat
         note_launch();
         sc_finish<<<m, 256, 0, s>>>(fin, mask, prz, precond_partials<T>(op, m));
       }
+      return;
+    }
+  }
+  if constexpr (sizeof(T) == 8) {
+    if (use_digits<T>(op)) {
+      digit_transform(op, m, op->nr, r, z, false, st, mask, s);
+      launch_tridiag<T>(tri_args<T>(op, m, z, z, st, mask), s);
+      digit_transform(op, m, op->nr, z, out, true, st, mask, s, nullptr, r, prz, fin);
       return;
     }
   }
@@ -1791,6 +1880,25 @@ void pcg_iteration(const ax_operator *op, int m, const PcgVecs<T> &v, RhsState *
         note_launch();
         sc_finish<<<m, 256, 0, s>>>(beta, kLive, prz, precond_partials<T>(op, m));
       }
+      return;
+    }
+  }
+  if constexpr (sizeof(T) == 8) {
+    if (use_digits<T>(op)) {
+      DigitArgs u{};
+      u.x = v.x;
+      u.r = v.r;
+      u.pa = v.pa;
+      u.pb = v.pb;
+      u.partial = prr;
+      u.fin = upd;
+      {
+        ProfScope ps(w, kProfDstFwd, units, s);
+        digit_transform(op, m, op->nr, v.q, v.z, false, st, kLive, s, &u);
+      }
+      { ProfScope ps(w, kProfTridiag, units, s); launch_tridiag<T>(tri_args<T>(op, m, v.z, v.z, st, kLive), s); }
+      ProfScope ps(w, kProfDstInv, units, s);
+      digit_transform(op, m, op->nr, v.z, v.z, true, st, kLive, s, nullptr, v.r, prz, beta);
       return;
     }
   }
@@ -2531,6 +2639,7 @@ int ax_destroy_operator(ax_operator *op) {
     dfree(w->stage_a);
     dfree(w->stage_b);
     dfree(w->split);
+    dfree(w->digits);
     dfree(w->small_buf);
     dfree(w->small_bar);
     if (w->h_flag) cudaFreeHost(w->h_flag);
@@ -3063,6 +3172,28 @@ static int apply_step(ax_operator *op, const double *in, double *out, int m, int
   int rc = ensure_scratch(op, (field + fb) * m * sizeof(T));
   if (rc != AX_OK) return rc;
   if (tc && (rc = ensure_split(op, (size_t)m * split_geom(op, rows_per).bytes_per_rhs)) != AX_OK) return rc;
+  // FP64 transforms by integer products
+  bool dg = sizeof(T) == 8 && (which == 1 || which == 3 || which == 4) && !w->digits_off &&
+            digits_apply(rows_per, op->nz);
+  if (dg) digit_prepare(op, m, rows_per, s);
+  dg = dg && !w->digits_off;
+  if constexpr (sizeof(T) == 8) {
+    if (dg) {
+      // from and to the caller's dense rows; these calls do not wait for the GPU,
+      // so an expired wait shows as NaN rows
+      double *z = reinterpret_cast<double *>(w->scratch);
+      const bool all = which == 3;
+      digit_transform(op, m, rows_per, in, all ? z : out, which == 4, nullptr, -1, s, nullptr, nullptr, nullptr,
+                      Finish{}, false, true, !all);
+      if (all) {
+        launch_tridiag<double>(tri_args<double>(op, m, z, z, nullptr, -1), s);
+        digit_transform(op, m, rows_per, z, out, true, nullptr, -1, s, nullptr, nullptr, nullptr, Finish{}, false,
+                        false, true);
+      }
+      AX_CHECK_LAUNCH();
+      return AX_OK;
+    }
+  }
   T *a = reinterpret_cast<T *>(w->scratch);
   T *b = a + field * m;
   AX_TRY(cudaMemsetAsync(w->scratch, 0, (field + fb) * m * sizeof(T), s));
@@ -3320,6 +3451,7 @@ int ax_solve(ax_operator *op, const double *f, double *u, int32_t m, double tol,
 
   if (method == AX_PCG_FP64 || method == AX_CHEB_FP64) {
     if ((rc = ensure_vec64(op, m, cheb)) != AX_OK) return rc;
+    if (use_digits<double>(op)) digit_prepare(op, m, nr, s);
     // r = phi - A x, start
     StencilArgs<double> ra = stencil_args<double>(op, m, w->st, -1);
     ra.in = w->x64;
@@ -3461,7 +3593,7 @@ int ax_solve(ax_operator *op, const double *f, double *u, int32_t m, double tol,
     AX_TRY(cudaMemcpyAsync(u, ud, dense * sizeof(double), cudaMemcpyDeviceToHost, s));
     AX_TRY(cudaStreamSynchronize(s));
   }
-  if (op->dst_tc) {
+  if (op->dst_tc || use_digits<double>(op)) {
     // a bounded wait of the tensor-core transform expired: report and re-arm
     int *flag = tc_flag(op->device), hf = 0;
     if (flag) {
