@@ -184,6 +184,16 @@ __device__ __forceinline__ float bf16_round(float a) { return __bfloat162float(_
 // The two BF16 halves of a packed pair as FP32 (exact).
 __device__ __forceinline__ float bf16_lo(unsigned p) { return __uint_as_float(p << 16); }
 __device__ __forceinline__ float bf16_hi(unsigned p) { return __uint_as_float(p & 0xFFFF0000u); }
+// The same operand stored by modes, for the inverse transform (the tensor core reads
+// either): in each 16 KB half of a tile, blocks of 64 rows x 8 positions (1 KB), the
+// positions' blocks consecutive, each position a run of 64 rows (128 bytes) whose
+// 16-byte pieces are swizzled by the position (the 128-byte swizzle).  Byte of 8
+// consecutive rows from `row` on:
+__device__ __forceinline__ size_t split_t_byte(int m, int row, int pos, int mtiles, int ktiles) {
+  return (((size_t)m * mtiles + (row >> 7)) * ktiles + (pos >> 6)) * (size_t)kSplitTileBytes +
+         ((row & 127) >> 6) * 8192 + ((pos & 63) >> 3) * 1024 + (pos & 7) * 128 +
+         ((((row & 63) >> 3) ^ (pos & 7)) << 4) + (row & 7) * 2;
+}
 // Writes the 8 consecutive columns col .. col + 7 (col % 8 == 0) of one row:
 // the 4 even ones and the 4 odd ones each as 8 bytes of high and of low parts.
 __device__ __forceinline__ void split_store8(unsigned char *split, int m, int row, int col, int mtiles, int ktiles,

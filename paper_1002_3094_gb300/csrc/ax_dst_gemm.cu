@@ -74,19 +74,34 @@ __device__ __forceinline__ uint64_t smem_desc(const void *p) {
   return (uint64_t)((a >> 4) & 0x3FFFu) | ((uint64_t)(128u >> 4) << 16) | ((uint64_t)(1024u >> 4) << 32) |
          (1ull << 46);
 }
+// The input tile: the same, or by modes (ax_common.cuh): rows contiguous, 128-byte
+// swizzle, blocks of 64 rows 8192 bytes apart, of 8 positions 1024 bytes.
+struct InputTile {
+  uint64_t desc;   // without the address
+  unsigned step;   // bytes per K = 16 step
+  unsigned major;  // instruction descriptor bit 15
+};
+__device__ __forceinline__ InputTile input_tile(int by_modes) {
+  if (by_modes)
+    return {((uint64_t)(8192u >> 4) << 16) | ((uint64_t)(1024u >> 4) << 32) | (1ull << 46) | (2ull << 61), 2048u, 1u << 15};
+  return {((uint64_t)(128u >> 4) << 16) | ((uint64_t)(1024u >> 4) << 32) | (1ull << 46), 256u, 0u};
+}
+__device__ __forceinline__ uint64_t input_desc(const InputTile &t, const void *p) {
+  return t.desc | (uint64_t)((smem_u32(p) >> 4) & 0x3FFFu);
+}
 // Instruction descriptor, kind::f16: D FP32 (bits 4-5 = 1), A and B BF16
-// (bits 7-9 = 1, 10-12 = 1), both K-major, N >> 3 at bits 17-22, M >> 4 at 24-28.
+// (bits 7-9 = 1, 10-12 = 1), K-major unless bit 15 (A) is set, N >> 3 at bits 17-22, M >> 4 at 24-28.
 template <int N>
 constexpr unsigned kIdesc = (1u << 4) | (1u << 7) | (1u << 10) | ((unsigned)(N >> 3) << 17) |
                             ((unsigned)(kBM >> 4) << 24);
 
 template <int N = kBN>
-__device__ __forceinline__ void umma(unsigned d_tmem, uint64_t a, uint64_t b, unsigned accumulate) {
+__device__ __forceinline__ void umma(unsigned d_tmem, uint64_t a, uint64_t b, unsigned accumulate, unsigned major) {
   asm volatile(
       "{\n\t.reg .pred p;\n\t"
       "setp.ne.b32 p, %4, 0;\n\t"
       "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
-      "l"(a), "l"(b), "r"(kIdesc<N>), "r"(accumulate)
+      "l"(a), "l"(b), "r"(kIdesc<N> | major), "r"(accumulate)
       : "memory");
 }
 __device__ __forceinline__ void umma_commit(uint64_t *bar) {
@@ -173,6 +188,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) dst_gemm_kernel(const GemmDst
   if (warp == 0) {
     // ---- MMA issuer ----
     if (lane == 0) {
+      const InputTile in = input_tile(a.by_modes);
       bool ok = true;
       int kk = 0;  // k blocks consumed so far (ring position)
       int it = 0;  // tiles processed so far (TMEM buffer = it & 1)
@@ -201,11 +217,11 @@ __global__ void __launch_bounds__(kGemmThreads, 1) dst_gemm_kernel(const GemmDst
           const int first = odd ? a.kbe : 0;
 #pragma unroll
           for (int j = 0; j < kBK / 16; ++j) {
-            const uint64_t ahi = smem_desc(st + j * 256), alo = smem_desc(st + kATileBytes / 2 + j * 256);
+            const uint64_t ahi = input_desc(in, st + j * in.step), alo = input_desc(in, st + kATileBytes / 2 + j * in.step);
             const uint64_t bhi = smem_desc(st + kATileBytes + j * 256);
-            umma(acc_t, ahi, bhi, (kb != first || j != 0) ? 1u : 0u);
-            umma(acc_t, alo, bhi, 1u);
-            if (THREE) umma(acc_t, ahi, smem_desc(st + kATileBytes + kBTileBytes + j * 256), 1u);
+            umma(acc_t, ahi, bhi, (kb != first || j != 0) ? 1u : 0u, in.major);
+            umma(acc_t, alo, bhi, 1u, in.major);
+            if (THREE) umma(acc_t, ahi, smem_desc(st + kATileBytes + kBTileBytes + j * 256), 1u, in.major);
           }
           umma_commit(&empty_bar[s]);
         }
@@ -582,6 +598,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) dst_gemm_small_kernel(const G
   if (warp == 0) {
     // ---- MMA issuer ----
     if (lane == 0) {
+      const InputTile in = input_tile(a.by_modes);
       bool ok = true;
       for (int kb = 0; kb < KB; ++kb) {
         const int s = kb % kSStages;
@@ -596,11 +613,11 @@ __global__ void __launch_bounds__(kGemmThreads, 1) dst_gemm_small_kernel(const G
         const int first = odd ? a.kbe : 0;
 #pragma unroll
         for (int j = 0; j < kBK / 16; ++j) {
-          const uint64_t ahi = smem_desc(st + j * 256), alo = smem_desc(st + kATileBytes / 2 + j * 256);
+          const uint64_t ahi = input_desc(in, st + j * in.step), alo = input_desc(in, st + kATileBytes / 2 + j * in.step);
           const uint64_t bhi = smem_desc(st + kATileBytes + j * 256);
-          umma<kSN>(acc_t, ahi, bhi, (kb != first || j != 0) ? 1u : 0u);
-          umma<kSN>(acc_t, alo, bhi, 1u);
-          if (THREE) umma<kSN>(acc_t, ahi, smem_desc(st + kATileBytes + kSBTileBytes + j * 256), 1u);
+          umma<kSN>(acc_t, ahi, bhi, (kb != first || j != 0) ? 1u : 0u, in.major);
+          umma<kSN>(acc_t, alo, bhi, 1u, in.major);
+          if (THREE) umma<kSN>(acc_t, ahi, smem_desc(st + kATileBytes + kSBTileBytes + j * 256), 1u, in.major);
         }
         umma_commit(&empty_bar[s]);
       }

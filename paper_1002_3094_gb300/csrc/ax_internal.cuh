@@ -347,6 +347,7 @@ __host__ __device__ inline int dst_buffer_len(int L, int n) {
 // of ax_common.cuh, BF16 DST matrix, FP32 accumulation).
 struct GemmDstArgs {
   const unsigned char *A;  // split input, tiles (m, mtiles, ktiles), even columns first
+  int by_modes;            // the tiles' layout: by rows, or by modes (ax_common.cuh)
   float *out;              // rows of the output field (columns < n written)
   const uint16_t *SB;      // S_hi / S_lo tiles (dst_gemm_table)
   int n, nr, pitch;        // n = nz; rows per RHS

@@ -83,6 +83,9 @@ struct Workspace {
   size_t scratch_bytes = 0;
   unsigned char *split = nullptr;  // BF16 split operand of the tensor-core transform
   size_t split_bytes = 0;
+  unsigned char *split_t = nullptr;  // split operand by modes (ax_common.cuh)
+  size_t split_t_bytes = 0;
+  bool split_t_off = false;
   unsigned char *digits = nullptr;  // digits and row exponents of the FP64 tensor-core transform
   size_t digits_bytes = 0;
   bool digits_off = false;  // no memory for them: FP64 transforms by FFT
@@ -323,15 +326,31 @@ int ensure_stage(ax_operator *op, size_t elems) {
   return AX_OK;
 }
 
+// Split operands of `bytes` for the tensor-core transforms: the rows' (split) and,
+// where the mode solves can be fed mode-major, the solutions' (split_t; without
+// memory for it the mode solves run staged).
 int ensure_split(ax_operator *op, size_t bytes) {
   std::lock_guard<std::recursive_mutex> lock(g_alloc_capture_mutex);
   Workspace *w = op->ws;
-  if (w->split_bytes >= bytes) return AX_OK;
-  dfree(w->split);
-  free_graph(w->g32); free_graph(w->gc32);  // they hold its address
-  w->split_bytes = 0;
-  AX_TRY(dalloc(&w->split, bytes));  // zero: padding rows and columns stay zero
-  w->split_bytes = bytes;
+  if (w->split_bytes < bytes) {
+    dfree(w->split);
+    free_graph(w->g32); free_graph(w->gc32);  // they hold its address
+    w->split_bytes = 0;
+    AX_TRY(dalloc(&w->split, bytes));  // zero: padding rows and columns stay zero
+    w->split_bytes = bytes;
+  }
+  if (op->c32.IPST != nullptr && op->tpitch > 0 && !w->split_t_off && w->split_t_bytes < bytes) {
+    dfree(w->split_t);
+    free_graph(w->g32); free_graph(w->gc32);
+    w->split_t_bytes = 0;
+    if (dalloc(&w->split_t, bytes) != cudaSuccess) {
+      cudaGetLastError();
+      w->split_t = nullptr;
+      w->split_t_off = true;
+    } else {
+      w->split_t_bytes = bytes;
+    }
+  }
   return AX_OK;
 }
 
@@ -1538,14 +1557,16 @@ SplitGeom split_geom(const ax_operator *op, int rows) {
 // whether it is a pipelined one, which works on the row-scaled systems: the
 // transforms around it then take the scaling D in their epilogues.
 int tc_mode_variant(const ax_operator *op, int m) {
-  return tridiag_effective(op->nr, op->tri_variant, m, op->c32.IPS != nullptr && op->c32.RS != nullptr);
+  const int v = tridiag_effective(op->nr, op->tri_variant, m, op->c32.IPS != nullptr && op->c32.RS != nullptr);
+  return v == 14 && (op->c32.IPST == nullptr || op->tpitch == 0 || op->ws->split_t == nullptr) ? 9 : v;
 }
 bool tc_scaled(const ax_operator *op, int m) { return tc_mode_variant(op, m) >= 2; }
-// The forward transform of a preconditioner application writes mode-major
-// for the mode-solve kernel 14 (the buffer holds either layout: see
-// ensure_vec32), when its factor table exists.
-bool tc_tr_mode(const ax_operator *op, int m) {
-  return tc_mode_variant(op, m) == 14 && op->c32.IPST != nullptr && op->tpitch > 0;
+// The forward transform of a preconditioner application writes mode-major for the
+// mode-solve kernel 14 (the buffer holds either layout: see ensure_vec32), whose
+// solutions the inverse transform then reads from split_t.
+bool tc_tr_mode(const ax_operator *op, int m) { return tc_mode_variant(op, m) == 14; }
+unsigned char *tc_solution_split(const ax_operator *op, int m) {
+  return tc_tr_mode(op, m) ? op->ws->split_t : op->ws->split;
 }
 
 // scaled: multiply every output row by D (the row scale of the pipelined mode
@@ -1556,6 +1577,7 @@ void tc_transform(const ax_operator *op, int m, int rows, const unsigned char *A
                   float *pa = nullptr, float *pb = nullptr, float *x = nullptr, bool scaled = false,
                   bool tout = false) {
   GemmDstArgs g{};
+  g.by_modes = A == op->ws->split_t;
   if (tout) {  // mode-major output for the mode-solve kernel 14 (forward only)
     g.tout = 1;
     g.tpitch = op->tpitch;
@@ -1623,8 +1645,6 @@ void tc_mode_solve(const ax_operator *op, int m, const float *z, float *tmp, uns
     t.IPST = op->c32.IPST;
     t.tcstride = op->cstride != 0 ? (long long)op->nz * op->tpitch : 0;
     t.tpitch = op->tpitch;
-  } else if (t.variant == 14) {
-    t.variant = 9;
   }
   if (tridiag_split_ok(op->nr)) {
     t.split = split;
@@ -1760,9 +1780,10 @@ void precond_apply(const ax_operator *op, int m, const T *r, T *z, const RhsStat
       const bool sc = tc_scaled(op, m);
       tc_transform(op, m, op->nr, sp, false, z, st, mask, nullptr, nullptr, s, -1, nullptr, nullptr, nullptr, sc,
                    tc_tr_mode(op, m));
-      tc_mode_solve(op, m, z, tmp, sp, st, mask, s, dm ? prz : nullptr, dm ? fin : Finish{});
+      unsigned char *ss = tc_solution_split(op, m);
+      tc_mode_solve(op, m, z, tmp, ss, st, mask, s, dm ? prz : nullptr, dm ? fin : Finish{});
       if (dm && dot_only) return;
-      tc_transform(op, m, op->nr, sp, true, out, st, mask, dm ? nullptr : r, dm ? nullptr : prz, s, -1, nullptr,
+      tc_transform(op, m, op->nr, ss, true, out, st, mask, dm ? nullptr : r, dm ? nullptr : prz, s, -1, nullptr,
                    nullptr, nullptr, sc);
       if (!dm && fin.kind != kFinNone) {
         note_launch();
@@ -1863,16 +1884,17 @@ void pcg_iteration(const ax_operator *op, int m, const PcgVecs<T> &v, RhsState *
                      tc_tr_mode(op, m));
       }
       const bool dm = tc_dot_in_modes(op);
+      unsigned char *ss = tc_solution_split(op, m);
       {
         ProfScope ps(w, kProfTridiag, units, s);
-        tc_mode_solve(op, m, v.z, v.q, sp, st, kLive, s, dm ? prz : nullptr, dm ? beta : Finish{});
+        tc_mode_solve(op, m, v.z, v.q, ss, st, kLive, s, dm ? prz : nullptr, dm ? beta : Finish{});
       }
       {
         ProfScope ps(w, kProfDstInv, units, s);
         if (fused)
-          tc_transform(op, m, op->nr, sp, true, v.z, st, kLive, nullptr, nullptr, s, -1, v.pa, v.pb, v.x, sc);
+          tc_transform(op, m, op->nr, ss, true, v.z, st, kLive, nullptr, nullptr, s, -1, v.pa, v.pb, v.x, sc);
         else
-          tc_transform(op, m, op->nr, sp, true, v.z, st, kLive, dm ? nullptr : v.r, dm ? nullptr : prz, s, -1, nullptr,
+          tc_transform(op, m, op->nr, ss, true, v.z, st, kLive, dm ? nullptr : v.r, dm ? nullptr : prz, s, -1, nullptr,
                        nullptr, nullptr, sc);
       }
       if (!dm) {
@@ -2639,6 +2661,7 @@ int ax_destroy_operator(ax_operator *op) {
     dfree(w->stage_a);
     dfree(w->stage_b);
     dfree(w->split);
+    dfree(w->split_t);
     dfree(w->digits);
     dfree(w->small_buf);
     dfree(w->small_bar);
@@ -3253,8 +3276,9 @@ static int apply_step(ax_operator *op, const double *in, double *out, int m, int
       const bool sc = tc_scaled(op, m);
       tc_transform(op, m, rows_per, sp, false, b, nullptr, -1, nullptr, nullptr, s, tc_three, nullptr, nullptr, nullptr,
                    sc, rows_per == op->nr && tc_tr_mode(op, m));
-      tc_mode_solve(op, m, b, a, sp, nullptr, -1, s);
-      tc_transform(op, m, rows_per, sp, true, b, nullptr, -1, nullptr, nullptr, s, tc_three, nullptr, nullptr, nullptr,
+      unsigned char *ss = tc_solution_split(op, m);
+      tc_mode_solve(op, m, b, a, ss, nullptr, -1, s);
+      tc_transform(op, m, rows_per, ss, true, b, nullptr, -1, nullptr, nullptr, s, tc_three, nullptr, nullptr, nullptr,
                    sc);
     }
   } else {

@@ -939,24 +939,24 @@ __global__ void __launch_bounds__(32 * WPC * CW, (32 * WPC * CW <= 512) ? 2 : 1)
 // contiguous floats, and the lanes of a warp (consecutive chunks of the same
 // column) read one contiguous run: data and factors go straight from global
 // memory to registers with 16-byte loads, with no shared-memory staging (the
-// staged kernels are bound by the shared-memory pipe).  Recurrences, carries,
-// partials and the write-back of the result through the CTA's shared tile into
-// the split operand are those of tridiag_reg2_kernel, whose layout the tile
-// keeps.
+// staged kernels are bound by the shared-memory pipe).  The solution's split parts
+// leave the registers the same way, as runs of rows (the operand by modes,
+// ax_common.cuh): written by rows they went through a shared tile and, a CTA having 8
+// or 4 columns, in pieces of 8 or 4 bytes.  1024 x 1024 x 64: 195 -> 139 us, 4096 x
+// 4096 x 16: 1278 -> 631 us (the bytes at the copy rate: 79 and 316).  A CTA holds 4
+// or 2 columns (4 or 2 CTAs an SM), as the carries make a CTA's warps wait for each
+// other.  Recurrences, carries and partials are those of tridiag_reg2_kernel.
 // ---------------------------------------------------------------------------
 template <int C2, int WPC, int CW>
-__global__ void __launch_bounds__(32 * WPC * CW, (32 * WPC * CW <= 512) ? 2 : 1)
+__global__ void __launch_bounds__(32 * WPC * CW, 1024 / (32 * WPC * CW))
     tridiag_tr_kernel(const TriArgs<float> a) {
   constexpr int NT = 32 * WPC * CW;
-  constexpr int kChunkWords = C2 * CW + 2;
-  static_assert(NT <= 1024 && (CW == 4 || CW == 8) && C2 % 4 == 0, "tile shape");
-  extern __shared__ __align__(16) float tsm3[];
+  static_assert(NT <= 512 && (C2 == 4 || C2 == 8 || C2 == 16), "tile shape");
   __shared__ float xfa[CW][WPC], xfm[CW][WPC], xba[CW][WPC], xbm[CW][WPC];
   __shared__ double red[NT / 32];
   // one tile: column group cg (columns cg CW ..) of right-hand side m
   const int cg = blockIdx.x, m = blockIdx.y;
   const int nr = a.nr;
-  float *ds = tsm3;
   const int col0 = cg * CW;
   if (!rhs_selected(a.st, a.mask, m)) return;  // uniform over the CTA
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -1062,14 +1062,11 @@ __global__ void __launch_bounds__(32 * WPC * CW, (32 * WPC * CW <= 512) ? 2 : 1)
   const float yin = fmaf(Me, cin, Ae);
   pr = 1.f;
   float dot = 0.f;
-  float *pd = ds + ci * kChunkWords;
-  auto wc = [&](int t) { return 2 * ((w >> 1) ^ reg2_sw<CW>(rbase + t)) + (w & 1); };
 #pragma unroll
   for (int t = C2 - 1; t >= 0; --t) {
     pr *= ip[t];
     v[t] = fmaf(pr, yin, v[t]);
     dot = fmaf(b[t], v[t], dot);  // (b', y') of this chunk: the (rhat, yhat) partial
-    pd[CW * t + wc(t)] = v[t];
   }
   if (a.partial != nullptr) {
     const double sw = warp_sum_of(dot);
@@ -1084,32 +1081,49 @@ __global__ void __launch_bounds__(32 * WPC * CW, (32 * WPC * CW <= 512) ? 2 : 1)
   // this CTA's arrival for the scalar step, overlapped with the write-back
   __shared__ int s_last;
   if (threadIdx.x == 0) s_last = a.fin.kind != kFinNone && finish_arrive(a.fin, m, gridDim.x);
-  // ---- write back: one thread per row, its CW columns (as tridiag_reg2_kernel)
-  const int ncol = min(CW, a.nz - col0);
-  for (int row = threadIdx.x; row < nr; row += NT) {
-    float x[CW];
-    const float *src = ds + row * CW + 2 * (row / C2);
-    const int sw = reg2_sw<CW>(row);
+  // ---- the solution's split parts, from registers ----
+  if (rbase < a.split_mtiles * 128 || C2 == 16) {
+    unsigned hi[C2 / 2], lo[C2 / 2];
 #pragma unroll
-    for (int c = 0; c < CW; c += 2) {
-      const float2 f2 = *reinterpret_cast<const float2 *>(src + 2 * ((c >> 1) ^ sw));
-      x[c] = f2.x;
-      x[c + 1] = f2.y;
+    for (int t = 0; t < C2; t += 2) {
+      hi[t / 2] = bf16_pack2(v[t], v[t + 1]);
+      lo[t / 2] = bf16_pack2(v[t] - bf16_lo(hi[t / 2]), v[t + 1] - bf16_hi(hi[t / 2]));
     }
-    if (a.split != nullptr) {
-      if constexpr (CW == 8) {
-        split_store8(a.split, m, row, col0, a.split_mtiles, a.split_ktiles, a.split_kbe, x);
-      } else {
-        split_store4(a.split, m, row, col0, a.split_mtiles, a.split_ktiles, a.split_kbe, x);
+    const int pos = split_pos(col, a.split_kbe);
+    auto put = [&](int row, const unsigned *h, const unsigned *l) {  // 8 rows
+      if (!cok || row >= a.split_mtiles * 128) return;
+      unsigned char *p = a.split + split_t_byte(m, row, pos, a.split_mtiles, a.split_ktiles);
+      *reinterpret_cast<uint4 *>(p) = make_uint4(h[0], h[1], h[2], h[3]);
+      *reinterpret_cast<uint4 *>(p + kSplitTileBytes / 2) = make_uint4(l[0], l[1], l[2], l[3]);
+    };
+    if constexpr (C2 == 4) {
+      if (cok) {
+        unsigned char *p = a.split + split_t_byte(m, rbase, pos, a.split_mtiles, a.split_ktiles);
+        *reinterpret_cast<uint2 *>(p) = make_uint2(hi[0], hi[1]);
+        *reinterpret_cast<uint2 *>(p + kSplitTileBytes / 2) = make_uint2(lo[0], lo[1]);
       }
+    } else if constexpr (C2 == 8) {
+      put(rbase, hi, lo);
     } else {
-      float *o = a.out + (size_t)m * a.field + (size_t)row * a.pitch + col0;
-      if (ncol == CW) {
+      // two pieces per lane: the lanes of a pair trade one, so that each store
+      // fills whole 32-byte sectors
+      const bool odd = lane & 1;
+      unsigned h[4], l[4];
 #pragma unroll
-        for (int c = 0; c < CW; c += 4) *reinterpret_cast<float4 *>(o + c) = make_float4(x[c], x[c + 1], x[c + 2], x[c + 3]);
-      } else {
-        for (int c = 0; c < ncol; ++c) o[c] = x[c];
+      for (int i = 0; i < 4; ++i) {
+        h[i] = __shfl_xor_sync(0xffffffffu, odd ? hi[i] : hi[4 + i], 1);
+        l[i] = __shfl_xor_sync(0xffffffffu, odd ? lo[i] : lo[4 + i], 1);
       }
+      // rows of the even lane's chunk, then of the odd lane's
+      const int r0 = rbase & ~31;
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const unsigned th = odd ? h[i] : hi[i], tl = odd ? l[i] : lo[i];
+        const unsigned uh = odd ? hi[4 + i] : h[i], ul = odd ? lo[4 + i] : l[i];
+        hi[i] = th; lo[i] = tl; hi[4 + i] = uh; lo[4 + i] = ul;
+      }
+      put(r0 + (odd ? 8 : 0), hi, lo);
+      put(r0 + 16 + (odd ? 8 : 0), hi + 4, lo + 4);
     }
   }
   if (a.fin.kind == kFinNone) return;
@@ -1120,10 +1134,8 @@ __global__ void __launch_bounds__(32 * WPC * CW, (32 * WPC * CW <= 512) ? 2 : 1)
 template <int C2, int WPC, int CW>
 void launch_tridiag_tr(const TriArgs<float> &a, cudaStream_t s) {
   constexpr int NT = 32 * WPC * CW;
-  const size_t smem = (size_t)(32 * WPC) * (C2 * CW + 2) * sizeof(float);
-  ensure_smem_attr((const void *)tridiag_tr_kernel<C2, WPC, CW>, smem);
   dim3 grid((a.nz + CW - 1) / CW, a.m);
-  tridiag_tr_kernel<C2, WPC, CW><<<grid, NT, smem, s>>>(a);
+  tridiag_tr_kernel<C2, WPC, CW><<<grid, NT, 0, s>>>(a);
 }
 
 // ---------------------------------------------------------------------------
@@ -1387,11 +1399,12 @@ int pipe_max_rows(const PipeVariant &v) { return 16 * v.nt / v.cw; }
 
 int tridiag_variants(int nr, int *ids) {
   // the default first: the staged kernel on the row-scaled systems fed
-  // mode-major by the forward transform (14; measured 8.25 ms per
-  // 1024^2 x 64 solve and 99.9 ms per 4096^2 x 16 solve, against 9.7 and
-  // 140.6 for the same kernel staging a row-major input, 9, which runs where
-  // the input is row-major), then the others (10.4 ms for the plain register
-  // kernel 1, 11.3 to 12.5 for the pipelined kernels and for 10, 11, 12);
+  // mode-major by the forward transform (14: 139 us per call at 1024^2 x 64
+  // and 631 at 4096^2 x 16; 195 and 1278 while it wrote the solution by rows),
+  // then the same kernel staging a row-major input (9: 1.2 and 1.4 times the
+  // latter; where the input is row-major) and the others (1.26 times for the
+  // plain register kernel 1, 1.4 to 1.5 for the pipelined kernels and for 10,
+  // 11, 12, at 1024^2 x 64);
   // paths that cannot scale the rows (the FFT transforms) take kernel 1
   // (tridiag_effective)
   int n = 0;
@@ -1432,6 +1445,7 @@ int tridiag_reg_cols(int nr, int variant) {
   const int v = resolve_variant(nr, variant);
   if (v == 0) return 0;
   if (v == 12) return 16;
+  if (v == 14) return nr <= 2048 ? 4 : 2;  // the columns of a CTA
   if (v == 1 || v >= 9) return reg_cols(nr);
   return find_pipe(v)->cw;
 }
@@ -1486,11 +1500,11 @@ bool launch_tridiag_tile(const TriArgs<float> &a, cudaStream_t s) {
       v = 9;
     } else {
       const int c2 = (a.nr + 63) / 64;
-      if (c2 <= 4) launch_tridiag_tr<4, 2, 8>(a, s);
-      else if (c2 <= 8) launch_tridiag_tr<8, 2, 8>(a, s);
-      else if (c2 <= 16) launch_tridiag_tr<16, 2, 8>(a, s);
-      else if (a.nr <= 2048) launch_tridiag_tr<16, 4, 8>(a, s);
-      else launch_tridiag_tr<16, 8, 4>(a, s);
+      if (c2 <= 4) launch_tridiag_tr<4, 2, 4>(a, s);
+      else if (c2 <= 8) launch_tridiag_tr<8, 2, 4>(a, s);
+      else if (c2 <= 16) launch_tridiag_tr<16, 2, 4>(a, s);
+      else if (a.nr <= 2048) launch_tridiag_tr<16, 4, 4>(a, s);
+      else launch_tridiag_tr<16, 8, 2>(a, s);
       return true;
     }
   }
