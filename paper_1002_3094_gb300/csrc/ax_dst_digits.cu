@@ -33,14 +33,14 @@
 // Q).  A cluster of two CTAs computes 128 rows x 64 columns (or 32), one P and one Q,
 // whose 8 accumulators of 64 columns fill its TMEM; each then sends the other half of
 // its sums through distributed shared memory and finishes half of the columns.  (One
-// CTA for both, P before Q: 470 us in place of 405 at 8192 x 1024, and 1.6 times the
+// CTA for both, P before Q: 470 us in place of 405 at 8192 x 1024, then, and 1.6 times the
 // time where a launch has few tiles.)  K blocks of 32 (64 KB of input digits, 32 KB
 // of matrix digits) come by bulk copies through two stages (16 through four: 1.07
-// times the time).  What bounds it at 1024 points: 1152 MMAs of about 80 cycles per
-// CTA (50 for the same MMAs with nothing copied or waited for: 6 KB of operands each
-// through shared memory), then 16 000 cycles of FP64 pipe in the drain, with no MMAs
-// beside it as the accumulators fill TMEM.  Both kernels, 8192 rows of 1024: 405 us
-// against the FFT's 1503; 4000 rows of 511: 89 against 190.
+// times the time).  What bounds the products at 1024 points, some 90 000 cycles per
+// CTA: 1152 MMAs of 50 cycles (6 KB of operands each through shared memory), then
+// 16 000 cycles of FP64 pipe in the drain with no MMAs beside it, as the accumulators
+// fill TMEM, and the first copies.  Both kernels, 8192 rows of 1024: 392 us against
+// the FFT's 1503; 4000 rows of 511: 84 against 190.
 #include <algorithm>
 #include <cmath>
 #include <mutex>
@@ -137,16 +137,23 @@ __device__ __forceinline__ int digit_byte(int row, int k) {
   return (row >> 3) * (kDK * 16) + (k >> 3) * 128 + (row & 7) * 16 + (k & 7) * 2;
 }
 
-// X (|X| <= 2^56) as 8 digits, most significant first: [-64, 64], the first
-// [-128, 128].
-__device__ __forceinline__ void digits_of(long long X, int (&d)[kSlices]) {
+// X (|X| <= 2^56) as 8 digits, most significant first: [-64, 63], the first
+// [-256, 256].  With 64 added at each digit but the first, the digits are plain bit
+// fields; a field becomes a float by the bits of 2^23 + field (FP32 and integer
+// operations: the conversion instructions have an eighth of their rate).
+__device__ __forceinline__ void digits_of(long long X, float (&d)[kSlices]) {
+  constexpr long long kBias = 64ll * 0x40810204081ll;  // 64 sum of 128^k, k = 0 .. 6
+  const unsigned long long Y = (unsigned long long)(X + kBias);
 #pragma unroll
   for (int s = kSlices - 1; s > 0; --s) {
-    const int v = ((int)((unsigned)X + 64u) & 127) - 64;
-    d[s] = v;
-    X = (X - v) >> 7;
+    const int at = 7 * (kSlices - 1 - s);
+    d[s] = __uint_as_float(((unsigned)(Y >> at) & 127u) | 0x4B000000u) - 8388672.f;
   }
-  d[0] = (int)X;
+  d[0] = __int_as_float(0x4B400000 + (int)((long long)Y >> 49)) - 12582912.f;
+}
+// Two floats that BF16 holds exactly, packed.
+__device__ __forceinline__ unsigned bf16_pack_exact(float a, float b) {
+  return __byte_perm(__float_as_uint(a), __float_as_uint(b), 0x7632);
 }
 
 // v 2^(bits - e) rounded to an integer (bits = 54 or 55), for a finite v below
@@ -154,13 +161,11 @@ __device__ __forceinline__ void digits_of(long long X, int (&d)[kSlices]) {
 __device__ __forceinline__ long long fixed_point(double v, int e, int bits) {
   const long long b = __double_as_longlong(v);
   const int f = (int)((b >> 52) & 0x7FF);
-  long long mant = b & 0xFFFFFFFFFFFFFll;
-  if (f != 0) mant |= 1ll << 52;
-  const int sh = bits - 52 - (e - ((f != 0 ? f : 1) - 1023));  // mant 2^(ex - 52) 2^(bits - e)
-  long long X;
-  if (sh >= 0) X = mant << sh;
-  else if (sh < -60) X = 0;
-  else X = (mant + (1ll << (-sh - 1))) >> -sh;
+  unsigned long long mant = (unsigned long long)b << 11;  // 1.mantissa at bit 63
+  if (f != 0) mant |= 1ull << 63;
+  const int r = 62 - bits + (e - ((f != 0 ? f : 1) - 1023));  // one bit kept below the unit
+  const unsigned long long t = r < 64 ? mant >> r : 0ull;
+  const long long X = (long long)((t + 1) >> 1);
   return b < 0 ? -X : X;
 }
 
@@ -169,9 +174,11 @@ __device__ __forceinline__ long long fixed_point(double v, int e, int bits) {
 // x += alpha p, r -= alpha q and the ||r||^2 partials of PCG) and its largest
 // magnitude; then 8 rows x 64 columns per warp are cut into digits, whose 16-byte
 // pieces fill whole 128-byte core matrices.  Columns past n and the rest of the
-// last K block are written as zeros.
+// last K block are written as zeros.  Bound by integer issue (some 45 operations per
+// value for the digits) and, with update, the latency of the row pass: 63 us for 8192
+// rows of 1024 (30 at the copy rate).
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(256) digit_split_kernel(const DigitArgs a) {
+__global__ void __launch_bounds__(256, 4) digit_split_kernel(const DigitArgs a) {
   __shared__ double red[8];
   __shared__ int s_e[8];
   const int m = blockIdx.y;
@@ -273,11 +280,11 @@ __global__ void __launch_bounds__(256) digit_split_kernel(const DigitArgs a) {
       unsigned pk[kSlices][4];
 #pragma unroll
       for (int i = 0; i < 8; i += 2) {
-        int d0[kSlices], d1[kSlices];
+        float d0[kSlices], d1[kSlices];
         digits_of(fixed_point(v[h][i], e, 55), d0);
         digits_of(fixed_point(v[h][i + 1], e, 55), d1);
 #pragma unroll
-        for (int s = 0; s < kSlices; ++s) pk[s][i >> 1] = bf16_pack2((float)d0[s], (float)d1[s]);
+        for (int s = 0; s < kSlices; ++s) pk[s][i >> 1] = bf16_pack_exact(d0[s], d1[s]);
       }
       unsigned char *t = a.digits + (((size_t)m * a.mtiles + (row >> 7)) * 2 * kbh + h * kbh + kb) * (size_t)(kSlices * kDATile) +
                          digit_byte(row & 127, g % (kDK / 8) * 8);
@@ -615,12 +622,12 @@ __global__ void __launch_bounds__(256) digit_table_kernel(unsigned char *__restr
         }
       }
     }
-    int d[kSlices];
+    float d[kSlices];
     digits_of(fixed_point(v, e, 54) + llrint(ldexp(vlo, 54 - e)), d);
     unsigned char *p = t + ((size_t)nt * 2 * kbh + kb) * (size_t)(kSlices * kDBTile) + digit_byte(nl, kl);
 #pragma unroll
     for (int s = 0; s < kSlices; ++s)
-      *reinterpret_cast<__nv_bfloat16 *>(p + s * kDBTile) = __float2bfloat16((float)d[s]);
+      *reinterpret_cast<__nv_bfloat16 *>(p + s * kDBTile) = __float2bfloat16(d[s]);
   }
 }
 
@@ -680,7 +687,7 @@ static void digit_gemm_launch(const DigitArgs &a, cudaStream_t s) {
 
 // Output columns per CTA (the results are the same): 64, or 32 where 64 would leave
 // more than half of the SMs without a CTA.  An MMA of 32 columns takes 45 cycles, one
-// of 64 some 80, and the input digits are copied for each: 500 rows of 511 take
+// of 64 takes 50, and the input digits are copied for each: 500 rows of 511 take
 // 6 us less, 4000 rows 20 us more.
 void launch_digit_gemm(const DigitArgs &a, cudaStream_t s) {
   note_launch();
