@@ -183,6 +183,95 @@ __global__ void __launch_bounds__(1024) tridiag_kernel(const TriArgs<T> a, int W
   }
 }
 
+// FP64, nr <= 64 C.  Bound by the FP64 pipe (two operations per clock and SM), so it
+// is laid out for few of them: the factors alpha_t = -E_{t-1} ip_t and beta_t = -E_t
+// ip_t are formed once and stay in registers, and each recurrence runs twice, first
+// from a zero carry for the chunk's map, then from the true one (one fma per row; the
+// kernel above corrects with the running product, two more), 9 operations per row
+// against 13; the maps are composed by shuffles and then over at most 8 warps.  A CTA
+// holds 4 columns (32-byte rows); a warp 8 chunks of C rows of each.  1024 x 1024 x 8:
+// 267 -> 183 us; 500 x 511, cold caches, eight right-hand sides 73 -> 54, one 22 -> 12.
+template <int C>
+__global__ void __launch_bounds__(256, 2) tridiag_fp64_kernel(const TriArgs<double> a) {
+  __shared__ double xa[2][8][4], xm[2][8][4];  // the warps' maps, forward and backward
+  const int m = blockIdx.x;
+  if (!rhs_selected(a.st, a.mask, m)) return;
+  const int lane = threadIdx.x & 31, h = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  const int w = lane & 3, c = h * 8 + (lane >> 2);
+  const int col = blockIdx.y * 4 + w, s0 = c * C, nr = a.nr, pitch = a.pitch;
+  const int cnt = col < a.nz ? max(0, min(C, nr - s0)) : 0;
+  const size_t off = (size_t)s0 * pitch + col;
+  const double *__restrict__ in = a.in + (size_t)m * (size_t)a.field + off;
+  const double *__restrict__ ip = a.IP + (size_t)m * a.cstride + off;
+  const double *__restrict__ E = a.E + (size_t)m * a.estride + s0;  // E[t] couples rows s0 + t and s0 + t + 1
+  double v[C], al[C], be[C];
+#pragma unroll
+  for (int t = 0; t < C; ++t) {
+    v[t] = t < cnt ? in[(size_t)t * pitch] : 0.0;
+    be[t] = t < cnt ? ld_nc(ip + (size_t)t * pitch) : 0.0;
+  }
+  double eprev = s0 > 0 && cnt > 0 ? -ld_nc(E - 1) : 0.0;
+  double A = 0.0, M = 1.0;
+#pragma unroll
+  for (int t = 0; t < C; ++t) {
+    const double f = be[t], e = t < cnt ? -ld_nc(E + t) : 0.0;
+    al[t] = eprev * f;
+    be[t] = e * f;
+    eprev = e;
+    v[t] *= f;
+    A = fma(al[t], A, v[t]);
+    M *= al[t];
+  }
+  // carry into chunk c: the composed maps of the chunks before it (forward), after it
+  // (backward)
+  auto carry = [&](int dir) {
+#pragma unroll
+    for (int o = 4; o < 32; o <<= 1) {
+      const double pa = dir == 0 ? __shfl_up_sync(0xffffffffu, A, o) : __shfl_down_sync(0xffffffffu, A, o);
+      const double pm = dir == 0 ? __shfl_up_sync(0xffffffffu, M, o) : __shfl_down_sync(0xffffffffu, M, o);
+      if (dir == 0 ? lane >= o : lane + o < 32) {
+        A = fma(M, pa, A);
+        M *= pm;
+      }
+    }
+    if (lane >> 2 == (dir == 0 ? 7 : 0)) {
+      xa[dir][h][w] = A;
+      xm[dir][h][w] = M;
+    }
+    double ea = dir == 0 ? __shfl_up_sync(0xffffffffu, A, 4) : __shfl_down_sync(0xffffffffu, A, 4);
+    double em = dir == 0 ? __shfl_up_sync(0xffffffffu, M, 4) : __shfl_down_sync(0xffffffffu, M, 4);
+    if (lane >> 2 == (dir == 0 ? 0 : 7)) {
+      ea = 0.0;
+      em = 1.0;
+    }
+    __syncthreads();
+    double x = 0.0;
+    if (dir == 0)
+      for (int j = 0; j < h; ++j) x = fma(xm[0][j][w], x, xa[0][j][w]);
+    else
+      for (int j = nw - 1; j > h; --j) x = fma(xm[1][j][w], x, xa[1][j][w]);
+    return fma(em, x, ea);
+  };
+  double g = carry(0);
+#pragma unroll
+  for (int t = 0; t < C; ++t) v[t] = g = fma(al[t], g, v[t]);
+  // backward: y_t = g_t + beta_t y_{t+1}
+  A = 0.0;
+  M = 1.0;
+#pragma unroll
+  for (int t = C - 1; t >= 0; --t) {
+    A = fma(be[t], A, v[t]);
+    M *= be[t];
+  }
+  double y = carry(1);
+  double *__restrict__ out = a.out + (size_t)m * (size_t)a.field + off;
+#pragma unroll
+  for (int t = C - 1; t >= 0; --t) {
+    y = fma(be[t], y, v[t]);
+    if (t < cnt) out[(size_t)t * pitch] = y;
+  }
+}
+
 // Tiles of the register kernel below: a CTA stages an nr x CW column tile in
 // shared memory; idx(row, col) = row CW + col + row / C2 is padded by one word
 // per chunk of C2 rows, so the lanes of a warp (rows c C2 + t of one column,
@@ -1338,9 +1427,6 @@ __global__ void __launch_bounds__(32 * WPC * CW, (32 * WPC * CW <= 512) ? 2 : 1)
 // Chunk length C: short enough that the chunk stays in registers without
 // spilling (16 FP32 / 8 FP64 values); very tall systems use twice that so
 // that a CTA still spans >= 8 mode columns (32-byte row segments).
-template <typename T> struct TriChunk;
-template <> struct TriChunk<float> { static constexpr int small = 16, large = 32, switch_nr = 2048; };
-template <> struct TriChunk<double> { static constexpr int small = 8, large = 16, switch_nr = 1024; };
 
 template <typename T, int C>
 void launch_tridiag_c(const TriArgs<T> &a, cudaStream_t s) {
@@ -1554,8 +1640,21 @@ void launch_tridiag(const TriArgs<T> &a, cudaStream_t s) {
   if constexpr (sizeof(T) == 4) {
     if (launch_tridiag_tile(a, s)) return;
   }
-  if (a.nr > TriChunk<T>::switch_nr) launch_tridiag_c<T, TriChunk<T>::large>(a, s);
-  else launch_tridiag_c<T, TriChunk<T>::small>(a, s);
+  if constexpr (sizeof(T) == 8) {
+    if (a.nr <= 1024) {
+      const int c = a.nr <= 512 ? 8 : 16, warps = ((a.nr + c - 1) / c + 7) / 8;
+      const dim3 grid(a.m, (a.nz + 3) / 4);
+      if (c == 8) tridiag_fp64_kernel<8><<<grid, 32 * warps, 0, s>>>(a);
+      else tridiag_fp64_kernel<16><<<grid, 32 * warps, 0, s>>>(a);
+    } else {
+      launch_tridiag_c<T, 16>(a, s);
+    }
+    return;
+  }
+  if constexpr (sizeof(T) == 4) {
+    if (a.nr > 2048) launch_tridiag_c<T, 32>(a, s);
+    else launch_tridiag_c<T, 16>(a, s);
+  }
 }
 
 template void launch_tridiag<float>(const TriArgs<float> &, cudaStream_t);

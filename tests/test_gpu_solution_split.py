@@ -13,6 +13,7 @@ import pytest
 
 torch = pytest.importorskip("torch")
 
+import oracle as O  # noqa: E402
 import paper_1002_3094_gb300 as P  # noqa: E402
 from paper_1002_3094_gb300.inputs import sample_operator_inputs  # noqa: E402
 from workloads import layered_inclusion_medium  # noqa: E402
@@ -53,5 +54,40 @@ def test_by_modes_against_by_rows(nr, nz, bc_z):
         assert torch.equal(again[1], out[14][1])
         P.ax_apply_preconditioner(op, x, again, m, P.AX_PREC_FP32_TC3)
         assert torch.equal(again, out[14])
+    finally:
+        P.ax_destroy_operator(op)
+
+
+@pytest.mark.parametrize("bc_z", [0, 1])
+@pytest.mark.parametrize("nr,nz", [(1, 5), (7, 3), (8, 4), (9, 6), (63, 9), (65, 7), (449, 2), (511, 5), (512, 4),
+                                   (513, 5), (897, 1), (1023, 6), (1024, 3), (1025, 2)])
+def test_fp64_mode_solves_at_chunk_edges(nr, nz, bc_z):
+    """Backward error of every mode system where rows end at the edge of a chunk (8
+    or 16 rows), a warp (8 chunks) and the kernel's range, columns inside a CTA's 4:
+    the recurrences round each row a few times, 1e-14 as a stable solver."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    P.build()
+    P.load_library()
+    m = 2
+    dev = torch.device("cuda:0")
+    med = layered_inclusion_medium(n_rhs=m, nominal_n=64)
+    kr, kz, q = sample_operator_inputs(med, nr, nz, bc_z=bc_z)
+    grid = O.Grid(nr, nz, bc_z=bc_z)
+    kt, qt = O.preconditioner_constants(kr, kz, q)[:2]
+    op = P.ax_setup_operator(*[torch.from_numpy(x).to(dev) for x in (kr, kz, q)], nr, nz, bc_z=bc_z)
+    try:
+        b = np.random.default_rng(nr).normal(size=(m, nr, nz))
+        y = torch.zeros((m, nr, nz), dtype=torch.float64, device=dev)
+        P.ax_apply_mode_solve(op, torch.from_numpy(b).to(dev), y, m)
+        y = y.cpu().numpy()
+        lam = O.mode_eigenvalues(nz, grid.hz, bc_z)
+        for l in range(nz):
+            sub, diag, sup = O.mode_tridiagonal(kt, qt, lam[l], grid)
+            t = np.diag(diag) + (np.diag(sub, -1) + np.diag(sup, 1) if nr > 1 else 0.0)
+            norm = np.abs(t).sum(1).max()
+            for j in range(m):
+                r = t @ y[j, :, l] - b[j, :, l]
+                assert np.linalg.norm(r) <= 1e-14 * (norm * np.linalg.norm(y[j, :, l]) + np.linalg.norm(b[j, :, l]))
     finally:
         P.ax_destroy_operator(op)
