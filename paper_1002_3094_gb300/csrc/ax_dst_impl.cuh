@@ -639,30 +639,48 @@ __global__ void __launch_bounds__(256, DstOcc<T>::min_blocks) dst_kernel(const D
       f2 = __ldg(a.CW + 8 * o + 2);
       f3 = __ldg(a.CW + 8 * o + 3);
     }
-    for (int rr = 0; rr < nrows; ++rr) {
-      const C *Z = src + rr * L;
-      T v;
-      if (!cosine) {
-        const C zk = Z[o + 1], zm = Z[L - o - 1];
-        v = ((zm.y - zk.y) + c * (zk.x - zm.x) + sn * (zk.y + zm.y)) * sc;
-      } else if (!inv) {
-        const C zl = Z[o], zm = Z[o ? n - o : 0];
-        v = (zl.x + zm.x) * c + (zl.y - zm.y) * sn + (zl.y + zm.y) * f2 - (zl.x - zm.x) * f3;
-      } else {
-        const C w = Z[o >> 1];
-        v = ((o & 1) ? -w.y : w.x) * sc;
+    // rows in groups whose operands are all loaded before any is used: one memory
+    // round trip per group
+    constexpr int G = (MODE == kDstPcgInverse || MODE == kDstChebInverse) ? 4 : 1;
+    for (int r0 = 0; r0 < nrows; r0 += G) {
+      T g0[G], g1[G];
+#pragma unroll
+      for (int j = 0; j < G; ++j) {
+        const size_t e = base + (size_t)(r0 + j) * a.pitch + o;
+        g0[j] = g1[j] = T(0);
+        if (r0 + j >= nrows) continue;
+        if (MODE == kDstPcgInverse) g0[j] = a.r[e];
+        if (MODE == kDstChebInverse) {
+          g0[j] = a.y[e];
+          g1[j] = a.yprev[e];
+        }
       }
-      const size_t e = base + (size_t)rr * a.pitch + o;
-      if (MODE == kDstPlain || MODE == kDstPcgForward) {
-        outg[e] = v;
-      } else if (MODE == kDstPcgInverse) {
-        const T rv = a.r[e];
-        outg[e] = v;
-        acc = fma(rv, v, acc);
-      } else {  // Chebyshev: y_{k+1} = a (y_k - tau B^-1 res) + (1 - a) y_{k-1}
-        const T yb = fma(-tau, v, a.y[e]);
-        const T pv = a.yprev[e];
-        a.yprev[e] = fma(cheb_a, yb - pv, pv);
+#pragma unroll
+      for (int j = 0; j < G; ++j) {
+        const int rr = r0 + j;
+        if (rr >= nrows) continue;
+        const C *Z = src + rr * L;
+        T v;
+        if (!cosine) {
+          const C zk = Z[o + 1], zm = Z[L - o - 1];
+          v = ((zm.y - zk.y) + c * (zk.x - zm.x) + sn * (zk.y + zm.y)) * sc;
+        } else if (!inv) {
+          const C zl = Z[o], zm = Z[o ? n - o : 0];
+          v = (zl.x + zm.x) * c + (zl.y - zm.y) * sn + (zl.y + zm.y) * f2 - (zl.x - zm.x) * f3;
+        } else {
+          const C w = Z[o >> 1];
+          v = ((o & 1) ? -w.y : w.x) * sc;
+        }
+        const size_t e = base + (size_t)rr * a.pitch + o;
+        if (MODE == kDstPlain || MODE == kDstPcgForward) {
+          outg[e] = v;
+        } else if (MODE == kDstPcgInverse) {
+          outg[e] = v;
+          acc = fma(g0[j], v, acc);
+        } else {  // Chebyshev: y_{k+1} = a (y_k - tau B^-1 res) + (1 - a) y_{k-1}
+          const T yb = fma(-tau, v, g0[j]);
+          a.yprev[e] = fma(cheb_a, yb - g1[j], g1[j]);
+        }
       }
     }
   }
