@@ -508,11 +508,21 @@ __global__ void __launch_bounds__(256, DstOcc<T>::min_blocks) dst_kernel(const D
   const T *__restrict__ ing = a.in;
   const int spitch = (n + 3) & ~3;  // staging row length (16-byte aligned rows)
   T *stg = reinterpret_cast<T *>(buf1);
-  for (int rr = 0; rr < nrows; ++rr) {
-    const size_t rb = base + (size_t)rr * a.pitch;
-    for (int k0 = threadIdx.x * V; k0 < n; k0 += blockDim.x * V) {
-      const size_t e = rb + k0;
-      T v[V];
+  // The rows' vectors as one run over the threads (a row of 511 has 128), several
+  // loaded before the first is used: one memory round trip per group (511 x 511 x 16
+  // in FP32: 27 -> 22 us plain, 33 -> 28 in the Chebyshev form).
+  const int nv = (n + V - 1) / V, items = nrows * nv;
+  constexpr int G = MODE == kDstPcgForward ? 1 : 4;
+  for (int i0 = threadIdx.x; i0 < items; i0 += G * blockDim.x) {
+    T v[G][V];
+    int at[G];
+#pragma unroll
+    for (int g = 0; g < G; ++g) {
+      const int it = i0 + g * blockDim.x;
+      if (it >= items) continue;
+      const int rr = it / nv, k0 = (it - rr * nv) * V;
+      const size_t e = base + (size_t)rr * a.pitch + k0;
+      at[g] = rr * spitch + k0;
       if (MODE == kDstPcgForward) {
         T xv[V], pv[V], rv[V], qv[V];
         if (x_fresh) {
@@ -529,15 +539,17 @@ __global__ void __launch_bounds__(256, DstOcc<T>::min_blocks) dst_kernel(const D
           xv[t] = fma(alpha, pv[t], xv[t]);
           rv[t] = fma(-alpha, qv[t], rv[t]);
           acc = fma(rv[t], rv[t], acc);
-          v[t] = rv[t];
+          v[g][t] = rv[t];
         }
         store_vec<T>(xg + e, xv);
         store_vec<T>(rg + e, rv);
       } else {
-        load_vec<T>(ing + e, v);
+        load_vec<T>(ing + e, v[g]);
       }
-      store_vec<T>(stg + rr * spitch + k0, v);
     }
+#pragma unroll
+    for (int g = 0; g < G; ++g)
+      if (i0 + g * blockDim.x < items) store_vec<T>(stg + at[g], v[g]);
   }
   __syncthreads();
   for (int rr = 0; rr < nrows; ++rr) {
@@ -640,7 +652,7 @@ __global__ void __launch_bounds__(256, DstOcc<T>::min_blocks) dst_kernel(const D
       f3 = __ldg(a.CW + 8 * o + 3);
     }
     // rows in groups whose operands are all loaded before any is used: one memory
-    // round trip per group
+    // round trip per group (Chebyshev form, 511 x 511 x 16: 41 -> 33 us)
     constexpr int G = (MODE == kDstPcgInverse || MODE == kDstChebInverse) ? 4 : 1;
     for (int r0 = 0; r0 < nrows; r0 += G) {
       T g0[G], g1[G];
