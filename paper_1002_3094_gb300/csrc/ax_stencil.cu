@@ -66,7 +66,11 @@ struct StripShape {
   static constexpr int row = 32 * V;                          // elements of a strip row
   static constexpr int array = (kStripRows + 2) * row + 16 / (int)sizeof(T) * kStripRows;  // rows, then edges
   static constexpr int stage = arrays * array;
-  static constexpr size_t warp_bytes = (size_t)stages * stage * sizeof(T);
+  // a warp's ring: no more stages than right-hand sides (few: more CTAs fit an SM, a
+  // solve of three 1024 x 1024 or one of 1500 x 1500 takes 1 per cent less)
+  __host__ __device__ static size_t warp_bytes(int chunk) {
+    return (size_t)(chunk < stages ? chunk : stages) * stage * sizeof(T);
+  }
 };
 
 template <typename T, int MODE, int NW>
@@ -104,7 +108,7 @@ __global__ void __launch_bounds__(32 * NW, (MODE == kStencilPcg ? 16 : 24) / NW)
   __syncthreads();
   const int n = s_n;
   if (n == 0) return;
-  T *ring = reinterpret_cast<T *>(ssm + (size_t)warp * S::warp_bytes);
+  T *ring = reinterpret_cast<T *>(ssm + warp * S::warp_bytes(chunk));
   // rows i0 - 1 .. i0 + R of the c-th right-hand side's grid function (mode Pcg:
   // z and, unless beta is 0 (p_1 = z), p_old), and nodes k0 - 1 (lane 0) and
   // k0 + V (lane 31) of rows i0 .. i0 + R - 1
@@ -736,7 +740,7 @@ static void launch_stencil_mode(const StencilArgs<T> &a, cudaStream_t s) {
     const long long c = (long long)a.m * sx * sy * nw / (152 * 48);
     const int chunk = a.cstride != 0 ? 1 : (int)std::max<long long>(1, std::min<long long>(c, kStripChunk));
     const dim3 grid(sx, sy, (a.m + chunk - 1) / chunk);
-    const size_t smem = nw * StripShape<T, MODE>::warp_bytes;
+    const size_t smem = nw * StripShape<T, MODE>::warp_bytes(chunk);
     if (nw == 8) {
       ensure_smem_attr((const void *)strip_kernel<T, MODE, 8>, smem);
       strip_kernel<T, MODE, 8><<<grid, 256, smem, s>>>(a, chunk);
