@@ -187,7 +187,8 @@ __global__ void __launch_bounds__(256, 4) digit_split_kernel(const DigitArgs a) 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const size_t base = (size_t)m * (size_t)a.in_field;
   const double *src = a.r != nullptr ? a.r : a.in;
-  const bool pairs = (a.in_pitch & 1) == 0 && (a.in_field & 1) == 0;  // 16-byte loads
+  // 16-byte loads (a caller's rows may start at any element)
+  const bool pairs = (a.in_pitch & 1) == 0 && (a.in_field & 1) == 0 && (reinterpret_cast<uintptr_t>(src) & 15) == 0;
   double acc = 0.0;
   {
     const int row = row0 + warp;
@@ -503,7 +504,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kDThreads, 1) digit_
       const double e = a.scale[(size_t)m * a.mtiles * kDM + row];
       const int sh = e == e ? max((int)e, -900) + a.table_exp - 60 : 1 << 20;
       const size_t rb = (size_t)m * (size_t)a.field + (size_t)row * a.pitch;
-      const bool even = ((a.pitch | (int)a.field) & 1) == 0;  // 16-byte stores
+      // 16-byte stores
+      const bool even = ((a.pitch | (int)a.field) & 1) == 0 &&
+                        ((reinterpret_cast<uintptr_t>(a.out) | reinterpret_cast<uintptr_t>(a.dot)) & 15) == 0;
       auto put = [&](int col, double v, double &acc) {
         if (a.dot != nullptr) acc = fma(a.dot[rb + col], v, acc);
         a.out[rb + col] = v;

@@ -75,6 +75,11 @@ def test_transform_against_extended_sums(nz, rows, bc_z):
             assert (err <= TOL * norm[np.arange(rows) % 8]).all(), (f.__name__, err.max())
             f(op, xd, xd, rows)  # in place
             assert torch.equal(xd, y)
+            # buffers that start 8 bytes off a 16-byte boundary
+            flat_x, flat_y = (torch.zeros(rows * nz + 1, dtype=torch.float64, device=dev) for _ in range(2))
+            flat_x[1:] = torch.from_numpy(x).to(dev).flatten()
+            f(op, flat_x[1:].view(rows, nz), flat_y[1:].view(rows, nz), rows)
+            assert torch.equal(flat_y[1:].view(rows, nz), y)
             # a row that is not finite stays alone
             xn = torch.from_numpy(x).to(dev)
             xn[3, 2], xn[17, nz - 1] = float("nan"), float("inf")
