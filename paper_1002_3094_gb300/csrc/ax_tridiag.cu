@@ -1424,9 +1424,9 @@ __global__ void __launch_bounds__(32 * WPC * CW, (32 * WPC * CW <= 512) ? 2 : 1)
 
 }  // namespace
 
-// Chunk length C: short enough that the chunk stays in registers without
-// spilling (16 FP32 / 8 FP64 values); very tall systems use twice that so
-// that a CTA still spans >= 8 mode columns (32-byte row segments).
+// Chunk length C: short enough that the chunk stays in registers without spilling
+// (16 values; 32 FP32 values for very tall systems, so that a CTA still spans >= 8
+// mode columns).
 
 template <typename T, int C>
 void launch_tridiag_c(const TriArgs<T> &a, cudaStream_t s) {
