@@ -95,7 +95,7 @@ struct Coef {
 };
 
 // Scalar state of one right-hand side during an iteration.  Lives in device
-// memory; written only by the scalar kernels.
+// memory; written only by the scalar steps (ax_finish.cuh) and the starts.
 struct RhsState {
   double rho;      // (r, z)
   double alpha;    // step length
