@@ -502,7 +502,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kDThreads, 1) digit_
       // out = V 2^sh: 2^(e - 55) 2^(eS - 54) 2^49 (the 8 highest of 15 digit
       // weights, 128^14 .. 128^7); a row that is not finite: NaN
       const double e = a.scale[(size_t)m * a.mtiles * kDM + row];
-      const int sh = e == e ? max((int)e, -900) + a.table_exp - 60 : 1 << 20;
+      const int sh = e == e ? (int)e + a.table_exp - 60 : 1 << 20;
       const size_t rb = (size_t)m * (size_t)a.field + (size_t)row * a.pitch;
       // 16-byte stores
       const bool even = ((a.pitch | (int)a.field) & 1) == 0 &&
