@@ -249,6 +249,9 @@ __global__ void __launch_bounds__(256, 4) digit_split_kernel(const DigitArgs a) 
   __syncthreads();
   const int ne = (n + 1) >> 1, kbh = (ne + kDK - 1) / kDK;  // K blocks per half
   const int r = lane >> 2, row = row0 + r, e = s_e[r];
+  // a folded sum of entries from 2^1023 on can exceed the FP64 range: halves are folded
+  const bool halves = a.fold && e > 1023;
+  const int ef = halves ? e - 1 : e;
   const size_t rb = base + (size_t)row * a.in_pitch;
   const bool row_ok = row < a.rows && e < (1 << 20);
   // a task: 8 positions of both halves (16 columns)
@@ -269,7 +272,11 @@ __global__ void __launch_bounds__(256, 4) digit_split_kernel(const DigitArgs a) 
           if (2 * k + 1 < n) v[1][i] = t.y;
         }
       } else if (k < ne) {  // u_k = r_k + r_{n-1-k}, w_k = r_k - r_{n-1-k} (the middle entry of odd n once)
-        const double x = src[rb + k], y = src[rb + n - 1 - k];
+        double x = src[rb + k], y = src[rb + n - 1 - k];
+        if (halves) {
+          x *= 0.5;
+          y *= 0.5;
+        }
         const bool mid = 2 * k + 1 == n;
         v[0][i] = mid ? x : x + y;
         v[1][i] = mid ? 0.0 : x - y;
@@ -282,8 +289,8 @@ __global__ void __launch_bounds__(256, 4) digit_split_kernel(const DigitArgs a) 
 #pragma unroll
       for (int i = 0; i < 8; i += 2) {
         float d0[kSlices], d1[kSlices];
-        digits_of(fixed_point(v[h][i], e, 55), d0);
-        digits_of(fixed_point(v[h][i + 1], e, 55), d1);
+        digits_of(fixed_point(v[h][i], ef, 55), d0);
+        digits_of(fixed_point(v[h][i + 1], ef, 55), d1);
 #pragma unroll
         for (int s = 0; s < kSlices; ++s) pk[s][i >> 1] = bf16_pack_exact(d0[s], d1[s]);
       }

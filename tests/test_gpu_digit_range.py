@@ -39,3 +39,20 @@ def test_rows_of_every_exponent(nz, bc_z):
         _check(op, x, nz, bc_z, dev)
     finally:
         P.ax_destroy_operator(op)
+
+
+@pytest.mark.parametrize("nz,bc_z", [(128, 0), (300, 1), (301, 1)])
+def test_rows_near_the_largest_number(nz, bc_z):
+    """Entries whose sums (the cosine transform folds its input) exceed the range, with
+    transforms that do not."""
+    op, _, _, dev = _problem(48, nz, 1, bc_z)
+    big = 1.75 * 2.0 ** 1023
+    x = np.zeros((48, nz))
+    x[:, 5] = np.resize([big, -big, 0.5 * big], 48)
+    x[::2, nz - 6] = big
+    x[4:, 9] = np.ldexp(np.arange(44) - 21.5, 1010)
+    x[40:, nz // 2] = 0.25 * big
+    try:
+        _check(op, x, nz, bc_z, dev)
+    finally:
+        P.ax_destroy_operator(op)
