@@ -67,7 +67,7 @@ struct Workspace {
   // partial sums [4][m][kPartialStride]
   double *part = nullptr;
   double *chp = nullptr;      // Chebyshev (tau, rho0^2) per right-hand side [m][2]
-  double *rscale = nullptr;   // mixed methods: power-of-two scale of phi and x per right-hand side [m]
+  int *rexp = nullptr;        // mixed methods: exponent of the power-of-two scale of phi and x per right-hand side [m]
   RhsState *st = nullptr, *st_outer = nullptr;
   int mfield64 = 0;           // right-hand sides that phi64 and x64 hold
   unsigned *arrive = nullptr; // CTA arrivals per right-hand side (Finish::count)
@@ -219,10 +219,10 @@ void free_vectors32(Workspace *w) {
 void free_base(Workspace *w) {
   dfree(w->phi64); dfree(w->base);
   w->x64 = nullptr;
-  w->part = w->chp = w->rscale = w->par = nullptr;
+  w->part = w->chp = w->par = nullptr;
   w->st = w->st_outer = nullptr;
   w->arrive = nullptr;
-  w->chk = nullptr;
+  w->chk = w->rexp = nullptr;
   if (w->h_st) cudaFreeHost(w->h_st);
   w->h_st = nullptr;
   w->mbase = w->mfield64 = 0;
@@ -237,16 +237,16 @@ int ensure_base(ax_operator *op, int m) {
   if (w->mbase >= m) return AX_OK;
   free_base(w);
   // one zeroed allocation (each costs tens of microseconds, as does its release)
-  const size_t mm = (size_t)m, nd = 4 * mm * kPartialStride + 3 * mm + 2;
-  AX_TRY(dalloc(&w->base, nd * sizeof(double) + 2 * mm * sizeof(RhsState) + (mm + 1) * sizeof(unsigned)));
+  const size_t mm = (size_t)m, nd = 4 * mm * kPartialStride + 2 * mm + 2;
+  AX_TRY(dalloc(&w->base, nd * sizeof(double) + 2 * mm * sizeof(RhsState) + (2 * mm + 1) * sizeof(unsigned)));
   w->part = reinterpret_cast<double *>(w->base);
   w->chp = w->part + 4 * mm * kPartialStride;
-  w->rscale = w->chp + 2 * mm;
-  w->par = w->rscale + mm;
+  w->par = w->chp + 2 * mm;
   w->st = reinterpret_cast<RhsState *>(w->part + nd);
   w->st_outer = w->st + mm;
   w->arrive = reinterpret_cast<unsigned *>(w->st_outer + mm);
-  w->chk = reinterpret_cast<int *>(w->arrive + mm);
+  w->rexp = reinterpret_cast<int *>(w->arrive + mm);
+  w->chk = w->rexp + mm;
   AX_TRY(cudaMallocHost((void **)&w->h_st, sizeof(RhsState) * 2 * m));
   w->mbase = m;
   return AX_OK;
@@ -430,20 +430,32 @@ __global__ void padded_to_dense(const T *__restrict__ src, double *__restrict__ 
 // right-hand side has its largest magnitude in [1/2, 1) for any finite
 // nonzero phi of FP64 (no square is formed, so nothing overflows or
 // underflows on the way); 1 for phi = 0 or non-finite phi.  pmax holds the
-// per-CTA maxima of |phi| (nb per right-hand side).
-__global__ void rhs_scale(double *scale, const double *pmax, int nb, int m) {
+// per-CTA maxima of |phi| (nb per right-hand side).  What is kept is e: sigma itself
+// is no normal number where max |phi| is below 2^-1024 or from 2^1022 on.
+__device__ __forceinline__ int peak_exponent(double mx) {
+  int e = 0;
+  if (mx > 0.0 && isfinite(mx)) frexp(mx, &e);
+  return e;
+}
+__global__ void rhs_scale(int *rexp, const double *pmax, int nb, int m) {
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= m) return;
   double mx = 0.0;
   for (int b = 0; b < nb; ++b) mx = fmax(mx, pmax[(size_t)j * kPartialStride + b]);
-  double sc = 1.0;
-  if (mx > 0.0 && isfinite(mx)) {
-    int e = 0;
-    frexp(mx, &e);
-    sc = ldexp(1.0, -e);
-  }
-  scale[j] = sc;
+  rexp[j] = peak_exponent(mx);
 }
+
+// 2^e (|e| <= 1100) as two factors, each a normal number; the second is 1 (and need
+// not be multiplied by) but at the ends of the range.
+struct Pow2 {
+  double a, b;
+  bool one;
+};
+__device__ __forceinline__ Pow2 pow2(int e) {
+  const int h = abs(e) <= 1000 ? e : e >> 1;
+  return {__hiloint2double((1023 + h) << 20, 0), __hiloint2double((1023 + e - h) << 20, 0), h == e};
+}
+__device__ __forceinline__ double times(double v, const Pow2 &p) { return p.one ? v * p.a : v * p.a * p.b; }
 
 // Per-CTA partials of ||phi||^2 in the block structure of prep_rhs (grid
 // (m, ceil(nr / 16)), 256 threads), for the scaled right-hand side.
@@ -460,19 +472,16 @@ __global__ void phi_norm2(const double *__restrict__ phi, int nr, int nz, int pi
   if (threadIdx.x == 0) part[(size_t)m * kPartialStride + blockIdx.y] = s;
 }
 
-// phi *= sigma and x *= sigma (x may be null) with the ||phi||^2 partials *=
-// sigma^2 (inverse = false), or x /= sigma (inverse = true).  grid (., m).
-__global__ void apply_rhs_scale(double *phi, double *x, const double *scale, double *part, int nb, size_t field,
-                                bool inverse) {
+// phi *= sigma and x *= sigma (x may be null; inverse = false), or x /= sigma
+// (inverse = true).  grid (., m).
+__global__ void apply_rhs_scale(double *phi, double *x, const int *rexp, size_t field, bool inverse) {
   const int m = blockIdx.y;
-  const double sc = inverse ? 1.0 / scale[m] : scale[m];
+  const Pow2 sc = pow2(inverse ? rexp[m] : -rexp[m]);
   const size_t b = (size_t)m * field;
   for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < field; e += (size_t)gridDim.x * blockDim.x) {
-    if (phi) phi[b + e] *= sc;
-    if (x) x[b + e] *= sc;
+    if (phi) phi[b + e] = times(phi[b + e], sc);
+    if (x) x[b + e] = times(x[b + e], sc);
   }
-  if (part && blockIdx.x == 0)
-    for (int k = threadIdx.x; k < nb; k += blockDim.x) part[(size_t)m * kPartialStride + k] *= sc * sc;
 }
 
 // phi = r_i f (Eq. diff_approx1), FP64, plus per-CTA partials of ||phi||^2
@@ -569,13 +578,13 @@ __device__ __forceinline__ void split_df(double v, float &h, float &l) {
   l = (float)rest * unit * 1.862645149230957e-9f;  // 2^-29
 }
 
-// Mixed PCG: sigma of every right-hand side, the power of two that brings
-// max |r f| into [1/2, 1) (1 for a zero or non-finite right-hand side), so that
+// Mixed PCG: the exponent of every right-hand side's peak (see rhs_scale): sigma, its
+// negative power, brings max |r f| into [1/2, 1) (1 for a zero or non-finite right-hand side), so that
 // the FP32 inner iteration works on values of order one whatever the units of f.
 // |f| is compared as integers (its bits, sign cleared), and r >= 0 multiplies the
 // row maxima only (rounding is monotone).  grid (m, .); par: tol^2, delta^2.
 __global__ void __launch_bounds__(256) mixed_peak(const double *__restrict__ f, const double *__restrict__ R, int nr,
-                                                  int nz, double *__restrict__ pmax, double *__restrict__ scale,
+                                                  int nz, double *__restrict__ pmax, int *__restrict__ rexp,
                                                   unsigned *count, double *par, double tol2, double delta2, int *chk) {
   __shared__ double red[8];
   __shared__ int s_last;
@@ -626,15 +635,7 @@ __global__ void __launch_bounds__(256) mixed_peak(const double *__restrict__ f, 
   for (int i = threadIdx.x; i < (int)gridDim.y; i += 256)
     mx = fmax(mx, __ldcg(pmax + (size_t)m * kPartialStride + i));
   mx = cta_max(mx);
-  if (threadIdx.x == 0) {
-    double sc = 1.0;
-    if (mx > 0.0 && isfinite(mx)) {
-      int e = 0;
-      frexp(mx, &e);
-      sc = ldexp(1.0, -e);
-    }
-    scale[m] = sc;
-  }
+  if (threadIdx.x == 0) rexp[m] = peak_exponent(mx);
 }
 
 constexpr int kPrepRows = 4;  // rows per CTA of the two kernels below
@@ -643,7 +644,7 @@ constexpr int kPrepRows = 4;  // rows per CTA of the two kernels below
 // partials; with r32 the residual of the zero start too, r = phi.  With u (a
 // guess, dense) instead x = sigma u as a pair.  grid (m, ceil(nr / kPrepRows)).
 __global__ void __launch_bounds__(256) mixed_prep(const double *__restrict__ f, const double *__restrict__ u,
-                                                  const double *__restrict__ R, const double *__restrict__ scale,
+                                                  const double *__restrict__ R, const int *__restrict__ rexp,
                                                   int nr, int nz, int pitch, float *__restrict__ ph,
                                                   float *__restrict__ pl, float *__restrict__ r32,
                                                   float *__restrict__ xh, float *__restrict__ xl,
@@ -651,14 +652,18 @@ __global__ void __launch_bounds__(256) mixed_prep(const double *__restrict__ f, 
   __shared__ double red[8];
   const int m = blockIdx.x;
   const int i0 = blockIdx.y * kPrepRows, i1 = min(i0 + kPrepRows, nr);
-  const double sc = scale[m];
+  const Pow2 sc = pow2(-rexp[m]);
   double acc = 0.0;
   for (int i = i0; i < i1; ++i) {
-    const double rs = R[i] * sc;  // exact: sc is a power of two
+    const double ri = R[i], rs = ri * sc.a;
+    // R sigma, a normal number but at the ends of the range, is exact, and so is its
+    // product with f but for the one rounding of R f
+    const unsigned ex = (unsigned)__double2hiint(rs) >> 20;
+    const bool exact = sc.one && ex >= 1 && ex <= 2046;
     const size_t src = ((size_t)m * nr + i) * nz, dst = ((size_t)m * nr + i) * pitch;
 #pragma unroll 4
     for (int k = threadIdx.x; k < nz; k += 256) {
-      const double v = rs * f[src + k];
+      const double v = exact ? rs * f[src + k] : ri * (f[src + k] * sc.a) * sc.b;
       float h, l;
       split_df(v, h, l);
       ph[dst + k] = h;
@@ -666,7 +671,7 @@ __global__ void __launch_bounds__(256) mixed_prep(const double *__restrict__ f, 
       if (r32 != nullptr) r32[dst + k] = h;
       acc = fma(v, v, acc);
       if (u != nullptr) {
-        split_df(u[src + k] * sc, h, l);
+        split_df(times(u[src + k], sc), h, l);
         xh[dst + k] = h;
         xl[dst + k] = l;
       }
@@ -683,27 +688,33 @@ __global__ void __launch_bounds__(256) mixed_prep(const double *__restrict__ f, 
 // addition per value remains.  grid (m, .).
 __global__ void __launch_bounds__(256) mixed_result(const float *__restrict__ xh0, const float *__restrict__ xl0,
                                                     const float *__restrict__ xh1, const float *__restrict__ xl1,
-                                                    const double *__restrict__ scale, const RhsState *st,
+                                                    const int *__restrict__ rexp, const RhsState *st,
                                                     int zero_start, int nr, int nz, int pitch,
                                                     double *__restrict__ u) {
   const int m = blockIdx.x;
   const int nrep = (int)st[m].tmp;
   const bool zero = zero_start && nrep == 0;
   const float *xh = (nrep & 1) ? xh1 : xh0, *xl = (nrep & 1) ? xl1 : xl0;
-  // scale is a power of two, normal: its inverse 2^e2 from the exponent bits
-  const int e2 = 1023 - (int)((__double_as_longlong(scale[m]) >> 52) & 0x7FF);
-  auto widen = [&](float v) -> double {
+  const int e = rexp[m];  // 1 / sigma = 2^e
+  // v 2^e by its exponent bits; false: neither a normal number nor 0
+  auto widen = [&](float v, double &o) -> bool {
     const unsigned b = __float_as_uint(v);
-    const int ex = (int)((b >> 23) & 0xFF), en = ex - 127 + e2;
-    if (ex == 0 || ex == 255 || en < -1022 || en > 1023) return ldexp((double)v, e2);
-    const unsigned long long o = ((unsigned long long)(b >> 31) << 63) | ((unsigned long long)(en + 1023) << 52) |
-                                 ((unsigned long long)(b & 0x7FFFFFu) << 29);
-    return __longlong_as_double((long long)o);
+    const int ex = (int)((b >> 23) & 0xFF), en = ex - 127 + e;
+    o = __longlong_as_double((long long)(((unsigned long long)(b >> 31) << 63) |
+                                         ((unsigned long long)(unsigned)(en + 1023) << 52) |
+                                         ((unsigned long long)(b & 0x7FFFFFu) << 29)));
+    if ((b << 1) == 0) o = 0.0;
+    return (b << 1) == 0 || (ex != 0 && ex != 255 && en >= -1022 && en <= 1023);
+  };
+  auto value = [&](float h, float l) -> double {
+    double a, b;
+    const bool ha = widen(h, a), lb = widen(l, b);
+    return ha && lb ? a + b : ldexp((double)h + (double)l, e);
   };
   for (int i = blockIdx.y; i < nr; i += gridDim.y) {
     const size_t src = ((size_t)m * nr + i) * pitch, dst = ((size_t)m * nr + i) * nz;
 #pragma unroll 4
-    for (int k = threadIdx.x; k < nz; k += 256) u[dst + k] = zero ? 0.0 : widen(xh[src + k]) + widen(xl[src + k]);
+    for (int k = threadIdx.x; k < nz; k += 256) u[dst + k] = zero ? 0.0 : value(xh[src + k], xl[src + k]);
   }
 }
 
@@ -2482,14 +2493,14 @@ int pcg_mixed_solve(ax_operator *op, const double *fd, double *ud, int m, double
   {
     const int nb = std::max(1, std::min((nr + 3) / 4, std::max(16, 2432 / m)));
     note_launch();
-    mixed_peak<<<dim3(m, nb), 256, 0, s>>>(fd, op->c64.R, nr, nz, part_ptr(w, kPartC), w->rscale, w->arrive, w->par,
+    mixed_peak<<<dim3(m, nb), 256, 0, s>>>(fd, op->c64.R, nr, nz, part_ptr(w, kPartC), w->rexp, w->arrive, w->par,
                                            tol * tol, delta * delta, w->chk);
     Finish fin = make_fin(w, st, guess ? kFinNone : kFinStart);
     fin.xoff = xoff;
     fin.max_iter = max_iter;
     note_launch();
     mixed_prep<<<dim3(m, (nr + kPrepRows - 1) / kPrepRows), 256, 0, s>>>(
-        fd, guess ? ud : nullptr, op->c64.R, w->rscale, nr, nz, P, w->phh, w->phl, guess ? nullptr : w->r32, w->xh[0],
+        fd, guess ? ud : nullptr, op->c64.R, w->rexp, nr, nz, P, w->phh, w->phl, guess ? nullptr : w->r32, w->xh[0],
         w->xl[0], part_ptr(w, kPartD), fin);
   }
   if (guess) residual(false, -1, kFinStart, s);
@@ -2550,7 +2561,7 @@ int pcg_mixed_solve(ax_operator *op, const double *fd, double *ud, int m, double
   }
   note_launch();
   mixed_result<<<dim3(m, std::max(1, std::min(nr, std::max(64, 9728 / m)))), 256, 0, s>>>(
-      w->xh[0], w->xl[0], w->xh[1], w->xl[1], w->rscale, st, guess ? 0 : 1, nr, nz, P, ud);
+      w->xh[0], w->xl[0], w->xh[1], w->xl[1], w->rexp, st, guess ? 0 : 1, nr, nz, P, ud);
   AX_CHECK_LAUNCH();
   return AX_OK;
 }
@@ -3466,10 +3477,10 @@ int ax_solve(ax_operator *op, const double *f, double *u, int32_t m, double tol,
   }
   if (scaled) {
     note_launch();
-    rhs_scale<<<(m + 31) / 32, 32, 0, s>>>(w->rscale, part_ptr(w, kPartC), nbf, m);
+    rhs_scale<<<(m + 31) / 32, 32, 0, s>>>(w->rexp, part_ptr(w, kPartC), nbf, m);
     note_launch();
-    apply_rhs_scale<<<dim3(sblocks, m), 256, 0, s>>>(w->phi64, guess ? w->x64 : nullptr, w->rscale, nullptr, 0,
-                                                     field, false);
+    apply_rhs_scale<<<dim3(sblocks, m), 256, 0, s>>>(w->phi64, guess ? w->x64 : nullptr, w->rexp, field,
+                                                     false);
     // ||phi||^2 of the scaled right-hand side, formed anew (the unscaled
     // squares may have overflowed or underflowed)
     note_launch();
@@ -3620,7 +3631,7 @@ int ax_solve(ax_operator *op, const double *f, double *u, int32_t m, double tol,
     for (int i = 0; i < m; ++i) info[i].iters += lz_steps[i];
   if (scaled) {
     note_launch();
-    apply_rhs_scale<<<dim3(sblocks, m), 256, 0, s>>>(nullptr, w->x64, w->rscale, nullptr, 0, field, true);
+    apply_rhs_scale<<<dim3(sblocks, m), 256, 0, s>>>(nullptr, w->x64, w->rexp, field, true);
   }
   if (!direct_mixed) {
     note_launch();
