@@ -663,13 +663,14 @@ int digit_gemm_partials(int rows, int n) { return 4 * digit_mtiles(rows) * (((n 
 
 // Digits of the transform matrix per (device, n, kind), kept for the life of the
 // process like the BF16 tables.
-const unsigned char *digit_table(int device, int n, int kind, cudaStream_t s) {
+const unsigned char *digit_table(int device, int n, int kind, cudaStream_t s, bool make) {
   static std::mutex mu;
   static std::vector<std::pair<long long, unsigned char *>> tables;
   std::lock_guard<std::mutex> lock(mu);
   const long long key = (long long)device << 32 | (unsigned)n | (long long)kind << 24;
   for (auto &e : tables)
     if (e.first == key) return e.second;
+  if (!make) return nullptr;
   const int ne = (n + 1) >> 1, kbh = (ne + kDK - 1) / kDK, nts = (ne + kDN - 1) / kDN;
   const size_t bytes = (size_t)nts * 2 * kbh * kSlices * kDBTile;
   unsigned char *d = nullptr;

@@ -442,7 +442,7 @@ size_t digit_bytes(int rows, int n);       // per RHS
 int digit_table_exp(int n, int kind);
 int digit_split_blocks(int rows);          // partials per RHS of the split
 int digit_gemm_partials(int rows, int n);    // partials per RHS of the products
-const unsigned char *digit_table(int device, int n, int kind, cudaStream_t s);
+const unsigned char *digit_table(int device, int n, int kind, cudaStream_t s, bool make = true);
 void launch_digit_split(const DigitArgs &a, cudaStream_t s);
 void launch_digit_gemm(const DigitArgs &a, cudaStream_t s);
 

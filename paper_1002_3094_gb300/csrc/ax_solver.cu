@@ -1410,11 +1410,12 @@ const uint16_t *tc_table(int device, int n, int kind = kTableSine) {
   c.tables.push_back({key, d});
   return d;
 }
-int *tc_flag(int device) {
+int *tc_flag(int device, bool make = true) {
   TcCache &c = tc_cache();
   std::lock_guard<std::mutex> lock(c.mu);
   for (auto &e : c.flags)
     if (e.first == device) return e.second;
+  if (!make) return nullptr;
   int *d = nullptr;
   std::lock_guard<std::recursive_mutex> lock2(g_alloc_capture_mutex);
   if (dalloc(&d, 1) != cudaSuccess) return nullptr;
@@ -1703,13 +1704,25 @@ bool use_digits(const ax_operator *op) {
   return sizeof(T) == 8 && !op->ws->digits_off && digits_apply(op->nr, op->nz);
 }
 
-// Buffers and tables for `rows` rows of m right-hand sides (before any capture):
-// 16 bytes per point.  Where they do not fit, the operator's FP64 transforms go
-// back to the FFT, which needs none.
+// Digits and row exponents of `rows` rows of m right-hand sides: 16 bytes per point.
+size_t digit_need(const ax_operator *op, int m, int rows) {
+  return m * (digit_bytes(rows, op->nz) + (size_t)digit_mtiles(rows) * 128 * sizeof(double));
+}
+// The matrix digits of both directions and the error flag exist; make: they are made
+// where they do not.
+bool digit_tables(const ax_operator *op, cudaStream_t s, bool make) {
+  const bool cz = op->bc_z == 1;
+  return digit_table(op->device, op->nz, cz ? kTableCosForward : kTableSine, s, make) != nullptr &&
+         digit_table(op->device, op->nz, cz ? kTableCosInverse : kTableSine, s, make) != nullptr &&
+         tc_flag(op->device, make) != nullptr;
+}
+
+// Buffers and tables of a solve of m right-hand sides (before any capture).  Where
+// they do not fit, the operator's FP64 transforms go back to the FFT, which needs none.
 void digit_prepare(ax_operator *op, int m, int rows, cudaStream_t s) {
   std::lock_guard<std::recursive_mutex> lock(g_alloc_capture_mutex);
   Workspace *w = op->ws;
-  const size_t need = m * (digit_bytes(rows, op->nz) + (size_t)digit_mtiles(rows) * 128 * sizeof(double));
+  const size_t need = digit_need(op, m, rows);
   if (w->digits_bytes < need) {
     dfree(w->digits);
     w->digits_bytes = 0;
@@ -1722,9 +1735,7 @@ void digit_prepare(ax_operator *op, int m, int rows, cudaStream_t s) {
     }
     w->digits_bytes = need;
   }
-  const bool cz = op->bc_z == 1;
-  if (!digit_table(op->device, op->nz, cz ? kTableCosForward : kTableSine, s) ||
-      !digit_table(op->device, op->nz, cz ? kTableCosInverse : kTableSine, s) || !tc_flag(op->device)) {
+  if (!digit_tables(op, s, true)) {
     cudaGetLastError();
     w->digits_off = true;
     free_graph(w->g64);
@@ -1734,12 +1745,15 @@ void digit_prepare(ax_operator *op, int m, int rows, cudaStream_t s) {
 // out = transform of the rows `in`; with upd.r the PCG update of r and x comes
 // first (upd.in = q; upd.partial and upd.fin its ||r||^2).  dot: (dot, out)
 // partials with the scalar step fin.  report: an expired wait sets the device's
-// error flag (callers that read it); it always makes the rows NaN.
+// error flag (callers that read it); it always makes the rows NaN.  buf: digit_need
+// bytes for the digits (null: the solves' own).
 void digit_transform(const ax_operator *op, int m, int rows, const double *in, double *out, bool inverse,
                      const RhsState *st, int mask, cudaStream_t s, const DigitArgs *upd = nullptr,
                      const double *dot = nullptr, double *partial = nullptr, const Finish &fin = Finish{},
-                     bool report = true, bool dense_in = false, bool dense_out = false) {
+                     bool report = true, bool dense_in = false, bool dense_out = false,
+                     unsigned char *buf = nullptr) {
   Workspace *w = op->ws;
+  if (buf == nullptr) buf = w->digits;
   DigitArgs a{};
   if (upd != nullptr) a = *upd;
   const int kind = op->bc_z == 1 ? (inverse ? kTableCosInverse : kTableCosForward) : kTableSine;
@@ -1753,8 +1767,8 @@ void digit_transform(const ax_operator *op, int m, int rows, const double *in, d
   a.mtiles = digit_mtiles(rows);
   a.in = in;
   a.fold = kind == kTableCosForward;
-  a.digits = w->digits;
-  a.scale = reinterpret_cast<double *>(w->digits + (size_t)m * digit_bytes(rows, op->nz));
+  a.digits = buf;
+  a.scale = reinterpret_cast<double *>(buf + (size_t)m * digit_bytes(rows, op->nz));
   a.st = st;
   a.mask = mask;
   launch_digit_split(a, s);
@@ -3211,38 +3225,58 @@ __global__ void scale_rows(float *__restrict__ x, const float *__restrict__ rs, 
 }
 
 // ---- single-step entry points --------------------------------------------
+// Whether a single FP64 step transforms by integer products: its staging (the digits
+// and `extra` FP64 elements per right-hand side) and tables are made where they are
+// missing; where they cannot be, for want of memory or under stream capture, the FFT
+// runs, whose staging is no larger.
+static bool digit_step_ready(ax_operator *op, int m, int rows, size_t extra, cudaStream_t s) {
+  Workspace *w = op->ws;
+  if (w->digits_off || !digits_apply(rows, op->nz)) return false;
+  const size_t need = digit_need(op, m, rows) + extra * m * sizeof(double);
+  if (w->scratch_bytes >= need && digit_tables(op, s, false)) return true;
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) {
+    cudaGetLastError();
+    return false;
+  }
+  if (ensure_scratch(op, need) == AX_OK && digit_tables(op, s, true)) return true;
+  cudaGetLastError();
+  std::lock_guard<std::recursive_mutex> lock(g_alloc_capture_mutex);
+  w->digits_off = true;
+  free_graph(w->g64);
+  return false;
+}
+
 template <typename T>
 static int apply_step(ax_operator *op, const double *in, double *out, int m, int rows_per, int which,
                       cudaStream_t s, bool tc = false, int tc_three = 0) {
   Workspace *w = op->ws;
   const size_t field = (size_t)rows_per * op->pitch;
-  // b also holds the mode-major field between the tensor-core transforms
-  const size_t fb = tc ? std::max(field, (size_t)op->nz * op->tpitch) : field;
-  int rc = ensure_scratch(op, (field + fb) * m * sizeof(T));
-  if (rc != AX_OK) return rc;
-  if (tc && (rc = ensure_split(op, (size_t)m * split_geom(op, rows_per).bytes_per_rhs)) != AX_OK) return rc;
-  // FP64 transforms by integer products
-  bool dg = sizeof(T) == 8 && (which == 1 || which == 3 || which == 4) && !w->digits_off &&
-            digits_apply(rows_per, op->nz);
-  if (dg) digit_prepare(op, m, rows_per, s);
-  dg = dg && !w->digits_off;
   if constexpr (sizeof(T) == 8) {
-    if (dg) {
-      // from and to the caller's dense rows; these calls do not wait for the GPU,
-      // so an expired wait shows as NaN rows
+    // FP64 transforms by integer products, from and to the caller's dense rows, the
+    // digits in the single steps' own staging (graphs that a caller captured of them
+    // hold its address).  These calls do not wait for the GPU, so an expired wait shows
+    // as NaN rows
+    if ((which == 1 || which == 3 || which == 4) && digit_step_ready(op, m, rows_per, which == 3 ? field : 0, s)) {
       double *z = reinterpret_cast<double *>(w->scratch);
       const bool all = which == 3;
+      unsigned char *buf = reinterpret_cast<unsigned char *>(z + (all ? field * m : 0));
       digit_transform(op, m, rows_per, in, all ? z : out, which == 4, nullptr, -1, s, nullptr, nullptr, nullptr,
-                      Finish{}, false, true, !all);
+                      Finish{}, false, true, !all, buf);
       if (all) {
         launch_tridiag<double>(tri_args<double>(op, m, z, z, nullptr, -1), s);
         digit_transform(op, m, rows_per, z, out, true, nullptr, -1, s, nullptr, nullptr, nullptr, Finish{}, false,
-                        false, true);
+                        false, true, buf);
       }
       AX_CHECK_LAUNCH();
       return AX_OK;
     }
   }
+  // b also holds the mode-major field between the tensor-core transforms
+  const size_t fb = tc ? std::max(field, (size_t)op->nz * op->tpitch) : field;
+  int rc = ensure_scratch(op, (field + fb) * m * sizeof(T));
+  if (rc != AX_OK) return rc;
+  if (tc && (rc = ensure_split(op, (size_t)m * split_geom(op, rows_per).bytes_per_rhs)) != AX_OK) return rc;
   T *a = reinterpret_cast<T *>(w->scratch);
   T *b = a + field * m;
   AX_TRY(cudaMemsetAsync(w->scratch, 0, (field + fb) * m * sizeof(T), s));

@@ -1,0 +1,45 @@
+"""Which calls take the integer-product transforms, and what the others need not pay."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+import paper_1002_3094_gb300 as P  # noqa: E402
+from test_gpu_digit_transform import TOL, _problem  # noqa: E402
+
+pytestmark = pytest.mark.gpu
+
+
+def test_capture_before_the_first_transform():
+    """A capture of FP64 single steps whose staging exists already, but not the
+    digits' buffers: nothing may be allocated there."""
+    op, _, f, dev = _problem(64, 256, 1, 0)
+    x = torch.randn((1, 64, 256), dtype=torch.float64, device=dev)
+    y, z = torch.zeros_like(x), torch.zeros_like(x)
+    try:
+        P.ax_apply_operator(op, x, y, 1)  # makes the staging
+        torch.cuda.synchronize()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g):
+            P.ax_apply_dst(op, x, y, 64)
+            P.ax_apply_dst_inverse(op, y, z, 64)
+        g.replay()
+        torch.cuda.synchronize()
+        assert (z - x).norm() <= 2 * TOL * x.norm()
+        P.ax_apply_dst(op, x, z, 64)  # outside a capture: the digits
+        assert (z - y).norm() <= 2 * TOL * x.norm()
+        g.replay()
+        torch.cuda.synchronize()
+        P.ax_apply_preconditioner(op, x, y, 1)
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g):
+            P.ax_apply_preconditioner(op, x, z, 1)
+        # a larger solve on the operator leaves the captured staging alone
+        fm = torch.from_numpy(np.repeat(f[:1], 4, 0)).to(dev)
+        P.ax_solve(op, fm, torch.zeros_like(fm), 4, 1e-8, 500, P.AX_PCG_FP64)
+        z.zero_()
+        g.replay()
+        torch.cuda.synchronize()
+        assert torch.equal(y, z)
+    finally:
+        P.ax_destroy_operator(op)
