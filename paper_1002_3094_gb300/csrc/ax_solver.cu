@@ -1699,9 +1699,11 @@ void tc_mode_solve(const ax_operator *op, int m, const float *z, float *tmp, uns
 bool tc_dot_in_modes(const ax_operator *op) { return tridiag_split_ok(op->nr); }
 
 // ---- FP64 transform by integer products (ax_dst_digits.cu) -------------------
+// (their launches have a right-hand side per block of grid dimension y)
+constexpr int kMaxGridY = 65535;
 template <typename T>
-bool use_digits(const ax_operator *op) {
-  return sizeof(T) == 8 && !op->ws->digits_off && digits_apply(op->nr, op->nz);
+bool use_digits(const ax_operator *op, int m) {
+  return sizeof(T) == 8 && m <= kMaxGridY && !op->ws->digits_off && digits_apply(op->nr, op->nz);
 }
 
 // Digits and row exponents of `rows` rows of m right-hand sides: 16 bytes per point.
@@ -1833,7 +1835,7 @@ void precond_apply(const ax_operator *op, int m, const T *r, T *z, const RhsStat
     }
   }
   if constexpr (sizeof(T) == 8) {
-    if (use_digits<T>(op)) {
+    if (use_digits<T>(op, m)) {
       digit_transform(op, m, op->nr, r, z, false, st, mask, s);
       launch_tridiag<T>(tri_args<T>(op, m, z, z, st, mask), s);
       digit_transform(op, m, op->nr, z, out, true, st, mask, s, nullptr, r, prz, fin);
@@ -1946,7 +1948,7 @@ void pcg_iteration(const ax_operator *op, int m, const PcgVecs<T> &v, RhsState *
     }
   }
   if constexpr (sizeof(T) == 8) {
-    if (use_digits<T>(op)) {
+    if (use_digits<T>(op, m)) {
       DigitArgs u{};
       u.x = v.x;
       u.r = v.r;
@@ -3231,7 +3233,7 @@ __global__ void scale_rows(float *__restrict__ x, const float *__restrict__ rs, 
 // runs, whose staging is no larger.
 static bool digit_step_ready(ax_operator *op, int m, int rows, size_t extra, cudaStream_t s) {
   Workspace *w = op->ws;
-  if (w->digits_off || !digits_apply(rows, op->nz)) return false;
+  if (w->digits_off || m > kMaxGridY || !digits_apply(rows, op->nz)) return false;
   const size_t need = digit_need(op, m, rows) + extra * m * sizeof(double);
   if (w->scratch_bytes >= need && digit_tables(op, s, false)) return true;
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
@@ -3535,7 +3537,7 @@ int ax_solve(ax_operator *op, const double *f, double *u, int32_t m, double tol,
 
   if (method == AX_PCG_FP64 || method == AX_CHEB_FP64) {
     if ((rc = ensure_vec64(op, m, cheb)) != AX_OK) return rc;
-    if (use_digits<double>(op)) digit_prepare(op, m, nr, s);
+    if (use_digits<double>(op, m)) digit_prepare(op, m, nr, s);
     // r = phi - A x, start
     StencilArgs<double> ra = stencil_args<double>(op, m, w->st, -1);
     ra.in = w->x64;
@@ -3677,7 +3679,7 @@ int ax_solve(ax_operator *op, const double *f, double *u, int32_t m, double tol,
     AX_TRY(cudaMemcpyAsync(u, ud, dense * sizeof(double), cudaMemcpyDeviceToHost, s));
     AX_TRY(cudaStreamSynchronize(s));
   }
-  if (op->dst_tc || use_digits<double>(op)) {
+  if (op->dst_tc || use_digits<double>(op, m)) {
     // a bounded wait of the tensor-core transform expired: report and re-arm
     int *flag = tc_flag(op->device), hf = 0;
     if (flag) {

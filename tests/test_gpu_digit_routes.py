@@ -43,3 +43,22 @@ def test_capture_before_the_first_transform():
         assert torch.equal(y, z)
     finally:
         P.ax_destroy_operator(op)
+
+
+def test_many_right_hand_sides():
+    """More right-hand sides than a grid dimension y holds blocks."""
+    m, nr, nz = 65536, 48, 128
+    op, _, _, dev = _problem(nr, nz, 1, 0)
+    x = torch.randn((nr, nz), dtype=torch.float64, device=dev).expand(m, nr, nz).contiguous()
+    x[m - 1] *= 2.0
+    y = torch.zeros_like(x)
+    try:
+        P.ax_apply_preconditioner(op, x, y, m)
+        assert torch.equal(y[1], y[0]) and torch.equal(y[m - 2], y[0]) and torch.equal(y[m - 1], 2.0 * y[0])
+        one = torch.zeros_like(x[:1])
+        P.ax_apply_preconditioner(op, x[:1], one, 1)
+        assert (one[0] - y[0]).norm() <= 1e-12 * one.norm()
+    finally:
+        P.ax_destroy_operator(op)
+        del x, y
+        torch.cuda.empty_cache()
