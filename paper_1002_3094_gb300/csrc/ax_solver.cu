@@ -3525,6 +3525,7 @@ int ax_solve(ax_operator *op, const double *f, double *u, int32_t m, double tol,
   AX_CHECK_LAUNCH();
   const int nbs64 = stencil_blocks_per_rhs(nr, nz, 2);
   const bool cheb = (method == AX_CHEB_FP64 || method == AX_CHEB_MIXED);
+  bool digits = false;  // some transform runs by integer products
   // Chebyshev bounds from a Lanczos estimate where they are needed (see
   // cheb_estimate); its PCG steps count as iterations of this solve
   std::vector<int> lz_steps;
@@ -3537,7 +3538,11 @@ int ax_solve(ax_operator *op, const double *f, double *u, int32_t m, double tol,
 
   if (method == AX_PCG_FP64 || method == AX_CHEB_FP64) {
     if ((rc = ensure_vec64(op, m, cheb)) != AX_OK) return rc;
-    if (use_digits<double>(op, m)) digit_prepare(op, m, nr, s);
+    // the integer-product transforms serve the conjugate gradients and the guess gate
+    if (use_digits<double>(op, m) && (check_guess || (!cheb && !small_applies(op, m)))) {
+      digit_prepare(op, m, nr, s);
+      digits = use_digits<double>(op, m);
+    }
     // r = phi - A x, start
     StencilArgs<double> ra = stencil_args<double>(op, m, w->st, -1);
     ra.in = w->x64;
@@ -3679,7 +3684,7 @@ int ax_solve(ax_operator *op, const double *f, double *u, int32_t m, double tol,
     AX_TRY(cudaMemcpyAsync(u, ud, dense * sizeof(double), cudaMemcpyDeviceToHost, s));
     AX_TRY(cudaStreamSynchronize(s));
   }
-  if (op->dst_tc || use_digits<double>(op, m)) {
+  if (op->dst_tc || digits) {
     // a bounded wait of the tensor-core transform expired: report and re-arm
     int *flag = tc_flag(op->device), hf = 0;
     if (flag) {

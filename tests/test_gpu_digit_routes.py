@@ -62,3 +62,22 @@ def test_many_right_hand_sides():
         P.ax_destroy_operator(op)
         del x, y
         torch.cuda.empty_cache()
+
+
+def test_chebyshev_solves_hold_no_digits():
+    """AX_CHEB_FP64 transforms by FFT: the digits' 16 bytes per point are first
+    allocated by the AX_PCG_FP64 solve after it, whose vectors exist by then."""
+    nr, nz, m = 256, 511, 32
+    op, _, f, dev = _problem(nr, nz, 1, 0)
+    fd = torch.from_numpy(np.repeat(f[:1], m, 0)).to(dev)
+    u = torch.zeros_like(fd)
+    free = lambda: (torch.cuda.synchronize(), torch.cuda.mem_get_info()[0])[1]  # noqa: E731
+    try:
+        st, _ = P.ax_solve(op, fd, u, m, 1e-6, 500, P.AX_CHEB_FP64)
+        assert st == P.AX_OK
+        before = free()
+        st, _ = P.ax_solve(op, fd, u, m, 1e-6, 500, P.AX_PCG_FP64)
+        assert st == P.AX_OK
+        assert before - free() >= 16 * nr * nz * m
+    finally:
+        P.ax_destroy_operator(op)
