@@ -92,6 +92,39 @@ __device__ __forceinline__ double warp_sum_of(T v) {
   return s.warp_total();
 }
 
+// Sums of many FP32 values as three FP32 numbers, h + m + l: the rounding errors of h
+// (two-sum, exact) are summed in m and those of m in l, so that only roundings of l are
+// lost.  A sum that leaves FP32's range is infinite, one of values that are not finite
+// what their FP32 sum is.
+struct Sum3 {
+  float h = 0.f, m = 0.f, l = 0.f;
+  __device__ __forceinline__ static float two_sum(float a, float b, float &err) {
+    const float s = a + b, bb = s - a;
+    err = (a - (s - bb)) + (b - bb);
+    return s;
+  }
+  __device__ __forceinline__ void add(float v) {
+    float e1, e2;
+    h = two_sum(h, v, e1);
+    m = two_sum(m, e1, e2);
+    l += e2;
+  }
+  __device__ __forceinline__ void add(const Sum3 &o) {
+    float e1, e2, e3;
+    h = two_sum(h, o.h, e1);
+    m = two_sum(m, o.m, e2);
+    m = two_sum(m, e1, e3);
+    l = (l + o.l) + (e2 + e3);
+  }
+  // to words of at most 2^-24 each of the one before (every 256 values: the errors of
+  // l then stay below those of FP64 sums)
+  __device__ __forceinline__ void renorm() {
+    h = two_sum(h, m, m);
+    m = two_sum(m, l, l);
+  }
+  __device__ __forceinline__ float value() const { return isfinite(h) ? h + (m + l) : h; }
+};
+
 template <typename T>
 __device__ __forceinline__ double block_sum_of(T v, double *red) {
   const double w = warp_sum_of(v);

@@ -498,37 +498,69 @@ __global__ void __launch_bounds__(256) sum_partials(const float *__restrict__ pa
   }
 }
 
-// Per-block sums of gz over pixels, per channel: partial[block][c] (pairs of FP32
-// numbers inside a thread and over the block's threads, fixed order).  blockDim
-// = 256: groups of cp / 4 threads walk the pixels, 4 channels each.
+// s[t][.] += s[t + k q][.] over the `groups` groups of q threads, in a fixed order; the
+// first group holds the result.  Every thread of the block calls it.
+template <int N>
+__device__ __forceinline__ void add_groups(Sum3 (*s)[N], int q, int groups) {
+  const int grp = threadIdx.x / q;
+  for (int left = groups; left > 1;) {
+    const int half = (left + 1) >> 1;
+    if (grp < left - half)
+#pragma unroll
+      for (int i = 0; i < N; ++i) s[threadIdx.x][i].add(s[threadIdx.x + half * q][i]);
+    __syncthreads();
+    left = half;
+  }
+}
+
+// out[i] = sum over the slots of partial[slot][i], a warp per element in a fixed order,
+// rounded to FP32 once.  (The sums of gradients cancel: rounded to FP32 per block, 912
+// of them, they were some 100 times as far off as the plane sums in FP64 before.)
+__global__ void __launch_bounds__(256) sum_sum3(const Sum3 *__restrict__ partial, int slots, int n,
+                                                float *__restrict__ out) {
+  const int i = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  if (i >= n) return;
+  Sum3 s;
+#pragma unroll 4
+  for (int k = lane; k < slots; k += 32) s.add(partial[(size_t)k * n + i]);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const Sum3 t{__shfl_xor_sync(0xffffffffu, s.h, o), __shfl_xor_sync(0xffffffffu, s.m, o),
+                 __shfl_xor_sync(0xffffffffu, s.l, o)};
+    s.add(t);
+  }
+  if (lane == 0) out[i] = s.value();
+}
+
+// Per-block sums of gz over pixels, per channel: partial[block][c].  blockDim = 256:
+// groups of cp / 4 threads walk the pixels, 4 channels each.
 __global__ void __launch_bounds__(256) channel_sums(const float *__restrict__ g, int C, int cp, size_t pixels,
-                                                    float *__restrict__ partial) {
-  __shared__ float sh[256][4], sl[256][4];
+                                                    Sum3 *__restrict__ partial) {
+  __shared__ Sum3 sd[256][4];
   const int q = cp / 4, groups = max(1, 256 / q);
   // channels beyond what one pass of the threads covers are taken in turn
   for (int c0 = 0; c0 < q; c0 += 256) {
     const int c = c0 + (q <= 256 ? (int)threadIdx.x % q : (int)threadIdx.x), grp = q <= 256 ? threadIdx.x / q : 0;
-    SumOf<float> s[4];
+    Sum3 s[4];
     if (c < q && grp < groups) {
+      unsigned seen = 0;
       for (size_t p = (size_t)blockIdx.x * groups + grp; p < pixels; p += (size_t)gridDim.x * groups) {
         const float4 v = *reinterpret_cast<const float4 *>(g + p * cp + c * 4);
         s[0].add(v.x); s[1].add(v.y); s[2].add(v.z); s[3].add(v.w);
+        if ((++seen & 255u) == 0)
+#pragma unroll
+          for (int i = 0; i < 4; ++i) s[i].renorm();
       }
     }
     __syncthreads();
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      sh[threadIdx.x][i] = s[i].h;
-      sl[threadIdx.x][i] = s[i].l;
-    }
+    for (int i = 0; i < 4; ++i) sd[threadIdx.x][i] = s[i];
     __syncthreads();
+    add_groups(sd, min(q, 256), groups);
     if ((int)threadIdx.x < min(q, 256) && c < q) {
 #pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        SumOf<float> tot;
-        for (int k = 0; k < groups; ++k) tot.add(sh[threadIdx.x + k * q][i], sl[threadIdx.x + k * q][i]);
-        if (c * 4 + i < C) partial[(size_t)blockIdx.x * C + c * 4 + i] = tot.h + tot.l;
-      }
+      for (int i = 0; i < 4; ++i)
+        if (c * 4 + i < C) partial[(size_t)blockIdx.x * C + c * 4 + i] = sd[threadIdx.x][i];
     }
   }
 }
@@ -642,16 +674,17 @@ __global__ void head_fwd(const bf16 *__restrict__ a, const float *__restrict__ w
 // of the bias gradient sum_p gy.  Threads as in channel_sums (4 channels each).
 __global__ void __launch_bounds__(256) head_bwd(const float *__restrict__ gy, const bf16 *__restrict__ a,
                                                 const float *__restrict__ w, float *__restrict__ gz, size_t pixels,
-                                                int C, int cp, float *__restrict__ partial) {
-  __shared__ float sh[256][5], sl[256][5];
+                                                int C, int cp, Sum3 *__restrict__ partial) {
+  __shared__ Sum3 sd[256][5];
   const int q = cp / 4, groups = max(1, 256 / q);
   for (int c0 = 0; c0 < q; c0 += 256) {
     const int c = c0 + (q <= 256 ? (int)threadIdx.x % q : (int)threadIdx.x), grp = q <= 256 ? threadIdx.x / q : 0;
-    SumOf<float> s[5];
+    Sum3 s[5];
     if (c < q && grp < groups) {
       float wv[4];
 #pragma unroll
       for (int i = 0; i < 4; ++i) wv[i] = c * 4 + i < C ? w[c * 4 + i] : 0.f;
+      unsigned seen = 0;
       for (size_t p = (size_t)blockIdx.x * groups + grp; p < pixels; p += (size_t)gridDim.x * groups) {
         const float gv = gy[p];
         const uint2 u = *reinterpret_cast<const uint2 *>(a + p * cp + c * 4);
@@ -665,25 +698,25 @@ __global__ void __launch_bounds__(256) head_bwd(const float *__restrict__ gy, co
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
           const float pr = av[i] * gv;
-          s[i].add(pr, fmaf(av[i], gv, -pr));
+          s[i].add(pr);
+          s[i].add(fmaf(av[i], gv, -pr));
         }
         s[4].add(gv);
+        if ((++seen & 127u) == 0)
+#pragma unroll
+          for (int i = 0; i < 5; ++i) s[i].renorm();
       }
     }
     __syncthreads();
 #pragma unroll
-    for (int i = 0; i < 5; ++i) {
-      sh[threadIdx.x][i] = s[i].h;
-      sl[threadIdx.x][i] = s[i].l;
-    }
+    for (int i = 0; i < 5; ++i) sd[threadIdx.x][i] = s[i];
     __syncthreads();
+    add_groups(sd, min(q, 256), groups);
     if ((int)threadIdx.x < min(q, 256) && c < q) {
 #pragma unroll
       for (int i = 0; i < 5; ++i) {
-        SumOf<float> tot;
-        for (int k = 0; k < groups; ++k) tot.add(sh[threadIdx.x + k * q][i], sl[threadIdx.x + k * q][i]);
         const int slot = i < 4 ? c * 4 + i : C;
-        if (i < 4 ? slot < C : c == 0) partial[(size_t)blockIdx.x * (C + 1) + slot] = tot.h + tot.l;
+        if (i < 4 ? slot < C : c == 0) partial[(size_t)blockIdx.x * (C + 1) + slot] = sd[threadIdx.x][i];
       }
     }
   }
@@ -866,7 +899,8 @@ struct GuessNet {
   float *y = nullptr, *gy = nullptr;                             // head output and its gradient [cap][hw][hw]
   float *gbuf[3] = {nullptr, nullptr, nullptr};                  // gradients (largest activation)
   std::vector<float *> gskip;                                    // skip gradients per level
-  float *partial = nullptr;                                      // weight- and bias-gradient partials
+  float *partial = nullptr;                                      // weight-gradient partials
+  Sum3 *spart = nullptr;                                         // partials of the bias and head gradients
   double *lpart = nullptr;                                       // loss partials
   float h1 = 0.f;                                                // weight of the loss's edge term
   int step = 0;
@@ -1008,7 +1042,7 @@ void net_free(GuessNet *n) {
   for (auto *a : n->gskip) cudaFree(a);
   cudaFree(n->y);
   for (float *g : n->gbuf) cudaFree(g);
-  cudaFree(n->partial); cudaFree(n->lpart);
+  cudaFree(n->partial); cudaFree(n->spart); cudaFree(n->lpart);
   delete n;
 }
 
@@ -1069,9 +1103,9 @@ void launch_wgrad(GuessNet *n, const bf16 *in, const float *gz, float *gw, int B
 
 void bias_grad(GuessNet *n, const float *gz, float *gb, int B, int C, int res, cudaStream_t s) {
   note_launch();
-  channel_sums<<<kSumBlocks, 256, 0, s>>>(gz, C, pad8(C), (size_t)B * res * res, n->partial);
+  channel_sums<<<kSumBlocks, 256, 0, s>>>(gz, C, pad8(C), (size_t)B * res * res, n->spart);
   note_launch();
-  sum_partials<<<(C + 31) / 32, 256, 0, s>>>(n->partial, kSumBlocks, (size_t)C, gb, 1, C);
+  sum_sum3<<<(C + 7) / 8, 256, 0, s>>>(n->spart, kSumBlocks, C, gb);
 }
 
 void pack_all(GuessNet *n, cudaStream_t s) {
@@ -1114,9 +1148,9 @@ void backward_pass(GuessNet *n, int B, cudaStream_t s) {
     const NetLayer &L = n->layers[last];
     note_launch();
     head_bwd<<<kSumBlocks, 256, 0, s>>>(n->gy, n->act[L.in], n->p + L.woff, g, (size_t)B * H * H, L.cin, pad8(L.cin),
-                                        n->partial);
+                                        n->spart);
     note_launch();
-    sum_partials<<<(L.cin + 32) / 32, 256, 0, s>>>(n->partial, kSumBlocks, (size_t)L.cin + 1, n->g + L.woff, 1, L.cin + 1);
+    sum_sum3<<<(L.cin + 8) / 8, 256, 0, s>>>(n->spart, kSumBlocks, L.cin + 1, n->g + L.woff);
   }
   for (int li = last - 1; li >= 0; --li) {
     const NetLayer &L = n->layers[li];
@@ -1226,14 +1260,15 @@ int ax_guessnet_create(int32_t hw, const int32_t *channels, int32_t batch_capaci
     n->gskip.push_back(sg);
   }
   // partials of the weight gradients (splits x 9 cin cout) and of the channel sums
-  size_t pn = 0;
+  size_t pn = 0, sn = 0;
   for (const NetLayer &L : n->layers) {
     const int cin = L.in < 0 ? 9 : L.cin;
     if (L.kind == 'c' || L.kind == 's')
       pn = std::max(pn, (size_t)wgrad_splits(cin, L.cout, 1LL << 40) * 9 * cin * L.cout);
-    pn = std::max(pn, (size_t)kSumBlocks * (std::max(L.cin, L.cout) + 1));
+    sn = std::max(sn, (size_t)kSumBlocks * (std::max(L.cin, L.cout) + 1));
   }
   if (e == cudaSuccess) e = zalloc(&n->partial, pn);
+  if (e == cudaSuccess) e = zalloc(&n->spart, sn);
   if (e == cudaSuccess) e = zalloc(&n->lpart, 1024);
   if (e == cudaSuccess) e = cudaMemcpy(n->p, h.data(), n->nparams * sizeof(float), cudaMemcpyHostToDevice);
   if (e == cudaSuccess) {
