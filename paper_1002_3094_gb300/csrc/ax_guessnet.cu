@@ -579,7 +579,8 @@ __global__ void pack_input(const float *__restrict__ x, bf16 *__restrict__ y, in
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
       const bf16 h = __float2bfloat16(v[c]);
-      const float r = v[c] - __bfloat162float(h);
+      // no rest beside an infinite high part: its NaN times the zero weights would hide it
+      const float r = isinf(__bfloat162float(h)) ? 0.f : v[c] - __bfloat162float(h);
       const bf16 m = __float2bfloat16(r);
       o[c] = h;
       o[3 + c] = m;

@@ -118,3 +118,22 @@ def test_sums_that_cancel(ch, hw, batch):
     c = ch[0]
     got = grad[-(2 * c + 1):]  # biases of the last convolution, the head's weights and bias
     assert np.abs(got - math.fsum(each)).max() <= tol
+
+
+@pytest.mark.parametrize("value", [float("inf"), 3.4e38])
+def test_an_infinite_input_stays_visible(value):
+    """3.4e38 is infinite in BF16.  All weights are positive, so the outputs that
+    depend on the value are infinite."""
+    _cuda()
+    ch, hw = (8, 8, 8, 8), 64
+    net = P.ax_guessnet_create(hw, ch, batch_capacity=1, seed=3)
+    try:
+        P.ax_guessnet_set_params(net, _constant_net(ch, 0.125, 1.0, 1.0, 0.0))
+        x = torch.zeros((1, 3, hw, hw), dtype=torch.float32, device="cuda")
+        x[0, 1, 20, 30] = value
+        y = torch.zeros((1, hw, hw), dtype=torch.float32, device="cuda")
+        P.ax_guessnet_forward(net, x, y, 1)
+        assert torch.isinf(y[0, 17:24, 27:34]).all()
+        assert not torch.isnan(y).any()
+    finally:
+        P.ax_guessnet_destroy(net)
