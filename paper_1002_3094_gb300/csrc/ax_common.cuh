@@ -57,40 +57,55 @@ __device__ __forceinline__ double block_sum(double v, double *red) {
   return s;
 }
 
-// Sums of FP32 values, returned in FP64.  GB300 adds two FP64 numbers per clock
-// and SM, so a warp's FP64 shuffle tree holds that pipe for 80 cycles; here the
-// sums are pairs of FP32 numbers (two-sum, about 48 bits) instead: some 50 FP32
-// operations per tree, 13 cycles.  FP64 values are summed in FP64.
-template <typename T> struct SumOf;
-template <>
-struct SumOf<float> {
-  float h = 0.f, l = 0.f;
-  __device__ __forceinline__ void add(float oh, float ol = 0.f) {
-    const float s = h + oh, bb = s - h;
-    l = (l + ol) + ((h - (s - bb)) + (oh - bb));
-    h = s;
-  }
-  __device__ __forceinline__ double warp_total() {
+// Sum of N FP32 values of every lane of a warp, returned in FP64.  GB300 adds two FP64
+// numbers per clock and SM, so an FP64 shuffle tree holds that pipe for 80 cycles a
+// warp.  Here the values are cut to integers of 60 bits below the largest one's exponent
+// (three words of 20 bits with room for the sums) and added exactly by the warp's
+// integer reductions: what is lost is at most 32 N 2^-60 of the largest value and the
+// rounding of the result, less than an FP64 tree loses (5 2^-53 of the sum of
+// magnitudes for N = 1), and no sum overflows.  Values that are not finite are summed in
+// FP64.
+template <int N>
+__device__ __forceinline__ double warp_sum_fp32(const float (&v)[N]) {
+  unsigned top = 1;
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      const float oh = __shfl_xor_sync(0xffffffffu, h, o), ol = __shfl_xor_sync(0xffffffffu, l, o);
-      add(oh, ol);
-    }
-    return (double)h + (double)l;
+  for (int i = 0; i < N; ++i) top = max(top, (__float_as_uint(v[i]) >> 23) & 255u);
+  top = __reduce_max_sync(0xffffffffu, top);
+  if (top == 255u) {
+    double d = 0.0;
+    for (int i = 0; i < N; ++i) d += (double)v[i];
+    return warp_sum(d);
   }
-};
-template <>
-struct SumOf<double> {
-  double v = 0.0;
-  __device__ __forceinline__ void add(double o) { v += o; }
-  __device__ __forceinline__ double warp_total() { return warp_sum(v); }
-};
-template <typename T>
-__device__ __forceinline__ double warp_sum_of(T v) {
-  SumOf<T> s;
-  s.add(v);
-  return s.warp_total();
+  int w0 = 0, w1 = 0, w2 = 0;
+#pragma unroll
+  for (int i = 0; i < N; ++i) {
+    const unsigned b = __float_as_uint(v[i]), f = (b >> 23) & 255u;
+    const unsigned mant = (b & 0x7FFFFFu) | (f != 0 ? 0x800000u : 0u);
+    const unsigned long long X = ((unsigned long long)mant << 36) >> min(top - max(f, 1u), 63u);
+    const int sgn = (int)b >> 31;  // 0 or -1
+    w0 += ((int)(X >> 40) ^ sgn) - sgn;
+    w1 += ((int)(X >> 20 & 0xFFFFF) ^ sgn) - sgn;
+    w2 += ((int)(X & 0xFFFFF) ^ sgn) - sgn;
+  }
+  w0 = __reduce_add_sync(0xffffffffu, w0);
+  w1 = __reduce_add_sync(0xffffffffu, w1);
+  w2 = __reduce_add_sync(0xffffffffu, w2);
+  // sum 2^-5 in units of 2^(top - 127 - 23 - 36) as one integer of at most 63 bits
+  // (N <= 8), rounded to a double by its bits
+  const long long S = ((long long)w0 << 35) + ((((long long)w1 << 20) + w2) >> 5);
+  if (S == 0) return 0.0;
+  const unsigned long long a = (unsigned long long)(S < 0 ? -S : S);
+  const int lz = __clzll((long long)a);
+  unsigned long long r = a << lz;
+  r = (r >> 11) + ((r >> 10) & 1);  // 2^52 .. 2^53
+  const unsigned long long bits = ((unsigned long long)(1023 + 63 - lz + 5 + (int)top - 186 - 1) << 52) + r;
+  return __longlong_as_double((long long)(bits | (S < 0 ? 1ull << 63 : 0ull)));
 }
+__device__ __forceinline__ double warp_sum_of(float v) {
+  const float w[1] = {v};
+  return warp_sum_fp32(w);
+}
+__device__ __forceinline__ double warp_sum_of(double v) { return warp_sum(v); }
 
 // Sums of many FP32 values as three FP32 numbers, h + m + l: the rounding errors of h
 // (two-sum, exact) are summed in m and those of m in l, so that only roundings of l are

@@ -294,10 +294,17 @@ __global__ void __launch_bounds__(32 * NW, (MODE == kStencilPcg ? 16 : 24) / NW)
   const unsigned nb = gridDim.x * gridDim.y;
   __syncthreads();
   for (int c = warp; c < n; c += NW) {
-    SumOf<T> sum;
+    double tot;
+    if constexpr (sizeof(T) == 4) {
+      float v[NW];
 #pragma unroll
-    for (int i = 0; i < NW; ++i) sum.add(s_acc[c][i * 32 + lane]);
-    const double tot = sum.warp_total();
+      for (int i = 0; i < NW; ++i) v[i] = s_acc[c][i * 32 + lane];
+      tot = warp_sum_fp32(v);
+    } else {
+      tot = 0.0;
+      for (int i = 0; i < NW; ++i) tot += s_acc[c][i * 32 + lane];
+      tot = warp_sum(tot);
+    }
     if (lane == 0) {
       if (a.partial != nullptr)
         a.partial[(size_t)s_m[c] * kPartialStride + blockIdx.y * gridDim.x + blockIdx.x] = tot;
