@@ -22,10 +22,10 @@
 // and rounded to FP64 once.  A row whose entries are small beside its largest (the sum
 // of |X_0| stays below 512 128 with one bit more) gets that bit, |X_0| <= 256: there
 // the rounding of the digits, not that of the result, would be the larger error.
-// Error against 113-bit sums, of the row's norm, mean over rows of normal deviates, of
-// a few large entries, constant and smooth ones, 128 to 1024 columns: 0.9-1.9e-16 by
-// length (the FFT: 2.1-5.3e-16), at most 4.8e-16 (6.7e-16): a constant row under the
-// cosine of length 511 = 7 73, where the matrix entries' own rounding adds up.
+// Error against 64-bit significands, in 2^-53 of the row's norm, rows of normal deviates
+// and single, wide-ranged, constant, smooth and decaying ones, 11 lengths from 128 to
+// 1024, both boundaries: 0.65-0.80 on average over the normal deviates, at most 2.7 (the
+// FFT: 1.9-6.8, 7.3).
 //
 // Even / odd split as in ax_dst_gemm.cu: P = (even input columns) S and Q = (odd
 // input columns) S over the first ceil(n/2) output columns, out[l] = P + Q,
@@ -597,9 +597,52 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kDThreads, 1) digit_
   }
 }
 
+// Numbers as pairs of FP64 numbers, v = h + l, for the matrix entries (two-sum and
+// two-product; some 100 bits).
+struct Pair {
+  double h, l;
+};
+__device__ __forceinline__ Pair pair_sum(double a, double b) {
+  const double s = a + b, bb = s - a;
+  return {s, (a - (s - bb)) + (b - bb)};
+}
+__device__ __forceinline__ Pair pair_add(Pair a, Pair b) {
+  const Pair s = pair_sum(a.h, b.h);
+  return pair_sum(s.h, s.l + (a.l + b.l));
+}
+__device__ __forceinline__ Pair pair_mul(Pair a, Pair b) {
+  const double p = a.h * b.h;
+  return pair_sum(p, fma(a.h, b.h, -p) + (a.h * b.l + a.l * b.h));
+}
+__device__ __forceinline__ Pair pair_div(Pair a, double d) {
+  const double q = a.h / d;
+  return pair_sum(q, (fma(-q, d, a.h) + a.l) / d);
+}
+
+// t[j] = sin(pi j / den), j <= den / 2, by the Taylor series of the sine or cosine of at
+// most pi / 4.  FP64 functions would leave an error of about 2^-53 in every entry of the
+// matrix, and the argument's rounding one that neighbouring entries share: it showed in
+// constant rows (511 columns: 4.3 2^-53 of the row's norm; now 0.8).
+__global__ void __launch_bounds__(128) sine_list_kernel(Pair *t, int den) {
+  const int j = blockIdx.x * 128 + threadIdx.x;
+  if (j > den / 2) return;
+  const bool co = 4 * j > den;  // cos(pi (den - 2 j) / (2 den))
+  const Pair x = pair_mul(pair_div(Pair{co ? (double)(den - 2 * j) : (double)j, 0.0}, co ? 2.0 * den : (double)den),
+                          Pair{3.14159265358979312, 1.2246467991473532e-16});
+  const Pair x2 = pair_mul(x, x);
+  Pair term = co ? Pair{1.0, 0.0} : x, sum = term;
+  for (int k = co ? 1 : 2; k < 24; k += 2) {  // -x^2 / (k (k + 1))
+    term = pair_div(pair_mul(term, x2), -(double)(k * (k + 1)));
+    sum = pair_add(sum, term);
+  }
+  t[j] = sum;
+}
+
 // Matrix digits: tiles (N tile, K block, slice) as the stages copy them; row l of a
-// tile the output column, k the position of the half.
-__global__ void __launch_bounds__(256) digit_table_kernel(unsigned char *__restrict__ t, int n, int kind, int e) {
+// tile the output column, k the position of the half.  sine: sine_list_kernel's, of
+// den = n + 1 for the sine, 2 n for the cosines.
+__global__ void __launch_bounds__(256) digit_table_kernel(unsigned char *__restrict__ t, const Pair *__restrict__ sine,
+                                                          int n, int kind, int e) {
   const int ne = (n + 1) >> 1, kbh = (ne + kDK - 1) / kDK, nts = (ne + kDN - 1) / kDN, L = n + 1;
   const size_t total = (size_t)nts * 2 * kbh * kDN * kDK;
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
@@ -607,19 +650,22 @@ __global__ void __launch_bounds__(256) digit_table_kernel(unsigned char *__restr
     const int nt = (int)(i / ((size_t)kDK * kDN * 2 * kbh));
     const bool second = kb >= kbh;
     const int l = nt * kDN + nl, kk = (second ? kb - kbh : kb) * kDK + kl;
-    double v = 0.0, vlo = 0.0;  // the entry as a pair
+    Pair v{0.0, 0.0};
     if (l < ne && kk < ne) {
-      // sqrt(num / den) c, the root as a pair: its rounding would be the same in
-      // every entry and show in rows that are nearly constant
-      auto entry = [&](int num, int den, double c) {
-        const double q = (double)num / den, ql = fma(-q, (double)den, (double)num) / den;
-        const double r = sqrt(q), rl = (fma(-r, r, q) + ql) / (2.0 * r);
-        v = r * c;
-        vlo = fma(r, c, -v) + rl * c;
+      // sqrt(num / den) c, the angles of c reduced exactly
+      auto entry = [&](int num, int den, Pair c) {
+        const Pair q = pair_div(Pair{(double)num, 0.0}, (double)den);
+        const double r = sqrt(q.h);
+        v = pair_mul(c, Pair{r, (fma(-r, r, q.h) + q.l) / (2.0 * r)});
       };
-      // orthonormal cosine entry of mode f at node k, the angle reduced exactly
+      auto sign = [](Pair c, bool minus) { return minus ? Pair{-c.h, -c.l} : c; };
+      // orthonormal cosine entry of mode f at node k, cos(pi m / (2 n)) = sin(pi (n - m) / (2 n))
       auto cosm = [&](int f, int k) {
-        entry(f == 0 ? 1 : 2, n, cospi((double)((long long)(2 * k + 1) * f % (4LL * n)) / (2.0 * n)));
+        int m = (int)((long long)(2 * k + 1) * f % (4LL * n));
+        if (m > 2 * n) m = 4 * n - m;
+        const bool minus = m > n;
+        if (minus) m = 2 * n - m;
+        entry(f == 0 ? 1 : 2, n, sign(sine[n - m], minus));
       };
       if (kind == kTableCosForward) {
         const int f = second ? 2 * l + 1 : 2 * l;
@@ -627,13 +673,22 @@ __global__ void __launch_bounds__(256) digit_table_kernel(unsigned char *__restr
       } else {
         const int k = second ? 2 * kk + 1 : 2 * kk;
         if (k < n) {
-          if (kind == kTableCosInverse) cosm(k, l);
-          else entry(2, L, sinpi((double)((long long)(k + 1) * (l + 1) % (2LL * L)) / L));
+          if (kind == kTableCosInverse) {
+            cosm(k, l);
+          } else {
+            int m = (int)((long long)(k + 1) * (l + 1) % (2LL * L));
+            const bool minus = m > L;
+            if (minus) m -= L;
+            entry(2, L, sign(sine[m > L - m ? L - m : m], minus));
+          }
         }
       }
     }
+    // v 2^(54 - e) rounded to an integer
+    const double w = ldexp(v.h, 54 - e);
+    const long long X = llrint(w);
     float d[kSlices];
-    digits_of(fixed_point(v, e, 54) + llrint(ldexp(vlo, 54 - e)), d);
+    digits_of(X + llrint((w - (double)X) + ldexp(v.l, 54 - e)), d);
     unsigned char *p = t + ((size_t)nt * 2 * kbh + kb) * (size_t)(kSlices * kDBTile) + digit_byte(nl, kl);
 #pragma unroll
     for (int s = 0; s < kSlices; ++s)
@@ -673,10 +728,15 @@ const unsigned char *digit_table(int device, int n, int kind, cudaStream_t s, bo
   if (!make) return nullptr;
   const int ne = (n + 1) >> 1, kbh = (ne + kDK - 1) / kDK, nts = (ne + kDN - 1) / kDN;
   const size_t bytes = (size_t)nts * 2 * kbh * kSlices * kDBTile;
+  // the matrix and, behind it, the list of sines it is made from
+  const int den = kind == kTableSine ? n + 1 : 2 * n;
   unsigned char *d = nullptr;
-  if (cudaMalloc((void **)&d, bytes) != cudaSuccess) return nullptr;
+  if (cudaMalloc((void **)&d, bytes + (den / 2 + 1) * sizeof(Pair)) != cudaSuccess) return nullptr;
+  Pair *sine = reinterpret_cast<Pair *>(d + bytes);
   note_launch();
-  digit_table_kernel<<<608, 256, 0, s>>>(d, n, kind, digit_table_exp(n, kind));
+  sine_list_kernel<<<den / 256 + 1, 128, 0, s>>>(sine, den);
+  note_launch();
+  digit_table_kernel<<<608, 256, 0, s>>>(d, sine, n, kind, digit_table_exp(n, kind));
   if (cudaGetLastError() != cudaSuccess || cudaStreamSynchronize(s) != cudaSuccess) {
     cudaFree(d);
     return nullptr;

@@ -56,3 +56,24 @@ def test_rows_near_the_largest_number(nz, bc_z):
         _check(op, x, nz, bc_z, dev)
     finally:
         P.ax_destroy_operator(op)
+
+
+@pytest.mark.parametrize("nz,bc_z", [(511, 1), (512, 0), (513, 1), (300, 0), (255, 1)])
+def test_constant_rows(nz, bc_z):
+    """Errors of the matrix entries that neighbours share would add up here.  Rounding P,
+    Q and their sum costs at most 2 2^-53 of the row's norm, the entries' own rounding
+    (2^-56 of the largest, of random sign) little: 3 2^-53."""
+    rows = 64 if nz <= 512 else 384  # (fewer take the FFT above 512 columns)
+    op, _, _, dev = _problem(64, nz, 1, bc_z)
+    k = np.arange(nz)
+    base = np.stack([np.ones(nz), np.where(k % 2, 1.0, -1.0), np.where(k < nz // 2, 1.0, 2.0), np.where(k % 7, 1.0, 3.0)])
+    x = np.resize(base, (rows, nz))
+    mat, xl = _matrix(nz, bc_z), x.astype(np.longdouble)
+    try:
+        for f, r in ((P.ax_apply_dst, mat.T), (P.ax_apply_dst_inverse, mat)):
+            y = torch.zeros((rows, nz), dtype=torch.float64, device=dev)
+            f(op, torch.from_numpy(x).to(dev), y, rows)
+            err = np.sqrt(((y.cpu().numpy() - xl @ r) ** 2).sum(1) / (xl ** 2).sum(1))
+            assert (err <= 3 * 2.0 ** -53).all(), (f.__name__, err[:4] * 2.0 ** 53)
+    finally:
+        P.ax_destroy_operator(op)
