@@ -2104,7 +2104,7 @@ bool unfinished(const RhsState *h, int m) {
 
 // PCG for the vectors v with right-hand side phi (in v.r on entry as the
 // residual).  Assumes st has been started (sc_start) and x holds the start.
-// If `true_check`, right-hand sides whose recursive residual passes get an
+// If `true_check` (FP64), right-hand sides whose recursive residual passes get an
 // FP64-exact test with the true residual phi - A x (plain method); otherwise
 // they finish at once (inner solves).
 template <typename T>
@@ -2122,13 +2122,15 @@ int pcg_loop(ax_operator *op, int m, const PcgVecs<T> &v, const T *phi, RhsState
   // fails it takes z, beta and p from the new r in the next iteration (kRedo).
   auto check_step = [&](cudaStream_t ss) {
     if (!true_check) return;
-    StencilArgs<T> ra = stencil_args<T>(op, m, st, kCheck);
-    ra.in = v.x;
-    ra.phi = phi;
-    ra.out_res = v.r;
-    ra.partial = part_ptr(w, kPartB);
-    ra.fin = make_fin(w, st, kFinTrueCheck);
-    launch_stencil<T>(kStencilResidual, ra, ss);
+    if constexpr (sizeof(T) == 8) {
+      StencilArgs<T> ra = stencil_args<T>(op, m, st, kCheck);
+      ra.in = v.x;
+      ra.phi = phi;
+      ra.out_res = v.r;
+      ra.partial = part_ptr(w, kPartB);
+      ra.fin = make_fin(w, st, kFinTrueCheck);
+      launch_stencil<T>(kStencilResidual, ra, ss);
+    }
   };
   const double per_rhs = (double)op->nr * op->nz;
   for (int guard = 0; guard < 1000000; ++guard) {

@@ -66,8 +66,10 @@ struct StripShape {
   static constexpr int row = 32 * V;                          // elements of a strip row
   static constexpr int array = (kStripRows + 2) * row + 16 / (int)sizeof(T) * kStripRows;  // rows, then edges
   static constexpr int stage = arrays * array;
-  // a warp's ring: no more stages than right-hand sides (few: more CTAs fit an SM, a
-  // solve of three 1024 x 1024 or one of 1500 x 1500 takes 1 per cent less)
+  // a warp's ring: no more stages than right-hand sides (few: more CTAs fit an SM.
+  // Mixed solves, all stages and these, four alternating runs of each within 0.2%: one
+  // 1024 x 1024 2.087 and 2.068 ms, three 4.273 and 4.233, one 1500 x 1500 5.056 and
+  // 4.994; 700 x 700 to 3000 x 3000 the same)
   __host__ __device__ static size_t warp_bytes(int chunk) {
     return (size_t)(chunk < stages ? chunk : stages) * stage * sizeof(T);
   }
@@ -186,7 +188,7 @@ __global__ void __launch_bounds__(32 * NW, (MODE == kStencilPcg ? 16 : 24) / NW)
   load_coefs(s_m[0]);
   for (int c = 0; c < n; ++c) {
     T ph[R][V];  // phi, requested before the wait for this right-hand side's rows
-    if (MODE == kStencilResidual || MODE == kStencilCheb) {
+    if (MODE == kStencilCheb) {
 #pragma unroll
       for (int j = 0; j < R; ++j) {
 #pragma unroll
@@ -271,18 +273,10 @@ __global__ void __launch_bounds__(32 * NW, (MODE == kStencilPcg ? 16 : 24) / NW)
         T res[V];
 #pragma unroll
         for (int e = 0; e < V; ++e) {
-          res[e] = (k0 + e < nz) ? ((MODE == kStencilResidual) ? ph[j][e] - o[e] : o[e] - ph[j][e]) : T(0);
+          res[e] = (k0 + e < nz) ? o[e] - ph[j][e] : T(0);
           acc = fma(res[e], res[e], acc);
         }
-        if (MODE == kStencilResidual) {
-          if (a.out_res) store_vec<T>(a.out_res + ro, res);
-          if (a.out32) {
-#pragma unroll
-            for (int e = 0; e < V; ++e) a.out32[ro + e] = (float)res[e];
-          }
-        } else {
-          store_vec<T>(a.out + ro, res);
-        }
+        store_vec<T>(a.out + ro, res);
       }
     }
     if (MODE != kStencilApply) s_acc[c][threadIdx.x] = acc;
@@ -294,17 +288,10 @@ __global__ void __launch_bounds__(32 * NW, (MODE == kStencilPcg ? 16 : 24) / NW)
   const unsigned nb = gridDim.x * gridDim.y;
   __syncthreads();
   for (int c = warp; c < n; c += NW) {
-    double tot;
-    if constexpr (sizeof(T) == 4) {
-      float v[NW];
+    T v[NW];
 #pragma unroll
-      for (int i = 0; i < NW; ++i) v[i] = s_acc[c][i * 32 + lane];
-      tot = warp_sum_fp32(v);
-    } else {
-      tot = 0.0;
-      for (int i = 0; i < NW; ++i) tot += s_acc[c][i * 32 + lane];
-      tot = warp_sum(tot);
-    }
+    for (int i = 0; i < NW; ++i) v[i] = s_acc[c][i * 32 + lane];
+    const double tot = warp_sum_fp32(v);
     if (lane == 0) {
       if (a.partial != nullptr)
         a.partial[(size_t)s_m[c] * kPartialStride + blockIdx.y * gridDim.x + blockIdx.x] = tot;
@@ -483,14 +470,7 @@ __global__ void __launch_bounds__(256) stencil_kernel(const StencilArgs<T> a, in
         if (MODE == kStencilResidual) {
           if (a.out_res) store_vec<T>(a.out_res + rowoff + k0, res);
           if (a.out32) {
-            float r32[4];
-#pragma unroll
-            for (int e = 0; e < V; ++e) r32[e] = (float)res[e];
-            if (V == 4) {
-              *reinterpret_cast<float4 *>(a.out32 + rowoff + k0) = make_float4(r32[0], r32[1], r32[2], r32[3]);
-            } else {
-              *reinterpret_cast<float2 *>(a.out32 + rowoff + k0) = make_float2(r32[0], r32[1]);
-            }
+            *reinterpret_cast<float2 *>(a.out32 + rowoff + k0) = make_float2((float)res[0], (float)res[1]);
           }
         } else {
           store_vec<T>(a.out + rowoff + k0, res);
@@ -703,8 +683,9 @@ int column_warps(int nz, int vec) {
 
 // Warps per CTA of the strip kernel, by the grid alone (see there); 0 where its
 // partials, one per CTA, would not fit the array: the 16-row kernel runs.
-// FP64 (vec = 2) runs it too: it is bound by the FP64 pipe, and the strips form
-// p = z + beta p_old twice on their shared rows (500 x 511 x 8: 81 us against 64).
+// FP64 (vec = 2) runs the 16-row kernel always: it is bound by the FP64 pipe, and
+// strips form p = z + beta p_old twice on their shared rows (500 x 511 x 8: 81 us
+// against 64).
 static int strip_warps(int nr, int nz, int vec, int *gx, int *gy) {
   if (vec != 4) return 0;
   *gy = (nz + 32 * vec - 1) / (32 * vec);
@@ -770,7 +751,9 @@ void launch_stencil(int mode, const StencilArgs<T> &a, cudaStream_t s) {
     case kStencilApply: launch_stencil_mode<T, kStencilApply>(a, s); break;
     case kStencilPcg: launch_stencil_mode<T, kStencilPcg>(a, s); break;
     case kStencilPcgP: launch_stencil_mode<T, kStencilPcgP>(a, s); break;
-    case kStencilResidual: launch_stencil_mode<T, kStencilResidual>(a, s); break;
+    case kStencilResidual:  // FP64 only (the mixed PCG's is launch_residual_df)
+      if constexpr (sizeof(T) == 8) launch_stencil_mode<T, kStencilResidual>(a, s);
+      break;
     default: launch_stencil_mode<T, kStencilCheb>(a, s); break;
   }
 }
