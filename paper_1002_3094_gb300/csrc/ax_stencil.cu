@@ -495,6 +495,8 @@ __global__ void __launch_bounds__(256) stencil_kernel(const StencilArgs<T> a, in
       const double s = block_sum_of(acc, red);
       if (threadIdx.x == 0)
         a.partial[(size_t)m * kPartialStride + blockIdx.y * gridDim.z + blockIdx.z] = s;
+    } else {
+      __syncthreads();  // every warp has read the state before this CTA arrives
     }
     const int nb = (int)(gridDim.y * gridDim.z);
     finish_rhs(a.fin, m, (unsigned)nb, a.partial ? a.partial + (size_t)m * kPartialStride : nullptr, nb, red);
