@@ -241,7 +241,8 @@ int ax_chebyshev_bounds(const ax_operator *op, int32_t m, double *gamma1, double
  *                    stops its copies before the first stage, one of its bounded
  *                    waits (short limit) runs out, the kernel sets the device's
  *                    error flag, frees its tensor memory and returns; the call
- *                    returns AX_ERR_TIMEOUT and the context stays usable
+ *                    returns AX_ERR_TIMEOUT (a single FP64 step: NaN rows) and the
+ *                    context stays usable
  * Unknown names or out-of-range values: AX_ERR_INVALID_ARG. */
 int ax_set_option(ax_operator *op, const char *name, double value);
 
@@ -365,7 +366,12 @@ int ax_solve_learned(ax_operator *op, void *net, const double *kappa, const doub
 /* ---- single steps of the hot path, for testing each kernel -----------------
  * All take FP64 device arrays [m][nr][nz]; precision selects the kernel
  * (AX_PREC_FP64 or AX_PREC_FP32 — the FP32 kernels round the input to FP32
- * first and widen the output).  in and out must not overlap. */
+ * first and widen the output).  in and out must not overlap.
+ * The FP64 transforms of 128 to 1024 columns and enough rows run as integer
+ * products on the tensor cores, with bounded waits.  The FP64 calls do not wait for the GPU (and
+ * may be captured into a CUDA graph once their staging exists), so a wait that
+ * expires there shows as NaN in the rows concerned and not in the status; the
+ * tensor-core FP32 calls and the solves return AX_ERR_TIMEOUT. */
 
 /* out = A in (the 5-point stencil of Eqs. poisson_diff_2, scheme_op_r_z). */
 int ax_apply_operator(ax_operator *op, const double *in, double *out, int32_t m,

@@ -137,7 +137,7 @@ __device__ __forceinline__ int digit_byte(int row, int k) {
   return (row >> 3) * (kDK * 16) + (k >> 3) * 128 + (row & 7) * 16 + (k & 7) * 2;
 }
 
-// X (|X| <= 2^56) as 8 digits, most significant first: [-64, 63], the first
+// X (|X| <= 2^57) as 8 digits, most significant first: [-64, 63], the first
 // [-256, 256].  With 64 added at each digit but the first, the digits are plain bit
 // fields; a field becomes a float by the bits of 2^23 + field (FP32 and integer
 // operations: the conversion instructions have an eighth of their rate).

@@ -432,9 +432,11 @@ struct DigitArgs {
 // The sums stay exact up to 512 positions per half, and one right-hand side's
 // partials fit their array up to 65536 rows.  From 128 columns on: below that the FFT
 // is short.  A transform of few rows takes its MMAs' time whatever their number, the
-// FFT its own (it is short for 255, 511, 1023): 48 rows of 128, 255, 511, 1023, 1024
+// FFT its own, by the factors of its length: 48 rows of 128, 255, 511, 1023, 1024
 // take 21, 25, 35, 57, 59 us (FFT 69, 41, 42, 46, 76), 1024 rows 23, 29, 38, 66, 66
-// (70, 42, 64, 123, 236).  Above 512 columns the lines cross between 128 and 512 rows.
+// (70, 42, 64, 123, 236).  Above 512 columns the lines cross between 128 and 512 rows
+// for 1023 (length 2^10) and below 48 for 1024 (5^2 41): one line for all, drawn where
+// no length loses.
 constexpr int kDigitMinN = 128, kDigitMaxN = 1024, kDigitMinRows = 48, kDigitMinRowsLong = 384, kDigitMaxRows = 65536;
 bool digits_apply(int rows, int n);
 int digit_mtiles(int rows);

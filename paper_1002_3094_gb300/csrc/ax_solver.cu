@@ -9,16 +9,18 @@
 // GPU organisation.  Scalars (alpha, beta, rho, norms) live on the device in
 // one RhsState per right-hand side and are produced by the last CTA of the
 // kernel that forms the sum, which reduces the per-CTA FP64 partial sums in a
-// fixed order (ax_finish.cuh; deterministic).  Every iteration kernel reads its RHS's state and returns at once
-// unless the state matches the kernel's mask, so converged right-hand sides
-// stop costing bandwidth while the others continue.  A block of iterations is
-// captured once into a CUDA graph and replayed; the host reads the states
-// between replays.
+// fixed order (ax_finish.cuh; deterministic).  Every iteration kernel reads its
+// RHS's state and returns at once unless the state matches the kernel's mask, so
+// converged right-hand sides stop costing bandwidth while the others continue.  A
+// block of iterations is launched directly the first two times, then captured into
+// a CUDA graph and replayed; the host reads the states between blocks.
 //
-// Mixed precision (AX_PCG_MIXED / AX_CHEB_MIXED): iterative refinement.  The
-// outer loop forms the true residual r = phi - A x in FP64 (FP64 stencil,
-// FP64 coefficients), the inner loop solves A d = r in FP32 to a relative
-// tolerance eta_in (or a fixed number of steps), and x += d in FP64.
+// Mixed precision.  AX_PCG_MIXED: FP32 PCG whose residual is replaced, now and then,
+// by the true residual phi - A x of a double-float iterate (pcg_mixed_solve).
+// AX_CHEB_MIXED, and AX_PCG_MIXED with option "mixed_restart": iterative refinement.
+// The outer loop forms r = phi - A x in FP64 (FP64 stencil and coefficients), the
+// inner loop solves A d = r in FP32 to a relative tolerance eta_in (or a fixed number
+// of steps), and x += d in FP64.
 #include <cmath>
 #include <cstdio>
 #include <cstdlib>
@@ -422,10 +424,9 @@ __global__ void padded_to_dense(const T *__restrict__ src, double *__restrict__ 
     for (int k = threadIdx.x; k < nz; k += blockDim.x) dst[row * nz + k] = (double)src[row * pitch + k];
 }
 
-// Mixed methods: sigma_m = 2^-round(log2(rms(phi_m))) (1 for phi_m = 0), from
-// the ||phi||^2 partials, so that the FP32 inner iteration works on values of
-// order one whatever the units of f (FP32 squares of residuals near 1e-20
-// would underflow).  A power of two scales FP64 values exactly.
+// Mixed methods: each right-hand side is scaled by a power of two (exact in FP64), so
+// that the FP32 inner iteration works on values of order one whatever the units of f
+// (FP32 squares of residuals near 1e-20 would underflow).
 // sigma = 2^-e with max |phi| = f 2^e, 1/2 <= f < 1 (frexp): the scaled
 // right-hand side has its largest magnitude in [1/2, 1) for any finite
 // nonzero phi of FP64 (no square is formed, so nothing overflows or
