@@ -662,21 +662,28 @@ __global__ void __launch_bounds__(256) mixed_prep(const double *__restrict__ f, 
     const unsigned ex = (unsigned)__double2hiint(rs) >> 20;
     const bool exact = sc.one && ex >= 1 && ex <= 2046;
     const size_t src = ((size_t)m * nr + i) * nz, dst = ((size_t)m * nr + i) * pitch;
+    auto row = [&](auto phi, auto guess) {
 #pragma unroll 4
-    for (int k = threadIdx.x; k < nz; k += 256) {
-      const double v = exact ? rs * f[src + k] : ri * (f[src + k] * sc.a) * sc.b;
-      float h, l;
-      split_df(v, h, l);
-      ph[dst + k] = h;
-      pl[dst + k] = l;
-      if (r32 != nullptr) r32[dst + k] = h;
-      acc = fma(v, v, acc);
-      if (u != nullptr) {
-        split_df(times(u[src + k], sc), h, l);
-        xh[dst + k] = h;
-        xl[dst + k] = l;
+      for (int k = threadIdx.x; k < nz; k += 256) {
+        const double v = phi(f[src + k]);
+        float h, l;
+        split_df(v, h, l);
+        ph[dst + k] = h;
+        pl[dst + k] = l;
+        if (r32 != nullptr) r32[dst + k] = h;
+        acc = fma(v, v, acc);
+        if (u != nullptr) {
+          split_df(guess(u[src + k]), h, l);
+          xh[dst + k] = h;
+          xl[dst + k] = l;
+        }
       }
-    }
+    };
+    // two loops, so that the ordinary one issues no FP64 operation of the other
+    if (exact)
+      row([&](double x) { return rs * x; }, [&](double x) { return x * sc.a; });
+    else
+      row([&](double x) { return ri * (x * sc.a) * sc.b; }, [&](double x) { return x * sc.a * sc.b; });
   }
   const double s = block_sum(acc, red);
   if (threadIdx.x == 0) part[(size_t)m * kPartialStride + blockIdx.y] = s;
@@ -698,14 +705,13 @@ __global__ void __launch_bounds__(256) mixed_result(const float *__restrict__ xh
   const float *xh = (nrep & 1) ? xh1 : xh0, *xl = (nrep & 1) ? xl1 : xl0;
   const int e = rexp[m];  // 1 / sigma = 2^e
   // v 2^e by its exponent bits; false: neither a normal number nor 0
+  const int off = 1023 - 127 + e, low = max(1, 1 - off), span = min(254, 2046 - off) - low;
   auto widen = [&](float v, double &o) -> bool {
     const unsigned b = __float_as_uint(v);
-    const int ex = (int)((b >> 23) & 0xFF), en = ex - 127 + e;
-    o = __longlong_as_double((long long)(((unsigned long long)(b >> 31) << 63) |
-                                         ((unsigned long long)(unsigned)(en + 1023) << 52) |
-                                         ((unsigned long long)(b & 0x7FFFFFu) << 29)));
-    if ((b << 1) == 0) o = 0.0;
-    return (b << 1) == 0 || (ex != 0 && ex != 255 && en >= -1022 && en <= 1023);
+    const bool zero = (b << 1) == 0;
+    const int hi = (int)((((b >> 3) & 0x0FFFFFFFu) + ((unsigned)off << 20)) | (b & 0x80000000u));
+    o = zero ? 0.0 : __hiloint2double(hi, (int)(b << 29));
+    return zero || (span >= 0 && ((b >> 23) & 255u) - (unsigned)low <= (unsigned)span);
   };
   auto value = [&](float h, float l) -> double {
     double a, b;
