@@ -1249,52 +1249,59 @@ __global__ void __launch_bounds__(256) setup_fields(const SetupArgs a) {
 // relative accuracy where differences of the diagonals lost it to rounding (the mode
 // solves' error at 1024 rows, 2-norm: 5e-13 to 3e-12 before, some 1e-15 now).  IP = 1 /
 // delta; IPS = IP / RS^2 the inverse pivots of the row-scaled systems D T D, and
-// IPST the same mode-major, through a 32 x 32 shared tile.  One warp per CTA.
-__global__ void __launch_bounds__(32) setup_factors(const SetupArgs a) {
-  __shared__ float tile[32][33];
-  const int lane = threadIdx.x, l = blockIdx.x * 32 + lane, nr = a.nr;
-  const bool ok = l < a.nz;
+// IPST the same mode-major.  Every FP64 operation of a warp holds its quarter of the SM
+// for 64 cycles, so warp 0 takes the three operations and the division of each row
+// alone; warps 1 to 3 form the products r_a shift of the next 32 rows and convert and
+// store the 32 before, through shared tiles (all in one warp: 122 us at 256 rows, now
+// 88; set-up of 1024 x 1024 0.74 and 0.59 ms, 0.69 with the differences).
+__global__ void __launch_bounds__(128) setup_factors(const SetupArgs a) {
+  __shared__ double rs[2][32][32], ipt[2][32][33];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, l0 = blockIdx.x * 32, l = l0 + lane, nr = a.nr;
   const double *R = a.stage + nr, *G = a.stage + 3 * nr, *I2 = a.stage + 4 * nr;
   // mode eigenvalue of the z second difference: sine modes l + 1 = 1..nz, or the
   // cosine modes of Eq. eq_trid, 4/h^2 sin^2(pi l / (2 nz)) (0 for l = 0)
   const double sn = a.cosine ? sinpi(l / (2.0 * a.nz)) : sinpi((l + 1) / (2.0 * (a.nz + 1)));
   const double shift = a.kt * (4.0 / (a.hz * a.hz) * sn * sn) + a.qt;
-  double ip = 0.0, gs = 0.0;  // 1 / delta and g s of the row before
-  // the rows' constants, a row per lane and 32 rows ahead, so that no load stands in
-  // the chain (500 rows: 295 -> 208 us)
-  double rn, gn, i2n;
-  auto fetch = [&](int i) {
-    const bool in = i < nr;
-    rn = in ? R[i] : 0.0;
-    gn = in ? G[i] : 0.0;
-    i2n = in ? I2[i] : 0.0;
+  const int tiles = (nr + 31) / 32;
+  auto products = [&](int t) {
+    for (int j = warp - 1; j < 32; j += 3) rs[t & 1][j][lane] = t * 32 + j < nr ? R[t * 32 + j] * shift : 0.0;
   };
-  fetch(lane);
-  for (int a0 = 0; a0 < nr; a0 += 32) {
-    const int cnt = min(32, nr - a0);
-    const double r = rn, g = gn, i2 = i2n;
-    fetch(a0 + 32 + lane);
+  auto store = [&](int t) {
+    const double(*ip)[33] = ipt[t & 1];
+    for (int j = warp - 1; j < 32; j += 3) {
+      const int i = t * 32 + j;
+      if (i < nr) {  // row i, a column per lane
+        const double v = l < a.nz ? ip[j][lane] : 0.0;
+        const size_t o = (size_t)i * a.pitch + l;
+        a.c64.IP[o] = v;
+        a.c32.IP[o] = (float)v;
+        a.c32.IPS[o] = (float)(v * I2[i]);
+      }
+      if (l0 + j < a.nz)  // column l0 + j, a row per lane
+        a.c32.IPST[(size_t)(l0 + j) * a.tpitch + t * 32 + lane] =
+            t * 32 + lane < nr ? (float)(ip[lane][j] * I2[t * 32 + lane]) : 0.f;
+    }
+  };
+  if (warp != 0) products(0);
+  __syncthreads();
+  double ip = 0.0, gs = 0.0, gn = lane < nr ? G[lane] : 0.0;  // 1 / delta and g s of the row before
+  for (int t = 0; t <= tiles; ++t) {
+    if (warp != 0) {
+      if (t + 1 < tiles) products(t + 1);
+      if (t > 0) store(t - 1);
+    } else if (t < tiles) {
+      const int cnt = min(32, nr - t * 32), next = (t + 1) * 32 + lane;
+      const double g = gn;
+      gn = next < nr ? G[next] : 0.0;  // a row per lane, 32 rows ahead of the chain
 #pragma unroll 4
-    for (int j = 0; j < cnt; ++j) {
-      const int i = a0 + j;
-      const double ga = __shfl_sync(0xffffffffu, g, j), di = __shfl_sync(0xffffffffu, i2, j);
-      const double ex = fma(gs, ip, __shfl_sync(0xffffffffu, r, j) * shift);
-      ip = 1.0 / (ga + ex);
-      gs = ga * ex;
-      const size_t o = (size_t)i * a.pitch + l;
-      const float ips = ok ? (float)(ip * di) : 0.f;
-      a.c64.IP[o] = ok ? ip : 0.0;
-      a.c32.IP[o] = ok ? (float)ip : 0.f;
-      a.c32.IPS[o] = ips;
-      tile[j][lane] = ips;
+      for (int j = 0; j < cnt; ++j) {
+        const double ga = __shfl_sync(0xffffffffu, g, j), ex = fma(gs, ip, rs[t & 1][j][lane]);
+        ip = 1.0 / (ga + ex);
+        gs = ga * ex;
+        ipt[t & 1][j][lane] = ip;
+      }
     }
-    for (int j = cnt; j < 32; ++j) tile[j][lane] = 0.f;
-    __syncwarp();
-    for (int j = 0; j < 32; ++j) {
-      const int col = blockIdx.x * 32 + j;
-      if (col < a.nz) a.c32.IPST[(size_t)col * a.tpitch + a0 + lane] = tile[lane][j];
-    }
-    __syncwarp();
+    __syncthreads();
   }
 }
 
@@ -3197,7 +3204,7 @@ int ax_setup_operator(const double *kappa_r, const double *kappa_z, const double
     note_launch();
     setup_fields<<<(unsigned)std::min(nr, 8192), 256, 0, s>>>(a);
     note_launch();
-    setup_factors<<<(nz + 31) / 32, 32, 0, s>>>(a);
+    setup_factors<<<(nz + 31) / 32, 128, 0, s>>>(a);
     e = cudaGetLastError();
   }
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
