@@ -513,23 +513,23 @@ __device__ __forceinline__ void add_groups(Sum3 (*s)[N], int q, int groups) {
   }
 }
 
-// out[i] = sum over the slots of partial[slot][i], a warp per element in a fixed order,
-// rounded to FP32 once.  (The sums of gradients cancel: rounded to FP32 per block, 912
-// of them, they were some 100 times as far off as the plane sums in FP64 before.)
+// out[i] = sum over the slots of partial[slot][i], rounded to FP32 once.  (The sums of
+// gradients cancel: rounded to FP32 per block, 912 of them, they were some 100 times as
+// far off as the plane sums in FP64 before.)  256 threads: 8 elements x 32 groups of
+// slots, added in a fixed order.
 __global__ void __launch_bounds__(256) sum_sum3(const Sum3 *__restrict__ partial, int slots, int n,
                                                 float *__restrict__ out) {
-  const int i = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-  if (i >= n) return;
+  __shared__ Sum3 red[256][1];
+  const int i = blockIdx.x * 8 + (threadIdx.x & 7);
   Sum3 s;
-#pragma unroll 4
-  for (int k = lane; k < slots; k += 32) s.add(partial[(size_t)k * n + i]);
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const Sum3 t{__shfl_xor_sync(0xffffffffu, s.h, o), __shfl_xor_sync(0xffffffffu, s.m, o),
-                 __shfl_xor_sync(0xffffffffu, s.l, o)};
-    s.add(t);
+  if (i < n) {
+#pragma unroll 8
+    for (int k = threadIdx.x >> 3; k < slots; k += 32) s.add(partial[(size_t)k * n + i]);
   }
-  if (lane == 0) out[i] = s.value();
+  red[threadIdx.x][0] = s;
+  __syncthreads();
+  add_groups(red, 8, 32);
+  if (threadIdx.x < 8 && i < n) out[i] = red[threadIdx.x][0].value();
 }
 
 // Per-block sums of gz over pixels, per channel: partial[block][c].  blockDim = 256:
