@@ -422,10 +422,10 @@ def _reference_laguerre(args):
 
 def arm_config(args, nr: int, nz: int, m: int, world: int) -> dict:
     """The config of a single-operator workload's line (the same on both arms)."""
-    # working set of the mixed solve: f and u (FP64), the double-float x and
-    # phi, six FP32 vectors and the split operand, about 64 B per unknown
+    # working set of the mixed solve: f and u (FP64), the double-float x (two
+    # buffers) and phi, six FP32 vectors and two split operands, 72 B per unknown
     unknowns = nr * nz * m
-    ws_mb = (unknowns * 64) >> 20
+    ws_mb = (unknowns * 72) >> 20
     l2_note = ("inputs larger than L2 (f is %d MB, solver working set ~%d MB)" % ((unknowns * 8) >> 20, ws_mb)
                if ws_mb > 129 else
                "working set ~%d MB fits in L2, no flush between steps (a solve this small is launch-bound)"
