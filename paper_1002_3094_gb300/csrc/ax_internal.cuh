@@ -261,6 +261,7 @@ struct DfResidualArgs {
   Finish fin;
 };
 void launch_residual_df(const DfResidualArgs &a, cudaStream_t s);
+int residual_df_blocks(int nr, int nz);  // CTAs (and partial sums) per right-hand side
 
 // Persistent FP64 PCG of one right-hand side on a small grid (ax_small.cu):
 // the whole iteration in one cooperative launch, phases separated by bounded

@@ -66,8 +66,10 @@ struct Workspace {
   float *x32 = nullptr, *r32 = nullptr, *pa32 = nullptr, *pb32 = nullptr, *q32 = nullptr, *z32 = nullptr,
         *y32prev = nullptr;
   unsigned char *base = nullptr;  // one allocation: part .. chk below
-  // partial sums [4][m][kPartialStride]
+  // partial sums of four kinds, rows of kPartialStride per right-hand side; two kinds
+  // share a row where half of one holds every kernel's (part_half, see part_ptr)
   double *part = nullptr;
+  bool part_half = false;
   double *chp = nullptr;      // Chebyshev (tau, rho0^2) per right-hand side [m][2]
   int *rexp = nullptr;        // mixed methods: exponent of the power-of-two scale of phi and x per right-hand side [m]
   RhsState *st = nullptr, *st_outer = nullptr;
@@ -239,10 +241,13 @@ int ensure_base(ax_operator *op, int m) {
   if (w->mbase >= m) return AX_OK;
   free_base(w);
   // one zeroed allocation (each costs tens of microseconds, as does its release)
-  const size_t mm = (size_t)m, nd = 4 * mm * kPartialStride + 2 * mm + 2;
+  // (only the FP32 stencil's and the double-float residual's can be more than half a row)
+  w->part_half = std::max(stencil_blocks_per_rhs(op->nr, op->nz, 4), residual_df_blocks(op->nr, op->nz)) <=
+                 kPartialStride / 2;
+  const size_t mm = (size_t)m, np = (w->part_half ? 2 : 4) * mm * kPartialStride, nd = np + 2 * mm + 2;
   AX_TRY(dalloc(&w->base, nd * sizeof(double) + 2 * mm * sizeof(RhsState) + (2 * mm + 1) * sizeof(unsigned)));
   w->part = reinterpret_cast<double *>(w->base);
-  w->chp = w->part + 4 * mm * kPartialStride;
+  w->chp = w->part + np;
   w->par = w->chp + 2 * mm;
   w->st = reinterpret_cast<RhsState *>(w->part + nd);
   w->st_outer = w->st + mm;
@@ -404,7 +409,11 @@ void prof_collect(Workspace *w) {
   w->prof_events.clear();
 }
 
-double *part_ptr(Workspace *w, int kind) { return w->part + (size_t)kind * w->mbase * kPartialStride; }
+double *part_ptr(Workspace *w, int kind) {
+  const size_t block = (size_t)w->mbase * kPartialStride;
+  return w->part_half ? w->part + (size_t)(kind >> 1) * block + (kind & 1) * (kPartialStride / 2)
+                      : w->part + (size_t)kind * block;
+}
 enum { kPartA = 0, kPartB = 1, kPartC = 2, kPartD = 3 };
 
 // ---------------------------------------------------------------------------
@@ -3481,7 +3490,7 @@ int ax_solve(ax_operator *op, const double *f, double *u, int32_t m, double tol,
   if (!op || !f || !u || m < 1) return AX_ERR_INVALID_ARG;
   if (!(tol > 0.0) || !std::isfinite(tol) || max_iter < 1) return AX_ERR_INVALID_ARG;
   if (method < AX_PCG_FP64 || method > AX_CHEB_MIXED) return AX_ERR_INVALID_ARG;
-  if ((size_t)m * kPartialStride * 4 > ((size_t)1 << 40)) return AX_ERR_INVALID_ARG;
+  if ((size_t)m * kPartialStride * 2 > ((size_t)1 << 40)) return AX_ERR_INVALID_ARG;
   cudaStream_t s = (cudaStream_t)stream;
   Workspace *w = op->ws;
   if ((flags & AX_FLAG_HOST_BUFFERS) && w->host_chunks > 1 && m >= 2 * w->host_chunks)

@@ -772,6 +772,12 @@ static int df_warps(int nr, int nz, int *gx, int *gy) {
   }
 }
 
+int residual_df_blocks(int nr, int nz) {
+  int gx, gy;
+  df_warps(nr, nz, &gx, &gy);
+  return gx * gy;
+}
+
 template <bool FOLD>
 static void launch_df(const DfResidualArgs &a, cudaStream_t s) {
   int gx, gy;
